@@ -1,10 +1,10 @@
 // Tensor-core kernels of the generic decayed linear-attention operator for
 // bf16 inputs with Da = Ec = D, D = 128 or 64 (block formulas: la_common.cuh).  Two kernels share this file's
 // launchers: the half-width kernel below (every D = 64 launch, the state-only pre-pass at both head sizes, and the
-// D = 128 walk when an output is aligned to 16 but not 32 bytes) and the full-width walk of la_tc_full.cuh
-// (D = 128: one thread block per (batch*head, segment) with all four 128x128 accumulators in tensor memory),
-// which launch_walk_d prefers.  The text below describes the half-width kernel at D = 128; the differences at
-// D = 64 are described at the kernel's template parameter.
+// D = 128 walk when an output is aligned to 16 but not 32 bytes), the walk of la_tc_walk.cuh (D = 128: one thread block
+// per (batch*head, segment), all value columns, operands formed on chip in tensor memory), which launch_walk_d prefers,
+// and la_tc_full.cuh, the D = 128 walk with the gate in its epilogue.  The text below describes the half-width kernel at
+// D = 128; the differences at D = 64 are described at the kernel's template parameter.
 //
 // One thread block walks the 128-token blocks of one (batch*head, segment,
 // half of the value columns).  Per block it issues, on the 5th-generation
@@ -59,6 +59,8 @@
 // The value-like tile c and the state operand are MN-major B operands, b is used
 // K-major in M1 and MN-major (as b^T) in M3 from the same bytes.
 #include <cuda.h>
+
+#include <cstddef>
 
 #include "la_common.cuh"
 #include "sm100_ptx.cuh"
@@ -196,26 +198,28 @@ __device__ __forceinline__ void split8(const float (&x)[8], uint4& hi, uint4& lo
   lo = make_uint4(lw[0], lw[1], lw[2], lw[3]);
 }
 
-#define TC_WAIT(barid, par, code)                                        \
+#define TC_WAIT_TO(label, barid, par, code)                              \
   do {                                                                   \
     if (!wait_or_abort(&sm.bars[barid], (par), &sm.abort)) {             \
       if (!sm.abort) atomicCAS(&g_tc_status, 0u, (unsigned)(code));      \
       sm.abort = 1;                                                      \
-      goto teardown;                                                     \
+      goto label;                                                        \
     }                                                                    \
   } while (0)
+#define TC_WAIT(barid, par, code) TC_WAIT_TO(teardown, barid, par, code)
 
 // The same for a whole warp waiting together: the outcome is made warp-uniform so that the
 // warp-level synchronisation of the elected arrivals below can never be entered by a part of a warp.
-#define TC_WAIT_WARP(barid, par, code)                                                    \
+#define TC_WAIT_WARP_TO(label, barid, par, code)                                          \
   do {                                                                                    \
     const bool ok_ = wait_or_abort(&sm.bars[barid], (par), &sm.abort);                    \
     if (!__all_sync(0xffffffffu, ok_)) {                                                  \
       if (!ok_ && !sm.abort) atomicCAS(&g_tc_status, 0u, (unsigned)(code));               \
       sm.abort = 1;                                                                       \
-      goto teardown;                                                                      \
+      goto label;                                                                         \
     }                                                                                     \
   } while (0)
+#define TC_WAIT_WARP(barid, par, code) TC_WAIT_WARP_TO(teardown, barid, par, code)
 
 // One arrival per warp: every lane has fenced its own writes, the warp synchronises, lane 0
 // arrives.  (A barrier that 256 threads arrive on costs 256 serialised shared-memory atomics per
@@ -839,6 +843,7 @@ __global__ void bounded_wait_selftest_kernel(long long budget) {
 }
 
 #include "la_tc_full.cuh"
+#include "la_tc_walk.cuh"
 
 // ---------------------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -927,16 +932,11 @@ cudaError_t launch_walk_d(const OpArgs& args, const OpArgs* second, const DecayT
       !(second && (reinterpret_cast<uintptr_t>(second->out) & 31u))) {
     // full-width kernel: one thread block per (head, segment).  Its 32-byte output stores need that alignment;
     // an output that is only 16-byte aligned (the contract's minimum) takes the half-width kernels below.
-    if (second) {
-      if (!args.reverse) return cudaErrorInvalidValue;
-      return f32 ? launch_full_t<true, float, 2, false>(m0, m1, ta, tab, stream)
-                 : launch_full_t<true, __nv_bfloat16, 2, false>(m0, m1, ta, tab, stream);
-    }
     if (args.reverse)
-      return f32 ? launch_full_t<true, float, 1, false>(m0, m1, ta, tab, stream)
-                 : launch_full_t<true, __nv_bfloat16, 1, false>(m0, m1, ta, tab, stream);
-    return f32 ? launch_full_t<false, float, 1, false>(m0, m1, ta, tab, stream)
-               : launch_full_t<false, __nv_bfloat16, 1, false>(m0, m1, ta, tab, stream);
+      return f32 ? launch_walk_t<true, float>(m0, m1, ta, tab, stream)
+                 : launch_walk_t<true, __nv_bfloat16>(m0, m1, ta, tab, stream);
+    return f32 ? launch_walk_t<false, float>(m0, m1, ta, tab, stream)
+               : launch_walk_t<false, __nv_bfloat16>(m0, m1, ta, tab, stream);
   }
   if (second) {  // only the reverse direction is ever paired
     if (!args.reverse) return cudaErrorInvalidValue;

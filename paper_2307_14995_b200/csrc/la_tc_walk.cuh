@@ -1,0 +1,513 @@
+// Block walk for D = 128 (included by la_tc.cu, inside its anonymous namespace, after the helpers).
+//
+// One thread block walks the 128-token blocks of one (batch*head, segment) and produces all 128 value columns.  The
+// products whose one operand is formed on chip from fp32 values are turned so that this operand is the A operand and
+// lives in tensor memory (e: value columns, d: features, i, j: tokens of the block):
+//   M1  S    [i, j] = a b^T                               A, B in shared memory
+//   M2  O    [e, i] = Z^T a^T      Z^T  hi (+ lo)         A in tensor memory, lane e
+//   M3  dZ^T [e, d] = fc^T b       fc^T hi (+ lo)         A in tensor memory, lane e     (fc = diag(f_state) c)
+//   M4  O    [e, i] += c^T P^T     P    hi (+ lo)         A = c, B = P in shared memory; P is triangular, so K step k
+//                                                         only runs over the columns i it reaches (N = 128 - 16 k)
+// and O is scaled by diag(f_out) on the CUDA cores between M2 and M4.
+// Why: a shared-memory operand pair of an M = N = 128, K = 16 instruction is 8 KB, at the 128 bytes a clock of the
+// shared-memory pipe exactly the 64 clocks the instruction takes, and products win over loads: beside back-to-back
+// products of that kind a dependent 4-byte load takes 130 clocks with one warp loading and 480 with sixteen (41 and 44
+// without them, 64 beside products with A in tensor memory).  With [token, e] accumulators a block's products fetched
+// 384 KB and the CUDA cores moved 400 KB more through the same pipe (state and fc operand tiles, the output's
+// transposition); here the products fetch 290 KB, state and fc go to tensor memory, and since an accumulator lane is a
+// value column, a warp's plain store instruction writes 128 contiguous bytes of one token, so that the output needs no
+// transposition.
+//
+// Measured on B200 against the walk it replaces (la_tc_full.cuh without its gate): 7B-like shape, fp32 results, one walk
+// 0.654 -> 0.595 ms, the dV and dK walks in one launch 1.358 -> 1.166 ms; 3 x 8 heads x 3001 tokens, bf16 results, token-major,
+// one walk 75 -> 57 us, the pair 81 -> 60 us.
+//
+// Tensor memory (512 columns): R 128 (S, then dZ^T, in turn), O 128, fc^T hi/lo 2 x 64, Z^T hi/lo 2 x 64.
+// Shared memory: a, b twice, c twice, P hi/lo (32 KB each).
+// Order of the products per block n:  M2(n) M3(n) M4(n) M1(n+1).  They use O, R, O, R in turn, and what the CUDA cores
+// do with one region happens while the next product runs in the other: P reads S(n) during M2(n), O is scaled during
+// M3(n), dZ(n) is read during M4(n), O(n) is stored during M1(n+1).  Shared memory is read by the CUDA cores during M2
+// and M3 only (A in tensor memory); the F group therefore fetches c of the next block into registers during M3.
+//
+// Warp roles (32 warps): 0 TMA producer, 1 MMA issuer (all lanes converged, instructions on one elected lane), 4-11 P
+// group (two warps per 32 score rows), 12-19 O group (two warps per 32 value columns, 64 tokens each), 20-27 Z group
+// (fp32 state in registers: two warps per 32 value columns, 64 features each), 28-31 F group (fc).  Registers per thread
+// after start-up: W_REGS_*; they add up to the 2048 warp-registers of the launch.
+
+constexpr int W_THREADS = 1024;
+constexpr uint32_t WCOL_R = 0, WCOL_O = 128, WCOL_FH = 256, WCOL_FL = 320, WCOL_ZH = 384, WCOL_ZL = 448;
+constexpr int W_REGS_CTL = 32, W_REGS_P = 48, W_REGS_O = 40, W_REGS_Z = 104, W_REGS_F = 96;
+static_assert(4 * W_REGS_CTL + 8 * W_REGS_P + 8 * W_REGS_O + 8 * W_REGS_Z + 4 * W_REGS_F <= 2048, "registers of the launch");
+
+enum WBar {
+  W_FULL_C0 = 0, W_FULL_C1,  // TMA -> F group, MMA: c of an even / odd block
+  W_M1_OK0, W_M1_OK1,        // a and b landed (two arrivals with bytes) and the previous dZ read (8 warps)
+  W_M2_OK,                   // state operand written (8 warps) and the previous O read (8 warps)
+  W_M3_OK,                   // fc written (4 warps) and S read (8 warps)
+  W_M4_OK,                   // P written (8 warps) and O scaled (8 warps)
+  W_S_READY,                 // M1 done
+  W_M2_DONE,                 // M2 done: O_inter complete, a and the state operand free
+  W_DZ_READY,                // M3 done: dZ complete, b and fc free
+  W_O_READY,                 // M4 done: O complete, c and P free
+  W_DRAIN,
+  W_NUM_BARS
+};
+
+template <bool REV>
+struct alignas(1024) WSmem {
+  __nv_bfloat16 a[2][128 * 64];     // query-like tile, K-major, two 64-feature panels
+  __nv_bfloat16 b[2][2][128 * 64];  // key-like tile, two buffers (K-major in M1, MN-major in M3)
+  __nv_bfloat16 c[2][2][128 * 64];  // value-like tile, two buffers, MN-major: two 64-column chunks
+  __nv_bfloat16 p_hi[2][128 * 64];  // scores, K-major: two panels of 64 keys
+  __nv_bfloat16 p_lo[2][128 * 64];
+  // Factor of a token's O_inter.  REV: index 1 is for the edge block (the first one walked, which may be shorter than 128
+  // tokens), index 0 for every other.
+  float fout[REV ? 2 : 1][128];
+  float ptab[32];  // lambda^(31 - x)
+  uint64_t bars[W_NUM_BARS];
+  uint32_t tmem_slot;
+  int abort;
+};
+
+// args.njobs == 2: two walks of the same direction over the same tokens in one launch (the dV and dK walks of the
+// backward pass, which between them read Q, K, V and dO); the thread blocks of the two jobs alternate, so that the two
+// readers of a tile run side by side and the tile comes from HBM once.
+template <bool REV, typename TOut>
+__global__ void __launch_bounds__(W_THREADS, 1)
+tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps maps1,
+               const __grid_constant__ TcArgs args, const __grid_constant__ DecayTable tab) {
+  extern __shared__ unsigned char smem_raw[];
+  WSmem<REV>& sm = *reinterpret_cast<WSmem<REV>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int jobid = (args.njobs == 2) ? (int)(blockIdx.x & 1) : 0;
+  const int bidx = (args.njobs == 2) ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+  const TcJob& job = args.job[jobid];
+  const int seg = bidx % args.nseg;
+  int bh = bidx / args.nseg;
+  // packed batch: thread blocks take the sequences longest first, so that a long one is not what the launch ends on
+  if (args.seq_order) bh = args.seq_order[bh / args.H] * args.H + bh % args.H;
+  // Packed batch: "batch" entry bh / H is a sequence of its own length inside one [tokens, H, D] tensor; tok0 is its
+  // first token, and the maps' batch coordinate is 0.  Dense batch: tok0 = 0, every entry has N tokens.
+  const int n_tok = args.seq_len ? args.seq_len[bh / args.H] : args.N;
+  const int tok0 = args.seq_start ? args.seq_start[bh / args.H] : 0;
+  const int nseg_own = (n_tok + args.seg_len - 1) / args.seg_len;
+  if (seg >= nseg_own) return;  // the grid covers the longest sequence; nothing has been set up yet
+  const int seg_t0 = seg * args.seg_len;
+  const int seg_t1 = min(n_tok, seg_t0 + args.seg_len);
+  const int nblk = (seg_t1 - seg_t0 + 127) >> 7;
+  const int edge_len = seg_t1 - seg_t0 - (nblk - 1) * 128;  // tokens of the block that holds the segment's last ones
+  const float s2 = (float)tab.s2[bh % args.H];
+  const bool has_entry = job.entry != nullptr;  // without one the first block has no O_inter: M2 is skipped
+  const bool want_final = job.final_out && (REV ? seg == 0 : seg == nseg_own - 1);
+
+  if (tid == 0) {
+    for (int i = 0; i < W_NUM_BARS; ++i) {
+      uint32_t count = 1;
+      if (i == W_M1_OK0 || i == W_M1_OK1) count = 10;
+      if (i == W_M2_OK || i == W_M4_OK) count = 16;
+      if (i == W_M3_OK) count = 12;
+      mbar_init(&sm.bars[i], count);
+    }
+    sm.abort = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(&sm.tmem_slot, TMEM_COLS);
+    tmem_relinquish();
+  }
+  if (warp >= 4 && warp < 12) {
+    const int x = tid - 128, set = x >> 7, i = x & 127;
+    if (REV) {
+      const int Cr = set ? edge_len : 128;
+      sm.fout[REV ? set : 0][i] = i < Cr ? ex2_approx(-s2 * (float)(Cr - 1 - i)) : 0.f;
+    } else if (set == 0) {
+      sm.fout[0][i] = ex2_approx(-s2 * (float)(i + 1));
+    }
+    if (x < 32) sm.ptab[x] = ex2_approx(-s2 * (float)(31 - x));
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = sm.tmem_slot;
+  if (warp < 4) {
+    reg_dec<W_REGS_CTL>();
+    if (warp == 0) {
+      // ------------------------------------ TMA producer ------------------------------------
+      if (lane == 0) {
+        int armed_ab = 0, armed_c = 0;  // blocks whose loads have been started
+        const TcMaps* const maps = jobid ? &maps1 : &maps0;
+        const int hh_ = bh % args.H;  // head coordinate of the 4-D tensor maps
+        const int bb_ = args.seq_start ? 0 : bh / args.H;
+        auto token = [&](int it) { return tok0 + seg_t0 + (REV ? (nblk - 1 - it) : it) * 128; };
+        auto load = [&](int bar_id, __nv_bfloat16* dst, const CUtensorMap* map, int it) {
+          uint64_t* bar = &sm.bars[bar_id];
+          mbar_arrive_expect_tx(bar, 32768);
+          tma_load_4d(dst, map, bar, 0, token(it), hh_, bb_);
+          tma_load_4d(dst + 128 * 64, map, bar, 64, token(it), hh_, bb_);
+        };
+        auto load_a = [&](int it) { load(W_M1_OK0 + (it & 1), &sm.a[0][0], &maps->a, it); };
+        auto load_b = [&](int it) { load(W_M1_OK0 + (it & 1), &sm.b[it & 1][0][0], &maps->b, it); armed_ab = it + 1; };
+        auto load_c = [&](int it) { load(W_FULL_C0 + (it & 1), &sm.c[it & 1][0][0], &maps->c, it); armed_c = it + 1; };
+        load_b(0);
+        load_a(0);
+        load_c(0);
+        if (nblk > 1) {
+          load_b(1);
+          load_c(1);
+        }
+        for (int it = 0; it + 1 < nblk; ++it) {
+          TC_WAIT_TO(producer_done, W_M2_DONE, it & 1, 3);
+          load_a(it + 1);
+          if (it + 2 < nblk) {
+            TC_WAIT_TO(producer_done, W_DZ_READY, it & 1, 5);
+            load_b(it + 2);
+            TC_WAIT_TO(producer_done, W_O_READY, it & 1, 2);
+            load_c(it + 2);
+          }
+        }
+      producer_done:
+        // After an expired wait: nothing may be in flight when the block exits.  (A block that gave up before the Z group's
+        // arrivals leaves the a / b phases incomplete; these waits are bounded like every other.)
+        if (sm.abort) {
+          for (int k = 0; k < 2; ++k) {
+            const int ab = armed_ab - 1 - k, cc = armed_c - 1 - k;
+            if (ab >= 0) drain_wait(&sm.bars[W_M1_OK0 + (ab & 1)], (ab >> 1) & 1);
+            if (cc >= 0) drain_wait(&sm.bars[W_FULL_C0 + (cc & 1)], (cc >> 1) & 1);
+          }
+        }
+      }
+    } else if (warp == 1) {
+      // ------------------------------------ MMA issuer ------------------------------------
+      constexpr uint32_t ID_KK = umma_idesc_bf16(128, 128, false, false);  // K-major or tensor-memory A x K-major B
+      constexpr uint32_t ID_KN = umma_idesc_bf16(128, 128, false, true);   // tensor-memory A x MN-major B
+      constexpr uint32_t HI = UMMA_DESC_HI_SBO1024;
+      const uint32_t go = elect_one();
+      const bool split_p = (args.precision & 1) != 0, split_z = (args.precision & 2) != 0;
+      const bool split_c = (args.precision & 4) != 0 && s2 != 0.f;  // lambda == 1: the lo term is identically zero
+      // Low descriptor halves as one run-time base plus constants (16-byte units): this warp's few registers must hold
+      // everything, since a spilled value comes back through the pipe that the products keep busy.
+      using Sm = WSmem<REV>;
+      const uint32_t base = (smem_u32(&sm) & 0x3FFFFu) >> 4;
+      constexpr uint32_t KMAJ = 1u << 16, MNMAJ = 1024u << 16;  // leading-dimension offset 16 bytes / 16 KB
+      constexpr uint32_t OA = (uint32_t)(offsetof(Sm, a) >> 4) + KMAJ, OB = (uint32_t)(offsetof(Sm, b) >> 4);
+      constexpr uint32_t OC = (uint32_t)(offsetof(Sm, c) >> 4) + MNMAJ;
+      constexpr uint32_t OPH = (uint32_t)(offsetof(Sm, p_hi) >> 4) + KMAJ, OPL = (uint32_t)(offsetof(Sm, p_lo) >> 4) + KMAJ;
+      TC_WAIT_WARP_TO(mma_done, W_M1_OK0, 0, 7);
+      tc_fence_after_sync();
+      umma_group_ss<8, true, true>(tmem + WCOL_R, base + OA, base + OB + KMAJ, HI, ID_KK, 0, go);
+      umma_commit_if(&sm.bars[W_S_READY], go);
+      for (int it = 0; it < nblk; ++it) {
+        const uint32_t par = it & 1;
+        const bool inter = it > 0 || has_entry;
+        const uint32_t buf = base + par * 2048;  // base of this block's b and c buffers
+        TC_WAIT_WARP_TO(mma_done, W_M2_OK, par, 12);
+        tc_fence_after_sync();
+        if (inter) {
+          umma_group_tsd<true>(tmem + WCOL_O, tmem + WCOL_ZH, base + OA, HI, ID_KK, 0, go);
+          if (split_z) umma_group_tsd<true>(tmem + WCOL_O, tmem + WCOL_ZL, base + OA, HI, ID_KK, 1, go);
+        }
+        umma_commit_if(&sm.bars[W_M2_DONE], go);
+        if (it + 1 < nblk || want_final) {  // the state after the segment's last block is often not wanted
+          TC_WAIT_WARP_TO(mma_done, W_M3_OK, par, 13);
+          tc_fence_after_sync();
+          umma_group_tsd<false>(tmem + WCOL_R, tmem + WCOL_FH, buf + OB + MNMAJ, HI, ID_KN, 0, go);
+          if (split_c) umma_group_tsd<false>(tmem + WCOL_R, tmem + WCOL_FL, buf + OB + MNMAJ, HI, ID_KN, 1, go);
+        }
+        umma_commit_if(&sm.bars[W_DZ_READY], go);
+        TC_WAIT_WARP_TO(mma_done, W_FULL_C0 + par, (it >> 1) & 1, 15);
+        TC_WAIT_WARP_TO(mma_done, W_M4_OK, par, 14);
+        tc_fence_after_sync();
+        umma_tri4<REV ? 7 : 0, REV>(tmem + WCOL_O, buf + OC, base + OPH, HI, inter ? 1u : 0u, go);
+        umma_tri4<REV ? 3 : 4, REV>(tmem + WCOL_O, buf + OC, base + OPH, HI, 1, go);
+        if (split_p) {
+          umma_tri4<REV ? 7 : 0, REV>(tmem + WCOL_O, buf + OC, base + OPL, HI, 1, go);
+          umma_tri4<REV ? 3 : 4, REV>(tmem + WCOL_O, buf + OC, base + OPL, HI, 1, go);
+        }
+        umma_commit_if(&sm.bars[W_O_READY], go);
+        if (it + 1 < nblk) {
+          TC_WAIT_WARP_TO(mma_done, W_M1_OK0 + (par ^ 1), ((it + 1) >> 1) & 1, 11);
+          tc_fence_after_sync();
+          umma_group_ss<8, true, true>(tmem + WCOL_R, base + OA, base + (par ^ 1) * 2048 + OB + KMAJ, HI, ID_KK, 0, go);
+          umma_commit_if(&sm.bars[W_S_READY], go);
+        }
+      }
+    mma_done:
+      if (sm.abort) {
+        umma_commit_if(&sm.bars[W_DRAIN], go);
+        drain_wait(&sm.bars[W_DRAIN], 0);
+      }
+    }
+  } else if (warp < 12) {
+    // ------------------------------------ P group ------------------------------------
+    // S -> masked, decayed P as bf16 hi / lo rows in shared memory; the sub-tiles outside the causal band are never read
+    reg_dec<W_REGS_P>();
+    const int q = warp & 3;
+    const int phalf = (warp >= 8) ? 1 : 0;  // warps 4..7 take the 32-key chunks 0 and 3, warps 8..11 chunks 1 and 2
+    const int r = q * 32 + lane;            // score row
+    const uint32_t colS = tmem + ((uint32_t)(q * 32) << 16) + WCOL_R;
+    const bool split_p = (args.precision & 1) != 0;
+    const int c_first = phalf, c_second = phalf ? 2 : 3;
+    const bool use_first = REV ? (c_first >= q) : (c_first <= q), use_second = REV ? (c_second >= q) : (c_second <= q);
+    const int n_chunks = (use_first ? 1 : 0) + (use_second ? 1 : 0);
+    // Reverse walk of a packed batch: the keys past the end of the sequence lie inside the band of the edge block, and
+    // there they are the next sequence's tokens, not the zero fill a dense batch has.
+    const int cut = (REV && args.seq_start) ? edge_len : 128;
+    for (int it = 0; it < nblk; ++it) {
+      TC_WAIT_WARP(W_S_READY, it & 1, 17);
+      tc_fence_after_sync();
+      if (n_chunks == 0) WARP_ARRIVE(W_M3_OK);
+#pragma unroll 1
+      for (int ci = 0; ci < 2 * n_chunks; ++ci) {  // 16 keys at a time
+        const int j0 = ((use_first && ci < 2) ? c_first : c_second) * 32 + (ci & 1) * 16;
+        uint32_t sreg[16];
+        tmem_ld_x16(colS + j0, sreg);
+        const bool edge = REV && it == 0 && cut < 128;
+        const float base = ex2_approx(-s2 * (float)(REV ? j0 - r : r - j0 - 15));
+        tmem_ld_wait();
+        if (ci == 2 * n_chunks - 1) {
+          tc_fence_before_sync();
+          WARP_ARRIVE(W_M3_OK);  // all of S that this warp needs is in registers: M3 may overwrite it
+        }
+        float d[16];
+        if ((j0 >> 5) != q && !edge) {
+          // wholly inside the band: lambda^|i-j| = row factor * table entry (both at most 1), nothing to mask
+#pragma unroll
+          for (int x4 = 0; x4 < 4; ++x4) {
+            const float4 t = *reinterpret_cast<const float4*>(&sm.ptab[REV ? 28 - 4 * x4 : 16 + 4 * x4]);
+            d[4 * x4 + 0] = __uint_as_float(sreg[4 * x4 + 0]) * base * (REV ? t.w : t.x);
+            d[4 * x4 + 1] = __uint_as_float(sreg[4 * x4 + 1]) * base * (REV ? t.z : t.y);
+            d[4 * x4 + 2] = __uint_as_float(sreg[4 * x4 + 2]) * base * (REV ? t.y : t.z);
+            d[4 * x4 + 3] = __uint_as_float(sreg[4 * x4 + 3]) * base * (REV ? t.x : t.w);
+          }
+        } else {
+          const int n0 = REV ? j0 - r : r - j0;
+#pragma unroll
+          for (int x = 0; x < 16; ++x) {
+            const int n = REV ? n0 + x : n0 - x;
+            // a select, not a multiply by zero: masked-out tokens can never leak (n < 0: the power is not used)
+            const float f = ex2_approx(-s2 * (float)n);
+            d[x] = (n >= 0 && !(edge && j0 + x >= cut)) ? __uint_as_float(sreg[x]) * f : 0.f;
+          }
+        }
+        uint32_t h8[8], l8[8];
+        split16(d, h8, l8);
+        unsigned char* const row = reinterpret_cast<unsigned char*>(&sm.p_hi[j0 >> 6][0]) + r * 128;
+        const int u0 = ((((j0 & 63) >> 3)) ^ (r & 7)) << 4, u1 = u0 ^ 16;
+        *reinterpret_cast<uint4*>(row + u0) = make_uint4(h8[0], h8[1], h8[2], h8[3]);
+        *reinterpret_cast<uint4*>(row + u1) = make_uint4(h8[4], h8[5], h8[6], h8[7]);
+        if (split_p) {
+          *reinterpret_cast<uint4*>(row + sizeof(sm.p_hi) + u0) = make_uint4(l8[0], l8[1], l8[2], l8[3]);
+          *reinterpret_cast<uint4*>(row + sizeof(sm.p_hi) + u1) = make_uint4(l8[4], l8[5], l8[6], l8[7]);
+        }
+      }
+      fence_proxy_async_smem();
+      WARP_ARRIVE(W_M4_OK);
+    }
+  } else if (warp < 20) {
+    // ------------------------------------ O group ------------------------------------
+    reg_dec<W_REGS_O>();
+    const int q = warp & 3;
+    const int th = (warp >= 16) ? 64 : 0;  // first of this warp's 64 tokens
+    const uint32_t colO = tmem + ((uint32_t)(q * 32) << 16) + WCOL_O + th;
+    const size_t head_off = (size_t)(args.seq_start ? 0 : bh / args.H) * args.sB + (size_t)(bh % args.H) * args.sH +
+                            (size_t)tok0 * args.sT;
+    TOut* const out = static_cast<TOut*>(job.out) + head_off + q * 32 + lane;
+    WARP_ARRIVE(W_M2_OK);  // there is no earlier O to read
+    for (int it = 0; it < nblk; ++it) {
+      // ---- O <- O diag(f_out), between M2 and M4 ----
+      TC_WAIT_WARP(W_M2_DONE, it & 1, 24);
+      if (it > 0 || has_entry) {
+        const float* const ft = &sm.fout[REV && it == 0 ? 1 : 0][th];
+        tc_fence_after_sync();
+#pragma unroll 1
+        for (int pc = 0; pc < 4; ++pc) {
+          uint32_t w[16];
+          tmem_ld_x16(colO + pc * 16, w);
+          tmem_ld_wait();
+#pragma unroll
+          for (int x4 = 0; x4 < 4; ++x4) {
+            const float4 t = *reinterpret_cast<const float4*>(ft + pc * 16 + 4 * x4);
+            w[4 * x4 + 0] = __float_as_uint(__uint_as_float(w[4 * x4 + 0]) * t.x);
+            w[4 * x4 + 1] = __float_as_uint(__uint_as_float(w[4 * x4 + 1]) * t.y);
+            w[4 * x4 + 2] = __float_as_uint(__uint_as_float(w[4 * x4 + 2]) * t.z);
+            w[4 * x4 + 3] = __float_as_uint(__uint_as_float(w[4 * x4 + 3]) * t.w);
+          }
+          tmem_st_x16(colO + pc * 16, w);
+        }
+        tmem_st_wait();
+        tc_fence_before_sync();
+      }
+      WARP_ARRIVE(W_M4_OK);
+      // ---- store O ----
+      const int t0 = seg_t0 + (REV ? (nblk - 1 - it) : it) * 128 + th;
+      const int rows = seg_t1 - t0;  // tokens of this warp's 64 that exist (may be <= 0)
+      TOut* dst = out + (size_t)t0 * args.sT;
+      TC_WAIT_WARP(W_O_READY, it & 1, 25);
+      tc_fence_after_sync();
+#pragma unroll 1
+      for (int pc = 0; pc < 4; ++pc) {
+        uint32_t w[16];
+        tmem_ld_x16(colO + pc * 16, w);
+        tmem_ld_wait();
+        if (pc == 3) {
+          tc_fence_before_sync();
+          WARP_ARRIVE(W_M2_OK);  // M2 of the next block may overwrite O
+        }
+#pragma unroll
+        for (int x = 0; x < 16; ++x) {
+          if (pc * 16 + x < rows) *dst = from_f32<TOut>(__uint_as_float(w[x]));
+          dst += args.sT;
+        }
+      }
+    }
+  } else if (warp < 28) {
+    // ------------------------------------ Z group ------------------------------------
+    reg_inc<W_REGS_Z>();
+    const int q = warp & 3;
+    const int zhalf = (warp >= 24) ? 1 : 0;  // which 64 of the 128 features this warp owns
+    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
+    const uint32_t colDZ = lane_addr + WCOL_R + zhalf * 64;
+    const uint32_t colZ = lane_addr + WCOL_ZH + zhalf * 32;  // (the lo terms follow 64 columns further)
+    const bool split_z = (args.precision & 2) != 0;
+    float zreg[64];  // Z[zhalf * 64 + x][value column q * 32 + lane]
+    if (has_entry) {
+      const float* src = job.entry + ((size_t)bh * args.nseg + seg) * (128 * 128) + (size_t)(zhalf * 64) * 128 + q * 32 + lane;
+#pragma unroll
+      for (int x = 0; x < 64; ++x) zreg[x] = __ldg(src + x * 128);
+    } else {
+#pragma unroll
+      for (int x = 0; x < 64; ++x) zreg[x] = 0.f;
+    }
+    auto write_state_operand = [&]() {
+#pragma unroll
+      for (int pc = 0; pc < 8; ++pc) {
+        float x8[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) x8[x] = zreg[pc * 8 + x];
+        uint4 h, l;
+        split8(x8, h, l);
+        tmem_st_x4(colZ + pc * 4, h);
+        if (split_z) tmem_st_x4(colZ + 64 + pc * 4, l);
+      }
+      tmem_st_wait();
+      tc_fence_before_sync();
+    };
+    WARP_ARRIVE(W_M1_OK0);  // there is no earlier dZ to read
+    if (has_entry) write_state_operand();
+    WARP_ARRIVE(W_M2_OK);
+    for (int it = 0; it < nblk; ++it) {
+      if (it + 1 == nblk && !want_final) break;
+      // ---- Z <- Gamma Z + dZ ----
+      const float gamma = ex2_approx(-s2 * (float)(it == (REV ? 0 : nblk - 1) ? edge_len : 128));
+      TC_WAIT_WARP(W_DZ_READY, it & 1, 22);
+      tc_fence_after_sync();
+#pragma unroll
+      for (int pc = 0; pc < 4; ++pc) {
+        uint32_t dh[16];
+        tmem_ld_x16(colDZ + pc * 16, dh);
+        tmem_ld_wait();
+#pragma unroll
+        for (int x = 0; x < 16; ++x) zreg[pc * 16 + x] = fmaf(gamma, zreg[pc * 16 + x], __uint_as_float(dh[x]));
+      }
+      tc_fence_before_sync();
+      if (it + 1 < nblk) {
+        WARP_ARRIVE(W_M1_OK0 + ((it + 1) & 1));  // M1 of the next block may overwrite dZ
+        TC_WAIT_WARP(W_M2_DONE, it & 1, 23);     // M2 of this block has read the old state operand
+        tc_fence_after_sync();
+        write_state_operand();
+        WARP_ARRIVE(W_M2_OK);
+      }
+    }
+    if (want_final) {
+      float* dst = job.final_out + (size_t)bh * (128 * 128) + (size_t)(zhalf * 64) * 128 + q * 32 + lane;
+#pragma unroll
+      for (int x = 0; x < 64; ++x) dst[x * 128] = zreg[x];
+    }
+  } else {
+    // ------------------------------------ F group ------------------------------------
+    // fc^T = (diag(f_state) c)^T as hi / lo terms in tensor memory.  ldmatrix transposes 8 x 8 pieces of the c tile: a
+    // register holds a token pair of one value column, as the A operand wants it.
+    reg_inc<W_REGS_F>();
+    const int q = warp & 3;
+    const uint32_t colF = tmem + ((uint32_t)(q * 32) << 16) + WCOL_FH;
+    const bool split_c = (args.precision & 4) != 0 && s2 != 0.f;
+    // lane l points at token row (l >> 4) * 8 + (l & 7), value columns q * 32 + half * 16 + ((l >> 3) & 1) * 8
+    const uint32_t unit0 = (uint32_t)((q >> 1) * 16384 + (((lane >> 4) << 3) + (lane & 7)) * 128 +
+                                      ((((q & 1) * 4 + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
+    uint32_t raw[64];  // [32-token group][half][octet][8 value columns]
+    auto fetch = [&](int it) {
+      const uint32_t ctile = smem_u32(&sm.c[it & 1][0][0]);
+#pragma unroll
+      for (int g = 0; g < 8; ++g) {  // 16 tokens
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          uint32_t* w = &raw[g * 8 + half * 4];
+          ldmatrix_x4_trans(ctile + (unit0 ^ (half << 5)) + g * 2048, w[0], w[1], w[2], w[3]);
+        }
+      }
+    };
+    TC_WAIT_WARP(W_FULL_C0, 0, 20);
+    fetch(0);
+    for (int it = 0; it < nblk; ++it) {
+      if (it + 1 == nblk && !want_final) break;
+      if (it > 0) TC_WAIT_WARP(W_DZ_READY, (it - 1) & 1, 21);  // M3 of the previous block has read fc
+      tc_fence_after_sync();
+      const int Cr = (it == (REV ? 0 : nblk - 1)) ? edge_len : 128;
+      const int j0 = 2 * (lane & 3);
+      float s2v = s2;
+      asm volatile("" : "+f"(s2v));  // keeps the 32 factors from being held in registers across blocks
+#pragma unroll
+      for (int g = 0; g < 8; ++g) {  // 16 tokens
+        float f[4];                  // of this thread's token pairs in the two octets
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const int j = j0 + 16 * g + 8 * (o >> 1) + (o & 1);
+          f[o] = j < Cr ? ex2_approx(-s2v * (float)(REV ? j + 1 : Cr - 1 - j)) : 0.f;
+        }
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          uint32_t h[4], l[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {  // octet x >> 1, value columns (x & 1) * 8
+            const uint32_t w = raw[g * 8 + half * 4 + x];
+            const float x0 = __uint_as_float(w << 16) * f[(x >> 1) * 2], x1 = __uint_as_float(w & 0xffff0000u) * f[(x >> 1) * 2 + 1];
+            const __nv_bfloat162 hp = __floats2bfloat162_rn(x0, x1);
+            h[x] = *reinterpret_cast<const uint32_t*>(&hp);
+            const __nv_bfloat162 lp =
+                __floats2bfloat162_rn(x0 - __uint_as_float(h[x] << 16), x1 - __uint_as_float(h[x] & 0xffff0000u));
+            l[x] = *reinterpret_cast<const uint32_t*>(&lp);
+          }
+          const uint32_t at = colF + ((uint32_t)(half * 16) << 16) + g * 8;
+          tmem_st_16x128b_x2(at, h);
+          if (split_c) tmem_st_16x128b_x2(at + 64, l);
+        }
+      }
+      tmem_st_wait();
+      tc_fence_before_sync();
+      WARP_ARRIVE(W_M3_OK);
+      if (it + 1 < nblk) {
+        TC_WAIT_WARP(W_FULL_C0 + ((it + 1) & 1), ((it + 1) >> 1) & 1, 20);
+        fetch(it + 1);
+      }
+    }
+  }
+
+teardown:
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
+}
+
+template <bool REV, typename TOut>
+cudaError_t launch_walk_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, const DecayTable& tab, cudaStream_t stream) {
+  const size_t smem = sizeof(WSmem<REV>) + 1024;
+  static_assert(sizeof(WSmem<REV>) + 1024 <= 232448, "shared memory of one SM");
+  auto kern = tc_walk_kernel<REV, TOut>;
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  KernelTimer timer(ta.njobs == 2 ? K_WALK_PAIR : K_WALK, stream);
+  kern<<<(unsigned)(ta.BH * ta.nseg * ta.njobs), W_THREADS, smem, stream>>>(m0, m1, ta, tab);
+  count_launch();
+  return cudaGetLastError();
+}

@@ -200,6 +200,35 @@ __device__ __forceinline__ void tmem_st_x8(uint32_t taddr, const uint32_t (&r)[8
                "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                : "memory");
 }
+__device__ __forceinline__ void tmem_st_x4(uint32_t taddr, const uint4& r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r.x), "r"(r.y), "r"(r.z),
+               "r"(r.w)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_x16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+      : "memory");
+}
+// Sixteen lanes (those of taddr) x 8 columns: register 2 x of thread t is lane t / 4, column 4 x + t % 4, register
+// 2 x + 1 lane t / 4 + 8 of the same column -- two by two 8 x 8 matrices of 16-bit pairs, each spread over the
+// warp as ldmatrix leaves it.
+__device__ __forceinline__ void tmem_st_16x128b_x2(uint32_t taddr, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3])
+               : "memory");
+}
+// Four 8 x 8 matrices of 16-bit elements, transposed: thread t gets elements (row 2 (t % 4), row 2 (t % 4) + 1) of column
+// t / 4 of each; lane 8 m + i supplies the address of row i of matrix m (16 bytes).
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+               : "r"(saddr)
+               : "memory");
+}
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // D[tmem] (+)= A[tmem] * B[smem].  A is M x 16 bf16 for one instruction: row m in lane m, the 16
@@ -315,7 +344,58 @@ __device__ __forceinline__ void umma_group_ts8(uint32_t d_tmem, uint32_t a_tmem,
       "}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc0), "r"(go)
       : "memory");
 }
+// Eight K steps with a dense A operand in tensor memory (8 columns per step) and a B tile of 128 x 128 in shared
+// memory, K-major (BK) or MN-major.
+template <bool BK>
+__device__ __forceinline__ void umma_group_tsd(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi,
+                                               uint32_t idesc, uint32_t acc0, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred p, g, t;\n\t.reg .b64 db;\n\t.reg .b32 at, bl;\n\t"
+      "setp.ne.b32 g, %6, 0;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "mov.b64 db, {%2, %3};\n\t"
+      "@g tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t"
+      LA_UMMA_TS_STEP(8, %7) LA_UMMA_TS_STEP(16, %8) LA_UMMA_TS_STEP(24, %9) LA_UMMA_TS_STEP(32, %10)
+      LA_UMMA_TS_STEP(40, %11) LA_UMMA_TS_STEP(48, %12) LA_UMMA_TS_STEP(56, %13)
+      "}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc0), "r"(go),
+      "n"(umma_kstep<BK>(1)), "n"(umma_kstep<BK>(2)), "n"(umma_kstep<BK>(3)), "n"(umma_kstep<BK>(4)),
+      "n"(umma_kstep<BK>(5)), "n"(umma_kstep<BK>(6)), "n"(umma_kstep<BK>(7))
+      : "memory");
+}
 #undef LA_UMMA_TS_STEP
+// Four K steps of D[e, i] (+)= A[e, j] B[j, i] where B[j, i] = 0 for i < j (REV: for i > j): step k covers
+// j = 16 k .. 16 k + 15 and touches only the columns of D that it can change.  Steps K0, K0 + 1, .. (REV: K0, K0 - 1, ..),
+// so that step 0 (REV: 7), which covers every column, comes first.  A is MN-major, B K-major, both in shared memory.
+template <int K, bool REV>
+struct TriStep {
+  static constexpr uint32_t n = REV ? 16 * (K + 1) : 128 - 16 * K;        // columns of D
+  static constexpr uint32_t dcol = REV ? 0 : 16 * K;                        // first of them
+  static constexpr uint32_t a = K * 128;                                    // 2 KB per 16 tokens
+  static constexpr uint32_t b = (K >> 2) * 1024 + (K & 3) * 2 + dcol * 8;  // panel, 32 bytes per step, 128 bytes per row
+  static constexpr uint32_t idesc = umma_idesc_bf16(128, n, true, false);
+};
+#define LA_UMMA_TRI_STEP(DO, AO, BO, ID, PRED)                                              \
+  "add.u32 dt, %0, " #DO ";\n\tadd.u32 al, %1, " #AO ";\n\tadd.u32 bl, %2, " #BO ";\n\t"  \
+  "mov.b64 da, {al, %3};\n\tmov.b64 db, {bl, %3};\n\tmov.b32 id, " #ID ";\n\t"           \
+  "@g tcgen05.mma.cta_group::1.kind::f16 [dt], da, db, id, " #PRED ";\n\t"
+template <int K0, bool REV>
+__device__ __forceinline__ void umma_tri4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t acc0,
+                                          uint32_t go) {
+  constexpr int S = REV ? -1 : 1;
+  using T0 = TriStep<K0, REV>;
+  using T1 = TriStep<K0 + S, REV>;
+  using T2 = TriStep<K0 + 2 * S, REV>;
+  using T3 = TriStep<K0 + 3 * S, REV>;
+  asm volatile(
+      "{\n\t.reg .pred p, g, t;\n\t.reg .b64 da, db;\n\t.reg .b32 dt, al, bl, id;\n\t"
+      "setp.ne.b32 g, %5, 0;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      LA_UMMA_TRI_STEP(%6, %7, %8, %9, p) LA_UMMA_TRI_STEP(%10, %11, %12, %13, t)
+      LA_UMMA_TRI_STEP(%14, %15, %16, %17, t) LA_UMMA_TRI_STEP(%18, %19, %20, %21, t)
+      "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(acc0), "r"(go),
+      "n"(T0::dcol), "n"(T0::a), "n"(T0::b), "n"(T0::idesc), "n"(T1::dcol), "n"(T1::a), "n"(T1::b), "n"(T1::idesc),
+      "n"(T2::dcol), "n"(T2::a), "n"(T2::b), "n"(T2::idesc), "n"(T3::dcol), "n"(T3::a), "n"(T3::b), "n"(T3::idesc)
+      : "memory");
+}
+#undef LA_UMMA_TRI_STEP
 __device__ __forceinline__ void umma_commit_if(uint64_t* bar, uint32_t go) {
   asm volatile(
       "{\n\t.reg .pred g;\n\tsetp.ne.b32 g, %1, 0;\n\t"
