@@ -19,32 +19,35 @@
 // transposition.
 //
 // Measured on B200 against the walk it replaces (la_tc_full.cuh without its gate): 7B-like shape, fp32 results, one walk
-// 0.654 -> 0.595 ms, the dV and dK walks in one launch 1.358 -> 1.166 ms; 3 x 8 heads x 3001 tokens, bf16 results, token-major,
-// one walk 75 -> 57 us, the pair 81 -> 60 us.
+// 0.594 -> 0.467 ms, the dV and dK walks in one launch 1.186 -> 0.949 ms; 3 x 8 heads x 3001 tokens, bf16 results, one walk
+// 60 -> 49 us, the pair 65 -> 54 us.
 //
 // Tensor memory (512 columns): R 128 (S, then dZ^T, in turn), O 128, fc^T hi/lo 2 x 64, Z^T hi/lo 2 x 64.
 // Shared memory: a, b twice, c twice, P hi/lo (32 KB each).
 // Order of the products per block n:  M2(n) M3(n) M4(n) M1(n+1).  They use O, R, O, R in turn, and what the CUDA cores
-// do with one region happens while the next product runs in the other: P reads S(n) during M2(n), O is scaled during
+// do with one region happens while the next product runs in the other: S(n) is read during M2(n), O is scaled during
 // M3(n), dZ(n) is read during M4(n), O(n) is stored during M1(n+1).  Shared memory is read by the CUDA cores during M2
-// and M3 only (A in tensor memory); the F group therefore fetches c of the next block into registers during M3.
+// and M3 only (A in tensor memory), so that the value rows of the next block are fetched into registers during M3.
 //
-// Warp roles (32 warps): 0 TMA producer, 1 MMA issuer (all lanes converged, instructions on one elected lane), 4-11 P
-// group (two warps per 32 score rows), 12-19 O group (two warps per 32 value columns, 64 tokens each), 20-27 Z group
-// (fp32 state in registers: two warps per 32 value columns, 64 features each), 28-31 F group (fc).  Registers per thread
-// after start-up: W_REGS_*; they add up to the 2048 warp-registers of the launch.
+// Warp roles (28 warps): 0 TMA producer, 1 MMA issuer (all lanes converged, instructions on one elected lane), 4-19
+// workers, 20-27 O group (two warps per 32 value columns, 64 tokens each).  A worker warp does, one after the other, its
+// share of three jobs whose turns come at different times of a block: P (scores of up to 2 x 16 keys of 32 rows, during
+// M2 and M3), Z (32 value columns x 32 features of the fp32 state in registers, from M3 on; the chain that M2 of the next
+// block waits for, so it comes before F) and F (fc of 32 value columns x 32 tokens, until M3 of the next block).  With
+// eight warps for P, eight for Z and four for F the state's conversion alone took 2900 of a block's 7100 clocks.
+// Registers per thread after start-up: W_REGS_*; they add up to what the launch has.
 
-constexpr int W_THREADS = 1024;
+constexpr int W_THREADS = 896;
 constexpr uint32_t WCOL_R = 0, WCOL_O = 128, WCOL_FH = 256, WCOL_FL = 320, WCOL_ZH = 384, WCOL_ZL = 448;
-constexpr int W_REGS_CTL = 32, W_REGS_P = 48, W_REGS_O = 40, W_REGS_Z = 104, W_REGS_F = 96;
-static_assert(4 * W_REGS_CTL + 8 * W_REGS_P + 8 * W_REGS_O + 8 * W_REGS_Z + 4 * W_REGS_F <= 2048, "registers of the launch");
+constexpr int W_REGS_LAUNCH = 72, W_REGS_CTL = 24, W_REGS_W = 88, W_REGS_O = 64;
+static_assert(4 * W_REGS_CTL + 16 * W_REGS_W + 8 * W_REGS_O <= 28 * W_REGS_LAUNCH, "registers of the launch");
 
 enum WBar {
-  W_FULL_C0 = 0, W_FULL_C1,  // TMA -> F group, MMA: c of an even / odd block
-  W_M1_OK0, W_M1_OK1,        // a and b landed (two arrivals with bytes) and the previous dZ read (8 warps)
-  W_M2_OK,                   // state operand written (8 warps) and the previous O read (8 warps)
-  W_M3_OK,                   // fc written (4 warps) and S read (8 warps)
-  W_M4_OK,                   // P written (8 warps) and O scaled (8 warps)
+  W_FULL_C0 = 0, W_FULL_C1,  // TMA -> workers, MMA: c of an even / odd block
+  W_M1_OK0, W_M1_OK1,        // a and b landed (two arrivals with bytes) and the previous dZ read (16 worker warps)
+  W_M2_OK,                   // state operand written (16 worker warps) and the previous O read (8 warps)
+  W_M3_OK,                   // fc written and S read (16 worker warps)
+  W_M4_OK,                   // P written (16 worker warps) and O scaled (8 warps)
   W_S_READY,                 // M1 done
   W_M2_DONE,                 // M2 done: O_inter complete, a and the state operand free
   W_DZ_READY,                // M3 done: dZ complete, b and fc free
@@ -63,11 +66,22 @@ struct alignas(1024) WSmem {
   // Factor of a token's O_inter.  REV: index 1 is for the edge block (the first one walked, which may be shorter than 128
   // tokens), index 0 for every other.
   float fout[REV ? 2 : 1][128];
-  float ptab[32];  // lambda^(31 - x)
+  float ptab[16];  // lambda^(15 - x)
   uint64_t bars[W_NUM_BARS];
   uint32_t tmem_slot;
   int abort;
 };
+
+// p + x * stride (elements) as one multiply-add, which leaves the integer pipe (half rate, and what the conversions to
+// hi / lo terms need) alone.
+template <typename T>
+__device__ __forceinline__ T* elem_at(T* p, int x, long long stride) {
+  uint64_t r;
+  asm("mad.wide.u32 %0, %1, %2, %3;"
+      : "=l"(r)
+      : "r"((uint32_t)stride * (uint32_t)sizeof(T)), "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)));
+  return reinterpret_cast<T*>(r);
+}
 
 // args.njobs == 2: two walks of the same direction over the same tokens in one launch (the dV and dK walks of the
 // backward pass, which between them read Q, K, V and dO); the thread blocks of the two jobs alternate, so that the two
@@ -104,9 +118,9 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   if (tid == 0) {
     for (int i = 0; i < W_NUM_BARS; ++i) {
       uint32_t count = 1;
-      if (i == W_M1_OK0 || i == W_M1_OK1) count = 10;
-      if (i == W_M2_OK || i == W_M4_OK) count = 16;
-      if (i == W_M3_OK) count = 12;
+      if (i == W_M1_OK0 || i == W_M1_OK1) count = 18;
+      if (i == W_M2_OK || i == W_M4_OK) count = 24;
+      if (i == W_M3_OK) count = 16;
       mbar_init(&sm.bars[i], count);
     }
     sm.abort = 0;
@@ -124,7 +138,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     } else if (set == 0) {
       sm.fout[0][i] = ex2_approx(-s2 * (float)(i + 1));
     }
-    if (x < 32) sm.ptab[x] = ex2_approx(-s2 * (float)(31 - x));
+    if (x < 16) sm.ptab[x] = ex2_approx(-s2 * (float)(15 - x));
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -238,43 +252,124 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
         drain_wait(&sm.bars[W_DRAIN], 0);
       }
     }
-  } else if (warp < 12) {
-    // ------------------------------------ P group ------------------------------------
-    // S -> masked, decayed P as bf16 hi / lo rows in shared memory; the sub-tiles outside the causal band are never read
-    reg_dec<W_REGS_P>();
-    const int q = warp & 3;
-    const int phalf = (warp >= 8) ? 1 : 0;  // warps 4..7 take the 32-key chunks 0 and 3, warps 8..11 chunks 1 and 2
-    const int r = q * 32 + lane;            // score row
-    const uint32_t colS = tmem + ((uint32_t)(q * 32) << 16) + WCOL_R;
-    const bool split_p = (args.precision & 1) != 0;
-    const int c_first = phalf, c_second = phalf ? 2 : 3;
-    const bool use_first = REV ? (c_first >= q) : (c_first <= q), use_second = REV ? (c_second >= q) : (c_second <= q);
-    const int n_chunks = (use_first ? 1 : 0) + (use_second ? 1 : 0);
+  } else if (warp < 20) {
+    // ------------------------------------ workers ------------------------------------
+    reg_inc<W_REGS_W>();
+    const int q = warp & 3;                // quarter of tensor memory: score rows / value columns q * 32 + lane
+    const int w4 = (warp - 4) >> 2;        // this warp's share within the quarter
+    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
+    const uint32_t colDZ = lane_addr + WCOL_R + w4 * 32;
+    const uint32_t colZ = lane_addr + WCOL_ZH + w4 * 16;  // (the lo terms follow 64 columns further)
+    const uint32_t colF = lane_addr + WCOL_FH + w4 * 16;
+    const bool split_p = (args.precision & 1) != 0, split_z = (args.precision & 2) != 0;
+    const bool split_c = (args.precision & 4) != 0 && s2 != 0.f;
+    // P: the 16-key pieces w4 and w4 + 4 of the band's 2 (q + 1), forward from key 0, reverse from key 127 downwards
+    const int pieces = (REV ? 4 - q : q + 1) * 2;
+    const int n_pieces = w4 < pieces ? (w4 + 4 < pieces ? 2 : 1) : 0;
     // Reverse walk of a packed batch: the keys past the end of the sequence lie inside the band of the edge block, and
     // there they are the next sequence's tokens, not the zero fill a dense batch has.
     const int cut = (REV && args.seq_start) ? edge_len : 128;
+    // F: lane l points ldmatrix at token row w4 * 32 + (l >> 4) * 8 + (l & 7), value columns q * 32 + ((l >> 3) & 1) * 8
+    const uint32_t unit0 = (uint32_t)((q >> 1) * 16384 + (w4 * 32 + ((lane >> 4) << 3) + (lane & 7)) * 128 +
+                                      ((((q & 1) * 4 + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
+    const bool need_state = nblk > 1 || want_final;
+
+    float zreg[32];    // Z[w4 * 32 + x][value column q * 32 + lane]
+    uint32_t raw[16];  // c of the next block: [16 tokens][16 value columns][8 tokens][8 value columns]
+    auto write_state_operand = [&]() {
+#pragma unroll
+      for (int pc = 0; pc < 4; ++pc) {
+        float x8[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) x8[x] = zreg[pc * 8 + x];
+        uint4 h, l;
+        split8(x8, h, l);
+        tmem_st_x4(colZ + pc * 4, h);
+        if (split_z) tmem_st_x4(colZ + 64 + pc * 4, l);
+      }
+      tmem_st_wait();
+      tc_fence_before_sync();
+    };
+    auto fetch_c = [&](int it) {
+      const uint32_t ctile = smem_u32(&sm.c[it & 1][0][0]) + unit0;
+#pragma unroll
+      for (int g = 0; g < 4; ++g)  // 16 tokens (g >> 1), 16 value columns (g & 1)
+        ldmatrix_x4_trans((ctile ^ ((g & 1) << 5)) + (g >> 1) * 2048, raw[4 * g], raw[4 * g + 1], raw[4 * g + 2], raw[4 * g + 3]);
+    };
+    // fc^T = (diag(f_state) c)^T: ldmatrix has transposed 8 x 8 pieces of the c tile, a register holds a token pair of one
+    // value column, as the A operand wants it
+    auto write_fc = [&](int it) {
+      const int Cr = (it == (REV ? 0 : nblk - 1)) ? edge_len : 128;
+#pragma unroll
+      for (int g2 = 0; g2 < 2; ++g2) {  // 16 tokens
+        float f[4];                     // of this thread's token pairs in the two octets
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const int j = w4 * 32 + g2 * 16 + 8 * (o >> 1) + 2 * (lane & 3) + (o & 1);
+          f[o] = j < Cr ? ex2_approx(-s2 * (float)(REV ? j + 1 : Cr - 1 - j)) : 0.f;
+        }
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          uint32_t h[4], l[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {  // octet x >> 1, value columns (x & 1) * 8
+            const uint32_t w = raw[g2 * 8 + half * 4 + x];
+            const float x0 = __uint_as_float(w << 16) * f[(x >> 1) * 2], x1 = __uint_as_float(w & 0xffff0000u) * f[(x >> 1) * 2 + 1];
+            const __nv_bfloat162 hp = __floats2bfloat162_rn(x0, x1);
+            h[x] = *reinterpret_cast<const uint32_t*>(&hp);
+            const __nv_bfloat162 lp =
+                __floats2bfloat162_rn(x0 - __uint_as_float(h[x] << 16), x1 - __uint_as_float(h[x] & 0xffff0000u));
+            l[x] = *reinterpret_cast<const uint32_t*>(&lp);
+          }
+          const uint32_t at = colF + ((uint32_t)(half * 16) << 16) + g2 * 8;
+          tmem_st_16x128b_x2(at, h);
+          if (split_c) tmem_st_16x128b_x2(at + 64, l);
+        }
+      }
+      tmem_st_wait();
+      tc_fence_before_sync();
+    };
+
+    if (has_entry) {
+      const float* src = job.entry + ((size_t)bh * args.nseg + seg) * (128 * 128) + (size_t)(w4 * 32) * 128 + q * 32 + lane;
+#pragma unroll
+      for (int x = 0; x < 32; ++x) zreg[x] = __ldg(src + x * 128);
+    } else {
+#pragma unroll
+      for (int x = 0; x < 32; ++x) zreg[x] = 0.f;
+    }
+    WARP_ARRIVE(W_M1_OK0);  // there is no earlier dZ to read
+    if (has_entry) write_state_operand();
+    WARP_ARRIVE(W_M2_OK);
+    if (need_state) {
+      TC_WAIT_WARP(W_FULL_C0, 0, 20);
+      fetch_c(0);
+      write_fc(0);
+    }
     for (int it = 0; it < nblk; ++it) {
+      // ---- P: S -> masked, decayed bf16 hi / lo rows in shared memory (what lies outside the band is never read) ----
       TC_WAIT_WARP(W_S_READY, it & 1, 17);
       tc_fence_after_sync();
-      if (n_chunks == 0) WARP_ARRIVE(W_M3_OK);
+      if (n_pieces == 0) WARP_ARRIVE(W_M3_OK);
 #pragma unroll 1
-      for (int ci = 0; ci < 2 * n_chunks; ++ci) {  // 16 keys at a time
-        const int j0 = ((use_first && ci < 2) ? c_first : c_second) * 32 + (ci & 1) * 16;
+      for (int pi = 0; pi < n_pieces; ++pi) {
+        const int r = q * 32 + lane;  // score row
+        const int j0 = REV ? 112 - 16 * (w4 + 4 * pi) : 16 * (w4 + 4 * pi);
         uint32_t sreg[16];
-        tmem_ld_x16(colS + j0, sreg);
+        tmem_ld_x16(lane_addr + WCOL_R + j0, sreg);
         const bool edge = REV && it == 0 && cut < 128;
         const float base = ex2_approx(-s2 * (float)(REV ? j0 - r : r - j0 - 15));
         tmem_ld_wait();
-        if (ci == 2 * n_chunks - 1) {
+        if (pi == n_pieces - 1) {
           tc_fence_before_sync();
-          WARP_ARRIVE(W_M3_OK);  // all of S that this warp needs is in registers: M3 may overwrite it
+          WARP_ARRIVE(W_M3_OK);  // all of S that this warp needs is in registers, and its fc is written
         }
         float d[16];
         if ((j0 >> 5) != q && !edge) {
           // wholly inside the band: lambda^|i-j| = row factor * table entry (both at most 1), nothing to mask
 #pragma unroll
           for (int x4 = 0; x4 < 4; ++x4) {
-            const float4 t = *reinterpret_cast<const float4*>(&sm.ptab[REV ? 28 - 4 * x4 : 16 + 4 * x4]);
+            const float4 t = *reinterpret_cast<const float4*>(&sm.ptab[REV ? 12 - 4 * x4 : 4 * x4]);
             d[4 * x4 + 0] = __uint_as_float(sreg[4 * x4 + 0]) * base * (REV ? t.w : t.x);
             d[4 * x4 + 1] = __uint_as_float(sreg[4 * x4 + 1]) * base * (REV ? t.z : t.y);
             d[4 * x4 + 2] = __uint_as_float(sreg[4 * x4 + 2]) * base * (REV ? t.y : t.z);
@@ -303,12 +398,42 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       }
       fence_proxy_async_smem();
       WARP_ARRIVE(W_M4_OK);
+      const bool more = it + 1 < nblk;
+      if (!more && !want_final) break;
+      if (more) {
+        TC_WAIT_WARP(W_FULL_C0 + ((it + 1) & 1), ((it + 1) >> 1) & 1, 20);
+        fetch_c(it + 1);
+      }
+      // ---- Z <- Gamma Z + dZ ----
+      const float gamma = ex2_approx(-s2 * (float)(it == (REV ? 0 : nblk - 1) ? edge_len : 128));
+      TC_WAIT_WARP(W_DZ_READY, it & 1, 22);  // M2 and M3 of this block are done
+      tc_fence_after_sync();
+#pragma unroll
+      for (int pc = 0; pc < 2; ++pc) {
+        uint32_t dh[16];
+        tmem_ld_x16(colDZ + pc * 16, dh);
+        tmem_ld_wait();
+#pragma unroll
+        for (int x = 0; x < 16; ++x) zreg[pc * 16 + x] = fmaf(gamma, zreg[pc * 16 + x], __uint_as_float(dh[x]));
+      }
+      tc_fence_before_sync();
+      if (more) {
+        WARP_ARRIVE(W_M1_OK0 + ((it + 1) & 1));  // M1 of the next block may overwrite dZ
+        write_state_operand();
+        WARP_ARRIVE(W_M2_OK);
+        write_fc(it + 1);
+      }
     }
-  } else if (warp < 20) {
+    if (want_final) {
+      float* dst = job.final_out + (size_t)bh * (128 * 128) + (size_t)(w4 * 32) * 128 + q * 32 + lane;
+#pragma unroll
+      for (int x = 0; x < 32; ++x) dst[x * 128] = zreg[x];
+    }
+  } else {
     // ------------------------------------ O group ------------------------------------
     reg_dec<W_REGS_O>();
     const int q = warp & 3;
-    const int th = (warp >= 16) ? 64 : 0;  // first of this warp's 64 tokens
+    const int th = (warp >= 24) ? 64 : 0;  // first of this warp's 64 tokens
     const uint32_t colO = tmem + ((uint32_t)(q * 32) << 16) + WCOL_O + th;
     const size_t head_off = (size_t)(args.seq_start ? 0 : bh / args.H) * args.sB + (size_t)(bh % args.H) * args.sH +
                             (size_t)tok0 * args.sT;
@@ -346,149 +471,24 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       TC_WAIT_WARP(W_O_READY, it & 1, 25);
       tc_fence_after_sync();
 #pragma unroll 1
-      for (int pc = 0; pc < 4; ++pc) {
-        uint32_t w[16];
-        tmem_ld_x16(colO + pc * 16, w);
+      for (int pc = 0; pc < 2; ++pc) {  // 32 tokens at a time
+        uint32_t w[32];
+        tmem_ld_x32(colO + pc * 32, w);
         tmem_ld_wait();
-        if (pc == 3) {
+        if (pc == 1) {
           tc_fence_before_sync();
           WARP_ARRIVE(W_M2_OK);  // M2 of the next block may overwrite O
         }
+        const int here = rows - pc * 32;
+        if (here >= 32) {
 #pragma unroll
-        for (int x = 0; x < 16; ++x) {
-          if (pc * 16 + x < rows) *dst = from_f32<TOut>(__uint_as_float(w[x]));
-          dst += args.sT;
+          for (int x = 0; x < 32; ++x) *elem_at(dst, x, args.sT) = from_f32<TOut>(__uint_as_float(w[x]));
+        } else {
+#pragma unroll
+          for (int x = 0; x < 32; ++x)
+            if (x < here) *elem_at(dst, x, args.sT) = from_f32<TOut>(__uint_as_float(w[x]));
         }
-      }
-    }
-  } else if (warp < 28) {
-    // ------------------------------------ Z group ------------------------------------
-    reg_inc<W_REGS_Z>();
-    const int q = warp & 3;
-    const int zhalf = (warp >= 24) ? 1 : 0;  // which 64 of the 128 features this warp owns
-    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    const uint32_t colDZ = lane_addr + WCOL_R + zhalf * 64;
-    const uint32_t colZ = lane_addr + WCOL_ZH + zhalf * 32;  // (the lo terms follow 64 columns further)
-    const bool split_z = (args.precision & 2) != 0;
-    float zreg[64];  // Z[zhalf * 64 + x][value column q * 32 + lane]
-    if (has_entry) {
-      const float* src = job.entry + ((size_t)bh * args.nseg + seg) * (128 * 128) + (size_t)(zhalf * 64) * 128 + q * 32 + lane;
-#pragma unroll
-      for (int x = 0; x < 64; ++x) zreg[x] = __ldg(src + x * 128);
-    } else {
-#pragma unroll
-      for (int x = 0; x < 64; ++x) zreg[x] = 0.f;
-    }
-    auto write_state_operand = [&]() {
-#pragma unroll
-      for (int pc = 0; pc < 8; ++pc) {
-        float x8[8];
-#pragma unroll
-        for (int x = 0; x < 8; ++x) x8[x] = zreg[pc * 8 + x];
-        uint4 h, l;
-        split8(x8, h, l);
-        tmem_st_x4(colZ + pc * 4, h);
-        if (split_z) tmem_st_x4(colZ + 64 + pc * 4, l);
-      }
-      tmem_st_wait();
-      tc_fence_before_sync();
-    };
-    WARP_ARRIVE(W_M1_OK0);  // there is no earlier dZ to read
-    if (has_entry) write_state_operand();
-    WARP_ARRIVE(W_M2_OK);
-    for (int it = 0; it < nblk; ++it) {
-      if (it + 1 == nblk && !want_final) break;
-      // ---- Z <- Gamma Z + dZ ----
-      const float gamma = ex2_approx(-s2 * (float)(it == (REV ? 0 : nblk - 1) ? edge_len : 128));
-      TC_WAIT_WARP(W_DZ_READY, it & 1, 22);
-      tc_fence_after_sync();
-#pragma unroll
-      for (int pc = 0; pc < 4; ++pc) {
-        uint32_t dh[16];
-        tmem_ld_x16(colDZ + pc * 16, dh);
-        tmem_ld_wait();
-#pragma unroll
-        for (int x = 0; x < 16; ++x) zreg[pc * 16 + x] = fmaf(gamma, zreg[pc * 16 + x], __uint_as_float(dh[x]));
-      }
-      tc_fence_before_sync();
-      if (it + 1 < nblk) {
-        WARP_ARRIVE(W_M1_OK0 + ((it + 1) & 1));  // M1 of the next block may overwrite dZ
-        TC_WAIT_WARP(W_M2_DONE, it & 1, 23);     // M2 of this block has read the old state operand
-        tc_fence_after_sync();
-        write_state_operand();
-        WARP_ARRIVE(W_M2_OK);
-      }
-    }
-    if (want_final) {
-      float* dst = job.final_out + (size_t)bh * (128 * 128) + (size_t)(zhalf * 64) * 128 + q * 32 + lane;
-#pragma unroll
-      for (int x = 0; x < 64; ++x) dst[x * 128] = zreg[x];
-    }
-  } else {
-    // ------------------------------------ F group ------------------------------------
-    // fc^T = (diag(f_state) c)^T as hi / lo terms in tensor memory.  ldmatrix transposes 8 x 8 pieces of the c tile: a
-    // register holds a token pair of one value column, as the A operand wants it.
-    reg_inc<W_REGS_F>();
-    const int q = warp & 3;
-    const uint32_t colF = tmem + ((uint32_t)(q * 32) << 16) + WCOL_FH;
-    const bool split_c = (args.precision & 4) != 0 && s2 != 0.f;
-    // lane l points at token row (l >> 4) * 8 + (l & 7), value columns q * 32 + half * 16 + ((l >> 3) & 1) * 8
-    const uint32_t unit0 = (uint32_t)((q >> 1) * 16384 + (((lane >> 4) << 3) + (lane & 7)) * 128 +
-                                      ((((q & 1) * 4 + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
-    uint32_t raw[64];  // [32-token group][half][octet][8 value columns]
-    auto fetch = [&](int it) {
-      const uint32_t ctile = smem_u32(&sm.c[it & 1][0][0]);
-#pragma unroll
-      for (int g = 0; g < 8; ++g) {  // 16 tokens
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t* w = &raw[g * 8 + half * 4];
-          ldmatrix_x4_trans(ctile + (unit0 ^ (half << 5)) + g * 2048, w[0], w[1], w[2], w[3]);
-        }
-      }
-    };
-    TC_WAIT_WARP(W_FULL_C0, 0, 20);
-    fetch(0);
-    for (int it = 0; it < nblk; ++it) {
-      if (it + 1 == nblk && !want_final) break;
-      if (it > 0) TC_WAIT_WARP(W_DZ_READY, (it - 1) & 1, 21);  // M3 of the previous block has read fc
-      tc_fence_after_sync();
-      const int Cr = (it == (REV ? 0 : nblk - 1)) ? edge_len : 128;
-      const int j0 = 2 * (lane & 3);
-      float s2v = s2;
-      asm volatile("" : "+f"(s2v));  // keeps the 32 factors from being held in registers across blocks
-#pragma unroll
-      for (int g = 0; g < 8; ++g) {  // 16 tokens
-        float f[4];                  // of this thread's token pairs in the two octets
-#pragma unroll
-        for (int o = 0; o < 4; ++o) {
-          const int j = j0 + 16 * g + 8 * (o >> 1) + (o & 1);
-          f[o] = j < Cr ? ex2_approx(-s2v * (float)(REV ? j + 1 : Cr - 1 - j)) : 0.f;
-        }
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t h[4], l[4];
-#pragma unroll
-          for (int x = 0; x < 4; ++x) {  // octet x >> 1, value columns (x & 1) * 8
-            const uint32_t w = raw[g * 8 + half * 4 + x];
-            const float x0 = __uint_as_float(w << 16) * f[(x >> 1) * 2], x1 = __uint_as_float(w & 0xffff0000u) * f[(x >> 1) * 2 + 1];
-            const __nv_bfloat162 hp = __floats2bfloat162_rn(x0, x1);
-            h[x] = *reinterpret_cast<const uint32_t*>(&hp);
-            const __nv_bfloat162 lp =
-                __floats2bfloat162_rn(x0 - __uint_as_float(h[x] << 16), x1 - __uint_as_float(h[x] & 0xffff0000u));
-            l[x] = *reinterpret_cast<const uint32_t*>(&lp);
-          }
-          const uint32_t at = colF + ((uint32_t)(half * 16) << 16) + g * 8;
-          tmem_st_16x128b_x2(at, h);
-          if (split_c) tmem_st_16x128b_x2(at + 64, l);
-        }
-      }
-      tmem_st_wait();
-      tc_fence_before_sync();
-      WARP_ARRIVE(W_M3_OK);
-      if (it + 1 < nblk) {
-        TC_WAIT_WARP(W_FULL_C0 + ((it + 1) & 1), ((it + 1) >> 1) & 1, 20);
-        fetch(it + 1);
+        dst += 32 * args.sT;
       }
     }
   }
