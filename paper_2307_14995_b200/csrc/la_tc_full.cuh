@@ -90,6 +90,14 @@ __device__ __forceinline__ void reg_inc() {
   asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
 
+// This warp's registers per thread from now on, LAUNCH being what the launch gave: setmaxnreg.inc must not be given less
+// than the warp has, nor .dec more (an illegal instruction).
+template <int N, int LAUNCH>
+__device__ __forceinline__ void set_regs() {
+  if (N < LAUNCH) reg_dec<N>();
+  if (N > LAUNCH) reg_inc<N>();
+}
+
 // NJOBS = 2: two walks of the same direction over the same tokens in one launch (the dV and dK walks of the backward
 // pass, which between them read Q, K, V and dO); the thread blocks of the two jobs alternate, so that the two
 // readers of a tile run side by side and the tile comes from HBM once.

@@ -19,8 +19,8 @@
 // transposition.
 //
 // Measured on B200 against the walk it replaces (la_tc_full.cuh without its gate): 7B-like shape, fp32 results, one walk
-// 0.594 -> 0.467 ms, the dV and dK walks in one launch 1.186 -> 0.949 ms; 3 x 8 heads x 3001 tokens, bf16 results, one walk
-// 60 -> 49 us, the pair 65 -> 54 us.
+// 0.594 -> 0.467 ms, the dV and dK walks in one launch 1.186 -> 0.90 ms; 3 x 8 heads x 3001 tokens, bf16 results, one walk
+// 60 -> 46 us, the pair 65 -> 50 us.
 //
 // Tensor memory (512 columns): R 128 (S, then dZ^T, in turn), O 128, fc^T hi/lo 2 x 64, Z^T hi/lo 2 x 64.
 // Shared memory: a, b twice, c twice, P hi/lo (32 KB each).
@@ -35,11 +35,12 @@
 // M2 and M3), Z (32 value columns x 32 features of the fp32 state in registers, from M3 on; the chain that M2 of the next
 // block waits for, so it comes before F) and F (fc of 32 value columns x 32 tokens, until M3 of the next block).  With
 // eight warps for P, eight for Z and four for F the state's conversion alone took 2900 of a block's 7100 clocks.
-// Registers per thread after start-up: W_REGS_*; they add up to what the launch has.
+// Registers per thread after start-up: W_REGS_*; they add up to what the launch has (workers with 88 and O with 64: the pair 978
+// instead of 908 us at the 7B-like shape).
 
 constexpr int W_THREADS = 896;
 constexpr uint32_t WCOL_R = 0, WCOL_O = 128, WCOL_FH = 256, WCOL_FL = 320, WCOL_ZH = 384, WCOL_ZL = 448;
-constexpr int W_REGS_LAUNCH = 72, W_REGS_CTL = 24, W_REGS_W = 88, W_REGS_O = 64;
+constexpr int W_REGS_LAUNCH = 72, W_REGS_CTL = 24, W_REGS_W = 96, W_REGS_O = 48;
 static_assert(4 * W_REGS_CTL + 16 * W_REGS_W + 8 * W_REGS_O <= 28 * W_REGS_LAUNCH, "registers of the launch");
 
 enum WBar {
@@ -55,6 +56,37 @@ enum WBar {
   W_DRAIN,
   W_NUM_BARS
 };
+
+// Arithmetic on two fp32 values in one register pair: half the issue slots, which is what the worker warps are short of
+// (the reverse pair at the 1B-like shape 126 -> 123 us; in the fc conversion it spilled registers and was slower).
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// A pair as packed bf16 hi and lo terms, hi + lo = v to 2^-17.
+__device__ __forceinline__ void split2(uint64_t v, uint32_t& h, uint32_t& l) {
+  float a, b;
+  f2_unpack(v, a, b);
+  const __nv_bfloat162 hp = __floats2bfloat162_rn(a, b);
+  h = *reinterpret_cast<const uint32_t*>(&hp);
+  f2_unpack(f2_sub(v, f2_pack(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u))), a, b);
+  const __nv_bfloat162 lp = __floats2bfloat162_rn(a, b);
+  l = *reinterpret_cast<const uint32_t*>(&lp);
+}
 
 template <bool REV>
 struct alignas(1024) WSmem {
@@ -72,15 +104,19 @@ struct alignas(1024) WSmem {
   int abort;
 };
 
-// p + x * stride (elements) as one multiply-add, which leaves the integer pipe (half rate, and what the conversions to
-// hi / lo terms need) alone.
+// *(p + x * stride) = v with the address as one multiply-add, which leaves the integer pipe (half rate, and what the
+// conversions to hi / lo terms need) alone; one unit, so that the compiler does not hold 32 addresses in registers.
 template <typename T>
-__device__ __forceinline__ T* elem_at(T* p, int x, long long stride) {
-  uint64_t r;
-  asm("mad.wide.u32 %0, %1, %2, %3;"
-      : "=l"(r)
-      : "r"((uint32_t)stride * (uint32_t)sizeof(T)), "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)));
-  return reinterpret_cast<T*>(r);
+__device__ __forceinline__ void store_at(T* p, uint32_t stride_bytes, int x, float v) {
+  if (sizeof(T) == 4) {
+    asm volatile("{\n\t.reg .b64 a;\n\tmad.wide.u32 a, %0, %1, %2;\n\tst.global.b32 [a], %3;\n\t}" ::"r"(stride_bytes),
+                 "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)), "f"(v)
+                 : "memory");
+  } else {
+    asm volatile("{\n\t.reg .b64 a;\n\tmad.wide.u32 a, %0, %1, %2;\n\tst.global.b16 [a], %3;\n\t}" ::"r"(stride_bytes),
+                 "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)), "h"(__bfloat16_as_ushort(__float2bfloat16_rn(v)))
+                 : "memory");
+  }
 }
 
 // args.njobs == 2: two walks of the same direction over the same tokens in one launch (the dV and dK walks of the
@@ -145,7 +181,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   tc_fence_after_sync();
   const uint32_t tmem = sm.tmem_slot;
   if (warp < 4) {
-    reg_dec<W_REGS_CTL>();
+    set_regs<W_REGS_CTL, W_REGS_LAUNCH>();
     if (warp == 0) {
       // ------------------------------------ TMA producer ------------------------------------
       if (lane == 0) {
@@ -254,7 +290,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     }
   } else if (warp < 20) {
     // ------------------------------------ workers ------------------------------------
-    reg_inc<W_REGS_W>();
+    set_regs<W_REGS_W, W_REGS_LAUNCH>();
     const int q = warp & 3;                // quarter of tensor memory: score rows / value columns q * 32 + lane
     const int w4 = (warp - 4) >> 2;        // this warp's share within the quarter
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
@@ -279,11 +315,11 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     auto write_state_operand = [&]() {
 #pragma unroll
       for (int pc = 0; pc < 4; ++pc) {
-        float x8[8];
-#pragma unroll
-        for (int x = 0; x < 8; ++x) x8[x] = zreg[pc * 8 + x];
         uint4 h, l;
-        split8(x8, h, l);
+        split2(f2_pack(zreg[pc * 8 + 0], zreg[pc * 8 + 1]), h.x, l.x);
+        split2(f2_pack(zreg[pc * 8 + 2], zreg[pc * 8 + 3]), h.y, l.y);
+        split2(f2_pack(zreg[pc * 8 + 4], zreg[pc * 8 + 5]), h.z, l.z);
+        split2(f2_pack(zreg[pc * 8 + 6], zreg[pc * 8 + 7]), h.w, l.w);
         tmem_st_x4(colZ + pc * 4, h);
         if (split_z) tmem_st_x4(colZ + 64 + pc * 4, l);
       }
@@ -386,7 +422,8 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           }
         }
         uint32_t h8[8], l8[8];
-        split16(d, h8, l8);
+#pragma unroll
+        for (int x = 0; x < 8; ++x) split2(f2_pack(d[2 * x], d[2 * x + 1]), h8[x], l8[x]);
         unsigned char* const row = reinterpret_cast<unsigned char*>(&sm.p_hi[j0 >> 6][0]) + r * 128;
         const int u0 = ((((j0 & 63) >> 3)) ^ (r & 7)) << 4, u1 = u0 ^ 16;
         *reinterpret_cast<uint4*>(row + u0) = make_uint4(h8[0], h8[1], h8[2], h8[3]);
@@ -414,7 +451,10 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
         tmem_ld_x16(colDZ + pc * 16, dh);
         tmem_ld_wait();
 #pragma unroll
-        for (int x = 0; x < 16; ++x) zreg[pc * 16 + x] = fmaf(gamma, zreg[pc * 16 + x], __uint_as_float(dh[x]));
+        for (int x = 0; x < 16; x += 2)
+          f2_unpack(f2_fma(f2_pack(gamma, gamma), f2_pack(zreg[pc * 16 + x], zreg[pc * 16 + x + 1]),
+                           f2_pack(__uint_as_float(dh[x]), __uint_as_float(dh[x + 1]))),
+                    zreg[pc * 16 + x], zreg[pc * 16 + x + 1]);
       }
       tc_fence_before_sync();
       if (more) {
@@ -431,7 +471,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     }
   } else {
     // ------------------------------------ O group ------------------------------------
-    reg_dec<W_REGS_O>();
+    set_regs<W_REGS_O, W_REGS_LAUNCH>();
     const int q = warp & 3;
     const int th = (warp >= 24) ? 64 : 0;  // first of this warp's 64 tokens
     const uint32_t colO = tmem + ((uint32_t)(q * 32) << 16) + WCOL_O + th;
@@ -470,6 +510,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       TOut* dst = out + (size_t)t0 * args.sT;
       TC_WAIT_WARP(W_O_READY, it & 1, 25);
       tc_fence_after_sync();
+      const uint32_t stride = (uint32_t)args.sT * (uint32_t)sizeof(TOut);
 #pragma unroll 1
       for (int pc = 0; pc < 2; ++pc) {  // 32 tokens at a time
         uint32_t w[32];
@@ -482,11 +523,11 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
         const int here = rows - pc * 32;
         if (here >= 32) {
 #pragma unroll
-          for (int x = 0; x < 32; ++x) *elem_at(dst, x, args.sT) = from_f32<TOut>(__uint_as_float(w[x]));
+          for (int x = 0; x < 32; ++x) store_at(dst, stride, x, __uint_as_float(w[x]));
         } else {
 #pragma unroll
           for (int x = 0; x < 32; ++x)
-            if (x < here) *elem_at(dst, x, args.sT) = from_f32<TOut>(__uint_as_float(w[x]));
+            if (x < here) store_at(dst, stride, x, __uint_as_float(w[x]));
         }
         dst += 32 * args.sT;
       }
