@@ -53,6 +53,8 @@ struct Packed {
 struct Plan {
   int BH, seg_len, nseg;
   bool tensor;      // tensor-core kernels
+  bool chains;      // the walk chains the segments' local states itself (tensor-core kernels at d = 128): no scan ...
+  bool scanned;     // ... but running sums of the slowly decaying heads' states
   int precision;    // LA_SPLIT_* bits (tensor path)
   Packed pk;        // start == NULL: dense batch
 };
@@ -85,36 +87,54 @@ bool tensor_path_available(const la_shape* s) {
   return tc_supported() && s->in_dtype == LA_BF16 && s->d == s->e && (s->d == 128 || s->d == 64);
 }
 
-la_status make_plan(const la_shape* s, Plan* p) {
+// `packed`: the plan of a packed batch, whose sequences of different lengths share one segment length.
+la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
   p->pk = Packed{nullptr, nullptr, nullptr, 0};
   p->BH = s->B * s->H;
   if (s->path == LA_PATH_TENSOR && !tensor_path_available(s)) return LA_ERR_UNSUPPORTED;
   p->tensor = (s->path == LA_PATH_TENSOR) || (s->path == LA_PATH_AUTO && tensor_path_available(s));
+  p->chains = p->tensor && s->d == 128;
+  p->scanned = false;
   p->precision = (s->precision == LA_PRECISION_DEFAULT)
                      ? (LA_SPLIT_SCORES | LA_SPLIT_STATE | LA_SPLIT_DECAYED)
                      : s->precision;
   long seg_len = s->seg_len;
   if (seg_len == 0) {
-    // One thread block per (batch*head, segment[, value-column half]) and one block per SM at a
-    // time: pick the segment count that minimises (waves over the 148 SMs) x (blocks walked per
-    // segment + pipeline fill), with segments no shorter than 1024 tokens so that the
-    // per-segment state traffic stays small.  Depends on the shape only.
-    // at d = 128 the half-width tensor kernels also split the value columns over two thread blocks
-    const long slices = (p->tensor && s->d == 128 && !tc_full_width()) ? 2 : 1;
-    const long sms = 148, fill = 2;
-    long most = s->N / 1024;
-    if (most < 1) most = 1;
-    if (most > 1024) most = 1024;
-    long best_n = 1, best_cost = -1;
-    for (long n = 1; n <= most; ++n) {
-      const long len = ((s->N + n - 1) / n + 127) / 128 * 128;
-      const long nseg = (s->N + len - 1) / len;
-      const long waves = (p->BH * slices * nseg + sms - 1) / sms;
-      const long cost = waves * (len / 128 + fill);
-      if (best_cost < 0 || cost < best_cost) {
-        best_cost = cost;
-        best_n = n;
+    // One thread block per (batch*head, segment) and one block per SM at a time: pick the segment count with the least
+    // cost, in units of one 128-token block (about 3 us).  Depends on the shape only.
+    // Where the walk chains the segment states itself: forward walk and dQ walk, the dV and dK walks in one launch (twice
+    // the thread blocks), each in waves over the 148 SMs of (blocks of a segment + start and end), and per direction the
+    // launch that makes the states, with what each further state costs to write, read and chain.  Measured, forward plus
+    // backward: 3 x 8 heads x 3001 tokens 172 us with 1536-token segments, 141 with 512; 8 heads x 2048 118 with 1024, 92
+    // with 512, 126 with 128; 2 x 16 x 8192 289 with 2048, 344 with 1024 (the model: 49.7, 34.5 / 38, 29, 33 / 85, 97).
+    // Elsewhere (d = 64, fp32, packed batches): waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.
+    auto choose = [&](long most, long unit_limit, auto cost_of) {
+      if (most < 1) most = 1;
+      if (most > 1024) most = 1024;
+      long best_n = 1;
+      double best = -1.0;
+      for (long n = 1; n <= most; ++n) {
+        const long len = ((s->N + n - 1) / n + 127) / 128 * 128;
+        const long nseg = (s->N + len - 1) / len;
+        if (n > 1 && p->BH * nseg > unit_limit) break;
+        const double cost = cost_of(nseg, len / 128);
+        if (best < 0.0 || cost < best) {
+          best = cost;
+          best_n = n;
+        }
       }
+      return best_n;
+    };
+    auto waves = [](long units) { return (double)((units + 147) / 148); };
+    long best_n = choose(s->N / 1024, 1L << 40, [&](long nseg, long blocks) { return waves(p->BH * nseg) * (blocks + 2); });
+    if (p->chains && !packed) {
+      // (la_fwd_noalloc's scratch holds the states of 256 segments: shapes that fit it with long segments still do)
+      const long limit = std::max(p->BH * best_n, (long)(LA_NOALLOC_SCRATCH_BYTES / (2 * s->d * s->e * sizeof(float))));
+      best_n = choose(s->N / 128, limit, [&](long nseg, long blocks) {
+        const double units = (double)p->BH * nseg;
+        return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 1.3) +
+               (nseg > 1 ? 2.0 * (4.0 + 0.01 * units + 0.6 * nseg) : 0.0);
+      });
     }
     seg_len = ((s->N + best_n - 1) / best_n + 127) / 128 * 128;
   }
@@ -153,18 +173,6 @@ la_status check_device() {
     if ((expr) != cudaSuccess) return LA_ERR_CUDA; \
   } while (0)
 
-// One generic-operator call: optional pre-pass + scan (when the sequence is cut
-// into segments or the incoming state needs transposing), then the walk.
-struct OpCall {
-  const void *a, *b, *c;
-  void* out;
-  int reverse;
-  const float* z_in;     // user state entering the sequence (kernel orientation unless transposed)
-  bool z_in_transposed;
-  float* final_out;      // state leaving the sequence, kernel orientation, or NULL
-  float* buf;            // [BH,nseg,D*E] scratch for entry states (may be NULL if not needed)
-};
-
 // Element strides of the token tensors for the shape's layout (d == e in every supported shape).
 void set_strides(const la_shape* s, int tokens, OpArgs* a) {
   const long long D = s->d;
@@ -180,7 +188,7 @@ void set_strides(const la_shape* s, int tokens, OpArgs* a) {
 }
 
 cudaError_t run_prepass(const la_shape* s, const Plan& p, const DecayTable& tab, const void* b,
-                        const void* c, int reverse, float* local_out, cudaStream_t st) {
+                        const void* c, int reverse, float* local_out, bool all_segments, cudaStream_t st) {
   OpArgs args{};
   args.b = b;
   args.c = c;
@@ -196,7 +204,7 @@ cudaError_t run_prepass(const la_shape* s, const Plan& p, const DecayTable& tab,
   args.seq_order = p.pk.order;
   args.total_tokens = p.pk.total_tokens;
   set_strides(s, p.pk.start ? p.pk.total_tokens : s->N, &args);
-  if (p.tensor) return launch_tc_prepass(args, tab, s->d, p.precision, st);
+  if (p.tensor) return launch_tc_prepass(args, tab, s->d, p.precision, all_segments, st);
   return launch_simt_prepass(args, tab, s->d, s->e, (int)s->in_dtype, st);
 }
 
@@ -219,14 +227,59 @@ cudaError_t run_scan(const la_shape* s, const Plan& p, const DecayTable& tab, fl
   return launch_scan(sa, tab, st);
 }
 
+// Running sums pay where a slow head would read many states: 7B-like shape, nine segments, 8 us of chain against 5 us of
+// launch; with four segments 3 against 5.  Packed batches: always, their sequences differ in how many segments they have.
+bool wants_running(const la_shape* s, const Plan& p, const DecayTable& tab) {
+  if (!p.chains || p.nseg < 3 || p.BH > 65535 || !(p.pk.start || p.nseg > 6)) return false;
+  for (int h = 0; h < s->H; ++h)
+    if (slow_head((float)tab.s2[h], p.seg_len)) return true;
+  return false;
+}
+cudaError_t run_prefix(const la_shape* s, const Plan& p, const DecayTable& tab, float* buf, int reverse, cudaStream_t st) {
+  ScanArgs sa{};
+  sa.buf = buf;
+  sa.BH = p.BH;
+  sa.H = s->H;
+  sa.N = s->N;
+  sa.seg_len = p.seg_len;
+  sa.nseg = p.nseg;
+  sa.seq_len = p.pk.len;
+  sa.Da = s->d;
+  sa.Ec = s->e;
+  sa.reverse = reverse;
+  return launch_prefix(sa, tab, st);
+}
+
+// What a walk starts from: the state entering each segment (entry), or, where the walk chains the segments itself
+// (Plan::chains), the state entering the sequence and the segments' local states, each possibly stored transposed.
+struct Carried {
+  const float* entry = nullptr;
+  const float* z_in = nullptr;
+  const float* local = nullptr;
+  bool z_in_t = false, local_t = false;
+};
+Carried chained(const float* z_in, bool z_in_t, const float* local, bool local_t) {
+  Carried c;
+  c.z_in = z_in;
+  c.z_in_t = z_in_t;
+  c.local = local;
+  c.local_t = local_t;
+  return c;
+}
+
 OpArgs walk_args(const la_shape* s, const Plan& p, const void* a, const void* b, const void* c, void* out,
-                 const float* entry, float* final_out, int reverse) {
+                 const Carried& from, float* final_out, int reverse) {
   OpArgs args{};
   args.a = a;
   args.b = b;
   args.c = c;
   args.out = out;
-  args.entry = entry;
+  args.entry = from.entry;
+  args.z_in = from.z_in;
+  args.local = from.local;
+  args.z_in_t = from.z_in_t;
+  args.local_t = from.local_t;
+  args.scanned = p.scanned;
   args.final_out = final_out;
   args.BH = p.BH;
   args.H = s->H;
@@ -243,9 +296,9 @@ OpArgs walk_args(const la_shape* s, const Plan& p, const void* a, const void* b,
 }
 
 cudaError_t run_walk(const la_shape* s, const Plan& p, const DecayTable& tab, const void* a,
-                     const void* b, const void* c, void* out, const float* entry, float* final_out,
+                     const void* b, const void* c, void* out, const Carried& from, float* final_out,
                      int reverse, cudaStream_t st) {
-  const OpArgs args = walk_args(s, p, a, b, c, out, entry, final_out, reverse);
+  const OpArgs args = walk_args(s, p, a, b, c, out, from, final_out, reverse);
   if (p.tensor) return launch_tc_walk(args, tab, s->d, (int)s->out_dtype, p.precision, st);
   return launch_simt_walk(args, tab, s->d, s->e, (int)s->in_dtype, (int)s->out_dtype, st);
 }
@@ -267,16 +320,18 @@ using namespace la;
 
 extern "C" {
 
-size_t la_workspace_bytes(int op, const la_shape* shape) {
+static size_t scratch_bytes(int op, const la_shape* shape, bool packed) {
   if (op != LA_OP_FWD && op != LA_OP_BWD && op != LA_OP_DECODE) return (size_t)-1;
   if (check_shape(shape, op != LA_OP_DECODE) != LA_OK) return (size_t)-1;
   if (op == LA_OP_DECODE) return 0;
   Plan p;
-  if (make_plan(shape, &p) != LA_OK) return (size_t)-1;
+  if (make_plan(shape, &p, packed) != LA_OK) return (size_t)-1;
   const size_t one = state_set_bytes(shape, p);
-  if (op == LA_OP_FWD) return p.nseg > 1 ? 2 * one : 0;  // the states entering each segment, and their transposes
+  if (op == LA_OP_FWD) return p.nseg > 1 ? 2 * one : 0;  // the segments' states, and (without chains) their transposes
   return 3 * one;
 }
+
+size_t la_workspace_bytes(int op, const la_shape* shape) { return scratch_bytes(op, shape, false); }
 
 int la_segment_length(const la_shape* shape) {
   if (check_shape(shape, true) != LA_OK) return 0;
@@ -340,8 +395,9 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   DecayTable tab;
   if ((st = make_table(shape, lambda_host, &tab)) != LA_OK) return st;
   Plan p;
-  if ((st = make_plan(shape, &p)) != LA_OK) return st;
+  if ((st = make_plan(shape, &p, pk != nullptr)) != LA_OK) return st;
   if (pk) p.pk = *pk;
+  p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
   const size_t need = p.nseg > 1 ? 2 * one : 0;
   if (need > 0 && (!workspace || workspace_bytes < need)) return LA_ERR_WORKSPACE;
@@ -349,29 +405,39 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   if ((st = check_device()) != LA_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
 
-  const float* entry = kv_in;  // single segment: the caller's state is the entry state
-  if (p.nseg > 1) {
-    float* buf = static_cast<float*>(workspace);
-    LA_TRY_CUDA(run_prepass(shape, p, tab, k, v, 0, buf, cs));
+  Carried from;
+  float* const buf = static_cast<float*>(workspace);
+  if (p.nseg > 1) LA_TRY_CUDA(run_prepass(shape, p, tab, k, v, 0, buf, false, cs));
+  if (p.chains) {
+    if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf, 0, cs));
+    from = chained(kv_in, false, buf, false);
+  } else if (p.nseg > 1) {
     // the transposed copy (second set) is what the dQ walk of la_bwd_reuse starts from
     LA_TRY_CUDA(run_scan(shape, p, tab, buf, buf + one / sizeof(float), kv_in, false, 0, cs));
-    entry = buf;
+    from.entry = buf;
+  } else {
+    from.entry = kv_in;  // single segment: the caller's state is the entry state
   }
   if (!u) {
-    LA_TRY_CUDA(run_walk(shape, p, tab, q, k, v, o, entry, kv_out, 0, cs));
+    LA_TRY_CUDA(run_walk(shape, p, tab, q, k, v, o, from, kv_out, 0, cs));
     return LA_OK;
   }
-  OpArgs wa = walk_args(shape, p, q, k, v, o, entry, kv_out, 0);
-  wa.u = u;
-  wa.y = y;
-  wa.rstd = rstd;
-  if (p.tensor && tc_can_fuse_gate(wa, shape->d)) {
+  // The d = 128 walk has the output stage as an epilogue, which costs it about 4 us per 128 tokens (four quarters of a row
+  // meet through shared memory).  With fp32 results a row kernel behind the plain walk gives the same and is faster where o
+  // is written anyway (1B-like shape: 137 us against 148) or y still sits in L2 when the row kernel reads it; past that the
+  // epilogue saves a pass over y (7B-like shape 991 us against 1027).  bf16 results: always the epilogue, which rounds once.
+  const double y_bytes = (double)p.BH * shape->N * shape->e * sizeof(float);
+  if (p.chains && (shape->out_dtype == LA_BF16 || (!o && y_bytes > 126e6))) {
+    OpArgs wa = walk_args(shape, p, q, k, v, o, from, kv_out, 0);
+    wa.u = u;
+    wa.y = y;
+    wa.rstd = rstd;
     LA_TRY_CUDA(launch_tc_walk(wa, tab, shape->d, (int)shape->out_dtype, p.precision, cs));
     return LA_OK;
   }
   // not fused: the attention output goes to o (or, if it is not wanted, to y itself) and a row kernel turns it into y
   void* att = o ? o : y;
-  LA_TRY_CUDA(run_walk(shape, p, tab, q, k, v, att, entry, kv_out, 0, cs));
+  LA_TRY_CUDA(run_walk(shape, p, tab, q, k, v, att, from, kv_out, 0, cs));
   LA_TRY_CUDA(launch_norm_gate_fwd(att, u, y, rstd, (long)p.BH * shape->N, shape->e, (int)shape->in_dtype,
                                    (int)shape->out_dtype, cs));
   return LA_OK;
@@ -415,8 +481,9 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   DecayTable tab;
   if ((st = make_table(shape, lambda_host, &tab)) != LA_OK) return st;
   Plan p;
-  if ((st = make_plan(shape, &p)) != LA_OK) return st;
+  if ((st = make_plan(shape, &p, pk != nullptr)) != LA_OK) return st;
   if (pk) p.pk = *pk;
+  p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
   if (!workspace || workspace_bytes < 3 * one) return LA_ERR_WORKSPACE;
   if (fwd_workspace == workspace) return LA_ERR_INVALID_ARG;
@@ -429,37 +496,46 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   float* buf_et = buf_e + one / sizeof(float);                     // its transpose
   const bool multi = p.nseg > 1;
 
-  // dQ = fwd(a = dO, b = V, c = K); its state is KV^T, so the caller's kv_in enters transposed.
-  const float* entry_q = nullptr;
-  if (multi && fwd_workspace) {
+  // dQ = fwd(a = dO, b = V, c = K); its state is KV^T, so the caller's kv_in (and what la_fwd left) enters transposed.
+  Carried from_q;
+  if (p.chains) {
+    if (multi && !fwd_workspace) {
+      LA_TRY_CUDA(run_prepass(shape, p, tab, v, k, 0, buf_kvt, false, cs));
+      if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf_kvt, 0, cs));
+    }
+    from_q = chained(kv_in, true, fwd_workspace ? static_cast<const float*>(fwd_workspace) : buf_kvt, fwd_workspace != nullptr);
+  } else if (multi && fwd_workspace) {
     // la_fwd left KV entering each segment (kv_in included) and its transpose in its workspace: no pre-pass, no scan
-    entry_q = static_cast<const float*>(fwd_workspace) + one / sizeof(float);
+    from_q.entry = static_cast<const float*>(fwd_workspace) + one / sizeof(float);
   } else if (multi || kv_in) {
-    if (multi) LA_TRY_CUDA(run_prepass(shape, p, tab, v, k, 0, buf_kvt, cs));
+    if (multi) LA_TRY_CUDA(run_prepass(shape, p, tab, v, k, 0, buf_kvt, false, cs));
     LA_TRY_CUDA(run_scan(shape, p, tab, buf_kvt, nullptr, kv_in, true, 0, cs));
-    entry_q = buf_kvt;
+    from_q.entry = buf_kvt;
   }
-  LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, entry_q, nullptr, 0, cs));
+  LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
 
   // dV = rev(a = K, b = Q, c = dO) carries dKV; dK = rev(a = V, b = dO, c = Q) carries dKV^T.
-  const float* entry_v = nullptr;
-  const float* entry_k = nullptr;
-  if (multi) LA_TRY_CUDA(run_prepass(shape, p, tab, q, d_o, 1, buf_e, cs));
-  if (multi || grad_kv_out) {
+  Carried from_v, from_k;
+  if (multi) LA_TRY_CUDA(run_prepass(shape, p, tab, q, d_o, 1, buf_e, false, cs));
+  if (p.chains) {
+    if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf_e, 1, cs));
+    from_v = chained(grad_kv_out, false, buf_e, false);
+    from_k = chained(grad_kv_out, true, buf_e, true);
+  } else if (multi || grad_kv_out) {
     LA_TRY_CUDA(run_scan(shape, p, tab, buf_e, buf_et, grad_kv_out, false, 1, cs));
-    entry_v = buf_e;
-    entry_k = buf_et;
+    from_v.entry = buf_e;
+    from_k.entry = buf_et;
   }
   if (p.tensor) {
     // both reverse walks in one launch: together they read Q, K, V and dO, and the thread blocks of the two are
     // interleaved so that each of those tiles comes from HBM once (Algorithm 4 accumulates dK_j and dV_j in the
     // same outer iteration for the same reason)
-    const OpArgs walk_v = walk_args(shape, p, k, q, d_o, dv, entry_v, grad_kv_in, 1);
-    const OpArgs walk_k = walk_args(shape, p, v, d_o, q, dk, entry_k, nullptr, 1);
+    const OpArgs walk_v = walk_args(shape, p, k, q, d_o, dv, from_v, grad_kv_in, 1);
+    const OpArgs walk_k = walk_args(shape, p, v, d_o, q, dk, from_k, nullptr, 1);
     LA_TRY_CUDA(launch_tc_walk_pair(walk_v, walk_k, tab, shape->d, (int)shape->out_dtype, p.precision, cs));
   } else {
-    LA_TRY_CUDA(run_walk(shape, p, tab, k, q, d_o, dv, entry_v, grad_kv_in, 1, cs));
-    LA_TRY_CUDA(run_walk(shape, p, tab, v, d_o, q, dk, entry_k, nullptr, 1, cs));
+    LA_TRY_CUDA(run_walk(shape, p, tab, k, q, d_o, dv, from_v, grad_kv_in, 1, cs));
+    LA_TRY_CUDA(run_walk(shape, p, tab, v, d_o, q, dk, from_k, nullptr, 1, cs));
   }
   return LA_OK;
 }
@@ -682,7 +758,7 @@ la_status la_chunk_state(const la_shape* shape, int reverse, const void* b, cons
   if ((st = check_device()) != LA_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   float* buf = static_cast<float*>(workspace);
-  LA_TRY_CUDA(run_prepass(shape, p, tab, b, c, reverse, buf, cs));
+  LA_TRY_CUDA(run_prepass(shape, p, tab, b, c, reverse, buf, true, cs));
   ChainArgs ca{};
   ca.src = buf;
   ca.DE = shape->d * shape->e;
@@ -751,9 +827,8 @@ la_status varlen_check(const la_shape* shape, const int* cu, int S, la_shape* su
 size_t esize(int dt) { return dt == LA_BF16 ? 2 : 4; }
 
 // The single-launch form: every sequence is a "batch" entry of its own length inside the packed tensors, and the
-// full-width tensor-core walk (with the state-only pre-pass and the scan where the longest sequence is cut into
-// segments) runs over all of them at once.  It exists for bf16 inputs at d = e = 128 with outputs aligned to 32
-// bytes; everything else runs one call per sequence.  `sp` is the shape that goes with it: B = sequences, N = longest.
+// tensor-core walk (with the pre-pass where the longest sequence is cut into segments) runs over all of them at once.
+// It exists for bf16 inputs at d = e = 128; everything else runs one call per sequence.  `sp` is the shape that goes with it: B = sequences, N = longest.
 bool packed_shape(const la_shape* shape, const int* cu, int S, la_shape* sp) {
   if (S < 2 || shape->d != 128 || shape->in_dtype != LA_BF16 || shape->path == LA_PATH_SIMT || !tc_supported())
     return false;
@@ -800,7 +875,7 @@ size_t la_varlen_workspace_bytes(int op, const la_shape* shape, const int* cu_se
   }
   la_shape sp;
   if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp)) {  // the single-launch form: its table and its state sets
-    const size_t w = la_workspace_bytes(op, &sp);
+    const size_t w = scratch_bytes(op, &sp, true);
     if (w != (size_t)-1 && packed_table_bytes(num_seqs) + w > most) most = packed_table_bytes(num_seqs) + w;
   }
   return most;
@@ -814,7 +889,7 @@ la_status la_fwd_varlen(const la_shape* shape, const void* q, const void* k, con
   if (st != LA_OK) return st;
   if (!q || !k || !v || !o) return LA_ERR_INVALID_ARG;
   la_shape sp;
-  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp) && tc_walk_is_full(shape->d, o, nullptr)) {
+  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp)) {
     const size_t tb = packed_table_bytes(num_seqs);
     if (!workspace || workspace_bytes < tb || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_WORKSPACE;
     if ((st = check_device()) != LA_OK) return st;
@@ -848,8 +923,7 @@ la_status la_bwd_varlen(const la_shape* shape, const void* q, const void* k, con
   if (st != LA_OK) return st;
   if (!q || !k || !v || !d_o || !dq || !dk || !dv) return LA_ERR_INVALID_ARG;
   la_shape sp;
-  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp) && tc_walk_is_full(shape->d, dq, dk) &&
-      tc_walk_is_full(shape->d, dv, nullptr)) {
+  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp)) {
     const size_t tb = packed_table_bytes(num_seqs);
     if (!workspace || workspace_bytes < tb || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_WORKSPACE;
     if ((st = check_device()) != LA_OK) return st;

@@ -43,6 +43,13 @@ struct OpArgs {
   const void* c;      // [BH, N, Ec]
   void* out;          // [BH, N, Ec]  (unused by the pre-pass)
   const float* entry; // [BH, nseg, Da*Ec] state entering each segment, or NULL = zeros
+  // Tensor-core walk at Da = Ec = 128 instead of `entry`: the state entering the sequence [BH, Da*Ec] (NULL = zeros) and
+  // the segments' local states [BH, nseg, Da*Ec] as the pre-pass leaves them, which the walk chains itself; each may be
+  // stored transposed.
+  const float* z_in;
+  const float* local;
+  int z_in_t, local_t;
+  int scanned;  // launch_prefix has turned the local states of the slowly decaying heads into running ones
   float* local_out;   // pre-pass: [BH, nseg, Da*Ec] segment-local states
   float* final_out;   // [BH, Da*Ec] state leaving the last-processed segment, or NULL
   int BH, H, N;
@@ -101,6 +108,14 @@ cudaError_t launch_simt_walk(const OpArgs& args, const DecayTable& tab, int Da, 
 cudaError_t launch_simt_prepass(const OpArgs& args, const DecayTable& tab, int Da, int Ec, int in_dt,
                                 cudaStream_t stream);
 cudaError_t launch_scan(const ScanArgs& args, const DecayTable& tab, cudaStream_t stream);
+// Running sums of the segments' local states, in place: afterwards buf[p] is the state leaving segment p with nothing
+// entering the sequence.  Only for heads whose states reach over more than one segment (slow_head); args.buf, BH, H, N,
+// seg_len, nseg, Da, Ec, reverse and seq_len are used.
+cudaError_t launch_prefix(const ScanArgs& args, const DecayTable& tab, cudaStream_t stream);
+// Whole segments of seg_len tokens through which a state can be followed before its decay is below 2^-160, exactly zero in
+// fp32 (no limit for lambda = 1), and whether a head's states are worth a running sum.
+__host__ __device__ inline float state_reach(float s2, int seg_len) { return s2 > 0.f ? 160.f / (s2 * (float)seg_len) : 3.0e38f; }
+__host__ __device__ inline bool slow_head(float s2, int seg_len) { return state_reach(s2, seg_len) >= 2.f; }
 cudaError_t launch_chain(const ChainArgs& args, const DecayTable& tab, cudaStream_t stream);
 // dst[m] = transpose(src[m]) for `count` row-major Da x Ec fp32 matrices.
 cudaError_t launch_transpose_states(const float* src, float* dst, long count, int Da, int Ec, cudaStream_t stream);
@@ -120,19 +135,13 @@ cudaError_t launch_norm_gate_bwd(const void* o, const void* u, const void* dy, v
 bool tc_supported();
 cudaError_t launch_tc_walk(const OpArgs& args, const DecayTable& tab, int D, int out_dt, int precision,
                            cudaStream_t stream);
-// Whether launch_tc_walk can fuse the epilogue described by args.u / args.y into the walk (d = 128, y and out
-// aligned to 32 bytes); otherwise the caller runs the walk and then launch_norm_gate_fwd.
-// True when launch_tc_walk / launch_tc_walk_pair take the full-width kernel for these outputs (D = 128, aligned to 32 bytes).
-bool tc_walk_is_full(int D, const void* out0, const void* out1);
-bool tc_can_fuse_gate(const OpArgs& args, int D);
 // Two walks of the same direction over the same tokens (same N, BH, segments) in one launch; the thread blocks of
 // the two are interleaved so that tiles both read come from HBM once.
-// Whether the d = 128 walk normally runs as one full-width thread block per (head, segment) rather than two
-// half-width ones (the segment plan counts thread blocks accordingly).
-bool tc_full_width();
 cudaError_t launch_tc_walk_pair(const OpArgs& first, const OpArgs& second, const DecayTable& tab, int D, int out_dt,
                                 int precision, cudaStream_t stream);
-cudaError_t launch_tc_prepass(const OpArgs& args, const DecayTable& tab, int D, int precision,
+// all_segments: false leaves out the segment that no other segment's state depends on (forward the last, reverse the
+// first); a hint, at D = 64 every state is made.
+cudaError_t launch_tc_prepass(const OpArgs& args, const DecayTable& tab, int D, int precision, bool all_segments,
                               cudaStream_t stream);
 
 // One warp runs the kernels' bounded wait on a barrier nothing arrives on (budget in SM clocks).

@@ -489,6 +489,40 @@ cudaError_t launch_chain(const ChainArgs& args, const DecayTable& tab, cudaStrea
   return cudaGetLastError();
 }
 
+// One thread per four state elements; the next segment's state is fetched one step ahead.
+__global__ void __launch_bounds__(256) prefix_kernel(const ScanArgs args, const DecayTable tab) {
+  const int bh = blockIdx.y;
+  const double s2 = tab.s2[bh % args.H];
+  if (!slow_head((float)s2, args.seg_len)) return;
+  const int n_tok = args.seq_len ? args.seq_len[bh / args.H] : args.N;
+  const int nseg = (n_tok + args.seg_len - 1) / args.seg_len;
+  if (nseg < 3) return;  // a single state is its own running sum
+  const size_t DE = (size_t)args.Da * args.Ec;
+  float4* buf = reinterpret_cast<float4*>(args.buf + (size_t)bh * args.nseg * DE) + blockIdx.x * 256 + threadIdx.x;
+  const long step = (long)(DE / 4);
+  const float full = decay_pow_d(s2, (double)args.seg_len);  // every segment but the sequence's last is whole
+  // forward: segments 0 .. nseg - 2 (nothing reads the state after the last), reverse: nseg - 1 .. 1
+  const long first = args.reverse ? nseg - 1 : 0, dir = args.reverse ? -1 : 1;
+  float4 z = buf[first * step], next = buf[(first + dir) * step];
+  for (int i = 1; i < nseg - 1; ++i) {
+    const float4 x = next;
+    if (i + 1 < nseg - 1) next = buf[(first + (i + 1) * dir) * step];
+    z.x = fmaf(full, z.x, x.x);
+    z.y = fmaf(full, z.y, x.y);
+    z.z = fmaf(full, z.z, x.z);
+    z.w = fmaf(full, z.w, x.w);
+    buf[(first + i * dir) * step] = z;
+  }
+}
+
+cudaError_t launch_prefix(const ScanArgs& args, const DecayTable& tab, cudaStream_t stream) {
+  if ((args.Da * args.Ec) % 1024 != 0 || args.BH > 65535) return cudaErrorInvalidValue;
+  KernelTimer timer(K_SCAN, stream);
+  prefix_kernel<<<dim3((unsigned)(args.Da * args.Ec / 1024), (unsigned)args.BH), 256, 0, stream>>>(args, tab);
+  count_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_scan(const ScanArgs& args, const DecayTable& tab, cudaStream_t stream) {
   if (args.nseg > SCAN_MAX_SEG || (args.Da % 32) != 0 || (args.Ec % 32) != 0) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)args.BH, (unsigned)((args.Da / 32) * (args.Ec / 32)));

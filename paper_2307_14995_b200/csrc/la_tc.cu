@@ -112,7 +112,11 @@ struct TcJob {
   void* out;
   const float* entry;
   float* final_out;
-  // gate epilogue of the forward walk (full-width kernel only): y = SRMSNorm(out) (.) u
+  // D = 128 walk: the state entering the sequence and the segments' local states (see OpArgs)
+  const float* z_in;
+  const float* local;
+  bool z_in_t, local_t;
+  // gate epilogue of the forward walk (D = 128 only): y = SRMSNorm(out) (.) u
   const void* u;
   void* y;
   float* rstd;
@@ -131,6 +135,7 @@ struct TcArgs {
   int njobs;
   int BH, H, N, seg_len, nseg;
   int precision;
+  int scanned;  // see OpArgs
   long long sT, sH, sB;  // element offset of token t of (b,h): b*sB + h*sH + t*sT (rows of D contiguous features)
 };
 
@@ -842,8 +847,8 @@ __global__ void bounded_wait_selftest_kernel(long long budget) {
   }
 }
 
-#include "la_tc_full.cuh"
 #include "la_tc_walk.cuh"
+#include "la_tc_state.cuh"
 
 // ---------------------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -862,9 +867,9 @@ EncodeTiledFn encode_fn() {
 }
 
 // Tensor map over a token tensor seen as {feature D, token N, head H, batch B} with element strides {1, sT, sH, sB}
-// (D = 64 or 128, bf16 or fp32), a box of 128 bytes x 128 tokens x 1 x 1 and 128-byte swizzle; tokens beyond N read
+// (D = 64 or 128, bf16 or fp32), a box of 128 bytes x box_tokens x 1 x 1 and 128-byte swizzle; tokens beyond N read
 // as zero and are not written.
-bool make_map(CUtensorMap* m, const void* ptr, const OpArgs& a, int D, bool f32 = false) {
+bool make_map(CUtensorMap* m, const void* ptr, const OpArgs& a, int D, bool f32 = false, int box_tokens = 128) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
   const cuuint64_t esz = f32 ? 4 : 2;
@@ -873,7 +878,7 @@ bool make_map(CUtensorMap* m, const void* ptr, const OpArgs& a, int D, bool f32 
   const int tokens = a.seq_start ? a.total_tokens : a.N;
   cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)tokens, (cuuint64_t)a.H, (cuuint64_t)B};
   cuuint64_t strides[3] = {(cuuint64_t)a.sT * esz, (cuuint64_t)a.sH * esz, (cuuint64_t)a.sB * esz};
-  cuuint32_t box[4] = {(cuuint32_t)(128 / esz), 128, 1, 1};
+  cuuint32_t box[4] = {(cuuint32_t)(128 / esz), (cuuint32_t)box_tokens, 1, 1};
   cuuint32_t es[4] = {1, 1, 1, 1};
   return enc(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr),
              dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -892,85 +897,96 @@ cudaError_t launch_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, const
   return cudaGetLastError();
 }
 
-bool make_maps(TcMaps* m, const OpArgs& args, int D, bool f32) {
-  return make_map(&m->a, args.a, args, D) && make_map(&m->b, args.b, args, D) && make_map(&m->c, args.c, args, D) &&
-         make_map(&m->out, args.out ? args.out : args.y, args, D, f32);  // (gated walk without `out`: y)
+// out_f32: the type of the map over `out`, or NULL where the kernel stores its output without one.
+bool make_maps(TcMaps* m, const OpArgs& args, int D, const bool* out_f32) {
+  if (!(make_map(&m->a, args.a, args, D) && make_map(&m->b, args.b, args, D) && make_map(&m->c, args.c, args, D))) return false;
+  if (!out_f32) {
+    m->out = m->c;
+    return true;
+  }
+  return make_map(&m->out, args.out, args, D, *out_f32);
 }
 
-// One walk (second == nullptr) or two walks of the same direction over the same tokens in one launch.
-template <int D>
-cudaError_t launch_walk_d(const OpArgs& args, const OpArgs* second, const DecayTable& tab, int out_dt, int precision,
-                          cudaStream_t stream) {
-  TcMaps m0, m1;
-  const bool f32 = (out_dt == DT_F32);
-  if (!make_maps(&m0, args, D, f32)) return cudaErrorInvalidValue;
-  if (second) {
-    if (!make_maps(&m1, *second, D, f32)) return cudaErrorInvalidValue;
-  } else {
-    m1 = m0;
-  }
+TcJob make_job(const OpArgs& a) {
+  return TcJob{a.c, a.out, a.entry, a.final_out, a.z_in, a.local, a.z_in_t != 0, a.local_t != 0, a.u, a.y, a.rstd};
+}
+
+TcArgs make_args(const OpArgs& args, const OpArgs* second, int precision) {
   TcArgs ta{};
-  ta.job[0] = TcJob{args.c, args.out, args.entry, args.final_out, args.u, args.y, args.rstd};
-  ta.job[1] = second ? TcJob{second->c, second->out, second->entry, second->final_out, nullptr, nullptr, nullptr} : ta.job[0];
-  ta.local_out = nullptr;
+  ta.job[0] = make_job(args);
+  ta.job[1] = make_job(second ? *second : args);
+  ta.local_out = args.local_out;
   ta.njobs = second ? 2 : 1;
   ta.BH = args.BH; ta.H = args.H; ta.N = args.N; ta.seg_len = args.seg_len; ta.nseg = args.nseg;
   ta.precision = precision;
+  ta.scanned = args.scanned;
   ta.sT = args.sT; ta.sH = args.sH; ta.sB = args.sB;
   ta.seq_start = args.seq_start;
   ta.seq_len = args.seq_len;
   ta.seq_order = args.seq_order;
-  if (args.seq_start && !tc_walk_is_full(D, args.out, second ? second->out : nullptr))
-    return cudaErrorInvalidValue;  // only the full-width kernel walks packed batches (the caller checks first)
-  if (args.u) {
-    // forward walk with the gate epilogue: only the full-width kernel has it (the caller asks tc_can_fuse_gate first)
-    if (D != 128 || second || args.reverse || !tc_can_fuse_gate(args, D)) return cudaErrorInvalidValue;
-    return f32 ? launch_full_t<false, float, 1, true>(m0, m1, ta, tab, stream)
-               : launch_full_t<false, __nv_bfloat16, 1, true>(m0, m1, ta, tab, stream);
-  }
-  if (D == 128 && !(reinterpret_cast<uintptr_t>(args.out) & 31u) &&
-      !(second && (reinterpret_cast<uintptr_t>(second->out) & 31u))) {
-    // full-width kernel: one thread block per (head, segment).  Its 32-byte output stores need that alignment;
-    // an output that is only 16-byte aligned (the contract's minimum) takes the half-width kernels below.
-    if (args.reverse)
-      return f32 ? launch_walk_t<true, float>(m0, m1, ta, tab, stream)
-                 : launch_walk_t<true, __nv_bfloat16>(m0, m1, ta, tab, stream);
-    return f32 ? launch_walk_t<false, float>(m0, m1, ta, tab, stream)
-               : launch_walk_t<false, __nv_bfloat16>(m0, m1, ta, tab, stream);
-  }
-  if (second) {  // only the reverse direction is ever paired
-    if (!args.reverse) return cudaErrorInvalidValue;
-    return f32 ? launch_t<true, false, float, D, 2>(m0, m1, ta, tab, stream)
-               : launch_t<true, false, __nv_bfloat16, D, 2>(m0, m1, ta, tab, stream);
-  }
-  if (args.reverse)
-    return f32 ? launch_t<true, false, float, D, 1>(m0, m1, ta, tab, stream)
-               : launch_t<true, false, __nv_bfloat16, D, 1>(m0, m1, ta, tab, stream);
-  return f32 ? launch_t<false, false, float, D, 1>(m0, m1, ta, tab, stream)
-             : launch_t<false, false, __nv_bfloat16, D, 1>(m0, m1, ta, tab, stream);
+  return ta;
 }
 
-template <int D>
-cudaError_t launch_prepass_d(const OpArgs& args, const DecayTable& tab, int precision, cudaStream_t stream) {
+// One walk (second == nullptr) or two walks of the same direction over the same tokens in one launch.
+cudaError_t launch_walk128(const OpArgs& args, const OpArgs* second, const DecayTable& tab, int out_dt, int precision,
+                           cudaStream_t stream) {
+  TcMaps m0, m1;
+  if (!make_maps(&m0, args, 128, nullptr)) return cudaErrorInvalidValue;
+  m1 = m0;
+  if (second && !make_maps(&m1, *second, 128, nullptr)) return cudaErrorInvalidValue;
+  const TcArgs ta = make_args(args, second, precision);
+  const bool f32 = (out_dt == DT_F32);
+  if (args.u) {  // the gate epilogue exists for the single forward walk
+    if (second || args.reverse) return cudaErrorInvalidValue;
+    return f32 ? launch_walk_t<false, float, true>(m0, m1, ta, tab, stream)
+               : launch_walk_t<false, __nv_bfloat16, true>(m0, m1, ta, tab, stream);
+  }
+  if (args.reverse)
+    return f32 ? launch_walk_t<true, float, false>(m0, m1, ta, tab, stream)
+               : launch_walk_t<true, __nv_bfloat16, false>(m0, m1, ta, tab, stream);
+  return f32 ? launch_walk_t<false, float, false>(m0, m1, ta, tab, stream)
+             : launch_walk_t<false, __nv_bfloat16, false>(m0, m1, ta, tab, stream);
+}
+
+cudaError_t launch_walk64(const OpArgs& args, const OpArgs* second, const DecayTable& tab, int out_dt, int precision,
+                          cudaStream_t stream) {
+  TcMaps m0, m1;
+  const bool f32 = (out_dt == DT_F32);
+  if (args.seq_start || args.u) return cudaErrorInvalidValue;  // packed batches and the gate: D = 128 only
+  if (!make_maps(&m0, args, 64, &f32)) return cudaErrorInvalidValue;
+  m1 = m0;
+  if (second && !make_maps(&m1, *second, 64, &f32)) return cudaErrorInvalidValue;
+  const TcArgs ta = make_args(args, second, precision);
+  if (second) {  // only the reverse direction is ever paired
+    if (!args.reverse) return cudaErrorInvalidValue;
+    return f32 ? launch_t<true, false, float, 64, 2>(m0, m1, ta, tab, stream)
+               : launch_t<true, false, __nv_bfloat16, 64, 2>(m0, m1, ta, tab, stream);
+  }
+  if (args.reverse)
+    return f32 ? launch_t<true, false, float, 64, 1>(m0, m1, ta, tab, stream)
+               : launch_t<true, false, __nv_bfloat16, 64, 1>(m0, m1, ta, tab, stream);
+  return f32 ? launch_t<false, false, float, 64, 1>(m0, m1, ta, tab, stream)
+             : launch_t<false, false, __nv_bfloat16, 64, 1>(m0, m1, ta, tab, stream);
+}
+
+cudaError_t launch_prepass64(const OpArgs& args, const DecayTable& tab, int precision, cudaStream_t stream) {
   TcMaps m;
   // the a and out maps are unused by the state-only kernel; valid descriptors are passed anyway
-  if (!make_map(&m.b, args.b, args, D) || !make_map(&m.c, args.c, args, D))
-    return cudaErrorInvalidValue;
+  if (!make_map(&m.b, args.b, args, 64) || !make_map(&m.c, args.c, args, 64)) return cudaErrorInvalidValue;
   m.a = m.b;
   m.out = m.c;
-  TcArgs ta{};
-  ta.job[0] = TcJob{args.c, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  ta.job[1] = ta.job[0];
-  ta.local_out = args.local_out;
-  ta.njobs = 1;
-  ta.BH = args.BH; ta.H = args.H; ta.N = args.N; ta.seg_len = args.seg_len; ta.nseg = args.nseg;
-  ta.precision = precision;
-  ta.sT = args.sT; ta.sH = args.sH; ta.sB = args.sB;
-  ta.seq_start = args.seq_start;
-  ta.seq_len = args.seq_len;
-  ta.seq_order = args.seq_order;
-  return args.reverse ? launch_t<true, true, float, D, 1>(m, m, ta, tab, stream)
-                      : launch_t<false, true, float, D, 1>(m, m, ta, tab, stream);
+  const TcArgs ta = make_args(args, nullptr, precision);
+  return args.reverse ? launch_t<true, true, float, 64, 1>(m, m, ta, tab, stream)
+                      : launch_t<false, true, float, 64, 1>(m, m, ta, tab, stream);
+}
+
+cudaError_t launch_states128(const OpArgs& args, const DecayTable& tab, int precision, bool all_segments, cudaStream_t stream) {
+  TcMaps m;
+  if (!make_map(&m.b, args.b, args, 128, false, 64) || !make_map(&m.c, args.c, args, 128, false, 64))
+    return cudaErrorInvalidValue;
+  const TcArgs ta = make_args(args, nullptr, precision);
+  return args.reverse ? launch_state_t<true>(m, ta, tab, all_segments, stream)
+                      : launch_state_t<false>(m, ta, tab, all_segments, stream);
 }
 
 }  // namespace
@@ -979,21 +995,8 @@ bool tc_supported() { return encode_fn() != nullptr; }
 
 cudaError_t launch_tc_walk(const OpArgs& args, const DecayTable& tab, int D, int out_dt, int precision,
                            cudaStream_t stream) {
-  return D == 128 ? launch_walk_d<128>(args, nullptr, tab, out_dt, precision, stream)
-                  : launch_walk_d<64>(args, nullptr, tab, out_dt, precision, stream);
-}
-
-bool tc_full_width() { return true; }
-
-bool tc_walk_is_full(int D, const void* out0, const void* out1) {
-  return D == 128 && !((reinterpret_cast<uintptr_t>(out0) | reinterpret_cast<uintptr_t>(out1)) & 31u);
-}
-
-bool tc_can_fuse_gate(const OpArgs& args, int D) {
-  if (D != 128 || !args.u || !args.y) return false;
-  if (reinterpret_cast<uintptr_t>(args.y) & 31u) return false;
-  if (args.out && (reinterpret_cast<uintptr_t>(args.out) & 31u)) return false;
-  return true;
+  return D == 128 ? launch_walk128(args, nullptr, tab, out_dt, precision, stream)
+                  : launch_walk64(args, nullptr, tab, out_dt, precision, stream);
 }
 
 cudaError_t launch_tc_walk_pair(const OpArgs& first, const OpArgs& second, const DecayTable& tab, int D, int out_dt,
@@ -1001,12 +1004,14 @@ cudaError_t launch_tc_walk_pair(const OpArgs& first, const OpArgs& second, const
   if (first.reverse != second.reverse || first.N != second.N || first.BH != second.BH || first.nseg != second.nseg ||
       first.seg_len != second.seg_len)
     return cudaErrorInvalidValue;
-  return D == 128 ? launch_walk_d<128>(first, &second, tab, out_dt, precision, stream)
-                  : launch_walk_d<64>(first, &second, tab, out_dt, precision, stream);
+  return D == 128 ? launch_walk128(first, &second, tab, out_dt, precision, stream)
+                  : launch_walk64(first, &second, tab, out_dt, precision, stream);
 }
 
-cudaError_t launch_tc_prepass(const OpArgs& args, const DecayTable& tab, int D, int precision, cudaStream_t stream) {
-  return D == 128 ? launch_prepass_d<128>(args, tab, precision, stream) : launch_prepass_d<64>(args, tab, precision, stream);
+cudaError_t launch_tc_prepass(const OpArgs& args, const DecayTable& tab, int D, int precision, bool all_segments,
+                              cudaStream_t stream) {
+  return D == 128 ? launch_states128(args, tab, precision, all_segments, stream)
+                  : launch_prepass64(args, tab, precision, stream);
 }
 
 cudaError_t launch_bounded_wait_selftest(long long budget_clocks, cudaStream_t stream) {

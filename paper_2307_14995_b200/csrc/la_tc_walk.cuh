@@ -18,7 +18,7 @@
 // value column, a warp's plain store instruction writes 128 contiguous bytes of one token, so that the output needs no
 // transposition.
 //
-// Measured on B200 against the walk it replaces (la_tc_full.cuh without its gate): 7B-like shape, fp32 results, one walk
+// Measured on B200 against a walk with [token, e] accumulators and its on-chip operands in shared memory: 7B-like shape, fp32 results, one walk
 // 0.594 -> 0.467 ms, the dV and dK walks in one launch 1.186 -> 0.90 ms; 3 x 8 heads x 3001 tokens, bf16 results, one walk
 // 60 -> 46 us, the pair 65 -> 50 us.
 //
@@ -35,13 +35,17 @@
 // M2 and M3), Z (32 value columns x 32 features of the fp32 state in registers, from M3 on; the chain that M2 of the next
 // block waits for, so it comes before F) and F (fc of 32 value columns x 32 tokens, until M3 of the next block).  With
 // eight warps for P, eight for Z and four for F the state's conversion alone took 2900 of a block's 7100 clocks.
-// Registers per thread after start-up: W_REGS_*; they add up to what the launch has (workers with 88 and O with 64: the pair 978
+// Registers per thread after start-up: W_REGS_CTL, WRegs; they add up to what the launch has (workers with 88 and O with 64: the pair 978
 // instead of 908 us at the 7B-like shape).
 
 constexpr int W_THREADS = 896;
 constexpr uint32_t WCOL_R = 0, WCOL_O = 128, WCOL_FH = 256, WCOL_FL = 320, WCOL_ZH = 384, WCOL_ZL = 448;
-constexpr int W_REGS_LAUNCH = 72, W_REGS_CTL = 24, W_REGS_W = 96, W_REGS_O = 48;
-static_assert(4 * W_REGS_CTL + 16 * W_REGS_W + 8 * W_REGS_O <= 28 * W_REGS_LAUNCH, "registers of the launch");
+constexpr int W_REGS_LAUNCH = 72, W_REGS_CTL = 24;
+template <bool GATED>
+struct WRegs {  // (the gate's row sums need more than the plain store)
+  static constexpr int W = GATED ? 72 : 96, O = GATED ? 96 : 48;
+  static_assert(4 * W_REGS_CTL + 16 * W + 8 * O <= 28 * W_REGS_LAUNCH, "registers of the launch");
+};
 
 enum WBar {
   W_FULL_C0 = 0, W_FULL_C1,  // TMA -> workers, MMA: c of an even / odd block
@@ -53,9 +57,27 @@ enum WBar {
   W_M2_DONE,                 // M2 done: O_inter complete, a and the state operand free
   W_DZ_READY,                // M3 done: dZ complete, b and fc free
   W_O_READY,                 // M4 done: O complete, c and P free
+  W_GATE0, W_GATE1,          // GATED: a block's sums of squares exchanged (4 warps), per half of the tokens
   W_DRAIN,
   W_NUM_BARS
 };
+
+template <int N>
+__device__ __forceinline__ void reg_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void reg_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+
+// This warp's registers per thread from now on, LAUNCH being what the launch gave: setmaxnreg.inc must not be given less
+// than the warp has, nor .dec more (an illegal instruction).
+template <int N, int LAUNCH>
+__device__ __forceinline__ void set_regs() {
+  if (N < LAUNCH) reg_dec<N>();
+  if (N > LAUNCH) reg_inc<N>();
+}
 
 // Arithmetic on two fp32 values in one register pair: half the issue slots, which is what the worker warps are short of
 // (the reverse pair at the 1B-like shape 126 -> 123 us; in the fc conversion it spilled registers and was slower).
@@ -99,6 +121,7 @@ struct alignas(1024) WSmem {
   // tokens), index 0 for every other.
   float fout[REV ? 2 : 1][128];
   float ptab[16];  // lambda^(15 - x)
+  float gseg[3];   // decay through a whole segment, through the sequence's last one, and through all before this one
   uint64_t bars[W_NUM_BARS];
   uint32_t tmem_slot;
   int abort;
@@ -119,10 +142,45 @@ __device__ __forceinline__ void store_at(T* p, uint32_t stride_bytes, int x, flo
   }
 }
 
+// The 32 bits at p + x * stride, likewise.
+__device__ __forceinline__ uint32_t load_u32_at(const void* p, uint32_t stride_bytes, int x) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .b64 a;\n\tmad.wide.u32 a, %1, %2, %3;\n\tld.global.nc.b32 %0, [a];\n\t}"
+               : "=r"(r)
+               : "r"(stride_bytes), "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)));
+  return r;
+}
+
+// Sum over the 32 lanes of each of 16 values per lane; lane l returns the total of value l >> 1.
+__device__ __forceinline__ float lane_sums16(const float (&v)[16], int lane) {
+  float t[8];
+  const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    const float keep = b4 ? v[8 + x] : v[x], send = b4 ? v[x] : v[8 + x];
+    t[x] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const float keep = b3 ? t[4 + x] : t[x], send = b3 ? t[x] : t[4 + x];
+    t[x] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const float keep = b2 ? t[2 + x] : t[x], send = b2 ? t[x] : t[2 + x];
+    t[x] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  }
+  const float keep = b1 ? t[1] : t[0], send = b1 ? t[0] : t[1];
+  const float r = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+  return r + __shfl_xor_sync(0xffffffffu, r, 1);
+}
+
 // args.njobs == 2: two walks of the same direction over the same tokens in one launch (the dV and dK walks of the
 // backward pass, which between them read Q, K, V and dO); the thread blocks of the two jobs alternate, so that the two
 // readers of a tile run side by side and the tile comes from HBM once.
-template <bool REV, typename TOut>
+// GATED (forward, single job): the epilogue y = SRMSNorm(out) (.) u of Eq. 3 with Eq. 8 is applied to the rows
+// before they leave (job.u, job.y; job.out and job.rstd optional).
+template <bool REV, typename TOut, bool GATED>
 __global__ void __launch_bounds__(W_THREADS, 1)
 tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps maps1,
                const __grid_constant__ TcArgs args, const __grid_constant__ DecayTable tab) {
@@ -148,7 +206,8 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   const int nblk = (seg_t1 - seg_t0 + 127) >> 7;
   const int edge_len = seg_t1 - seg_t0 - (nblk - 1) * 128;  // tokens of the block that holds the segment's last ones
   const float s2 = (float)tab.s2[bh % args.H];
-  const bool has_entry = job.entry != nullptr;  // without one the first block has no O_inter: M2 is skipped
+  const int before = REV ? nseg_own - 1 - seg : seg;  // segments walked before this one
+  const bool has_entry = job.z_in != nullptr || before > 0;  // else the first block has no O_inter: M2 is skipped
   const bool want_final = job.final_out && (REV ? seg == 0 : seg == nseg_own - 1);
 
   if (tid == 0) {
@@ -157,6 +216,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       if (i == W_M1_OK0 || i == W_M1_OK1) count = 18;
       if (i == W_M2_OK || i == W_M4_OK) count = 24;
       if (i == W_M3_OK) count = 16;
+      if (i == W_GATE0 || i == W_GATE1) count = 4;
       mbar_init(&sm.bars[i], count);
     }
     sm.abort = 0;
@@ -173,6 +233,10 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       sm.fout[REV ? set : 0][i] = i < Cr ? ex2_approx(-s2 * (float)(Cr - 1 - i)) : 0.f;
     } else if (set == 0) {
       sm.fout[0][i] = ex2_approx(-s2 * (float)(i + 1));
+    }
+    if (x >= 192 && x < 195) {
+      const int len = x == 192 ? args.seg_len : x == 193 ? n_tok - (nseg_own - 1) * args.seg_len : REV ? n_tok - seg_t1 : seg_t0;
+      sm.gseg[x - 192] = decay_pow_d(tab.s2[bh % args.H], (double)len);
     }
     if (x < 16) sm.ptab[x] = ex2_approx(-s2 * (float)(15 - x));
   }
@@ -290,7 +354,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     }
   } else if (warp < 20) {
     // ------------------------------------ workers ------------------------------------
-    set_regs<W_REGS_W, W_REGS_LAUNCH>();
+    set_regs<WRegs<GATED>::W, W_REGS_LAUNCH>();
     const int q = warp & 3;                // quarter of tensor memory: score rows / value columns q * 32 + lane
     const int w4 = (warp - 4) >> 2;        // this warp's share within the quarter
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
@@ -366,13 +430,58 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       tc_fence_before_sync();
     };
 
-    if (has_entry) {
-      const float* src = job.entry + ((size_t)bh * args.nseg + seg) * (128 * 128) + (size_t)(w4 * 32) * 128 + q * 32 + lane;
+    // The state entering the segment: z = z_in, then z <- lambda^(length) z + local state for the segments before this one.
+    // Only the nearest `near` of them are read: through so many whole segments the decay is below 2^-160, exactly zero in
+    // fp32.  Where a launch has made running sums of the slow heads' states (args.scanned), one state and z_in are enough.
+    // (A head that decays reads one state; a slow one all of them, about 1 us each, against 5 us for the extra launch.)
+    {
+      // (written so that the compiler does not know the zeros: with them it spilled the copies it made of this part)
 #pragma unroll
-      for (int x = 0; x < 32; ++x) zreg[x] = __ldg(src + x * 128);
-    } else {
+      for (int x = 0; x < 32; ++x) asm volatile("mov.b32 %0, 0;" : "=f"(zreg[x]));
+      auto add_state = [&](const float* src, bool transposed, float g) {
+        if (transposed) {
+          const float4* r4 = reinterpret_cast<const float4*>(src + (size_t)(q * 32 + lane) * 128 + w4 * 32);
 #pragma unroll
-      for (int x = 0; x < 32; ++x) zreg[x] = 0.f;
+          for (int x = 0; x < 8; ++x) {
+            const float4 v = __ldg(r4 + x);
+            zreg[4 * x + 0] = fmaf(g, zreg[4 * x + 0], v.x);
+            zreg[4 * x + 1] = fmaf(g, zreg[4 * x + 1], v.y);
+            zreg[4 * x + 2] = fmaf(g, zreg[4 * x + 2], v.z);
+            zreg[4 * x + 3] = fmaf(g, zreg[4 * x + 3], v.w);
+          }
+        } else {
+          const float* r1 = src + (size_t)(w4 * 32) * 128 + q * 32 + lane;
+#pragma unroll
+          for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], __ldg(r1 + x * 128));
+        }
+      };
+      const float reach = state_reach(s2, args.seg_len);
+      const bool running = args.scanned && slow_head(s2, args.seg_len) && before > 0;
+      const int near = running ? 1 : ((float)before <= reach ? before : (int)reach + 1);
+      if ((near >= before || running) && job.z_in) add_state(job.z_in + (size_t)bh * (128 * 128), job.z_in_t, 0.f);
+      if (running) {
+#pragma unroll
+        for (int x = 0; x < 32; ++x) zreg[x] *= sm.gseg[2];
+        add_state(job.local + ((size_t)bh * args.nseg + (REV ? seg + 1 : seg - 1)) * (128 * 128), job.local_t, 1.f);
+      } else {
+#pragma unroll 1
+        for (int k = min(near, before); k >= 1; --k) {
+          const int p = REV ? seg + k : seg - k;
+          if (k >= 2 && !job.local_t) {  // two states' loads in flight
+            const float g1 = sm.gseg[p == nseg_own - 1 ? 1 : 0], g2 = sm.gseg[0];
+            const float* r1 = job.local + ((size_t)bh * args.nseg + p) * (128 * 128) + (size_t)(w4 * 32) * 128 + q * 32 + lane;
+            const float* r2 = r1 + (REV ? -1 : 1) * (128 * 128);
+            float v[32];
+#pragma unroll
+            for (int x = 0; x < 32; ++x) v[x] = __ldg(r1 + x * 128);
+#pragma unroll
+            for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g2, fmaf(g1, zreg[x], v[x]), __ldg(r2 + x * 128));
+            --k;
+            continue;
+          }
+          add_state(job.local + ((size_t)bh * args.nseg + p) * (128 * 128), job.local_t, sm.gseg[p == nseg_own - 1 ? 1 : 0]);
+        }
+      }
     }
     WARP_ARRIVE(W_M1_OK0);  // there is no earlier dZ to read
     if (has_entry) write_state_operand();
@@ -471,7 +580,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     }
   } else {
     // ------------------------------------ O group ------------------------------------
-    set_regs<W_REGS_O, W_REGS_LAUNCH>();
+    set_regs<WRegs<GATED>::O, W_REGS_LAUNCH>();
     const int q = warp & 3;
     const int th = (warp >= 24) ? 64 : 0;  // first of this warp's 64 tokens
     const uint32_t colO = tmem + ((uint32_t)(q * 32) << 16) + WCOL_O + th;
@@ -508,28 +617,99 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       const int t0 = seg_t0 + (REV ? (nblk - 1 - it) : it) * 128 + th;
       const int rows = seg_t1 - t0;  // tokens of this warp's 64 that exist (may be <= 0)
       TOut* dst = out + (size_t)t0 * args.sT;
+      // u of this warp's 64 tokens, two value columns to a register: lanes 0..15 hold token 2 x, lanes 16..31 token 2 x + 1
+      uint32_t upair[GATED ? 32 : 1];
+      if constexpr (GATED) {
+        const __nv_bfloat16* up = static_cast<const __nv_bfloat16*>(job.u) + head_off +
+                                  (size_t)(t0 + (lane >> 4)) * args.sT + q * 32 + (lane & 15) * 2;
+        const int mine = rows - (lane >> 4);
+#pragma unroll
+        for (int x = 0; x < 32; ++x) {
+          upair[x] = 0u;
+          if (2 * x < mine) upair[x] = load_u32_at(up, (uint32_t)args.sT * 4u, x);
+        }
+      }
       TC_WAIT_WARP(W_O_READY, it & 1, 25);
       tc_fence_after_sync();
       const uint32_t stride = (uint32_t)args.sT * (uint32_t)sizeof(TOut);
+      if constexpr (GATED) {
+        // Sums of squares of 64 tokens over this quarter's value columns (lanes), exchanged between the four quarters through
+        // shared memory once per block (beside M1 a read takes hundreds of clocks); then each quarter's warp reads its
+        // columns again, scales them and multiplies by u, which was fetched before M4.
+        // (The buffer is a part of the score tile that the forward walk never uses: keys 64.. of rows 0..15.  All warps have
+        // read a block's sums before M2 of the next block can start.)
+        float(*const g)[64] = reinterpret_cast<float(*)[64]>(&sm.p_hi[1][0]) + (th >> 6) * 4;
+        float* const mine = g[q];
 #pragma unroll 1
-      for (int pc = 0; pc < 2; ++pc) {  // 32 tokens at a time
-        uint32_t w[32];
-        tmem_ld_x32(colO + pc * 32, w);
-        tmem_ld_wait();
-        if (pc == 1) {
-          tc_fence_before_sync();
-          WARP_ARRIVE(W_M2_OK);  // M2 of the next block may overwrite O
-        }
-        const int here = rows - pc * 32;
-        if (here >= 32) {
+        for (int pc = 0; pc < 2; ++pc) {
+          uint32_t w[32];
+          tmem_ld_x32(colO + pc * 32, w);
+          tmem_ld_wait();
+          float sq[16], sr[16];
 #pragma unroll
-          for (int x = 0; x < 32; ++x) store_at(dst, stride, x, __uint_as_float(w[x]));
-        } else {
-#pragma unroll
-          for (int x = 0; x < 32; ++x)
-            if (x < here) store_at(dst, stride, x, __uint_as_float(w[x]));
+          for (int x = 0; x < 16; ++x) {
+            sq[x] = __uint_as_float(w[x]) * __uint_as_float(w[x]);
+            sr[x] = __uint_as_float(w[16 + x]) * __uint_as_float(w[16 + x]);
+          }
+          const float p0 = lane_sums16(sq, lane), p1 = lane_sums16(sr, lane);
+          // (lane l: token l >> 1 of either half; even lanes store the first, odd lanes the second)
+          mine[pc * 32 + ((lane & 1) << 4) + (lane >> 1)] = (lane & 1) ? p1 : p0;
         }
-        dst += 32 * args.sT;
+        WARP_ARRIVE(W_GATE0 + (th >> 6));
+        TC_WAIT_WARP(W_GATE0 + (th >> 6), it & 1, 26);
+        float scale[2];  // of tokens lane and 32 + lane
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int t = 32 * k + lane;
+          const float ss = (g[0][t] + g[1][t]) + (g[2][t] + g[3][t]);
+          scale[k] = ss > 0.f ? rsqrtf(ss * (1.f / 128.f)) : 0.f;
+          // rstd has the layout of the token tensors without the feature dimension
+          if (job.rstd && q == 0 && t < rows) job.rstd[(head_off + (size_t)(t0 + t) * args.sT) >> 7] = scale[k];
+        }
+        TOut* const ydst = static_cast<TOut*>(job.y) + head_off + (size_t)t0 * args.sT + q * 32 + lane;
+#pragma unroll
+        for (int pc = 0; pc < 4; ++pc) {
+          uint32_t w[16];
+          tmem_ld_x16(colO + pc * 16, w);
+          tmem_ld_wait();
+          if (pc == 3) {
+            tc_fence_before_sync();
+            WARP_ARRIVE(W_M2_OK);  // M2 of the next block may overwrite O
+          }
+#pragma unroll
+          for (int x = 0; x < 16; ++x) {
+            const int t = pc * 16 + x;
+            const float v = __uint_as_float(w[x]);
+            const uint32_t uw = __shfl_sync(0xffffffffu, upair[t >> 1], ((t & 1) << 4) + (lane >> 1));
+            const float ug = __uint_as_float((lane & 1) ? (uw & 0xffff0000u) : (uw << 16));
+            const float y = v * __shfl_sync(0xffffffffu, scale[t >> 5], t & 31) * ug;
+            if (t < rows) {
+              store_at(ydst, stride, t, y);
+              if (job.out) store_at(dst, stride, t, v);
+            }
+          }
+        }
+      } else {
+#pragma unroll 1
+        for (int pc = 0; pc < 2; ++pc) {  // 32 tokens at a time
+          uint32_t w[32];
+          tmem_ld_x32(colO + pc * 32, w);
+          tmem_ld_wait();
+          if (pc == 1) {
+            tc_fence_before_sync();
+            WARP_ARRIVE(W_M2_OK);  // M2 of the next block may overwrite O
+          }
+          const int here = rows - pc * 32;
+          if (here >= 32) {
+#pragma unroll
+            for (int x = 0; x < 32; ++x) store_at(dst, stride, x, __uint_as_float(w[x]));
+          } else {
+#pragma unroll
+            for (int x = 0; x < 32; ++x)
+              if (x < here) store_at(dst, stride, x, __uint_as_float(w[x]));
+          }
+          dst += 32 * args.sT;
+        }
       }
     }
   }
@@ -540,11 +720,11 @@ teardown:
   if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-template <bool REV, typename TOut>
+template <bool REV, typename TOut, bool GATED>
 cudaError_t launch_walk_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, const DecayTable& tab, cudaStream_t stream) {
   const size_t smem = sizeof(WSmem<REV>) + 1024;
   static_assert(sizeof(WSmem<REV>) + 1024 <= 232448, "shared memory of one SM");
-  auto kern = tc_walk_kernel<REV, TOut>;
+  auto kern = tc_walk_kernel<REV, TOut, GATED>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ta.njobs == 2 ? K_WALK_PAIR : K_WALK, stream);

@@ -373,6 +373,20 @@ __device__ __forceinline__ void umma_group_tsd(uint32_t d_tmem, uint32_t a_tmem,
       "n"(umma_kstep<BK>(5)), "n"(umma_kstep<BK>(6)), "n"(umma_kstep<BK>(7))
       : "memory");
 }
+// Four such steps (64 rows of K).
+template <bool BK>
+__device__ __forceinline__ void umma_group_tsd4(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi,
+                                                uint32_t idesc, uint32_t acc0, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred p, g, t;\n\t.reg .b64 db;\n\t.reg .b32 at, bl;\n\t"
+      "setp.ne.b32 g, %6, 0;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "mov.b64 db, {%2, %3};\n\t"
+      "@g tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t"
+      LA_UMMA_TS_STEP(8, %7) LA_UMMA_TS_STEP(16, %8) LA_UMMA_TS_STEP(24, %9)
+      "}" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc0), "r"(go),
+      "n"(umma_kstep<BK>(1)), "n"(umma_kstep<BK>(2)), "n"(umma_kstep<BK>(3))
+      : "memory");
+}
 #undef LA_UMMA_TS_STEP
 // Four K steps of D[e, i] (+)= A[e, j] B[j, i] where B[j, i] = 0 for i < j (REV: for i > j): step k covers
 // j = 16 k .. 16 k + 15 and touches only the columns of D that it can change.  Steps K0, K0 + 1, .. (REV: K0, K0 - 1, ..),

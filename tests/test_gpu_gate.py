@@ -120,6 +120,16 @@ def test_gated_forward_ragged_states_and_options(N, d, out_dtype):
         assert_close(kv_out, ref_kv, TOL_BF16, "kv_out")
 
 
+def test_gated_forward_large_without_o():
+    """fp32 y just past the L2 size and no o: the epilogue inside the walk, ragged last block, several segments, rstd."""
+    B, H, N, d = 1, 32, 7800, 128
+    q, k, v, _ = inputs.make_qkvdo(B, H, N, d, d, seed=31, with_do=False)
+    u = draw_gate((B, H, N, d), seed=32)
+    lam = inputs.decay_rates(H, 0.9)
+    got = run_gated(q, k, v, u, lam, want_o=False)
+    check_gated(q, k, v, u, lam, got, TOL_BF16)
+
+
 def test_gated_forward_fp32_path():
     w = inputs.make_workload("pr1_ref")
     u = draw_gate(tuple(w["v"].shape), seed=3, dtype=torch.float32)
