@@ -55,6 +55,7 @@ struct Plan {
   bool tensor;      // tensor-core kernels
   bool chains;      // the walk chains the segments' local states itself (tensor-core kernels at d = 128): no scan ...
   bool scanned;     // ... but running sums of the slowly decaying heads' states
+  bool rows;        // CUDA-core kernels: short segments, every row tile by itself (no chain of blocks)
   int precision;    // LA_SPLIT_* bits (tensor path)
   Packed pk;        // start == NULL: dense batch
 };
@@ -107,7 +108,10 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
     // launch that makes the states, with what each further state costs to write, read and chain.  Measured, forward plus
     // backward: 3 x 8 heads x 3001 tokens 172 us with 1536-token segments, 141 with 512; 8 heads x 2048 118 with 1024, 92
     // with 512, 126 with 128; 2 x 16 x 8192 289 with 2048, 344 with 1024 (the model: 49.7, 34.5 / 38, 29, 33 / 85, 97).
-    // Elsewhere (d = 64, fp32, packed batches): waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.
+    // CUDA-core kernels: one segment up to 256 tokens, else 128-token segments.  Forward plus backward in fp32: 2 heads x 256
+    // tokens, d = 64, 38 us as one segment and 57 in two; 4 x 512 85 and 65; 2 x 2048 205 with 512-token segments, 122 with
+    // 256, 81 with 128; 16 x 2048, d = 128, 946, 652 and 488.
+    // Elsewhere (d = 64, packed batches): waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.
     auto choose = [&](long most, long unit_limit, auto cost_of) {
       if (most < 1) most = 1;
       if (most > 1024) most = 1024;
@@ -127,9 +131,11 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
     };
     auto waves = [](long units) { return (double)((units + 147) / 148); };
     long best_n = choose(s->N / 1024, 1L << 40, [&](long nseg, long blocks) { return waves(p->BH * nseg) * (blocks + 2); });
-    if (p->chains && !packed) {
-      // (la_fwd_noalloc's scratch holds the states of 256 segments: shapes that fit it with long segments still do)
-      const long limit = std::max(p->BH * best_n, (long)(LA_NOALLOC_SCRATCH_BYTES / (2 * s->d * s->e * sizeof(float))));
+    // (la_fwd_noalloc's scratch holds so many segments' states, 256 at d = 128: shapes that fit it with long segments still do)
+    const long limit = std::max(p->BH * best_n, (long)(LA_NOALLOC_SCRATCH_BYTES / (2 * s->d * s->e * sizeof(float))));
+    if (!p->tensor && !packed) {
+      if (s->N > 256) best_n = choose((s->N + 127) / 128, limit, [&](long, long blocks) { return (double)blocks; });
+    } else if (p->chains && !packed) {
       best_n = choose(s->N / 128, limit, [&](long nseg, long blocks) {
         const double units = (double)p->BH * nseg;
         return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 1.3) +
@@ -140,6 +146,7 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
   }
   p->seg_len = (int)seg_len;
   p->nseg = (int)((s->N + seg_len - 1) / seg_len);
+  p->rows = !p->tensor && p->seg_len <= ROWS_MAX_SEG;
   if (p->nseg > 1024) return LA_ERR_UNSUPPORTED;  // the state scan keeps one decay factor per segment on chip
   return LA_OK;
 }
@@ -300,6 +307,7 @@ cudaError_t run_walk(const la_shape* s, const Plan& p, const DecayTable& tab, co
                      int reverse, cudaStream_t st) {
   const OpArgs args = walk_args(s, p, a, b, c, out, from, final_out, reverse);
   if (p.tensor) return launch_tc_walk(args, tab, s->d, (int)s->out_dtype, p.precision, st);
+  if (p.rows) return launch_simt_rows(&args, 1, tab, s->d, (int)s->in_dtype, (int)s->out_dtype, st);
   return launch_simt_walk(args, tab, s->d, s->e, (int)s->in_dtype, (int)s->out_dtype, st);
 }
 
@@ -512,7 +520,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     LA_TRY_CUDA(run_scan(shape, p, tab, buf_kvt, nullptr, kv_in, true, 0, cs));
     from_q.entry = buf_kvt;
   }
-  LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
+  if (!p.rows) LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
 
   // dV = rev(a = K, b = Q, c = dO) carries dKV; dK = rev(a = V, b = dO, c = Q) carries dKV^T.
   Carried from_v, from_k;
@@ -526,7 +534,12 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     from_v.entry = buf_e;
     from_k.entry = buf_et;
   }
-  if (p.tensor) {
+  if (p.rows) {
+    const OpArgs walks[3] = {walk_args(shape, p, d_o, v, k, dq, from_q, nullptr, 0),
+                             walk_args(shape, p, k, q, d_o, dv, from_v, grad_kv_in, 1),
+                             walk_args(shape, p, v, d_o, q, dk, from_k, nullptr, 1)};
+    LA_TRY_CUDA(launch_simt_rows(walks, 3, tab, shape->d, (int)shape->in_dtype, (int)shape->out_dtype, cs));
+  } else if (p.tensor) {
     // both reverse walks in one launch: together they read Q, K, V and dO, and the thread blocks of the two are
     // interleaved so that each of those tiles comes from HBM once (Algorithm 4 accumulates dK_j and dV_j in the
     // same outer iteration for the same reason)

@@ -105,6 +105,10 @@ enum { DT_BF16 = 0, DT_F32 = 1 };
 // Each returns cudaGetLastError() of its launch.
 cudaError_t launch_simt_walk(const OpArgs& args, const DecayTable& tab, int Da, int Ec, int in_dt,
                              int out_dt, cudaStream_t stream);
+// Up to three independent walks in one launch, with segments of at most ROWS_MAX_SEG tokens.
+constexpr int ROWS_MAX_SEG = 512;
+cudaError_t launch_simt_rows(const OpArgs* jobs, int njobs, const DecayTable& tab, int D, int in_dt, int out_dt,
+                             cudaStream_t stream);
 cudaError_t launch_simt_prepass(const OpArgs& args, const DecayTable& tab, int Da, int Ec, int in_dt,
                                 cudaStream_t stream);
 cudaError_t launch_scan(const ScanArgs& args, const DecayTable& tab, cudaStream_t stream);

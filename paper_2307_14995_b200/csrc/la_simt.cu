@@ -8,6 +8,8 @@
 // (batch*head, segment).  Shared memory holds the a/b/c tiles (a and b also
 // transposed so that every inner loop reads consecutive addresses), the masked
 // score tile and the Da x Ec state.
+#include <algorithm>
+
 #include "la_common.cuh"
 
 namespace la {
@@ -354,6 +356,265 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanArgs args, const De
   }
 }
 
+// The walk of segments of at most ROWS_MAX_SEG tokens without a chain of blocks: out = P c over the whole segment plus
+// diag(f_out) a Z, each 32-row tile of it by a thread block of its own, and the final state in 32-row tiles too.  All of it
+// is one loop, acc[32, EC] += w[j, 32]^T t[j, EC] over 32-row tiles t: rows of c with w the masked scores, rows of Z with w
+// the decayed a, or (final state) rows of c with w the decayed b.
+// A walk that carries the state from block to block is bound by that chain where it has few heads: 8 us a block at d = 64
+// with two thread blocks on the chip.  Here the work grows with the square of the segment, but all tiles run at once, and the
+// walks of a launch do too (B = 1, H = 2, N = 256, d = 64 in fp32, forward
+// plus backward: 240 us before, 38 now; with N = 2048 and 128-token segments 1155 and 81).
+// 128 threads and 60 KB at d = 128, so that three thread blocks share an SM; the next tiles are loaded into registers while
+// the present ones are multiplied.
+constexpr int ROWS_THREADS = 128;
+constexpr int ROWS_MAX_JOBS = 3;
+static_assert(ROWS_MAX_SEG % C == 0, "whole tiles");
+
+struct RowsArgs {
+  OpArgs job[ROWS_MAX_JOBS];
+  int first_block[ROWS_MAX_JOBS + 1];  // thread blocks of job j: first_block[j] .. first_block[j + 1] - 1
+  int units[ROWS_MAX_JOBS];            // how many of them make rows; the others make the final state
+};
+
+template <int D>
+struct RowsSmem {
+  float a[C][D + 4];   // rows of a (final state: unused)
+  float b[C][D + 4];
+  float t[C][D];       // rows of c or Z
+  float w[C][AP];      // w[j][i]
+  float f_out[C];
+  float dtab[ROWS_MAX_SEG + 1];  // lambda^n
+};
+
+// 32 rows of D values into registers, 16 bytes (fp32) at a time; rows past `valid` are zero.
+template <typename TIn, int D>
+__device__ __forceinline__ void fetch_tile(float4 (&x)[D / 16], const TIn* src, long long row_stride, int valid) {
+#pragma unroll
+  for (int n = 0; n < D / 16; ++n) {
+    const int idx = threadIdx.x + n * ROWS_THREADS, row = idx / (D / 4), col = idx % (D / 4) * 4;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (row < valid) Vec4<TIn>::load(src + (size_t)row * row_stride + col, v);
+    x[n] = make_float4(v[0], v[1], v[2], v[3]);
+  }
+}
+template <int D, int W>
+__device__ __forceinline__ void put_tile(float (*dst)[W], const float4 (&x)[D / 16]) {
+#pragma unroll
+  for (int n = 0; n < D / 16; ++n) {
+    const int idx = threadIdx.x + n * ROWS_THREADS;
+    *reinterpret_cast<float4*>(&dst[idx / (D / 4)][idx % (D / 4) * 4]) = x[n];
+  }
+}
+
+template <typename TIn, typename TOut, int D>
+__global__ void __launch_bounds__(ROWS_THREADS)
+simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ DecayTable tab) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  RowsSmem<D>& sm = *reinterpret_cast<RowsSmem<D>*>(smem_raw);
+  const int tid = threadIdx.x;
+  int jb = 0;
+  while (jb + 1 < ROWS_MAX_JOBS && (int)blockIdx.x >= all.first_block[jb + 1]) ++jb;
+  const OpArgs& args = all.job[jb];
+  int unit = (int)blockIdx.x - all.first_block[jb];
+  const bool rev = args.reverse != 0;
+  const bool state = unit >= all.units[jb];
+  const int per_seg = (args.seg_len + C - 1) / C;
+  int bh, seg, tile;
+  if (state) {
+    unit -= all.units[jb];
+    tile = unit % (D / C);
+    bh = unit / (D / C);
+    seg = rev ? 0 : args.nseg - 1;
+  } else {
+    // the row tiles with the most tiles to add up first
+    tile = unit / (args.BH * args.nseg);
+    if (!rev) tile = per_seg - 1 - tile;
+    seg = unit % args.nseg;
+    bh = unit / args.nseg % args.BH;
+  }
+  const double s2 = tab.s2[bh % args.H];
+  const int seg_t0 = seg * args.seg_len;
+  const int L = min(args.N, seg_t0 + args.seg_len) - seg_t0;
+  if (!state && tile * C >= L) return;
+
+  const size_t head_off = (size_t)(bh / args.H) * args.sB + (size_t)(bh % args.H) * args.sH + (size_t)seg_t0 * args.sT;
+  const long long sT = args.sT;
+  const TIn* a = static_cast<const TIn*>(args.a) + head_off;
+  const TIn* b = static_cast<const TIn*>(args.b) + head_off;
+  const TIn* c = static_cast<const TIn*>(args.c) + head_off;
+  const float* Z = args.entry ? args.entry + ((size_t)bh * args.nseg + seg) * D * D : nullptr;
+  const int ntile = (L + C - 1) / C;
+  // tiles of c to add up: the row tile's own first and then away from it; for the state towards the segment's edge
+  const int step = (rev != state) ? 1 : -1;  // (rows: reverse looks at later tokens)
+  int count;
+  if (state) count = ntile;
+  else count = rev ? ntile - tile : tile + 1;
+  const int first = state ? (rev ? ntile - 1 : 0) : tile;
+  const int dir = state ? (rev ? -1 : 1) : step;
+
+  float4 nb[D / 16], nc[D / 16];
+  fetch_tile<TIn, D>(nb, b + (size_t)first * C * sT, sT, L - first * C);
+  fetch_tile<TIn, D>(nc, c + (size_t)first * C * sT, sT, L - first * C);
+  if (!state) {
+    float4 na[D / 16];
+    fetch_tile<TIn, D>(na, a + (size_t)tile * C * sT, sT, L - tile * C);
+    put_tile<D, D + 4>(sm.a, na);
+  }
+  for (int n = tid; n <= L; n += ROWS_THREADS) sm.dtab[n] = decay_pow_d(s2, (double)n);
+  __syncthreads();
+
+  constexpr int EM = D / 16;  // value columns of a thread
+  const int i4 = (tid / 16) * 4, e0 = (tid % 16) * 4;
+  float acc[4][EM];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int m = 0; m < EM; ++m) acc[r][m] = 0.f;
+  // acc += w^T t over 32 rows; a thread has rows i4 .. i4 + 3 and columns e0 .. e0 + 3 (d = 128: and 64 + those)
+  const auto accumulate = [&]() {
+#pragma unroll 4
+    for (int j = 0; j < C; ++j) {
+      const float4 w = *reinterpret_cast<const float4*>(&sm.w[j][i4]);
+      const float wr[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int g = 0; g < EM / 4; ++g) {
+        const float4 t = *reinterpret_cast<const float4*>(&sm.t[j][e0 + 64 * g]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          acc[r][4 * g + 0] = fmaf(wr[r], t.x, acc[r][4 * g + 0]);
+          acc[r][4 * g + 1] = fmaf(wr[r], t.y, acc[r][4 * g + 1]);
+          acc[r][4 * g + 2] = fmaf(wr[r], t.z, acc[r][4 * g + 2]);
+          acc[r][4 * g + 3] = fmaf(wr[r], t.w, acc[r][4 * g + 3]);
+        }
+      }
+    }
+  };
+
+  for (int n = 0; n < count; ++n) {
+    const int jt = first + n * dir;
+    put_tile<D, D + 4>(sm.b, nb);
+    put_tile<D, D>(sm.t, nc);
+    __syncthreads();
+    // the next tile, unless every weight past this one is zero in fp32
+    bool more = n + 1 < count;
+    if (!state && more) more = sm.dtab[n * C + 1] != 0.f;
+    if (more) {
+      const int nt = jt + dir;
+      fetch_tile<TIn, D>(nb, b + (size_t)nt * C * sT, sT, L - nt * C);
+      fetch_tile<TIn, D>(nc, c + (size_t)nt * C * sT, sT, L - nt * C);
+    }
+    if (state) {
+      for (int x = tid; x < C * C; x += ROWS_THREADS) {
+        const int j = x / C, i = x % C, t = jt * C + j;
+        sm.w[j][i] = t < L ? sm.b[j][tile * C + i] * sm.dtab[rev ? t + 1 : L - 1 - t] : 0.f;
+      }
+    } else {
+      // scores: a thread has rows i2, i2 + 1 and columns jc + 8 x
+      const int i2 = (tid / 8) * 2, jc = tid % 8;
+      float s[2][4];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) s[r][x] = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < D; k += 4) {
+        float4 av[2], bv[4];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) av[r] = *reinterpret_cast<const float4*>(&sm.a[i2 + r][k]);
+#pragma unroll
+        for (int x = 0; x < 4; ++x) bv[x] = *reinterpret_cast<const float4*>(&sm.b[jc + 8 * x][k]);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            s[r][x] = fmaf(av[r].x, bv[x].x, s[r][x]);
+            s[r][x] = fmaf(av[r].y, bv[x].y, s[r][x]);
+            s[r][x] = fmaf(av[r].z, bv[x].z, s[r][x]);
+            s[r][x] = fmaf(av[r].w, bv[x].w, s[r][x]);
+          }
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int i = i2 + r, j = jc + 8 * x;
+          const int dist = rev ? (jt - tile) * C + j - i : (tile - jt) * C + i - j;
+          // a select, not a multiply by zero: masked-out tokens can never leak
+          sm.w[j][i] = dist >= 0 && jt * C + j < L ? s[r][x] * sm.dtab[min(dist, L)] : 0.f;
+        }
+    }
+    __syncthreads();
+    accumulate();
+    __syncthreads();
+    if (!more) break;
+  }
+
+  if (state) {
+    // state leaving the last segment: lambda^L Z + sum
+    float* dst = args.final_out + (size_t)bh * D * D + (size_t)tile * C * D;
+    const float g = sm.dtab[L];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int gq = 0; gq < EM / 4; ++gq) {
+        const size_t at = (size_t)(i4 + r) * D + e0 + 64 * gq;
+        float4 z = Z ? *reinterpret_cast<const float4*>(Z + (size_t)tile * C * D + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(dst + at) = make_float4(fmaf(g, z.x, acc[r][4 * gq]), fmaf(g, z.y, acc[r][4 * gq + 1]),
+                                                           fmaf(g, z.z, acc[r][4 * gq + 2]), fmaf(g, z.w, acc[r][4 * gq + 3]));
+      }
+    return;
+  }
+  if (Z) {
+    const int at = tile * C;  // decay of row i to the entry state
+    const float lead = sm.dtab[rev ? max(L - at - C, 0) : at + 1];
+    if (lead != 0.f) {
+      for (int k0 = 0; k0 < D; k0 += C) {
+        float4 nz[D / 16];
+        fetch_tile<float, D>(nz, Z + (size_t)k0 * D, D, C);
+        put_tile<D, D>(sm.t, nz);
+        for (int x = tid; x < C * C; x += ROWS_THREADS) {
+          const int k = x / C, i = x % C;
+          const int dist = rev ? L - 1 - (at + i) : at + i + 1;
+          sm.w[k][i] = dist >= 0 && dist <= L ? sm.a[i][k0 + k] * sm.dtab[dist] : 0.f;
+        }
+        __syncthreads();
+        accumulate();
+        __syncthreads();
+      }
+    }
+  }
+  TOut* out = static_cast<TOut*>(args.out) + head_off;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int i = tile * C + i4 + r;
+    if (i >= L) continue;
+#pragma unroll
+    for (int g = 0; g < EM / 4; ++g) {
+      const float v[4] = {acc[r][4 * g], acc[r][4 * g + 1], acc[r][4 * g + 2], acc[r][4 * g + 3]};
+      Vec4<TOut>::store(out + (size_t)i * sT + e0 + 64 * g, v);
+    }
+  }
+}
+
+template <typename TIn, typename TOut, int D>
+cudaError_t launch_rows_t(const RowsArgs& ra, const DecayTable& tab, cudaStream_t stream) {
+  const size_t smem = sizeof(RowsSmem<D>);
+  auto kern = simt_rows_kernel<TIn, TOut, D>;
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  KernelTimer timer(K_WALK, stream);
+  kern<<<(unsigned)ra.first_block[ROWS_MAX_JOBS], ROWS_THREADS, smem, stream>>>(ra, tab);
+  count_launch();
+  return cudaGetLastError();
+}
+template <int D>
+cudaError_t launch_rows_dims(const RowsArgs& ra, const DecayTable& tab, int in_dt, int out_dt, cudaStream_t stream) {
+  if (in_dt == DT_F32 && out_dt == DT_F32) return launch_rows_t<float, float, D>(ra, tab, stream);
+  if (in_dt == DT_BF16 && out_dt == DT_F32) return launch_rows_t<__nv_bfloat16, float, D>(ra, tab, stream);
+  if (in_dt == DT_BF16 && out_dt == DT_BF16) return launch_rows_t<__nv_bfloat16, __nv_bfloat16, D>(ra, tab, stream);
+  return cudaErrorInvalidValue;
+}
+
 template <typename TIn, typename TOut, int DA, int EC>
 cudaError_t launch_walk_t(const OpArgs& args, const DecayTable& tab, cudaStream_t stream) {
   const size_t smem = sizeof(Smem<DA, EC>);
@@ -414,6 +675,29 @@ cudaError_t launch_simt_walk(const OpArgs& args, const DecayTable& tab, int Da, 
   if (Da == 64 && Ec == 64) return launch_walk_dims<64, 64>(args, tab, in_dt, out_dt, stream);
   if (Da == 128 && Ec == 128) return launch_walk_dims<128, 128>(args, tab, in_dt, out_dt, stream);
   return cudaErrorInvalidValue;
+}
+
+// Up to three independent walks (one launch) whose segments have at most ROWS_MAX_SEG tokens.
+cudaError_t launch_simt_rows(const OpArgs* jobs, int njobs, const DecayTable& tab, int D, int in_dt, int out_dt,
+                             cudaStream_t stream) {
+  if (njobs < 1 || njobs > ROWS_MAX_JOBS || (D != 64 && D != 128)) return cudaErrorInvalidValue;
+  RowsArgs ra{};
+  long at = 0;
+  for (int j = 0; j < ROWS_MAX_JOBS; ++j) {
+    ra.first_block[j] = (int)at;
+    if (j >= njobs) continue;
+    const OpArgs& a = jobs[j];
+    if (a.seg_len > ROWS_MAX_SEG) return cudaErrorInvalidValue;
+    const long tiles = (std::min(a.seg_len, a.N) + C - 1) / C;
+    const long rows = (long)a.BH * a.nseg * tiles, states = a.final_out ? (long)a.BH * (D / C) : 0;
+    ra.job[j] = a;
+    ra.job[j].seg_len = (int)std::min((long)a.seg_len, tiles * C);
+    ra.units[j] = (int)rows;
+    at += rows + states;
+    if (at > 2147483647L) return cudaErrorInvalidValue;
+  }
+  ra.first_block[ROWS_MAX_JOBS] = (int)at;
+  return D == 64 ? launch_rows_dims<64>(ra, tab, in_dt, out_dt, stream) : launch_rows_dims<128>(ra, tab, in_dt, out_dt, stream);
 }
 
 cudaError_t launch_simt_prepass(const OpArgs& args, const DecayTable& tab, int Da, int Ec, int in_dt,

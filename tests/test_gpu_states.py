@@ -1,0 +1,67 @@
+"""States entering the segments of a long sequence (d = 128 tensor-core path) against the fp64 oracle: segments that one
+thread block sums, that a cluster shares, that the walk chains itself and that reach it as running sums.
+
+Tolerance: on-chip operands are two bf16 terms, 2^-17 of each product; a chain of 57 blocks in one fp32 accumulator adds up
+to 912 products with a relative error of 2^-24 of the running sum each.  Against RMS(ref), with |sum| up to 5 RMS: 2^-17 * 5 +
+912 * 2^-24 * 5 = 3.1e-4."""
+import pytest
+import torch
+
+from la_check import assert_close
+from oracle import la_oracle as orc
+from paper_2307_14995_b200 import binding as la
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,N,seg_len,lam", [
+    (1, 8500, 4224, [1.0, 0.9995, 0.9, 1e-30]),   # 33 blocks, unshared; ragged tail
+    (1, 4097, 2048, [1.0, 0.9995]),               # shared by a cluster; a tail of one token
+    (2, 1211, 128, [1.0, 0.999, 0.5]),            # one block a segment, ten segments: running sums
+    (1, 700, 128, [0.9, 1.0, 0.9995]),            # chained by the walk
+    (3, 3001, 0, [1.0, 0.98]),                    # the library's own plan
+])
+def test_states_entering_segments(B, N, seg_len, lam):
+    H = len(lam)
+    gen = torch.Generator().manual_seed(N)
+    q, k, v, do = [torch.randn(B, H, N, 128, generator=gen).bfloat16() for _ in range(4)]
+    kv_in, gko = [torch.randn(B, H, 128, 128, generator=gen) * 0.1 for _ in range(2)]
+    lam = torch.tensor(lam)
+    dev = [x.cuda() for x in (q, k, v, do, kv_in, gko)]
+    o, kv = la.fwd(*dev[:3], lam, out_dtype=torch.float32, kv_in=dev[4], want_state=True, seg_len=seg_len)
+    dq, dk, dv, gin = la.bwd(*dev[:4], lam, out_dtype=torch.float32, kv_in=dev[4], grad_kv_out=dev[5], want_state_grad=True,
+                             seg_len=seg_len)
+    torch.cuda.synchronize()
+    lam64 = lam.double().numpy()
+    ref = orc.fwd_rec(q, k, v, lam64, kv_in=kv_in, want_state=True)
+    ref += orc.bwd_rec(q, k, v, do, lam64, kv_in=kv_in, grad_kv_out=gko, want_state_grad=True)
+    for name, g, r in zip(("o", "kv", "dq", "dk", "dv", "gin"), (o, kv, dq, dk, dv, gin), ref):
+        assert_close(g, r, 3.1e-4, name)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N,seg_len,layout", [(1, 0, 0), (33, 0, 1), (256, 0, 0), (257, 0, 1), (700, 512, 0), (641, 640, 0)])
+def test_full_precision_rows(d, N, seg_len, layout):
+    """fp32 inputs: row tiles by themselves (segments up to 512 tokens) and the block-by-block walk (640).  Sums of at most
+    640 + d fp32 products each: 768 * 2^-24 of the largest partial sum, itself at most 2 RMS: 9.2e-5."""
+    H = 3
+    gen = torch.Generator().manual_seed(N)
+    q, k, v, do = [torch.randn(2, H, N, d, generator=gen) * d ** -0.5 for _ in range(4)]
+    kv_in, gko = [torch.randn(2, H, d, d, generator=gen) * 0.1 for _ in range(2)]
+    lam = torch.tensor([1.0, 0.97, 1e-20])
+    lam64 = lam.double().numpy()
+    ref = orc.fwd_rec(q, k, v, lam64, kv_in=kv_in, want_state=True)
+    ref += orc.bwd_rec(q, k, v, do, lam64, kv_in=kv_in, grad_kv_out=gko, want_state_grad=True)
+    dev = [x.cuda() for x in (q, k, v, do)]
+    if layout:
+        dev = [x.transpose(1, 2).contiguous() for x in dev]
+    shape = la.make_shape(2, H, N, d, d, torch.float32, torch.float32, seg_len, la.LA_PATH_SIMT,
+                          layout=la.LA_LAYOUT_BNHD if layout else la.LA_LAYOUT_BHND)
+    o, dq, dk, dv = [torch.empty_like(x) for x in dev]
+    kv, gin = [torch.empty(2, H, d, d, device="cuda") for _ in range(2)]
+    la.la_fwd(shape, *dev[:3], lam, o, kv_in.cuda(), kv, la.alloc_workspace(la.LA_OP_FWD, shape, "cuda"))
+    la.la_bwd(shape, *dev, lam, dq, dk, dv, kv_in.cuda(), gko.cuda(), gin, la.alloc_workspace(la.LA_OP_BWD, shape, "cuda"))
+    torch.cuda.synchronize()
+    back = (lambda x: x.transpose(1, 2)) if layout else (lambda x: x)
+    for name, g, r in zip(("o", "kv", "dq", "dk", "dv", "gin"), (back(o), kv, back(dq), back(dk), back(dv), gin), ref):
+        assert_close(g, r, 9.2e-5, name)
