@@ -111,7 +111,10 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
     // CUDA-core kernels: one segment up to 256 tokens, else 128-token segments.  Forward plus backward in fp32: 2 heads x 256
     // tokens, d = 64, 38 us as one segment and 57 in two; 4 x 512 85 and 65; 2 x 2048 205 with 512-token segments, 122 with
     // 256, 81 with 128; 16 x 2048, d = 128, 946, 652 and 488.
-    // Elsewhere (d = 64, packed batches): waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.
+    // Tensor cores at d = 64: the same waves, at about 2.5 us a block; pre-passes and scans take about 24 us and 0.17 us a
+    // state.  Measured: 8 heads x 777 62 us as one segment, 43 with 128-token segments; 8 x 2048 94 with 1024, 54 with 256;
+    // 16 x 4096 100 with 1024, 89 with 512; 4 x 16 x 2048 130 with 1024, 161 with 512.
+    // Packed batches: waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.
     auto choose = [&](long most, long unit_limit, auto cost_of) {
       if (most < 1) most = 1;
       if (most > 1024) most = 1024;
@@ -140,6 +143,11 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
         const double units = (double)p->BH * nseg;
         return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 1.3) +
                (nseg > 1 ? 2.0 * (4.0 + 0.01 * units + 0.6 * nseg) : 0.0);
+      });
+    } else if (!packed) {
+      best_n = choose((s->N + 127) / 128, limit, [&](long nseg, long blocks) {
+        const double units = (double)p->BH * nseg;
+        return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 0.67) + (nseg > 1 ? 9.6 + 0.068 * units : 0.0);
       });
     }
     seg_len = ((s->N + best_n - 1) / best_n + 127) / 128 * 128;

@@ -1,16 +1,12 @@
 // Tensor-core kernels of the generic decayed linear-attention operator for
-// bf16 inputs with Da = Ec = D, D = 128 or 64 (block formulas: la_common.cuh).  Two kernels share this file's
-// launchers: the half-width kernel below (every D = 64 launch, the state-only pre-pass at both head sizes, and the
-// D = 128 walk when an output is aligned to 16 but not 32 bytes), the walk of la_tc_walk.cuh (D = 128: one thread block
-// per (batch*head, segment), all value columns, operands formed on chip in tensor memory), which launch_walk_d prefers,
-// and la_tc_full.cuh, the D = 128 walk with the gate in its epilogue.  The text below describes the half-width kernel at
-// D = 128; the differences at D = 64 are described at the kernel's template parameter.
+// bf16 inputs with Da = Ec = D (block formulas: la_common.cuh).  D = 128: the walk of la_tc_walk.cuh and the segment states of
+// la_tc_state.cuh.  D = 64: the kernel below, as the walk and, state-only, as the pre-pass that makes the segment states.
 //
-// One thread block walks the 128-token blocks of one (batch*head, segment,
-// half of the value columns).  Per block it issues, on the 5th-generation
+// One thread block walks the 128-token blocks of one (batch*head, segment).
+// Per block it issues, on the 5th-generation
 // tensor cores (tcgen05.mma, fp32 accumulators in tensor memory):
-//   M1  S        = a b^T                          128x128, K = 128
-//   M2  O_inter  = a Z_hi (+ a Z_lo)              128x64,  K = 128   (state of the previous block)
+//   M1  S        = a b^T                          128x128, K = 64
+//   M2  O_inter  = a Z_hi (+ a Z_lo)              128x64,  K = 64    (state of the previous block)
 //   M3  dZ       = b^T fc_hi (+ b^T fc_lo)        128x64,  K = 128   (fc = diag(f_state) c; the state-only
 //                                                                      pre-pass uses one N = 128 product)
 //   M4  O_intra  = P_hi c (+ P_lo c)              128x64,  K = 128   (P = S (.) D, read from tensor memory)
@@ -74,6 +70,10 @@ namespace {
 using namespace ptx;
 
 constexpr int TC_THREADS = 768;
+// Registers per thread of the walk's warpgroups (one control, two P, two Z, one O), out of the 6 x 80 of the launch: with 80
+// each the walks spilled (bf16 pair at 1 x 16 x 32768 tokens 182 us, now 161; fp32 pair at 1 x 32 x 65536 587, now 573).
+constexpr int REGS_LAUNCH = 80, REGS_CTL = 24, REGS_P = 64, REGS_Z = 112, REGS_O = 104;
+static_assert(REGS_CTL + 2 * REGS_P + 2 * REGS_Z + REGS_O == 6 * REGS_LAUNCH && TC_THREADS == 6 * 128, "all that the launch has");
 constexpr int TMEM_COLS = 512;
 // tensor-memory columns: two S/P buffers, O_intra, two O_inter buffers, dZ
 constexpr uint32_t COL_S0 = 0, COL_S1 = 128, COL_OI = 256, COL_OE0 = 320, COL_OE1 = 384, COL_DZ = 448;
@@ -235,7 +235,7 @@ __device__ __forceinline__ void split8(const float (&x)[8], uint4& hi, uint4& lo
     if (lane == 0) mbar_arrive(&sm.bars[barid]);         \
   } while (0)
 
-template <bool REV, bool STATE_ONLY, typename TOut, int D, int NJOBS>
+template <bool REV, bool STATE_ONLY, typename TOut, int NJOBS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps maps1, const TcArgs args,
           const DecayTable tab) {
@@ -245,38 +245,27 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
   TcSmem& sm = *reinterpret_cast<TcSmem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // D = 128: two thread blocks per (head, segment), one per half of the value columns.  D = 64: one
-  // thread block; the feature halves 64..127 of the a and b tiles do not exist (the K steps over them are
-  // skipped, and the second b panel, which M3 reads as rows 64..127 of b^T, is zeroed once below), so rows
-  // 64..127 of the state stay zero and are neither loaded nor stored.
-  static_assert(D == 64 || D == 128, "feature dimension");
-  constexpr int KD = D / 16;  // K steps over the feature dimension
-  // With two jobs the thread blocks of one (head, segment) -- both jobs, both value halves -- have adjacent
+  // One thread block per (head, segment).  The second b panel, which M3 reads as rows 64..127 of b^T, does not exist and
+  // is zeroed once below, so rows 64..127 of the state stay zero and are neither loaded nor stored.
+  constexpr int D = 64, KD = D / 16;  // K steps over the feature dimension
+  // With two jobs the two thread blocks of one (head, segment) have adjacent
   // indices, so they run at the same time and share their tiles through L2.
   const int jobid = (NJOBS == 2) ? (int)(blockIdx.x & 1) : 0;
   const unsigned bidx = (NJOBS == 2) ? (blockIdx.x >> 1) : blockIdx.x;
-  TcJob job = args.job[0];
-  if (NJOBS == 2 && jobid) job = args.job[1];
+  // (only the fields that are used: with a copy of the whole struct the fp32 forward walk spilled, 306 us against 288)
+  struct { const void* c; const float* entry; float* final_out; } job = {args.job[0].c, args.job[0].entry, args.job[0].final_out};
+  if (NJOBS == 2 && jobid) job = {args.job[1].c, args.job[1].entry, args.job[1].final_out};
   const CUtensorMap* const tm_a = (NJOBS == 2 && jobid) ? &maps1.a : &maps0.a;
   const CUtensorMap* const tm_b = (NJOBS == 2 && jobid) ? &maps1.b : &maps0.b;
   const CUtensorMap* const tm_c = (NJOBS == 2 && jobid) ? &maps1.c : &maps0.c;
   const CUtensorMap* const tm_out = (NJOBS == 2 && jobid) ? &maps1.out : &maps0.out;
-  const int ehalf = (D == 128) ? (int)(bidx & 1) : 0;
-  const int segid = (D == 128) ? (int)(bidx >> 1) : (int)bidx;
-  const int seg = segid % args.nseg;
-  int bh = segid / args.nseg;
-  if (args.seq_order) bh = args.seq_order[bh / args.H] * args.H + bh % args.H;  // packed batch: longest sequences first
-  const int hh_ = bh % args.H;  // head coordinate of the 4-D tensor maps
-  // Packed batch (state-only kernel; the walk of a packed batch is the full-width kernel's): entry bh / H is a
-  // sequence of its own length starting at token tok0 of one [tokens, H, D] tensor, the maps' batch coordinate is 0.
-  const int n_tok = args.seq_len ? args.seq_len[bh / args.H] : args.N;
-  const int tok0 = args.seq_start ? args.seq_start[bh / args.H] : 0;
-  const int bb_ = args.seq_start ? 0 : bh / args.H;
-  if (seg * args.seg_len >= n_tok) return;  // the grid covers the longest sequence; nothing has been set up yet
-  const size_t head_off = (size_t)bb_ * args.sB + (size_t)hh_ * args.sH + (size_t)tok0 * args.sT;
+  const int seg = (int)bidx % args.nseg;
+  const int bh = (int)bidx / args.nseg;
+  const int hh_ = bh % args.H, bb_ = bh / args.H;  // head and batch coordinates of the 4-D tensor maps
+  const size_t head_off = (size_t)bb_ * args.sB + (size_t)hh_ * args.sH;
   const int seg_t0 = seg * args.seg_len;
-  const int seg_t1 = min(n_tok, seg_t0 + args.seg_len);
-  const float s2 = (float)tab.s2[bh % args.H];
+  const int seg_t1 = min(args.N, seg_t0 + args.seg_len);
+  const float s2 = (float)tab.s2[hh_];
   int nblk = (seg_t1 - seg_t0 + 127) >> 7;
   int it0 = 0;  // forward pre-pass: index of the first block that is walked
   if (STATE_ONLY && s2 > 0.f) {
@@ -328,14 +317,12 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
     tmem_alloc(&sm.tmem_slot, TMEM_COLS);
     tmem_relinquish();
   }
-  if (D == 64) {
-    for (int i = tid; i < 2 * 1024; i += TC_THREADS)
-      reinterpret_cast<uint4*>(&sm.st[i >> 10].b[1][0])[i & 1023] = make_uint4(0u, 0u, 0u, 0u);
-    if (STATE_ONLY)  // the third load stage keeps its b tile where the walk kernel has stage 0's a tile
-      for (int i = tid; i < 1024; i += TC_THREADS)
-        reinterpret_cast<uint4*>(&sm.st[0].a[1][0])[i] = make_uint4(0u, 0u, 0u, 0u);
-    fence_proxy_async_smem();
-  }
+  for (int i = tid; i < 2 * 1024; i += TC_THREADS)
+    reinterpret_cast<uint4*>(&sm.st[i >> 10].b[1][0])[i & 1023] = make_uint4(0u, 0u, 0u, 0u);
+  if (STATE_ONLY)  // the third load stage keeps its b tile where the walk kernel has stage 0's a tile
+    for (int i = tid; i < 1024; i += TC_THREADS)
+      reinterpret_cast<uint4*>(&sm.st[0].a[1][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -350,136 +337,135 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
   auto b_tile = [&](int ls) { return ls == 0 ? &sm.st[0].b[0][0] : (ls == 1 ? &sm.st[1].b[0][0] : &sm.st[0].a[0][0]); };
   auto c_tile = [&](int ls) { return ls == 0 ? &sm.st[0].c[0] : (ls == 1 ? &sm.st[1].c[0] : &sm.st[1].a[0][0]); };
 
-  if (warp == 0) {
-    // ------------------------------------ TMA producer ------------------------------------
-    if (lane == 0) {
-      for (int it = 0; it < nblk; ++it) {
-        const int s = STATE_ONLY ? it % NLS : (it & 1);
-        const int use = STATE_ONLY ? it / NLS : (it >> 1);  // how often this stage has been used before
-        const uint32_t prev = (use - 1) & 1;                // parity of this stage's previous use
-        const int blk = REV ? (nblk - 1 - it) : (it + it0);
-        const int t0 = tok0 + seg_t0 + blk * 128;  // token coordinate of the maps
-        // State-only kernel: the tiles a few blocks ahead are pulled into L2 now, so that the loads proper are
-        // L2 hits (measured: 0.276 -> 0.245 ms per launch; the same in the walk kernel made it slower).
-        if (STATE_ONLY && it + NLS < nblk) {
-          const int tp = tok0 + seg_t0 + (REV ? (nblk - 1 - NLS - it) : (it + NLS + it0)) * 128;
-          tma_prefetch_4d(tm_b, 0, tp, hh_, bb_);
-          if (D == 128) tma_prefetch_4d(tm_b, 64, tp, hh_, bb_);
-          tma_prefetch_4d(tm_c, ehalf * 64, tp, hh_, bb_);
+  if (warp < 4) {
+    if (!STATE_ONLY) set_regs<REGS_CTL, REGS_LAUNCH>();
+    if (warp == 0) {
+      // ------------------------------------ TMA producer ------------------------------------
+      if (lane == 0) {
+        for (int it = 0; it < nblk; ++it) {
+          const int s = STATE_ONLY ? it % NLS : (it & 1);
+          const int use = STATE_ONLY ? it / NLS : (it >> 1);  // how often this stage has been used before
+          const uint32_t prev = (use - 1) & 1;                // parity of this stage's previous use
+          const int blk = REV ? (nblk - 1 - it) : (it + it0);
+          const int t0 = seg_t0 + blk * 128;  // token coordinate of the maps
+          // State-only kernel: the tiles a few blocks ahead are pulled into L2 now, so that the loads proper are
+          // L2 hits (measured: 0.276 -> 0.245 ms per launch; the same in the walk kernel made it slower).
+          if (STATE_ONLY && it + NLS < nblk) {
+            const int tp = seg_t0 + (REV ? (nblk - 1 - NLS - it) : (it + NLS + it0)) * 128;
+            tma_prefetch_4d(tm_b, 0, tp, hh_, bb_);
+            tma_prefetch_4d(tm_c, 0, tp, hh_, bb_);
+          }
+          if (STATE_ONLY) {
+            if (it >= NLS) TC_WAIT(B_FREE0 + s, prev, 1);
+            mbar_arrive_expect_tx(&sm.bars[FULL_B0 + s], D * 256);
+            tma_load_4d(b_tile(s), tm_b, &sm.bars[FULL_B0 + s], 0, t0, hh_, bb_);
+          } else {
+            Stage& stg = sm.st[s];
+            // walk kernel: the a and b tiles of a stage travel together (one barrier for both, FULL_B); A_FREE
+            // is committed after M2, the last product of the block that reads either of them
+            if (it >= 2) TC_WAIT(A_FREE0 + s, prev, 3);
+            mbar_arrive_expect_tx(&sm.bars[FULL_B0 + s], D * 512);
+            tma_load_4d(&stg.b[0][0], tm_b, &sm.bars[FULL_B0 + s], 0, t0, hh_, bb_);
+            tma_load_4d(&stg.a[0][0], tm_a, &sm.bars[FULL_B0 + s], 0, t0, hh_, bb_);
+          }
+          armed_b[s] = use + 1;
+          if (it >= NLS) TC_WAIT(C_FREE0 + s, prev, 2);
+          mbar_arrive_expect_tx(&sm.bars[FULL_C0 + s], 16384);
+          tma_load_4d(c_tile(s), tm_c, &sm.bars[FULL_C0 + s], 0, t0, hh_, bb_);
+          armed_c[s] = use + 1;
         }
-        if (STATE_ONLY) {
-          if (it >= NLS) TC_WAIT(B_FREE0 + s, prev, 1);
-          mbar_arrive_expect_tx(&sm.bars[FULL_B0 + s], D * 256);
-          tma_load_4d(b_tile(s), tm_b, &sm.bars[FULL_B0 + s], 0, t0, hh_, bb_);
-          if (D == 128) tma_load_4d(b_tile(s) + 128 * 64, tm_b, &sm.bars[FULL_B0 + s], 64, t0, hh_, bb_);
-        } else {
-          Stage& stg = sm.st[s];
-          // walk kernel: the a and b tiles of a stage travel together (one barrier for both, FULL_B); A_FREE
-          // is committed after M2, the last product of the block that reads either of them
-          if (it >= 2) TC_WAIT(A_FREE0 + s, prev, 3);
-          mbar_arrive_expect_tx(&sm.bars[FULL_B0 + s], D * 512);
-          tma_load_4d(&stg.b[0][0], tm_b, &sm.bars[FULL_B0 + s], 0, t0, hh_, bb_);
-          if (D == 128) tma_load_4d(&stg.b[1][0], tm_b, &sm.bars[FULL_B0 + s], 64, t0, hh_, bb_);
-          tma_load_4d(&stg.a[0][0], tm_a, &sm.bars[FULL_B0 + s], 0, t0, hh_, bb_);
-          if (D == 128) tma_load_4d(&stg.a[1][0], tm_a, &sm.bars[FULL_B0 + s], 64, t0, hh_, bb_);
-        }
-        armed_b[s] = use + 1;
-        if (it >= NLS) TC_WAIT(C_FREE0 + s, prev, 2);
-        mbar_arrive_expect_tx(&sm.bars[FULL_C0 + s], 16384);
-        tma_load_4d(c_tile(s), tm_c, &sm.bars[FULL_C0 + s], ehalf * 64, t0, hh_, bb_);
-        armed_c[s] = use + 1;
       }
-    }
-  } else if (warp == 1 && STATE_ONLY) {
-    // ------------------------------------ MMA issuer, state-only kernel ------------------------------------
-    // All 32 lanes run this loop converged (waits included); the tensor-core instructions and their commits
-    // take effect in the one elected lane only.  Issued this way the instructions cost the warp few issue
-    // slots (measured: 0.242 -> 0.229 ms per launch against the single-lane form the walk kernel uses,
-    // which did not gain from it).
-    {
-      constexpr uint32_t ID_MN64 = umma_idesc_bf16(128, 64, true, true);   // b^T (MN-major A) x MN-major B
-      constexpr uint32_t ID_MN128 = umma_idesc_bf16(128, 128, true, true); // same with [fc_hi | fc_lo], N = 128
-      constexpr uint32_t HI = UMMA_DESC_HI_SBO1024;
-      const uint32_t go = elect_one();
-      mma_elected = go;
-      // low descriptor halves (MN-major: 64-element chunks 16 KB apart); K step k adds k * 2 KB >> 4
-      const uint32_t bm0 = umma_desc_lo(smem_u32(b_tile(0)), 16384), bm1 = umma_desc_lo(smem_u32(b_tile(1)), 16384);
-      const uint32_t bm2 = umma_desc_lo(smem_u32(b_tile(2)), 16384);
-      const uint32_t fh_lo = umma_desc_lo(smem_u32(&sm.fc_hi[0]), 16384), zh_lo = umma_desc_lo(smem_u32(&sm.z_hi[0]), 16384);
-      for (int it = 0; it < nblk; ++it) {
-        const int ls = it % NLS;   // load stage of the b tile
-        const int s = it & 1;      // fc buffer
-        const uint32_t par2 = (it >> 1) & 1;
-        const uint32_t bm = ls == 0 ? bm0 : (ls == 1 ? bm1 : bm2);
-        const uint32_t fbuf_lo = s ? zh_lo : fh_lo;  // fc buffer of this iteration (hi then lo, 16 KB apart)
-        TC_WAIT_WARP(FULL_B0 + ls, (it / NLS) & 1, 4);
-        TC_WAIT_WARP(FC_READY0 + s, par2, 5);
-        tc_fence_after_sync();
-        // tensor memory is otherwise unused here, so hi and lo share one N = 128 instruction
-        // ([fc_hi | fc_lo]) into columns 0..127; the halves are summed at the end
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          umma_bf16_lh(tmem + COL_S0, bm + k * 128, fbuf_lo + k * 128, HI, split_c ? ID_MN128 : ID_MN64,
-                       (it > 0 || k > 0), go);
-        issued_mma = true;
-        umma_commit_if(&sm.bars[B_FREE0 + ls], go);
-        umma_commit_if(&sm.bars[FC_FREE0 + s], go);
-      }
-      umma_commit_if(&sm.bars[DZ_READY], go);
-    }
-  } else if (warp == 1) {
-    // ------------------------------------ MMA issuer, walk kernel ------------------------------------
-    // All 32 lanes run this loop converged (waits included); the tensor-core instructions and their commits take
-    // effect in one elected lane only, a whole K loop per instruction sequence (measured: 4 % faster than issuing
-    // from inside an `if (lane == 0)` region).
-    {
-      constexpr uint32_t ID_S = umma_idesc_bf16(128, 128, false, false);
-      constexpr uint32_t ID_KN = umma_idesc_bf16(128, 64, false, true);
-      constexpr uint32_t ID_MN64 = umma_idesc_bf16(128, 64, true, true);
-      constexpr uint32_t HI = UMMA_DESC_HI_SBO1024;
-      const uint32_t go = elect_one();
-      mma_elected = go;
-      // low descriptor halves.  K-major tiles (a, b in M1; a in M2): K step k adds (k >> 2) * 16 KB + (k & 3) * 32 B;
-      // MN-major tiles (b^T in M3, fc, the state operand, c): K step k adds k * 2 KB.
-      const uint32_t ak0 = umma_desc_lo(smem_u32(&sm.st[0].a[0][0]), 16), ak1 = umma_desc_lo(smem_u32(&sm.st[1].a[0][0]), 16);
-      const uint32_t bk0 = umma_desc_lo(smem_u32(&sm.st[0].b[0][0]), 16), bk1 = umma_desc_lo(smem_u32(&sm.st[1].b[0][0]), 16);
-      const uint32_t bm0 = umma_desc_lo(smem_u32(&sm.st[0].b[0][0]), 16384), bm1 = umma_desc_lo(smem_u32(&sm.st[1].b[0][0]), 16384);
-      const uint32_t cm0 = umma_desc_lo(smem_u32(&sm.st[0].c[0]), 16384), cm1 = umma_desc_lo(smem_u32(&sm.st[1].c[0]), 16384);
-      const uint32_t fh = umma_desc_lo(smem_u32(&sm.fc_hi[0]), 16384), fl = umma_desc_lo(smem_u32(&sm.fc_lo[0]), 16384);
-      const uint32_t zh = umma_desc_lo(smem_u32(&sm.z_hi[0]), 16384), zl = umma_desc_lo(smem_u32(&sm.z_lo[0]), 16384);
-      TC_WAIT_WARP(FULL_B0, 0, 7);
-      tc_fence_after_sync();
-      umma_group_ss<KD, true, true>(tmem + COL_S0, ak0, bk0, HI, ID_S, 0, go);
-      issued_mma = true;
-      umma_commit_if(&sm.bars[S_READY0], go);
-      for (int it = 0; it < nblk; ++it) {
-        const int s = it & 1;
-        const uint32_t par1 = it & 1, par2 = (it >> 1) & 1;
-        const uint32_t col_p = s ? COL_S1 : COL_S0;
-        const uint32_t aks = s ? ak1 : ak0, bms = s ? bm1 : bm0, cms = s ? cm1 : cm0;
-        const uint32_t akn = s ? ak0 : ak1, bkn = s ? bk0 : bk1;  // the other stage (next block)
-        TC_WAIT_WARP(Z_READY, par1, 12);
-        tc_fence_after_sync();
-        umma_group_ss<8, false, false>(tmem + COL_DZ, bms, fh, HI, ID_MN64, 0, go);
-        if (split_c) umma_group_ss<8, false, false>(tmem + COL_DZ, bms, fl, HI, ID_MN64, 1, go);
-        umma_commit_if(&sm.bars[DZ_READY], go);
-        const uint32_t col_oe = (it & 1) ? COL_OE1 : COL_OE0;
-        umma_group_ss<KD, true, false>(tmem + col_oe, aks, zh, HI, ID_KN, 0, go);
-        if (split_z) umma_group_ss<KD, true, false>(tmem + col_oe, aks, zl, HI, ID_KN, 1, go);
-        umma_commit_if(&sm.bars[A_FREE0 + s], go);
-        if (it + 1 < nblk) {
-          const int s1 = s ^ 1;
-          TC_WAIT_WARP(FULL_B0 + s1, ((it + 1) >> 1) & 1, 11);
+    } else if (warp == 1 && STATE_ONLY) {
+      // ------------------------------------ MMA issuer, state-only kernel ------------------------------------
+      // All 32 lanes run this loop converged (waits included); the tensor-core instructions and their commits
+      // take effect in the one elected lane only.  Issued this way the instructions cost the warp few issue
+      // slots (measured: 0.242 -> 0.229 ms per launch against the single-lane form the walk kernel uses,
+      // which did not gain from it).
+      {
+        constexpr uint32_t ID_MN64 = umma_idesc_bf16(128, 64, true, true);   // b^T (MN-major A) x MN-major B
+        constexpr uint32_t ID_MN128 = umma_idesc_bf16(128, 128, true, true); // same with [fc_hi | fc_lo], N = 128
+        constexpr uint32_t HI = UMMA_DESC_HI_SBO1024;
+        const uint32_t go = elect_one();
+        mma_elected = go;
+        // low descriptor halves (MN-major: 64-element chunks 16 KB apart); K step k adds k * 2 KB >> 4
+        const uint32_t bm0 = umma_desc_lo(smem_u32(b_tile(0)), 16384), bm1 = umma_desc_lo(smem_u32(b_tile(1)), 16384);
+        const uint32_t bm2 = umma_desc_lo(smem_u32(b_tile(2)), 16384);
+        const uint32_t fh_lo = umma_desc_lo(smem_u32(&sm.fc_hi[0]), 16384), zh_lo = umma_desc_lo(smem_u32(&sm.z_hi[0]), 16384);
+        for (int it = 0; it < nblk; ++it) {
+          const int ls = it % NLS;   // load stage of the b tile
+          const int s = it & 1;      // fc buffer
+          const uint32_t par2 = (it >> 1) & 1;
+          const uint32_t bm = ls == 0 ? bm0 : (ls == 1 ? bm1 : bm2);
+          const uint32_t fbuf_lo = s ? zh_lo : fh_lo;  // fc buffer of this iteration (hi then lo, 16 KB apart)
+          TC_WAIT_WARP(FULL_B0 + ls, (it / NLS) & 1, 4);
+          TC_WAIT_WARP(FC_READY0 + s, par2, 5);
           tc_fence_after_sync();
-          umma_group_ss<KD, true, true>(tmem + (s1 ? COL_S1 : COL_S0), akn, bkn, HI, ID_S, 0, go);
-          umma_commit_if(&sm.bars[S_READY0 + s1], go);
+          // tensor memory is otherwise unused here, so hi and lo share one N = 128 instruction
+          // ([fc_hi | fc_lo]) into columns 0..127; the halves are summed at the end
+  #pragma unroll
+          for (int k = 0; k < 8; ++k)
+            umma_bf16_lh(tmem + COL_S0, bm + k * 128, fbuf_lo + k * 128, HI, split_c ? ID_MN128 : ID_MN64,
+                         (it > 0 || k > 0), go);
+          issued_mma = true;
+          umma_commit_if(&sm.bars[B_FREE0 + ls], go);
+          umma_commit_if(&sm.bars[FC_FREE0 + s], go);
         }
-        TC_WAIT_WARP(P_READY0 + s, par2, 14);
-        TC_WAIT_WARP(FULL_C0 + s, par2, 15);
+        umma_commit_if(&sm.bars[DZ_READY], go);
+      }
+    } else if (warp == 1) {
+      // ------------------------------------ MMA issuer, walk kernel ------------------------------------
+      // All 32 lanes run this loop converged (waits included); the tensor-core instructions and their commits take
+      // effect in one elected lane only, a whole K loop per instruction sequence (measured: 4 % faster than issuing
+      // from inside an `if (lane == 0)` region).
+      {
+        constexpr uint32_t ID_S = umma_idesc_bf16(128, 128, false, false);
+        constexpr uint32_t ID_KN = umma_idesc_bf16(128, 64, false, true);
+        constexpr uint32_t ID_MN64 = umma_idesc_bf16(128, 64, true, true);
+        constexpr uint32_t HI = UMMA_DESC_HI_SBO1024;
+        const uint32_t go = elect_one();
+        mma_elected = go;
+        // low descriptor halves.  K-major tiles (a, b in M1; a in M2): K step k adds (k >> 2) * 16 KB + (k & 3) * 32 B;
+        // MN-major tiles (b^T in M3, fc, the state operand, c): K step k adds k * 2 KB.
+        const uint32_t ak0 = umma_desc_lo(smem_u32(&sm.st[0].a[0][0]), 16), ak1 = umma_desc_lo(smem_u32(&sm.st[1].a[0][0]), 16);
+        const uint32_t bk0 = umma_desc_lo(smem_u32(&sm.st[0].b[0][0]), 16), bk1 = umma_desc_lo(smem_u32(&sm.st[1].b[0][0]), 16);
+        const uint32_t bm0 = umma_desc_lo(smem_u32(&sm.st[0].b[0][0]), 16384), bm1 = umma_desc_lo(smem_u32(&sm.st[1].b[0][0]), 16384);
+        const uint32_t cm0 = umma_desc_lo(smem_u32(&sm.st[0].c[0]), 16384), cm1 = umma_desc_lo(smem_u32(&sm.st[1].c[0]), 16384);
+        const uint32_t fh = umma_desc_lo(smem_u32(&sm.fc_hi[0]), 16384), fl = umma_desc_lo(smem_u32(&sm.fc_lo[0]), 16384);
+        const uint32_t zh = umma_desc_lo(smem_u32(&sm.z_hi[0]), 16384), zl = umma_desc_lo(smem_u32(&sm.z_lo[0]), 16384);
+        TC_WAIT_WARP(FULL_B0, 0, 7);
         tc_fence_after_sync();
-        umma_group_ts8(tmem + COL_OI, tmem + col_p, cms, HI, ID_KN, 0, go);
-        if (split_p) umma_group_ts8(tmem + COL_OI, tmem + col_p + 8, cms, HI, ID_KN, 1, go);
-        umma_commit_if(&sm.bars[O_READY], go);
+        umma_group_ss<KD, true, true>(tmem + COL_S0, ak0, bk0, HI, ID_S, 0, go);
+        issued_mma = true;
+        umma_commit_if(&sm.bars[S_READY0], go);
+        for (int it = 0; it < nblk; ++it) {
+          const int s = it & 1;
+          const uint32_t par1 = it & 1, par2 = (it >> 1) & 1;
+          const uint32_t col_p = s ? COL_S1 : COL_S0;
+          const uint32_t aks = s ? ak1 : ak0, bms = s ? bm1 : bm0, cms = s ? cm1 : cm0;
+          const uint32_t akn = s ? ak0 : ak1, bkn = s ? bk0 : bk1;  // the other stage (next block)
+          TC_WAIT_WARP(Z_READY, par1, 12);
+          tc_fence_after_sync();
+          umma_group_ss<8, false, false>(tmem + COL_DZ, bms, fh, HI, ID_MN64, 0, go);
+          if (split_c) umma_group_ss<8, false, false>(tmem + COL_DZ, bms, fl, HI, ID_MN64, 1, go);
+          umma_commit_if(&sm.bars[DZ_READY], go);
+          const uint32_t col_oe = (it & 1) ? COL_OE1 : COL_OE0;
+          umma_group_ss<KD, true, false>(tmem + col_oe, aks, zh, HI, ID_KN, 0, go);
+          if (split_z) umma_group_ss<KD, true, false>(tmem + col_oe, aks, zl, HI, ID_KN, 1, go);
+          umma_commit_if(&sm.bars[A_FREE0 + s], go);
+          if (it + 1 < nblk) {
+            const int s1 = s ^ 1;
+            TC_WAIT_WARP(FULL_B0 + s1, ((it + 1) >> 1) & 1, 11);
+            tc_fence_after_sync();
+            umma_group_ss<KD, true, true>(tmem + (s1 ? COL_S1 : COL_S0), akn, bkn, HI, ID_S, 0, go);
+            umma_commit_if(&sm.bars[S_READY0 + s1], go);
+          }
+          TC_WAIT_WARP(P_READY0 + s, par2, 14);
+          TC_WAIT_WARP(FULL_C0 + s, par2, 15);
+          tc_fence_after_sync();
+          umma_group_ts8(tmem + COL_OI, tmem + col_p, cms, HI, ID_KN, 0, go);
+          if (split_p) umma_group_ts8(tmem + COL_OI, tmem + col_p + 8, cms, HI, ID_KN, 1, go);
+          umma_commit_if(&sm.bars[O_READY], go);
+        }
       }
     }
   } else if (STATE_ONLY && warp >= 4 && warp < 20) {
@@ -529,10 +515,10 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
       const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
       TC_WAIT_WARP(DZ_READY, 0, 20);
       tc_fence_after_sync();
-      float* dst = args.local_out + ((size_t)bh * args.nseg + seg) * (D * D) + (size_t)r * D + ehalf * 64 + zh * 32;
+      float* dst = args.local_out + ((size_t)bh * args.nseg + seg) * (D * D) + (size_t)r * D + zh * 32;
 #pragma unroll
       for (int pc = 0; pc < 2; ++pc) {
-        if (r >= D) break;  // D = 64: state rows 64..127 do not exist (warp-uniform: r = 32 q + lane)
+        if (r >= D) break;  // state rows 64..127 do not exist (warp-uniform: r = 32 q + lane)
         uint32_t dh[16], dl[16];
         tmem_ld_x16(lane_addr + COL_S0 + zh * 32 + pc * 16, dh);
         if (split_c) tmem_ld_x16(lane_addr + COL_S0 + 64 + zh * 32 + pc * 16, dl);
@@ -552,6 +538,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
   } else if (warp >= 4 && warp < 12) {
     // ------------------------------------ P group ------------------------------------
     if (!STATE_ONLY) {
+      set_regs<REGS_P, REGS_LAUNCH>();
       const int q = warp & 3;
       const int half = (warp - 4) >> 2;  // which two of the four 32-column chunks this warp converts
       const int r = q * 32 + lane;       // score row i
@@ -601,6 +588,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
     }
   } else if (warp >= 12 && warp < 20) {
     // ------------------------------------ Z group (walk kernel) ------------------------------------
+    set_regs<REGS_Z, REGS_LAUNCH>();
     const int q = warp & 3;
     const int zh = (warp - 12) >> 2;  // which 32 of the 64 state / value columns this warp owns
     const int r = q * 32 + lane;      // token row j of c / state row k of Z
@@ -610,7 +598,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
     // token row 32 i + (zt >> 3), so a warp reads whole 128-byte lines of c per load instruction (four rows of this
     // block's 64 value columns) and writes whole rows of the operand tile; row-per-thread loads would touch 32
     // lines per instruction, and the load/store unit's time per line is what every group's shared-memory traffic
-    // then waits behind (measured on the full-width kernel: 7 % of a step).
+    // then waits behind (measured: 7 % of a step).
     const int zt = (warp - 12) * 32 + lane;  // 0 .. 255
     const int frow = zt >> 3, fch = zt & 7;
     // decay factor of token row `row` of block iteration `it` in the state update
@@ -648,7 +636,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
       const int blk = REV ? (nblk - 1 - it) : it;
       const int t0 = seg_t0 + blk * 128;
       const __nv_bfloat16* src = static_cast<const __nv_bfloat16*>(job.c) + head_off + (size_t)(t0 + frow) * args.sT +
-                                 ehalf * 64 + fch * 8;
+                                 fch * 8;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         if (t0 + 32 * i + frow < args.N) raw[i] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)(32 * i) * args.sT));
@@ -660,7 +648,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
       float zreg[32];
       if (job.entry && r < D) {
         const float4* src = reinterpret_cast<const float4*>(
-            job.entry + ((size_t)bh * args.nseg + seg) * (D * D) + (size_t)r * D + ehalf * 64 + zh * 32);
+            job.entry + ((size_t)bh * args.nseg + seg) * (D * D) + (size_t)r * D + zh * 32);
 #pragma unroll
         for (int x = 0; x < 8; ++x) {
           const float4 v = __ldg(src + x);
@@ -722,7 +710,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
       }
       const bool last_processed = REV ? (seg == 0) : (seg == args.nseg - 1);
       if (job.final_out && last_processed && r < D) {
-        float* dst = job.final_out + (size_t)bh * (D * D) + (size_t)r * D + ehalf * 64 + zh * 32;
+        float* dst = job.final_out + (size_t)bh * (D * D) + (size_t)r * D + zh * 32;
 #pragma unroll
         for (int x = 0; x < 8; ++x)
           *reinterpret_cast<float4*>(dst + 4 * x) = make_float4(zreg[4 * x], zreg[4 * x + 1], zreg[4 * x + 2], zreg[4 * x + 3]);
@@ -731,6 +719,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
   } else if (warp >= 20) {
     // ------------------------------------ O group ------------------------------------
     if (!STATE_ONLY) {
+      set_regs<REGS_O, REGS_LAUNCH>();
       const int q = warp & 3;
       const int r = q * 32 + lane;  // output row i
       const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
@@ -797,7 +786,7 @@ tc_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps m
           ++og_uses;
           if (warp == 20 && lane == 0) {
             // rows beyond N are clipped by the tensor map (a ragged block is always the last of the sequence)
-            tma_store_4d(tm_out, stg, ehalf * 64 + pass * (int)(128 / sizeof(TOut)), t0, hh_, bb_);
+            tma_store_4d(tm_out, stg, pass * (int)(128 / sizeof(TOut)), t0, hh_, bb_);
             tma_store_commit();
           }
         }
@@ -885,14 +874,14 @@ bool make_map(CUtensorMap* m, const void* ptr, const OpArgs& a, int D, bool f32 
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool REV, bool STATE_ONLY, typename TOut, int D, int NJOBS>
+template <bool REV, bool STATE_ONLY, typename TOut, int NJOBS>
 cudaError_t launch_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, const DecayTable& tab, cudaStream_t stream) {
   const size_t smem = sizeof(TcSmem) + 1024;
-  auto kern = tc_kernel<REV, STATE_ONLY, TOut, D, NJOBS>;
+  auto kern = tc_kernel<REV, STATE_ONLY, TOut, NJOBS>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(STATE_ONLY ? K_PREPASS : (NJOBS == 2 ? K_WALK_PAIR : K_WALK), stream);
-  kern<<<(unsigned)(ta.BH * ta.nseg * (D == 128 ? 2 : 1) * NJOBS), TC_THREADS, smem, stream>>>(m0, m1, ta, tab);
+  kern<<<(unsigned)(ta.BH * ta.nseg * NJOBS), TC_THREADS, smem, stream>>>(m0, m1, ta, tab);
   count_launch();
   return cudaGetLastError();
 }
@@ -959,25 +948,26 @@ cudaError_t launch_walk64(const OpArgs& args, const OpArgs* second, const DecayT
   const TcArgs ta = make_args(args, second, precision);
   if (second) {  // only the reverse direction is ever paired
     if (!args.reverse) return cudaErrorInvalidValue;
-    return f32 ? launch_t<true, false, float, 64, 2>(m0, m1, ta, tab, stream)
-               : launch_t<true, false, __nv_bfloat16, 64, 2>(m0, m1, ta, tab, stream);
+    return f32 ? launch_t<true, false, float, 2>(m0, m1, ta, tab, stream)
+               : launch_t<true, false, __nv_bfloat16, 2>(m0, m1, ta, tab, stream);
   }
   if (args.reverse)
-    return f32 ? launch_t<true, false, float, 64, 1>(m0, m1, ta, tab, stream)
-               : launch_t<true, false, __nv_bfloat16, 64, 1>(m0, m1, ta, tab, stream);
-  return f32 ? launch_t<false, false, float, 64, 1>(m0, m1, ta, tab, stream)
-             : launch_t<false, false, __nv_bfloat16, 64, 1>(m0, m1, ta, tab, stream);
+    return f32 ? launch_t<true, false, float, 1>(m0, m1, ta, tab, stream)
+               : launch_t<true, false, __nv_bfloat16, 1>(m0, m1, ta, tab, stream);
+  return f32 ? launch_t<false, false, float, 1>(m0, m1, ta, tab, stream)
+             : launch_t<false, false, __nv_bfloat16, 1>(m0, m1, ta, tab, stream);
 }
 
 cudaError_t launch_prepass64(const OpArgs& args, const DecayTable& tab, int precision, cudaStream_t stream) {
   TcMaps m;
+  if (args.seq_start) return cudaErrorInvalidValue;  // packed batches: D = 128 only
   // the a and out maps are unused by the state-only kernel; valid descriptors are passed anyway
   if (!make_map(&m.b, args.b, args, 64) || !make_map(&m.c, args.c, args, 64)) return cudaErrorInvalidValue;
   m.a = m.b;
   m.out = m.c;
   const TcArgs ta = make_args(args, nullptr, precision);
-  return args.reverse ? launch_t<true, true, float, 64, 1>(m, m, ta, tab, stream)
-                      : launch_t<false, true, float, 64, 1>(m, m, ta, tab, stream);
+  return args.reverse ? launch_t<true, true, float, 1>(m, m, ta, tab, stream)
+                      : launch_t<false, true, float, 1>(m, m, ta, tab, stream);
 }
 
 cudaError_t launch_states128(const OpArgs& args, const DecayTable& tab, int precision, bool all_segments, cudaStream_t stream) {

@@ -62,23 +62,6 @@ enum WBar {
   W_NUM_BARS
 };
 
-template <int N>
-__device__ __forceinline__ void reg_dec() {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
-}
-template <int N>
-__device__ __forceinline__ void reg_inc() {
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
-}
-
-// This warp's registers per thread from now on, LAUNCH being what the launch gave: setmaxnreg.inc must not be given less
-// than the warp has, nor .dec more (an illegal instruction).
-template <int N, int LAUNCH>
-__device__ __forceinline__ void set_regs() {
-  if (N < LAUNCH) reg_dec<N>();
-  if (N > LAUNCH) reg_inc<N>();
-}
-
 // Arithmetic on two fp32 values in one register pair: half the issue slots, which is what the worker warps are short of
 // (the reverse pair at the 1B-like shape 126 -> 123 us; in the fc conversion it spilled registers and was slower).
 __device__ __forceinline__ uint64_t f2_pack(float a, float b) {

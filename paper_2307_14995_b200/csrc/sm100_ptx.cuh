@@ -43,6 +43,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// ---- registers per thread of a warpgroup ----------------------------------------------------
+template <int N>
+__device__ __forceinline__ void reg_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void reg_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+
+// This warp's registers per thread from now on, LAUNCH being what the launch gave: setmaxnreg.inc must not be given less
+// than the warp has, nor .dec more (an illegal instruction).
+template <int N, int LAUNCH>
+__device__ __forceinline__ void set_regs() {
+  if (N < LAUNCH) reg_dec<N>();
+  if (N > LAUNCH) reg_inc<N>();
+}
+
 // ---- proxy / tcgen05 fences -------------------------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

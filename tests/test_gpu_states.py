@@ -1,5 +1,6 @@
-"""States entering the segments of a long sequence (d = 128 tensor-core path) against the fp64 oracle: segments that one
-thread block sums, that a cluster shares, that the walk chains itself and that reach it as running sums.
+"""States entering the segments of a long sequence against the fp64 oracle.  d = 128: segments that one thread block sums,
+that a cluster shares, that the walk chains itself and that reach it as running sums; d = 64: the scan.  And the full-precision
+kernels.
 
 Tolerance: on-chip operands are two bf16 terms, 2^-17 of each product; a chain of 57 blocks in one fp32 accumulator adds up
 to 912 products with a relative error of 2^-24 of the running sum each.  Against RMS(ref), with |sum| up to 5 RMS: 2^-17 * 5 +
@@ -14,18 +15,19 @@ from paper_2307_14995_b200 import binding as la
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("B,N,seg_len,lam", [
     (1, 8500, 4224, [1.0, 0.9995, 0.9, 1e-30]),   # 33 blocks, unshared; ragged tail
     (1, 4097, 2048, [1.0, 0.9995]),               # shared by a cluster; a tail of one token
     (2, 1211, 128, [1.0, 0.999, 0.5]),            # one block a segment, ten segments: running sums
-    (1, 700, 128, [0.9, 1.0, 0.9995]),            # chained by the walk
+    (1, 700, 128, [0.9, 1.0, 0.9995]),            # five segments: chained by the walk
     (3, 3001, 0, [1.0, 0.98]),                    # the library's own plan
 ])
-def test_states_entering_segments(B, N, seg_len, lam):
+def test_states_entering_segments(B, N, seg_len, lam, d):
     H = len(lam)
     gen = torch.Generator().manual_seed(N)
-    q, k, v, do = [torch.randn(B, H, N, 128, generator=gen).bfloat16() for _ in range(4)]
-    kv_in, gko = [torch.randn(B, H, 128, 128, generator=gen) * 0.1 for _ in range(2)]
+    q, k, v, do = [torch.randn(B, H, N, d, generator=gen).bfloat16() for _ in range(4)]
+    kv_in, gko = [torch.randn(B, H, d, d, generator=gen) * 0.1 for _ in range(2)]
     lam = torch.tensor(lam)
     dev = [x.cuda() for x in (q, k, v, do, kv_in, gko)]
     o, kv = la.fwd(*dev[:3], lam, out_dtype=torch.float32, kv_in=dev[4], want_state=True, seg_len=seg_len)
