@@ -91,7 +91,7 @@ typedef struct {
   la_dtype out_dtype; /* o, dq, dk, dv */
   int seg_len;        /* 0 = library chooses.  Otherwise the sequence is cut into
                          segments of this many tokens (a positive multiple of 128)
-                         that run as independent thread blocks joined by a state scan. */
+                         that run as independent thread blocks, each from the state entering it. */
   int path;           /* la_path */
   int precision;      /* LA_PRECISION_DEFAULT or an OR of LA_SPLIT_* */
   int layout;         /* la_layout */
@@ -119,8 +119,8 @@ int la_segment_length(const la_shape* shape);
  * With kv_in the result is o_t = kv_t^T q_t where kv_{-1} = kv_in.
  * workspace: device scratch of at least la_workspace_bytes(LA_OP_FWD, shape)
  * bytes, 256-byte aligned; may be NULL when that size is 0.  Calls that share a
- * workspace must be stream-ordered.  Afterwards the workspace holds the state
- * entering each segment and its transpose; la_bwd_reuse can take it to skip recomputing those.
+ * workspace must be stream-ordered.  Afterwards the workspace holds the segments'
+ * states as the backward walk wants them; la_bwd_reuse can take it to skip recomputing those.
  */
 la_status la_fwd(const la_shape* shape, const void* q, const void* k, const void* v,
                  const float* lambda_host, void* o, const float* kv_in, float* kv_out,
@@ -212,7 +212,7 @@ la_status la_decode_step(const la_shape* shape, const void* q, const void* k, co
  *   kv_in, kv_out, grad_kv_out, grad_kv_in   [2,B,H,d,e] fp32 (cos half, then sin half) or NULL;
  *   other arguments as in la_fwd / la_bwd; requires d == e.
  * Workspace: la_lrpe_workspace_bytes(op, shape), 256-byte aligned: the four feature tensors, fp32 temporaries of
- * the tensors' size (1-2 forward, 5-6 backward) and the inner calls' own workspace.
+ * the tensors' size (1-2 forward, 5-6 backward), a table of angles and the inner calls' own workspace.
  * d_theta is a position-weighted sum whose q and k parts cancel down to the relative-position result; with
  * bf16 features its error grows with the absolute positions (see the tests for the bound that is checked).
  */

@@ -23,7 +23,9 @@
 namespace la {
 namespace {
 
-constexpr int TILE_TOKENS = 256;  // tokens of one (b,h) per block in the gradient kernel
+constexpr int RUN = 16;  // consecutive tokens a group of d/4 lanes walks
+// tokens of one (b,h) per block in the gradient kernel: 256 / (d/4) groups, 128 (d = 128) or 256 (d = 64)
+__host__ __device__ constexpr int tile_tokens(int d) { return RUN * (1024 / d); }
 
 __device__ __forceinline__ void rotation(float theta, long long pos, float* c, float* s) {
   double a = (double)theta * (double)pos;
@@ -36,16 +38,62 @@ struct Geometry {   // where token t of (b,h) lives: element offset b*sB + h*sH 
   int B, H, N, d;
 };
 
-// x -> x cos(theta t), x sin(theta t), same layout as x.  d/4 lanes share a token (four features each) and walk a
-// run of RUN consecutive tokens of one (b,h): the first angle of the run is exact (double product, reduced), the
-// following ones come from rotating (cos, sin) by the feature's own step angle, four multiply-adds instead of a
-// sincos per element; over RUN = 16 steps the recurrence drifts by a few 1e-7, far below the bf16 features' 2^-9.
-constexpr int RUN = 16;
+// The angles a call needs, once for all its kernels and batches: (cos, sin) of theta t at every RUN-th token, [H, runs, d],
+// and of theta itself behind them, [H, d].  The kernels get the tokens between by rotating (cos, sin) by the feature's own
+// step angle, four multiply-adds instead of a sincos per element; over 16 steps the recurrence
+// drifts by a few 1e-7, far below the bf16 features' 2^-9.  With the double products and sincos in the kernels themselves
+// a warp spent most of its 2100 instructions on them with nothing in flight (this kernel: 7 us at 16 heads x 8192 tokens).
+__global__ void __launch_bounds__(256) lrpe_angle_kernel(const float* __restrict__ theta, float2* __restrict__ table, int H, int d,
+                                                         int runs, long long pos0) {
+  const int hd = H * d, chunks = (hd + 255) / 256;
+  const int run = blockIdx.x / chunks, i = blockIdx.x % chunks * 256 + threadIdx.x;  // run == runs: the step angles
+  if (i >= hd) return;
+  float2 v;
+  rotation(theta[i], run < runs ? pos0 + (long long)run * RUN : 1, &v.x, &v.y);
+  table[run < runs ? ((size_t)(i / d) * runs + run) * d + i % d : (size_t)runs * hd + i] = v;
+}
+
+// (cos, sin) of four consecutive features.
+__device__ __forceinline__ void load_angles(const float2* __restrict__ at, float (&c)[4], float (&s)[4]) {
+  const float4 x = *reinterpret_cast<const float4*>(at), y = *reinterpret_cast<const float4*>(at + 2);
+  c[0] = x.x; s[0] = x.y; c[1] = x.z; s[1] = x.w;
+  c[2] = y.x; s[2] = y.y; c[3] = y.z; s[3] = y.w;
+}
+__device__ __forceinline__ void turn(float (&c)[4], float (&s)[4], const float (&cs)[4], const float (&ss)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float cn = fmaf(c[k], cs[k], -s[k] * ss[k]);
+    s[k] = fmaf(s[k], cs[k], c[k] * ss[k]);
+    c[k] = cn;
+  }
+}
+
+// x -> x cos(theta t), x sin(theta t) for x = q and k, same layout as x.  d/4 lanes share a token (four features each) and
+// walk a run of RUN consecutive tokens of one (b,h).  Bound by memory, 12 bytes a feature of q and k in bf16; BATCH tokens of
+// both are loaded before any is used (1 x 16 x 8192 x 128: 33 us, one tensor a launch
+// and a sincos in the kernel 66).
+constexpr int BATCH = 4;
 
 template <typename T>
-__global__ void __launch_bounds__(256) lrpe_feature_kernel(const T* __restrict__ x, const float* __restrict__ theta,
-                                                           T* __restrict__ xc, T* __restrict__ xs, Geometry g,
-                                                           long long pos0) {
+struct FeatureArgs {
+  const T* x[2];  // q, k
+  T* c[2];
+  T* s[2];
+};
+
+template <typename T>
+__device__ __forceinline__ void store_features(const FeatureArgs<T>& io, size_t off, const float (&q)[4], const float (&k)[4],
+                                               const float (&c)[4], const float (&s)[4]) {
+  const float qc[4] = {q[0] * c[0], q[1] * c[1], q[2] * c[2], q[3] * c[3]}, qs[4] = {q[0] * s[0], q[1] * s[1], q[2] * s[2], q[3] * s[3]};
+  const float kc[4] = {k[0] * c[0], k[1] * c[1], k[2] * c[2], k[3] * c[3]}, ks[4] = {k[0] * s[0], k[1] * s[1], k[2] * s[2], k[3] * s[3]};
+  Vec4<T>::store(io.c[0] + off, qc);
+  Vec4<T>::store(io.s[0] + off, qs);
+  Vec4<T>::store(io.c[1] + off, kc);
+  Vec4<T>::store(io.s[1] + off, ks);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256, 4) lrpe_feature_kernel(const FeatureArgs<T> io, const float2* __restrict__ table, Geometry g) {
   const int lanes = g.d >> 2;
   const int groups = 256 / lanes;
   const int lane = threadIdx.x % lanes, grp = threadIdx.x / lanes;
@@ -56,30 +104,29 @@ __global__ void __launch_bounds__(256) lrpe_feature_kernel(const T* __restrict__
     const int t_first = (int)(run % runs_per_head) * RUN;
     const long bh = run / runs_per_head;
     const int h = (int)(bh % g.H), b = (int)(bh / g.H);
-    const float4 th = *reinterpret_cast<const float4*>(theta + (size_t)h * g.d + c0);
-    const float tv[4] = {th.x, th.y, th.z, th.w};
     float c[4], s[4], cs[4], ss[4];
+    load_angles(table + ((size_t)h * runs_per_head + run % runs_per_head) * g.d + c0, c, s);
+    load_angles(table + ((size_t)g.H * runs_per_head + h) * g.d + c0, cs, ss);
+    size_t off = (size_t)b * g.sB + (size_t)h * g.sH + (size_t)t_first * g.sT + c0;
+    int left = min(g.N - t_first, RUN);
+    for (; left >= BATCH; left -= BATCH, off += BATCH * g.sT) {
+      float v[2][BATCH][4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      rotation(tv[k], pos0 + t_first, &c[k], &s[k]);
-      rotation(tv[k], 1, &cs[k], &ss[k]);
-    }
-    const size_t base = (size_t)b * g.sB + (size_t)h * g.sH + c0;
-    const int t_end = min(g.N, t_first + RUN);
-    for (int t = t_first; t < t_end; ++t) {
-      const size_t off = base + (size_t)t * g.sT;
-      float v[4], oc[4], os[4];
-      Vec4<T>::load(x + off, v);
+      for (int n = 0; n < BATCH; ++n)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        oc[k] = v[k] * c[k];
-        os[k] = v[k] * s[k];
-        const float cn = fmaf(c[k], cs[k], -s[k] * ss[k]);
-        s[k] = fmaf(s[k], cs[k], c[k] * ss[k]);
-        c[k] = cn;
+        for (int w = 0; w < 2; ++w) Vec4<T>::load(io.x[w] + off + n * g.sT, v[w][n]);
+#pragma unroll
+      for (int n = 0; n < BATCH; ++n) {
+        store_features(io, off + n * g.sT, v[0][n], v[1][n], c, s);
+        turn(c, s, cs, ss);
       }
-      Vec4<T>::store(xc + off, oc);
-      Vec4<T>::store(xs + off, os);
+    }
+    for (; left > 0; --left, off += g.sT) {
+      float v[2][4];
+#pragma unroll
+      for (int w = 0; w < 2; ++w) Vec4<T>::load(io.x[w] + off, v[w]);
+      store_features(io, off, v[0], v[1], c, s);
+      turn(c, s, cs, ss);
     }
   }
 }
@@ -98,15 +145,31 @@ __global__ void __launch_bounds__(256) lrpe_sum_kernel(const float* a, const flo
   }
 }
 
-// Chain rule through the feature map for one of q, k:
+// Chain rule through the feature map, blockIdx.y = 0 for q and 1 for k:
 //   dx = gc cos + gs sin,     part[(bh, tile), i] = sum over the tile's tokens of t (x cos gs - x sin gc)_i.
-// Block = one tile of TILE_TOKENS tokens of one (b,h); d/4 lanes per token, 256/(d/4) tokens per pass.
+// Block = one tile of one (b,h); d/4 lanes share a token and walk a run of RUN.  Bound by memory (14
+// bytes a feature): both in one launch, and the angles from the table (1 x 16 x 8192 x 128: 86 us,
+// before 91; unrolled by two 98, its registers cost more warps than the loads ahead gain).
+
 template <typename TIn, typename TOut>
-__global__ void __launch_bounds__(256) lrpe_grad_kernel(const TIn* __restrict__ x, const float* __restrict__ gc,
-                                                        const float* __restrict__ gs, const float* __restrict__ theta,
-                                                        TOut* __restrict__ dx, float* __restrict__ part, Geometry g,
-                                                        long long pos0, int ntiles) {
+struct GradArgs {
+  const TIn* x[2];
+  const float* gc[2];
+  const float* gs[2];
+  TOut* dx[2];
+  float* part[2];
+};
+
+template <typename TIn, typename TOut>
+__global__ void __launch_bounds__(256) lrpe_grad_kernel(const GradArgs<TIn, TOut> io, const float2* __restrict__ table, Geometry g,
+                                                           long long pos0, int ntiles) {
   __shared__ float red[2048];  // [tokens per pass][d]: 8 x 128 or 16 x 64
+  const bool second = blockIdx.y != 0;
+  const TIn* __restrict__ const x = second ? io.x[1] : io.x[0];
+  const float* __restrict__ const gc = second ? io.gc[1] : io.gc[0];
+  const float* __restrict__ const gs = second ? io.gs[1] : io.gs[0];
+  TOut* __restrict__ const dx = second ? io.dx[1] : io.dx[0];
+  float* __restrict__ const part = second ? io.part[1] : io.part[0];
   const int lanes = g.d >> 2;
   const int rows_per_pass = 256 / lanes;  // 8 (d = 128) or 16 (d = 64)
   const int lane = threadIdx.x % lanes, row0 = threadIdx.x / lanes;
@@ -114,21 +177,16 @@ __global__ void __launch_bounds__(256) lrpe_grad_kernel(const TIn* __restrict__ 
   const int h = bh % g.H, b = bh / g.H;
   const int c0 = lane * 4;
   const size_t head_off = (size_t)b * g.sB + (size_t)h * g.sH + c0;
-  const float4 th = *reinterpret_cast<const float4*>(theta + (size_t)h * g.d + c0);
-  const float tv[4] = {th.x, th.y, th.z, th.w};
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  // each group of d/4 lanes walks its own run of consecutive tokens, rotating (cos, sin) from an exact start
-  const int run = TILE_TOKENS / rows_per_pass;  // 32 (d = 128) or 16 (d = 64)
-  const int t_first = tile * TILE_TOKENS + row0 * run;
-  const int t_end = min(g.N, t_first + run);
+  const int t_first = tile * tile_tokens(g.d) + row0 * RUN;
+  const int t_end = min(g.N, t_first + RUN);
+  const int runs = (g.N + RUN - 1) / RUN;
   float c[4], s[4], cs[4], ss[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    rotation(tv[k], pos0 + t_first, &c[k], &s[k]);
-    rotation(tv[k], 1, &cs[k], &ss[k]);
-  }
-  for (int t = t_first; t < t_end; ++t) {
-    const size_t off = head_off + (size_t)t * g.sT;
+  load_angles(table + ((size_t)h * runs + min(t_first / RUN, runs - 1)) * g.d + c0, c, s);
+  load_angles(table + ((size_t)g.H * runs + h) * g.d + c0, cs, ss);
+  size_t off = head_off + (size_t)t_first * g.sT;
+#pragma unroll 1
+  for (int t = t_first; t < t_end; ++t, off += g.sT) {
     float v[4], a[4], bb[4], o[4];
     Vec4<TIn>::load(x + off, v);
     Vec4<float>::load(gc + off, a);
@@ -138,10 +196,8 @@ __global__ void __launch_bounds__(256) lrpe_grad_kernel(const TIn* __restrict__ 
     for (int k = 0; k < 4; ++k) {
       o[k] = fmaf(a[k], c[k], bb[k] * s[k]);
       acc[k] = fmaf(pos, v[k] * (c[k] * bb[k] - s[k] * a[k]), acc[k]);
-      const float cn = fmaf(c[k], cs[k], -s[k] * ss[k]);
-      s[k] = fmaf(s[k], cs[k], c[k] * ss[k]);
-      c[k] = cn;
     }
+    turn(c, s, cs, ss);
     Vec4<TOut>::store(dx + off, o);
   }
   // fixed-order sum over the token rows of the block
@@ -200,18 +256,35 @@ Geometry geometry(const la_shape* s) {
   return g;
 }
 
-cudaError_t run_features(const la_shape* s, const void* x, const float* theta, void* xc, void* xs, long long pos0,
-                         cudaStream_t st) {
+size_t angle_count(const la_shape* s) { return (size_t)s->H * s->d * ((s->N + RUN - 1) / RUN + 1); }
+
+cudaError_t run_angles(const la_shape* s, const float* theta, float2* table, long long pos0, cudaStream_t st) {
   KernelTimer timer(K_LRPE, st);
-  const Geometry g = geometry(s);
-  const unsigned grid = grid_for((long)s->B * s->H * ((s->N + RUN - 1) / RUN) * (s->d / 4));
-  if (s->in_dtype == LA_BF16)
-    lrpe_feature_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)x, theta, (__nv_bfloat16*)xc,
-                                                            (__nv_bfloat16*)xs, g, pos0);
-  else
-    lrpe_feature_kernel<float><<<grid, 256, 0, st>>>((const float*)x, theta, (float*)xc, (float*)xs, g, pos0);
+  const int runs = (s->N + RUN - 1) / RUN;
+  const long blocks = (runs + 1L) * ((s->H * s->d + 255) / 256);
+  if (blocks > 2147483647L) return cudaErrorInvalidValue;
+  lrpe_angle_kernel<<<(unsigned)blocks, 256, 0, st>>>(theta, table, s->H, s->d, runs, pos0);
   count_launch();
   return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t run_features_t(const la_shape* s, const void* q, const void* k, const float2* table, void* qc, void* qs, void* kc,
+                           void* ks, cudaStream_t st) {
+  KernelTimer timer(K_LRPE, st);
+  FeatureArgs<T> io;
+  io.x[0] = static_cast<const T*>(q); io.x[1] = static_cast<const T*>(k);
+  io.c[0] = static_cast<T*>(qc); io.c[1] = static_cast<T*>(kc);
+  io.s[0] = static_cast<T*>(qs); io.s[1] = static_cast<T*>(ks);
+  const unsigned grid = grid_for((long)s->B * s->H * ((s->N + RUN - 1) / RUN) * (s->d / 4));
+  lrpe_feature_kernel<T><<<grid, 256, 0, st>>>(io, table, geometry(s));
+  count_launch();
+  return cudaGetLastError();
+}
+cudaError_t run_features(const la_shape* s, const void* q, const void* k, const float2* table, void* qc, void* qs, void* kc,
+                         void* ks, cudaStream_t st) {
+  return s->in_dtype == LA_BF16 ? run_features_t<__nv_bfloat16>(s, q, k, table, qc, qs, kc, ks, st)
+                                : run_features_t<float>(s, q, k, table, qc, qs, kc, ks, st);
 }
 
 cudaError_t run_sum(const la_shape* s, const float* a, const float* b, void* dst, cudaStream_t st) {
@@ -226,25 +299,38 @@ cudaError_t run_sum(const la_shape* s, const float* a, const float* b, void* dst
   return cudaGetLastError();
 }
 
-cudaError_t run_grad(const la_shape* s, const void* x, const float* gc, const float* gs, const float* theta, void* dx,
-                     float* part, long long pos0, int ntiles, cudaStream_t st) {
+// The tensors of GradArgs for q and k, untyped.
+struct GradSet {
+  const void* x;
+  const float* gc;
+  const float* gs;
+  void* dx;
+  float* part;
+};
+template <typename TIn, typename TOut>
+cudaError_t run_grad_t(const la_shape* s, const GradSet& q, const GradSet& k, const float2* table, long long pos0, int ntiles,
+                       cudaStream_t st) {
   KernelTimer timer(K_LRPE, st);
-  const Geometry g = geometry(s);
-  const unsigned grid = (unsigned)((long)s->B * s->H * ntiles);
-  const bool ib = s->in_dtype == LA_BF16, ob = s->out_dtype == LA_BF16;
-  if (ib && ob)
-    lrpe_grad_kernel<__nv_bfloat16, __nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)x, gc, gs, theta,
-                                                                        (__nv_bfloat16*)dx, part, g, pos0, ntiles);
-  else if (ib)
-    lrpe_grad_kernel<__nv_bfloat16, float><<<grid, 256, 0, st>>>((const __nv_bfloat16*)x, gc, gs, theta, (float*)dx,
-                                                                part, g, pos0, ntiles);
-  else if (!ob)
-    lrpe_grad_kernel<float, float><<<grid, 256, 0, st>>>((const float*)x, gc, gs, theta, (float*)dx, part, g, pos0,
-                                                        ntiles);
-  else
-    return cudaErrorInvalidValue;
+  GradArgs<TIn, TOut> io;
+  for (int w = 0; w < 2; ++w) {
+    const GradSet& one = w ? k : q;
+    io.x[w] = static_cast<const TIn*>(one.x);
+    io.gc[w] = one.gc;
+    io.gs[w] = one.gs;
+    io.dx[w] = static_cast<TOut*>(one.dx);
+    io.part[w] = one.part;
+  }
+  lrpe_grad_kernel<TIn, TOut><<<dim3((unsigned)((long)s->B * s->H * ntiles), 2), 256, 0, st>>>(io, table, geometry(s), pos0, ntiles);
   count_launch();
   return cudaGetLastError();
+}
+cudaError_t run_grad(const la_shape* s, const GradSet& q, const GradSet& k, const float2* table, long long pos0, int ntiles,
+                     cudaStream_t st) {
+  const bool ib = s->in_dtype == LA_BF16, ob = s->out_dtype == LA_BF16;
+  if (ib && ob) return run_grad_t<__nv_bfloat16, __nv_bfloat16>(s, q, k, table, pos0, ntiles, st);
+  if (ib) return run_grad_t<__nv_bfloat16, float>(s, q, k, table, pos0, ntiles, st);
+  if (!ob) return run_grad_t<float, float>(s, q, k, table, pos0, ntiles, st);
+  return cudaErrorInvalidValue;
 }
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
@@ -265,6 +351,7 @@ struct Carve {
   size_t f32;        // bytes of one fp32 temporary of the tensors' size
   size_t part;       // bytes of one partial-sum array for dtheta
   size_t op;         // workspace of the inner la_fwd / la_bwd
+  size_t angles;     // bytes of the angle table
   int ntiles;
   int n_f32;         // fp32 temporaries
   size_t total;
@@ -278,16 +365,17 @@ bool carve(int op, const la_shape* s, Carve* c) {
   const size_t elems = (size_t)s->B * s->H * s->N * s->d;
   c->feat = up256(elems * (s->in_dtype == LA_BF16 ? 2 : 4));
   c->f32 = up256(elems * 4);
-  c->ntiles = (s->N + TILE_TOKENS - 1) / TILE_TOKENS;
+  c->ntiles = (s->N + tile_tokens(s->d) - 1) / tile_tokens(s->d);
   c->part = up256((size_t)s->B * s->H * c->ntiles * s->d * 4);
   c->op = up256(op_ws);
+  c->angles = up256(angle_count(s) * sizeof(float2));
   const bool out32 = s->out_dtype == LA_F32;
   if (op == LA_OP_FWD) {
     c->n_f32 = out32 ? 1 : 2;                    // the second run's result (and the first's when o is bf16)
-    c->total = 4 * c->feat + c->n_f32 * c->f32 + c->op;
+    c->total = 4 * c->feat + c->n_f32 * c->f32 + c->angles + c->op;
   } else {
     c->n_f32 = 4 + (out32 ? 1 : 2);              // gradients of the four feature tensors, dv of the runs
-    c->total = 4 * c->feat + c->n_f32 * c->f32 + 2 * c->part + c->op;
+    c->total = 4 * c->feat + c->n_f32 * c->f32 + 2 * c->part + c->angles + c->op;
   }
   return true;
 }
@@ -319,14 +407,15 @@ la_status la_lrpe_fwd(const la_shape* shape, const void* q, const void* k, const
   char* w = static_cast<char*>(workspace);
   void* qc = w; void* qs = w + c.feat; void* kc = w + 2 * c.feat; void* ks = w + 3 * c.feat;
   float* tmp = reinterpret_cast<float*>(w + 4 * c.feat);
-  void* op_ws = w + 4 * c.feat + c.n_f32 * c.f32;
+  float2* table = reinterpret_cast<float2*>(w + 4 * c.feat + c.n_f32 * c.f32);
+  void* op_ws = w + 4 * c.feat + c.n_f32 * c.f32 + c.angles;
   const bool out32 = shape->out_dtype == LA_F32;
   la_shape inner = *shape;
   inner.out_dtype = LA_F32;
   const size_t state = (size_t)shape->B * shape->H * shape->d * shape->e;
 
-  if (run_features(shape, q, theta, qc, qs, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
-  if (run_features(shape, k, theta, kc, ks, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
+  if (run_angles(shape, theta, table, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
+  if (run_features(shape, q, k, table, qc, qs, kc, ks, cs) != cudaSuccess) return LA_ERR_CUDA;
   float* first = out32 ? static_cast<float*>(o) : tmp + c.f32 / 4;
   la_status st = la_fwd(&inner, qc, kc, v, lambda_host, first, kv_in, kv_out, op_ws, c.op, stream);
   if (st != LA_OK) return st;
@@ -363,13 +452,14 @@ la_status la_lrpe_bwd(const la_shape* shape, const void* q, const void* k, const
   w += c.n_f32 * c.f32;
   float* part_q = reinterpret_cast<float*>(w);
   float* part_k = reinterpret_cast<float*>(w + c.part);
-  void* op_ws = w + 2 * c.part;
+  float2* table = reinterpret_cast<float2*>(w + 2 * c.part);
+  void* op_ws = w + 2 * c.part + c.angles;
   la_shape inner = *shape;
   inner.out_dtype = LA_F32;
   const size_t state = (size_t)shape->B * shape->H * shape->d * shape->e;
 
-  if (run_features(shape, q, theta, qc, qs, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
-  if (run_features(shape, k, theta, kc, ks, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
+  if (run_angles(shape, theta, table, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
+  if (run_features(shape, q, k, table, qc, qs, kc, ks, cs) != cudaSuccess) return LA_ERR_CUDA;
   la_status st = la_bwd(&inner, qc, kc, v, d_o, lambda_host, g_qc, g_kc, dv_c, kv_in, grad_kv_out, grad_kv_in, op_ws,
                         c.op, stream);
   if (st != LA_OK) return st;
@@ -378,8 +468,9 @@ la_status la_lrpe_bwd(const la_shape* shape, const void* q, const void* k, const
               stream);
   if (st != LA_OK) return st;
   if (run_sum(shape, dv_c, dv_s, dv, cs) != cudaSuccess) return LA_ERR_CUDA;
-  if (run_grad(shape, q, g_qc, g_qs, theta, dq, part_q, pos0, c.ntiles, cs) != cudaSuccess) return LA_ERR_CUDA;
-  if (run_grad(shape, k, g_kc, g_ks, theta, dk, part_k, pos0, c.ntiles, cs) != cudaSuccess) return LA_ERR_CUDA;
+  if (run_grad(shape, GradSet{q, g_qc, g_qs, dq, part_q}, GradSet{k, g_kc, g_ks, dk, part_k}, table, pos0, c.ntiles, cs) !=
+      cudaSuccess)
+    return LA_ERR_CUDA;
   {
     KernelTimer timer(K_LRPE, cs);
     const int n = shape->H * shape->d;
