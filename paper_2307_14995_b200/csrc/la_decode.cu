@@ -10,12 +10,16 @@
 // strides over the key rows, so a warp touches whole 512-byte rows with 16-byte
 // accesses, all row loads are issued before the first use, and the column sums
 // for o are reduced inside the block (no atomics, bitwise reproducible).
+// With several tokens the inputs of up to CHUNK of them are fetched together with the state, so that a token costs its
+// arithmetic and one barrier instead of a round trip to memory and two (16 x 32
+// states, d = 128, 4 tokens: 14.8 us before, 13.5 now; 32 states, 8 tokens: 8.0 and 6.6).
 #include "la_common.cuh"
 
 namespace la {
 namespace {
 
 constexpr int THREADS = 256;
+constexpr int CHUNK = 8;  // tokens whose inputs are on chip at a time
 
 template <typename TIn, typename TOut, int D, int E>
 __global__ void __launch_bounds__(THREADS)
@@ -25,11 +29,12 @@ decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* _
   constexpr int LPR = E / 4;              // lanes per state row (float4 each)
   constexpr int RPP = THREADS / LPR;      // rows per pass
   constexpr int PASSES = D / RPP;
-  static_assert(D % RPP == 0 && THREADS % LPR == 0, "shape");
+  static_assert(D == E && D % RPP == 0 && THREADS % LPR == 0, "shape");
 
-  __shared__ float sq[D];
-  __shared__ float sk[D];
-  __shared__ float4 red[RPP][LPR];
+  __shared__ float sq[CHUNK][D];
+  __shared__ float sk[CHUNK][D];
+  __shared__ float sv[CHUNK][E];
+  __shared__ float4 red[2][RPP][LPR];
 
   const int bh = blockIdx.x;
   const int tid = threadIdx.x;
@@ -46,22 +51,29 @@ decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* _
   for (int p = 0; p < PASSES; ++p) s[p] = __ldcs(&state[(size_t)(row0 + p * RPP) * LPR + col4]);
 
   for (int t = 0; t < T; ++t) {
-    if (tid < D) {
-      sq[tid] = to_f32<TIn>(q[head_off + (size_t)t * sT + tid]);
-      sk[tid] = to_f32<TIn>(k[head_off + (size_t)t * sT + tid]);
+    const int u = t % CHUNK;
+    if (u == 0) {
+      if (t > 0) __syncthreads();  // the chunk before has been read
+      const int n = min(CHUNK, T - t);
+      for (int x = tid; x < n * (D / 4); x += THREADS) {
+        const size_t at = head_off + (size_t)(t + x / (D / 4)) * sT + x % (D / 4) * 4;
+        float w[4];
+        Vec4<TIn>::load(q + at, w);
+        *reinterpret_cast<float4*>(&sq[x / (D / 4)][x % (D / 4) * 4]) = make_float4(w[0], w[1], w[2], w[3]);
+        Vec4<TIn>::load(k + at, w);
+        *reinterpret_cast<float4*>(&sk[x / (D / 4)][x % (D / 4) * 4]) = make_float4(w[0], w[1], w[2], w[3]);
+        Vec4<TIn>::load(v + at, w);
+        *reinterpret_cast<float4*>(&sv[x / (D / 4)][x % (D / 4) * 4]) = make_float4(w[0], w[1], w[2], w[3]);
+      }
+      __syncthreads();
     }
-    float4 vv;
-    {
-      const TIn* vp = v + head_off + (size_t)t * sT + 4 * col4;
-      vv = make_float4(to_f32<TIn>(vp[0]), to_f32<TIn>(vp[1]), to_f32<TIn>(vp[2]), to_f32<TIn>(vp[3]));
-    }
-    __syncthreads();
+    const float4 vv = *reinterpret_cast<const float4*>(&sv[u][4 * col4]);
 
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int p = 0; p < PASSES; ++p) {
       const int i = row0 + p * RPP;
-      const float ki = sk[i], qi = sq[i];
+      const float ki = sk[u][i], qi = sq[u][i];
       float4 x = s[p];
       x.x = fmaf(lam, x.x, ki * vv.x);
       x.y = fmaf(lam, x.y, ki * vv.y);
@@ -74,23 +86,20 @@ decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* _
       acc.z = fmaf(x.z, qi, acc.z);
       acc.w = fmaf(x.w, qi, acc.w);
     }
-    red[row0][col4] = acc;
+    red[t & 1][row0][col4] = acc;
     __syncthreads();
     if (tid < LPR) {
-      float4 sum = red[0][tid];
+      float4 sum = red[t & 1][0][tid];
 #pragma unroll
       for (int r = 1; r < RPP; ++r) {
-        const float4 u = red[r][tid];
-        sum.x += u.x; sum.y += u.y; sum.z += u.z; sum.w += u.w;
+        const float4 w = red[t & 1][r][tid];
+        sum.x += w.x; sum.y += w.y; sum.z += w.z; sum.w += w.w;
       }
       TOut* op = o + head_off + (size_t)t * sT + 4 * tid;
-      op[0] = from_f32<TOut>(sum.x);
-      op[1] = from_f32<TOut>(sum.y);
-      op[2] = from_f32<TOut>(sum.z);
-      op[3] = from_f32<TOut>(sum.w);
+      const float w[4] = {sum.x, sum.y, sum.z, sum.w};
+      Vec4<TOut>::store(op, w);
     }
-    // (the next token's q, k are written to sq, sk only after every thread has passed the barrier above; red is
-    // rewritten only after the next barrier)
+    // (red has two copies: the one read here is written again after the barrier of the next token)
   }
 }
 

@@ -67,3 +67,24 @@ def test_full_precision_rows(d, N, seg_len, layout):
     back = (lambda x: x.transpose(1, 2)) if layout else (lambda x: x)
     for name, g, r in zip(("o", "kv", "dq", "dk", "dv", "gin"), (back(o), kv, back(dq), back(dk), back(dv), gin), ref):
         assert_close(g, r, 9.2e-5, name)
+
+
+@pytest.mark.parametrize("d,T,layout", [(64, 8, 0), (128, 8, 1), (64, 9, 1), (128, 17, 0)])
+def test_decode_token_counts(d, T, layout):
+    """One chunk of tokens on chip, one more than that, two and one more.  Each o adds d fp32 products of a state that has
+    been rounded at most T times: (d + 2 T) * 2^-24 of up to 8 RMS, at most 7.8e-5."""
+    B, H = 2, 3
+    gen = torch.Generator().manual_seed(T)
+    q, k, v = [torch.randn(B, H, T, d, generator=gen).bfloat16() for _ in range(3)]
+    kv0 = torch.randn(B, H, d, d, generator=gen)
+    lam = torch.tensor([1.0, 0.97, 1e-20])
+    state = kv0.double().numpy().copy()
+    ref = [orc.decode_step(q[:, :, t], k[:, :, t], v[:, :, t], lam.double().numpy(), state) for t in range(T)]
+    move = (lambda x: x.transpose(1, 2).contiguous()) if layout else (lambda x: x)
+    shape = la.make_shape(B, H, T, d, d, torch.bfloat16, torch.float32, layout=la.LA_LAYOUT_BNHD if layout else la.LA_LAYOUT_BHND)
+    dev = [move(x).cuda() for x in (q, k, v)]
+    kv, o = kv0.cuda(), torch.empty(dev[0].shape, device="cuda")
+    la.la_decode_steps(shape, *dev, lam, kv, o)
+    for t in range(T):
+        assert_close(move(o)[:, :, t:t + 1], ref[t][:, :, None, :], 7.8e-5, "o[%d]" % t)
+    assert_close(kv, state, 7.8e-5, "state")
