@@ -50,6 +50,13 @@ struct Packed {
   int total_tokens;
 };
 
+// A folded batch: entries t and t + batches of the shape's B = 2 * batches read the same entry t of the tensors named here.
+struct Folded {
+  int batches;
+  const void* tensors[2];
+  bool has(const void* p) const { return batches && (p == tensors[0] || p == tensors[1]); }
+};
+
 struct Plan {
   int BH, seg_len, nseg;
   bool tensor;      // tensor-core kernels
@@ -58,6 +65,7 @@ struct Plan {
   bool rows;        // CUDA-core kernels: short segments, every row tile by itself (no chain of blocks)
   int precision;    // LA_SPLIT_* bits (tensor path)
   Packed pk;        // start == NULL: dense batch
+  Folded fold;      // batches == 0: none
 };
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -91,6 +99,7 @@ bool tensor_path_available(const la_shape* s) {
 // `packed`: the plan of a packed batch, whose sequences of different lengths share one segment length.
 la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
   p->pk = Packed{nullptr, nullptr, nullptr, 0};
+  p->fold = Folded{0, {nullptr, nullptr}};
   p->BH = s->B * s->H;
   if (s->path == LA_PATH_TENSOR && !tensor_path_available(s)) return LA_ERR_UNSUPPORTED;
   p->tensor = (s->path == LA_PATH_TENSOR) || (s->path == LA_PATH_AUTO && tensor_path_available(s));
@@ -218,6 +227,8 @@ cudaError_t run_prepass(const la_shape* s, const Plan& p, const DecayTable& tab,
   args.seq_len = p.pk.len;
   args.seq_order = p.pk.order;
   args.total_tokens = p.pk.total_tokens;
+  args.fold = p.fold.batches;
+  args.shared = (p.fold.has(b) ? SHARED_B : 0) | (p.fold.has(c) ? SHARED_C : 0);
   set_strides(s, p.pk.start ? p.pk.total_tokens : s->N, &args);
   if (p.tensor) return launch_tc_prepass(args, tab, s->d, p.precision, all_segments, st);
   return launch_simt_prepass(args, tab, s->d, s->e, (int)s->in_dtype, st);
@@ -306,6 +317,8 @@ OpArgs walk_args(const la_shape* s, const Plan& p, const void* a, const void* b,
   args.seq_len = p.pk.len;
   args.seq_order = p.pk.order;
   args.total_tokens = p.pk.total_tokens;
+  args.fold = p.fold.batches;
+  args.shared = (p.fold.has(a) ? SHARED_A : 0) | (p.fold.has(b) ? SHARED_B : 0) | (p.fold.has(c) ? SHARED_C : 0);
   set_strides(s, p.pk.start ? p.pk.total_tokens : s->N, &args);
   return args;
 }
@@ -321,11 +334,12 @@ cudaError_t run_walk(const la_shape* s, const Plan& p, const DecayTable& tab, co
 
 la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const void* v, const void* u,
                    const float* lambda_host, void* y, void* o, float* rstd, const float* kv_in, float* kv_out,
-                   void* workspace, size_t workspace_bytes, void* stream, const Packed* pk = nullptr);
+                   void* workspace, size_t workspace_bytes, void* stream, const Packed* pk = nullptr,
+                   const Folded* fold = nullptr);
 la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const void* v, const void* d_o,
                    const float* lambda_host, void* dq, void* dk, void* dv, const float* kv_in,
                    const float* grad_kv_out, float* grad_kv_in, const void* fwd_workspace, void* workspace,
-                   size_t workspace_bytes, void* stream, const Packed* pk);
+                   size_t workspace_bytes, void* stream, const Packed* pk, const Folded* fold = nullptr);
 la_status decode_impl(const la_shape* shape, int T, const void* q, const void* k, const void* v,
                       const float* lambda_host, float* kv, void* o, void* stream);
 
@@ -401,7 +415,7 @@ namespace {
 // y = SRMSNorm(o) (.) u, fused into the walk where the kernel can, else by a row kernel behind it.
 la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const void* v, const void* u,
                    const float* lambda_host, void* y, void* o, float* rstd, const float* kv_in, float* kv_out,
-                   void* workspace, size_t workspace_bytes, void* stream, const Packed* pk) {
+                   void* workspace, size_t workspace_bytes, void* stream, const Packed* pk, const Folded* fold) {
   la_status st = check_shape(shape, true);
   if (st != LA_OK) return st;
   if (!q || !k || !v || (!u && !o)) return LA_ERR_INVALID_ARG;
@@ -413,6 +427,7 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   Plan p;
   if ((st = make_plan(shape, &p, pk != nullptr)) != LA_OK) return st;
   if (pk) p.pk = *pk;
+  if (fold) p.fold = *fold;
   p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
   const size_t need = p.nseg > 1 ? 2 * one : 0;
@@ -486,7 +501,7 @@ namespace {
 la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const void* v, const void* d_o,
                    const float* lambda_host, void* dq, void* dk, void* dv, const float* kv_in,
                    const float* grad_kv_out, float* grad_kv_in, const void* fwd_workspace, void* workspace,
-                   size_t workspace_bytes, void* stream, const Packed* pk) {
+                   size_t workspace_bytes, void* stream, const Packed* pk, const Folded* fold) {
   la_status st = check_shape(shape, true);
   if (st != LA_OK) return st;
   if (!q || !k || !v || !d_o || !dq || !dk || !dv) return LA_ERR_INVALID_ARG;
@@ -499,6 +514,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   Plan p;
   if ((st = make_plan(shape, &p, pk != nullptr)) != LA_OK) return st;
   if (pk) p.pk = *pk;
+  if (fold) p.fold = *fold;
   p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
   if (!workspace || workspace_bytes < 3 * one) return LA_ERR_WORKSPACE;
@@ -561,6 +577,37 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   return LA_OK;
 }
 }  // namespace
+}  // namespace la
+
+namespace la {
+// Two runs over one batch as one run over twice the batch: q, k (and what they yield: o, dq, dk, dv and the states) have
+// 2 * half->B entries, v and d_o half->B.  Only where the kernels fold a batch.
+static la_shape doubled(const la_shape* half) {
+  la_shape s = *half;
+  s.B *= 2;
+  return s;
+}
+size_t halves_workspace(int op, const la_shape* half) {
+  const la_shape s = doubled(half);
+  Plan p;
+  if (half->B > (1 << 20) || check_shape(&s, true) != LA_OK || make_plan(&s, &p) != LA_OK || !p.chains) return (size_t)-1;
+  return la_workspace_bytes(op, &s);
+}
+la_status halves_fwd(const la_shape* half, const void* q, const void* k, const void* v, const float* lambda_host, void* o,
+                     const float* kv_in, float* kv_out, void* workspace, size_t workspace_bytes, void* stream) {
+  const la_shape s = doubled(half);
+  const Folded fold{half->B, {v, v}};
+  return fwd_impl(&s, q, k, v, nullptr, lambda_host, nullptr, o, nullptr, kv_in, kv_out, workspace, workspace_bytes, stream, nullptr,
+                  &fold);
+}
+la_status halves_bwd(const la_shape* half, const void* q, const void* k, const void* v, const void* d_o, const float* lambda_host,
+                     void* dq, void* dk, void* dv, const float* kv_in, const float* grad_kv_out, float* grad_kv_in, void* workspace,
+                     size_t workspace_bytes, void* stream) {
+  const la_shape s = doubled(half);
+  const Folded fold{half->B, {v, d_o}};
+  return bwd_impl(&s, q, k, v, d_o, lambda_host, dq, dk, dv, kv_in, grad_kv_out, grad_kv_in, nullptr, workspace, workspace_bytes,
+                  stream, nullptr, &fold);
+}
 }  // namespace la
 
 extern "C" {

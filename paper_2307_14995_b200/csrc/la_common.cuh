@@ -37,6 +37,7 @@ struct DecayTable {
 
 // Arguments of one generic-operator launch (either the walking kernel or the
 // state-only pre-pass).
+constexpr int SHARED_A = 1, SHARED_B = 2, SHARED_C = 4;
 struct OpArgs {
   const void* a;      // [BH, N, Da]  (unused by the pre-pass)
   const void* b;      // [BH, N, Da]
@@ -72,6 +73,10 @@ struct OpArgs {
   // bound below is the sequence's own length.
   const int* seq_start;
   const int* seq_len;
+  // Folded batch (tensor-core kernels at Da = Ec = 128 only; 0 elsewhere): batch entries t and t + fold read the same
+  // entry t of the operands in `shared` (SHARED_* bits), which have `fold` batch entries.
+  int fold;
+  int shared;
   const int* seq_order;  // the order in which thread blocks take the sequences (longest first), or NULL
   int total_tokens;
 };

@@ -21,6 +21,13 @@
 #include "la_common.cuh"
 
 namespace la {
+// Both halves of the features as one run over twice the batch (la_api.cu); the size is (size_t)-1 where that cannot be.
+size_t halves_workspace(int op, const la_shape* half);
+la_status halves_fwd(const la_shape* half, const void* q, const void* k, const void* v, const float* lambda_host, void* o,
+                     const float* kv_in, float* kv_out, void* workspace, size_t workspace_bytes, void* stream);
+la_status halves_bwd(const la_shape* half, const void* q, const void* k, const void* v, const void* d_o, const float* lambda_host,
+                     void* dq, void* dk, void* dv, const float* kv_in, const float* grad_kv_out, float* grad_kv_in, void* workspace,
+                     size_t workspace_bytes, void* stream);
 namespace {
 
 constexpr int RUN = 16;  // consecutive tokens a group of d/4 lanes walks
@@ -353,6 +360,9 @@ struct Carve {
   size_t op;         // workspace of the inner la_fwd / la_bwd
   size_t angles;     // bytes of the angle table
   int ntiles;
+  // One run over both halves: half the launches, and twice the heads to fill the chip with (1 x 16 heads x 8192, d = 128,
+  // forward plus backward 660 us as two runs, 565 as one).  Its operands lie one after the other, so tensors may not be padded.
+  bool one_run;
   int n_f32;         // fp32 temporaries
   size_t total;
 };
@@ -360,9 +370,12 @@ struct Carve {
 bool carve(int op, const la_shape* s, Carve* c) {
   la_shape inner = *s;
   inner.out_dtype = LA_F32;
-  const size_t op_ws = la_workspace_bytes(op, &inner);
+  size_t op_ws = la_workspace_bytes(op, &inner);
   if (op_ws == (size_t)-1 || s->d != s->e) return false;
   const size_t elems = (size_t)s->B * s->H * s->N * s->d;
+  const size_t both = elems % 128 == 0 ? halves_workspace(op, &inner) : (size_t)-1;
+  c->one_run = both != (size_t)-1;
+  if (c->one_run) op_ws = both;
   c->feat = up256(elems * (s->in_dtype == LA_BF16 ? 2 : 4));
   c->f32 = up256(elems * 4);
   c->ntiles = (s->N + tile_tokens(s->d) - 1) / tile_tokens(s->d);
@@ -371,10 +384,10 @@ bool carve(int op, const la_shape* s, Carve* c) {
   c->angles = up256(angle_count(s) * sizeof(float2));
   const bool out32 = s->out_dtype == LA_F32;
   if (op == LA_OP_FWD) {
-    c->n_f32 = out32 ? 1 : 2;                    // the second run's result (and the first's when o is bf16)
+    c->n_f32 = out32 && !c->one_run ? 1 : 2;                    // the second run's result (and the first's when o is bf16)
     c->total = 4 * c->feat + c->n_f32 * c->f32 + c->angles + c->op;
   } else {
-    c->n_f32 = 4 + (out32 ? 1 : 2);              // gradients of the four feature tensors, dv of the runs
+    c->n_f32 = 4 + (out32 && !c->one_run ? 1 : 2);              // gradients of the four feature tensors, dv of the runs
     c->total = 4 * c->feat + c->n_f32 * c->f32 + 2 * c->part + c->angles + c->op;
   }
   return true;
@@ -416,6 +429,11 @@ la_status la_lrpe_fwd(const la_shape* shape, const void* q, const void* k, const
 
   if (run_angles(shape, theta, table, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
   if (run_features(shape, q, k, table, qc, qs, kc, ks, cs) != cudaSuccess) return LA_ERR_CUDA;
+  if (c.one_run) {
+    const la_status st = halves_fwd(&inner, qc, kc, v, lambda_host, tmp, kv_in, kv_out, op_ws, c.op, stream);
+    if (st != LA_OK) return st;
+    return run_sum(shape, tmp, tmp + c.f32 / 4, o, cs) == cudaSuccess ? LA_OK : LA_ERR_CUDA;
+  }
   float* first = out32 ? static_cast<float*>(o) : tmp + c.f32 / 4;
   la_status st = la_fwd(&inner, qc, kc, v, lambda_host, first, kv_in, kv_out, op_ws, c.op, stream);
   if (st != LA_OK) return st;
@@ -443,12 +461,16 @@ la_status la_lrpe_bwd(const la_shape* shape, const void* q, const void* k, const
   void* qc = w; void* qs = w + c.feat; void* kc = w + 2 * c.feat; void* ks = w + 3 * c.feat;
   w += 4 * c.feat;
   float* g_qc = reinterpret_cast<float*>(w);
-  float* g_kc = reinterpret_cast<float*>(w + c.f32);
-  float* g_qs = reinterpret_cast<float*>(w + 2 * c.f32);
+  float* g_qs = reinterpret_cast<float*>(w + c.f32);
+  float* g_kc = reinterpret_cast<float*>(w + 2 * c.f32);
   float* g_ks = reinterpret_cast<float*>(w + 3 * c.f32);
   float* dv_s = reinterpret_cast<float*>(w + 4 * c.f32);
   const bool out32 = shape->out_dtype == LA_F32;
   float* dv_c = out32 ? static_cast<float*>(dv) : reinterpret_cast<float*>(w + 5 * c.f32);
+  if (c.one_run) {
+    dv_c = dv_s;
+    dv_s = reinterpret_cast<float*>(w + 5 * c.f32);
+  }
   w += c.n_f32 * c.f32;
   float* part_q = reinterpret_cast<float*>(w);
   float* part_k = reinterpret_cast<float*>(w + c.part);
@@ -460,13 +482,17 @@ la_status la_lrpe_bwd(const la_shape* shape, const void* q, const void* k, const
 
   if (run_angles(shape, theta, table, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
   if (run_features(shape, q, k, table, qc, qs, kc, ks, cs) != cudaSuccess) return LA_ERR_CUDA;
-  la_status st = la_bwd(&inner, qc, kc, v, d_o, lambda_host, g_qc, g_kc, dv_c, kv_in, grad_kv_out, grad_kv_in, op_ws,
-                        c.op, stream);
-  if (st != LA_OK) return st;
-  st = la_bwd(&inner, qs, ks, v, d_o, lambda_host, g_qs, g_ks, dv_s, kv_in ? kv_in + state : nullptr,
-              grad_kv_out ? grad_kv_out + state : nullptr, grad_kv_in ? grad_kv_in + state : nullptr, op_ws, c.op,
-              stream);
-  if (st != LA_OK) return st;
+  la_status st;
+  if (c.one_run) {
+    st = halves_bwd(&inner, qc, kc, v, d_o, lambda_host, g_qc, g_kc, dv_c, kv_in, grad_kv_out, grad_kv_in, op_ws, c.op, stream);
+    if (st != LA_OK) return st;
+  } else {
+    st = la_bwd(&inner, qc, kc, v, d_o, lambda_host, g_qc, g_kc, dv_c, kv_in, grad_kv_out, grad_kv_in, op_ws, c.op, stream);
+    if (st != LA_OK) return st;
+    st = la_bwd(&inner, qs, ks, v, d_o, lambda_host, g_qs, g_ks, dv_s, kv_in ? kv_in + state : nullptr,
+                grad_kv_out ? grad_kv_out + state : nullptr, grad_kv_in ? grad_kv_in + state : nullptr, op_ws, c.op, stream);
+    if (st != LA_OK) return st;
+  }
   if (run_sum(shape, dv_c, dv_s, dv, cs) != cudaSuccess) return LA_ERR_CUDA;
   if (run_grad(shape, GradSet{q, g_qc, g_qs, dq, part_q}, GradSet{k, g_kc, g_ks, dk, part_k}, table, pos0, c.ntiles, cs) !=
       cudaSuccess)

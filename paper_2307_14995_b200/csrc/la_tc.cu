@@ -116,6 +116,7 @@ struct TcJob {
   const float* z_in;
   const float* local;
   bool z_in_t, local_t;
+  int shared;  // see OpArgs
   // gate epilogue of the forward walk (D = 128 only): y = SRMSNorm(out) (.) u
   const void* u;
   void* y;
@@ -135,7 +136,7 @@ struct TcArgs {
   int njobs;
   int BH, H, N, seg_len, nseg;
   int precision;
-  int scanned;  // see OpArgs
+  int scanned, fold;  // see OpArgs
   long long sT, sH, sB;  // element offset of token t of (b,h): b*sB + h*sH + t*sT (rows of D contiguous features)
 };
 
@@ -857,13 +858,13 @@ EncodeTiledFn encode_fn() {
 
 // Tensor map over a token tensor seen as {feature D, token N, head H, batch B} with element strides {1, sT, sH, sB}
 // (D = 64 or 128, bf16 or fp32), a box of 128 bytes x box_tokens x 1 x 1 and 128-byte swizzle; tokens beyond N read
-// as zero and are not written.
-bool make_map(CUtensorMap* m, const void* ptr, const OpArgs& a, int D, bool f32 = false, int box_tokens = 128) {
+// as zero and are not written.  shared: one of the operands that the two halves of a folded batch have in common.
+bool make_map(CUtensorMap* m, const void* ptr, const OpArgs& a, int D, bool f32 = false, int box_tokens = 128, bool shared = false) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
   const cuuint64_t esz = f32 ? 4 : 2;
   // packed batch: one [total_tokens, H, D] tensor, batch extent 1
-  const int B = a.seq_start ? 1 : a.BH / a.H;
+  const int B = a.seq_start ? 1 : shared ? a.fold : a.BH / a.H;
   const int tokens = a.seq_start ? a.total_tokens : a.N;
   cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)tokens, (cuuint64_t)a.H, (cuuint64_t)B};
   cuuint64_t strides[3] = {(cuuint64_t)a.sT * esz, (cuuint64_t)a.sH * esz, (cuuint64_t)a.sB * esz};
@@ -888,7 +889,10 @@ cudaError_t launch_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, const
 
 // out_f32: the type of the map over `out`, or NULL where the kernel stores its output without one.
 bool make_maps(TcMaps* m, const OpArgs& args, int D, const bool* out_f32) {
-  if (!(make_map(&m->a, args.a, args, D) && make_map(&m->b, args.b, args, D) && make_map(&m->c, args.c, args, D))) return false;
+  if (!(make_map(&m->a, args.a, args, D, false, 128, args.shared & SHARED_A) &&
+        make_map(&m->b, args.b, args, D, false, 128, args.shared & SHARED_B) &&
+        make_map(&m->c, args.c, args, D, false, 128, args.shared & SHARED_C)))
+    return false;
   if (!out_f32) {
     m->out = m->c;
     return true;
@@ -897,7 +901,7 @@ bool make_maps(TcMaps* m, const OpArgs& args, int D, const bool* out_f32) {
 }
 
 TcJob make_job(const OpArgs& a) {
-  return TcJob{a.c, a.out, a.entry, a.final_out, a.z_in, a.local, a.z_in_t != 0, a.local_t != 0, a.u, a.y, a.rstd};
+  return TcJob{a.c, a.out, a.entry, a.final_out, a.z_in, a.local, a.z_in_t != 0, a.local_t != 0, a.shared, a.u, a.y, a.rstd};
 }
 
 TcArgs make_args(const OpArgs& args, const OpArgs* second, int precision) {
@@ -909,6 +913,7 @@ TcArgs make_args(const OpArgs& args, const OpArgs* second, int precision) {
   ta.BH = args.BH; ta.H = args.H; ta.N = args.N; ta.seg_len = args.seg_len; ta.nseg = args.nseg;
   ta.precision = precision;
   ta.scanned = args.scanned;
+  ta.fold = args.fold;
   ta.sT = args.sT; ta.sH = args.sH; ta.sB = args.sB;
   ta.seq_start = args.seq_start;
   ta.seq_len = args.seq_len;
@@ -941,7 +946,7 @@ cudaError_t launch_walk64(const OpArgs& args, const OpArgs* second, const DecayT
                           cudaStream_t stream) {
   TcMaps m0, m1;
   const bool f32 = (out_dt == DT_F32);
-  if (args.seq_start || args.u) return cudaErrorInvalidValue;  // packed batches and the gate: D = 128 only
+  if (args.seq_start || args.u || args.fold) return cudaErrorInvalidValue;  // packed and folded batches, the gate: D = 128 only
   if (!make_maps(&m0, args, 64, &f32)) return cudaErrorInvalidValue;
   m1 = m0;
   if (second && !make_maps(&m1, *second, 64, &f32)) return cudaErrorInvalidValue;
@@ -960,7 +965,7 @@ cudaError_t launch_walk64(const OpArgs& args, const OpArgs* second, const DecayT
 
 cudaError_t launch_prepass64(const OpArgs& args, const DecayTable& tab, int precision, cudaStream_t stream) {
   TcMaps m;
-  if (args.seq_start) return cudaErrorInvalidValue;  // packed batches: D = 128 only
+  if (args.seq_start || args.fold) return cudaErrorInvalidValue;  // packed and folded batches: D = 128 only
   // the a and out maps are unused by the state-only kernel; valid descriptors are passed anyway
   if (!make_map(&m.b, args.b, args, 64) || !make_map(&m.c, args.c, args, 64)) return cudaErrorInvalidValue;
   m.a = m.b;
@@ -972,7 +977,8 @@ cudaError_t launch_prepass64(const OpArgs& args, const DecayTable& tab, int prec
 
 cudaError_t launch_states128(const OpArgs& args, const DecayTable& tab, int precision, bool all_segments, cudaStream_t stream) {
   TcMaps m;
-  if (!make_map(&m.b, args.b, args, 128, false, 64) || !make_map(&m.c, args.c, args, 128, false, 64))
+  if (!make_map(&m.b, args.b, args, 128, false, 64, args.shared & SHARED_B) ||
+      !make_map(&m.c, args.c, args, 128, false, 64, args.shared & SHARED_C))
     return cudaErrorInvalidValue;
   const TcArgs ta = make_args(args, nullptr, precision);
   return args.reverse ? launch_state_t<true>(m, ta, tab, all_segments, stream)

@@ -84,6 +84,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
   const int n_tok = args.seq_len ? args.seq_len[b] : args.N;
   const int tok0 = args.seq_start ? args.seq_start[b] : 0;
   const int bb = args.seq_start ? 0 : b;
+  const int bf = args.fold && bb >= args.fold ? bb - args.fold : bb;  // of an operand that is shared
+  const int bat_b = args.job[0].shared & SHARED_B ? bf : bb, bat_c = args.job[0].shared & SHARED_C ? bf : bb;
   const int seg_t0 = seg * args.seg_len, seg_t1 = min(n_tok, seg_t0 + args.seg_len);
   if (seg_t0 >= n_tok) return;  // (all thread blocks of a cluster that shares a segment alike)
   const float s2 = (float)tab.s2[h];
@@ -141,10 +143,10 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
         const int t = tok0 + seg_t0 + piece(it) * 64;
         uint64_t* bar = &sm.bars[S_FULL0 + s];
         mbar_arrive_expect_tx(bar, 32768);
-        tma_load_4d(&sm.stage[s].c[0][0], &map_c, bar, 0, t, h, bb);
-        tma_load_4d(&sm.stage[s].c[1][0], &map_c, bar, 64, t, h, bb);
-        tma_load_4d(&sm.stage[s].b[0][0], &map_b, bar, 0, t, h, bb);
-        tma_load_4d(&sm.stage[s].b[1][0], &map_b, bar, 64, t, h, bb);
+        tma_load_4d(&sm.stage[s].c[0][0], &map_c, bar, 0, t, h, bat_c);
+        tma_load_4d(&sm.stage[s].c[1][0], &map_c, bar, 64, t, h, bat_c);
+        tma_load_4d(&sm.stage[s].b[0][0], &map_b, bar, 0, t, h, bat_b);
+        tma_load_4d(&sm.stage[s].b[1][0], &map_b, bar, 64, t, h, bat_b);
         armed = it + 1;
         if (++s == S_STAGES) s = 0, phase ^= 1;
       }

@@ -236,16 +236,18 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
         const TcMaps* const maps = jobid ? &maps1 : &maps0;
         const int hh_ = bh % args.H;  // head coordinate of the 4-D tensor maps
         const int bb_ = args.seq_start ? 0 : bh / args.H;
+        const int bf_ = args.fold && bb_ >= args.fold ? bb_ - args.fold : bb_;  // of an operand that is shared
         auto token = [&](int it) { return tok0 + seg_t0 + (REV ? (nblk - 1 - it) : it) * 128; };
-        auto load = [&](int bar_id, __nv_bfloat16* dst, const CUtensorMap* map, int it) {
+        auto load = [&](int bar_id, __nv_bfloat16* dst, const CUtensorMap* map, int it, int batch) {
           uint64_t* bar = &sm.bars[bar_id];
           mbar_arrive_expect_tx(bar, 32768);
-          tma_load_4d(dst, map, bar, 0, token(it), hh_, bb_);
-          tma_load_4d(dst + 128 * 64, map, bar, 64, token(it), hh_, bb_);
+          tma_load_4d(dst, map, bar, 0, token(it), hh_, batch);
+          tma_load_4d(dst + 128 * 64, map, bar, 64, token(it), hh_, batch);
         };
-        auto load_a = [&](int it) { load(W_M1_OK0 + (it & 1), &sm.a[0][0], &maps->a, it); };
-        auto load_b = [&](int it) { load(W_M1_OK0 + (it & 1), &sm.b[it & 1][0][0], &maps->b, it); armed_ab = it + 1; };
-        auto load_c = [&](int it) { load(W_FULL_C0 + (it & 1), &sm.c[it & 1][0][0], &maps->c, it); armed_c = it + 1; };
+        const int ba = job.shared & SHARED_A ? bf_ : bb_, bb = job.shared & SHARED_B ? bf_ : bb_, bc = job.shared & SHARED_C ? bf_ : bb_;
+        auto load_a = [&](int it) { load(W_M1_OK0 + (it & 1), &sm.a[0][0], &maps->a, it, ba); };
+        auto load_b = [&](int it) { load(W_M1_OK0 + (it & 1), &sm.b[it & 1][0][0], &maps->b, it, bb); armed_ab = it + 1; };
+        auto load_c = [&](int it) { load(W_FULL_C0 + (it & 1), &sm.c[it & 1][0][0], &maps->c, it, bc); armed_c = it + 1; };
         load_b(0);
         load_a(0);
         load_c(0);
