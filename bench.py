@@ -66,11 +66,11 @@ def bytes_per_token_head(d: int, out_bytes: int, what: str) -> float:
 
 
 # DRAM traffic of one walk launch per token-head, from the ncu capture summarised in
-# profiles/tc_walk_full_kernel_small_case.md: 412.4 MB read per 524288 token-heads (the algorithmic
-# 768 B plus 2.4 % for entry states and re-fetches).  The writes of that small launch (230 MB of the
-# 268 MB of output; the rest was still in L2 when it ended) do not grow in proportion: at full size
+# profiles/tc_walk_kernel_small_case.md: 207.7 MB read per 262144 token-heads (the algorithmic
+# 768 B plus 3.2 % for segment states and re-fetches).  The writes of that small launch (91 MB of the
+# 134 MB of output; the rest was still in L2 when it ended) do not grow in proportion: at full size
 # the 4.3 GB of output cannot stay in the 126 MB L2, so the output is counted in full (512 B).
-WALK_DRAM_BYTES_PER_TOKEN_HEAD = 412.4e6 / 524288 + 512.0
+WALK_DRAM_BYTES_PER_TOKEN_HEAD = 207.7e6 / 262144 + 512.0
 
 
 def load_peaks():
@@ -630,11 +630,11 @@ def run_ours(args):
             "kernel_launches_per_step": {kname: c / prof_steps for kname, (_, c) in prof.items()},
             "fwd_ms": split_ms.get("fwd"), "bwd_ms": split_ms.get("bwd"), "gated_forward": gated, "lrpe_d": lrpe, "sequence_parallel": seqpar_leg, "varlen_prefill": varlen_leg, "sustained": sustained,
             "roofline": {"scope": "ONE kernel, the dominant one; the whole-step figure the target is stated on is step_roofline",
-                         "kernel": "full-width block walk (tc_walk_full_kernel), single-job launches (O and dQ)", "bound": "hbm",
+                         "kernel": "block walk (tc_walk_kernel), single-job launches (O and dQ)", "bound": "hbm",
                          "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": (achieved / peaks["hbm_gbs"]) if achieved else None,
                          "traffic": WALK_DRAM_BYTES_PER_TOKEN_HEAD * th,
-                         "traffic_note": "ncu dram read bytes of a 524288-token-head launch scaled by token-heads + the full fp32 output",
+                         "traffic_note": "ncu dram read bytes of a 262144-token-head launch scaled by token-heads + the full fp32 output",
                          "peak_source": peaks["source"],
                          "avg_launch_ms": walk_avg_ms, "launches": walk_n, "bytes_per_launch": walk_bytes,
                          "walk_pair": {"what": "the dV and dK walks of the backward pass in one launch",

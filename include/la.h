@@ -389,7 +389,7 @@ unsigned long long la_launch_count(void);
  * the launches, so a loop timed as a whole should run with it off.
  */
 #define LA_KERNEL_PREPASS 0 /* segment-local states            */
-#define LA_KERNEL_SCAN 1    /* state scan across segments      */
+#define LA_KERNEL_SCAN 1    /* scan or running sums of states  */
 #define LA_KERNEL_WALK 2    /* block walk producing o/dq/dk/dv */
 #define LA_KERNEL_DECODE 3  /* recurrent decode step           */
 #define LA_KERNEL_WALK_PAIR 4 /* the dV and dK walks of the backward pass in one launch */

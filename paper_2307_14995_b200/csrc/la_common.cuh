@@ -126,8 +126,6 @@ cudaError_t launch_prefix(const ScanArgs& args, const DecayTable& tab, cudaStrea
 __host__ __device__ inline float state_reach(float s2, int seg_len) { return s2 > 0.f ? 160.f / (s2 * (float)seg_len) : 3.0e38f; }
 __host__ __device__ inline bool slow_head(float s2, int seg_len) { return state_reach(s2, seg_len) >= 2.f; }
 cudaError_t launch_chain(const ChainArgs& args, const DecayTable& tab, cudaStream_t stream);
-// dst[m] = transpose(src[m]) for `count` row-major Da x Ec fp32 matrices.
-cudaError_t launch_transpose_states(const float* src, float* dst, long count, int Da, int Ec, cudaStream_t stream);
 // T >= 1 consecutive tokens per (batch, head); token t of (b,h) is the row at element offset b*sB + h*sH + t*sT.
 cudaError_t launch_decode(const void* q, const void* k, const void* v, float* kv, void* o, int BH,
                           int H, int T, int d, int e, int in_dt, int out_dt, long long sT, long long sH, long long sB,

@@ -1,13 +1,11 @@
 // fp32 CUDA-core kernels of the generic decayed linear-attention operator
-// (see la_common.cuh for the block formulas).  They serve the fp32 workload,
-// head dimension 64, and are the full-precision second opinion for the
-// tensor-core kernels.  All arithmetic is fp32 FMA with fp32 accumulation;
-// bf16 inputs are widened exactly on load.
+// (see la_common.cuh for the block formulas).  They serve fp32 inputs and are the full-precision second opinion for the
+// tensor-core kernels.  All arithmetic is fp32 FMA with fp32 accumulation; bf16 inputs are widened exactly on load.
 //
-// Block size C = 32 tokens, 256 threads per thread block, one thread block per
-// (batch*head, segment).  Shared memory holds the a/b/c tiles (a and b also
-// transposed so that every inner loop reads consecutive addresses), the masked
-// score tile and the Da x Ec state.
+// Tiles of C = 32 tokens.  simt_rows_kernel: segments of up to ROWS_MAX_SEG tokens, every row tile by itself.
+// simt_walk_kernel: longer segments, one thread block of 256 threads per (batch*head, segment) that carries the Da x Ec state
+// from block to block; shared memory holds the a/b/c tiles (a and b also transposed so that every inner loop reads consecutive
+// addresses), the masked score tile and the state.
 #include <algorithm>
 
 #include "la_common.cuh"
@@ -711,32 +709,6 @@ cudaError_t launch_simt_prepass(const OpArgs& args, const DecayTable& tab, int D
                            : launch_prepass_t<__nv_bfloat16, 128, 128>(args, tab, stream);
   }
   return cudaErrorInvalidValue;
-}
-
-// dst[m] = src[m]^T for `count` row-major Da x Ec matrices (32x32 tiles through shared memory).
-__global__ void __launch_bounds__(256) transpose_states_kernel(const float* __restrict__ src, float* __restrict__ dst,
-                                                               int Da, int Ec) {
-  __shared__ float tile[32][33];
-  const size_t m = blockIdx.x;
-  const int tiles_y = Ec / 32;
-  const int x0 = (blockIdx.y / tiles_y) * 32, y0 = (blockIdx.y % tiles_y) * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const float* s = src + m * Da * Ec;
-  float* d = dst + m * Da * Ec;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) tile[ty + 8 * k][tx] = s[(size_t)(x0 + ty + 8 * k) * Ec + y0 + tx];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 4; ++k) d[(size_t)(y0 + ty + 8 * k) * Da + x0 + tx] = tile[tx][ty + 8 * k];
-}
-
-cudaError_t launch_transpose_states(const float* src, float* dst, long count, int Da, int Ec, cudaStream_t stream) {
-  if ((Da % 32) != 0 || (Ec % 32) != 0 || count < 1 || count > 2147483647L) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)count, (unsigned)((Da / 32) * (Ec / 32)));
-  KernelTimer timer(K_SCAN, stream);
-  transpose_states_kernel<<<grid, 256, 0, stream>>>(src, dst, Da, Ec);
-  count_launch();
-  return cudaGetLastError();
 }
 
 // One thread per four consecutive state elements; the pieces are few (ranks of a sequence-parallel group, or the
