@@ -30,9 +30,13 @@ struct StatePlan {
   unsigned char order[LA_MAX_H];
 };
 
+// The loads of piece p arrive on barrier p % S_FULLS: all pieces of one barrier belong to the same group of workers, which
+// waits for no others.  (With a barrier per stage a group had to see the other's pieces go by, and nothing kept a stage from
+// being loaded again, twice, before a warp that came late had looked; it then waited until its budget ran out.)
+constexpr int S_FULLS = 2 * S_STAGES;
 enum SBar {
   S_FULL0 = 0,
-  S_FREE0 = S_FULL0 + S_STAGES,
+  S_FREE0 = S_FULL0 + S_FULLS,
   S_FC_READY0 = S_FREE0 + S_STAGES,
   S_FC_FREE0 = S_FC_READY0 + 4,
   S_DONE = S_FC_FREE0 + 4,
@@ -138,10 +142,11 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     // ------------------------------------ TMA producer ------------------------------------
     if (lane == 0) {
       int armed = 0;
-      for (int it = 0, s = 0, phase = 0; it < count; ++it) {
+      for (int it = 0, s = 0, phase = 0, f = 0; it < count; ++it) {
         if (it >= S_STAGES) TC_WAIT_TO(producer_done, S_FREE0 + s, phase ^ 1, 31);
         const int t = tok0 + seg_t0 + piece(it) * 64;
-        uint64_t* bar = &sm.bars[S_FULL0 + s];
+        uint64_t* bar = &sm.bars[S_FULL0 + f];
+        if (++f == S_FULLS) f = 0;
         mbar_arrive_expect_tx(bar, 32768);
         tma_load_4d(&sm.stage[s].c[0][0], &map_c, bar, 0, t, h, bat_c);
         tma_load_4d(&sm.stage[s].c[1][0], &map_c, bar, 64, t, h, bat_c);
@@ -153,7 +158,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     producer_done:
       if (sm.abort)  // nothing may be in flight when the block exits
         for (int k = 0; k < S_STAGES; ++k)
-          if (armed - 1 - k >= 0) drain_wait(&sm.bars[S_FULL0 + (armed - 1 - k) % S_STAGES], ((armed - 1 - k) / S_STAGES) & 1);
+          if (armed - 1 - k >= 0) drain_wait(&sm.bars[S_FULL0 + (armed - 1 - k) % S_FULLS], ((armed - 1 - k) / S_FULLS) & 1);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -162,8 +167,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     constexpr uint32_t HI = UMMA_DESC_HI_SBO1024;
     const uint32_t go = elect_one();
     const uint32_t b0 = umma_desc_lo(smem_u32(&sm.stage[0].b[0][0]), 8192);
-    for (int it = 0, s = 0, phase = 0, f = 0, fphase = 0; it < count; ++it) {
-      TC_WAIT_WARP_TO(mma_done, S_FULL0 + s, phase, 32);
+    for (int it = 0, s = 0, u = 0, phase = 0, f = 0, fphase = 0; it < count; ++it) {
+      TC_WAIT_WARP_TO(mma_done, S_FULL0 + u, phase, 32);
       TC_WAIT_WARP_TO(mma_done, S_FC_READY0 + f, fphase, 33);
       tc_fence_after_sync();
       const uint32_t fcol = tmem + SCOL_F + f * fcols;
@@ -171,7 +176,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
       if (split_c) umma_group_tsd4<false>(tmem + SCOL_Z, fcol + 32, b0 + s * 2048, HI, ID_KN, 1, go);
       umma_commit_if(&sm.bars[S_FREE0 + s], go);
       umma_commit_if(&sm.bars[S_FC_FREE0 + f], go);
-      if (++s == S_STAGES) s = 0, phase ^= 1;
+      if (++s == S_STAGES) s = 0;
+      if (++u == S_FULLS) u = 0, phase ^= 1;
       if (++f == nf) f = 0, fphase ^= 1;
     }
     umma_commit_if(&sm.bars[S_DONE], go);
@@ -192,11 +198,11 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     // lane l points ldmatrix at token row (w4 & 1) * 32 + (l >> 4) * 8 + (l & 7), value columns q * 32 + ((l >> 3) & 1) * 8
     const uint32_t unit0 = (uint32_t)((q >> 1) * 8192 + ((w4 & 1) * 32 + ((lane >> 4) << 3) + (lane & 7)) * 128 +
                                       ((((q & 1) * 4 + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
-    for (int it = 0, s = 0, phase = 0, fb = group, fphase = 0; it < count; ++it) {
-      const int st = s;
-      TC_WAIT_WARP(S_FULL0 + st, phase, 34);  // (of every piece: a parity tells a stage's loads apart only one by one)
-      if (++s == S_STAGES) s = 0, phase ^= 1;
-      if ((it & 1) != group) continue;
+    for (int it = group, u = group, phase = 0, fb = group, fphase = 0; it < count; it += 2) {
+      const int st = u < S_STAGES ? u : u - S_STAGES;
+      TC_WAIT_WARP(S_FULL0 + u, phase, 34);
+      u += 2;
+      if (u >= S_FULLS) u -= S_FULLS, phase ^= 1;
       if (it >= nf) TC_WAIT_WARP(S_FC_FREE0 + fb, fphase ^ 1, 35);
       tc_fence_after_sync();
 #pragma unroll

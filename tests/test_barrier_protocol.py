@@ -1,0 +1,81 @@
+"""The hand-offs between the warp roles of the tensor-core kernels as a model on the CPU.
+
+An mbarrier wait names a phase by its parity only.  A waiter that comes so late that the next phase has completed as well
+sees the parity of the phase after that, and if this one needs the waiter's own work it waits until its budget runs out.  So
+no phase may complete while some role has not yet passed its wait for the phase before.
+
+The roles are written down as their sequences of waits and arrivals.  The system has no choices in it (a role only ever waits
+for one thing), so letting every other role run as far as it can shows the most that can happen while one is held up."""
+import pytest
+
+
+def overruns(roles, counts):
+    """roles: name -> list of ("wait", barrier, phase) and ("arrive", barrier); counts: arrivals that complete a phase.
+    Returns the waits (role, barrier, phase) whose following phase can complete before they are passed; the whole must end."""
+
+    def run(held=None, stop=None):
+        at = {r: 0 for r in roles}
+        arrived = {b: 0 for b in counts}
+        moved = True
+        while moved:
+            moved = False
+            for r, ops in roles.items():
+                while at[r] < len(ops) and not (r == held and at[r] == stop):
+                    op = ops[at[r]]
+                    if op[0] == "arrive":
+                        arrived[op[1]] += 1
+                    elif arrived[op[1]] // counts[op[1]] <= op[2]:
+                        break
+                    at[r] += 1
+                    moved = True
+        return at, {b: n // counts[b] for b, n in arrived.items()}
+
+    at, _ = run()
+    assert all(at[r] == len(ops) for r, ops in roles.items()), "the protocol does not end"
+    found = []
+    for r, ops in roles.items():
+        for i, op in enumerate(ops):
+            if op[0] == "wait" and run(r, i)[1][op[1]] > op[2] + 1:
+                found.append((r, op[1], op[2]))
+    return found
+
+
+STAGES = 3
+
+
+def state_kernel(pieces, fc_buffers, full_barriers):
+    """tc_state_kernel: loads in STAGES stages, two groups of workers that take turns (one warp of each here), products.
+    full_barriers: how many barriers the loads' arrivals go round; with one per stage a group must follow every phase."""
+    full = lambda p: "full%d" % (p % full_barriers)
+    n = STAGES
+    producer, mma = [], []
+    groups = {0: [], 1: []}
+    for p in range(pieces):
+        if p >= n:
+            producer.append(("wait", "free%d" % (p % n), p // n - 1))
+        producer.append(("arrive", full(p)))
+        mma += [("wait", full(p), p // full_barriers), ("wait", "fc_ready%d" % (p % fc_buffers), p // fc_buffers),
+                ("arrive", "free%d" % (p % n)), ("arrive", "fc_free%d" % (p % fc_buffers))]
+        for g, ops in groups.items():
+            own = p % 2 == g
+            if own or full_barriers == n:
+                ops.append(("wait", full(p), p // full_barriers))
+            if own:
+                if p >= fc_buffers:
+                    ops.append(("wait", "fc_free%d" % (p % fc_buffers), p // fc_buffers - 1))
+                ops.append(("arrive", "fc_ready%d" % (p % fc_buffers)))
+    roles = {"producer": producer, "mma": mma, "even": groups[0], "odd": groups[1]}
+    return roles, {op[1]: 1 for ops in roles.values() for op in ops}
+
+
+@pytest.mark.parametrize("fc_buffers", [2, 4])
+@pytest.mark.parametrize("pieces", [1, 2, 3, 7, 13, 30])
+def test_state_kernel_phases_are_never_overrun(pieces, fc_buffers):
+    assert overruns(*state_kernel(pieces, fc_buffers, 2 * STAGES)) == []
+
+
+@pytest.mark.parametrize("fc_buffers", [2, 4])
+def test_state_kernel_with_one_barrier_a_stage_would_be_overrun(fc_buffers):
+    # (the group that does not own a piece is held back by nothing)
+    found = overruns(*state_kernel(7, fc_buffers, STAGES))
+    assert ("odd", "full0", 0) in found and ("even", "full1", 0) in found
