@@ -55,8 +55,11 @@ enum WBar {
   W_M4_OK,                   // P written (16 worker warps) and O scaled (8 warps)
   W_S_READY,                 // M1 done
   W_M2_DONE,                 // M2 done: O_inter complete, a and the state operand free
-  W_DZ_READY,                // M3 done: dZ complete, b and fc free
-  W_O_READY,                 // M4 done: O complete, c and P free
+  // M3 done: dZ complete, b and fc free; M4 done: O complete, c and P free.  Of an even / odd block: the producer waits for
+  // those of block n when nothing that M3 and M4 of block n + 1 need is still to come from it, so with one barrier they could
+  // complete as well before a late producer has looked; those of block n + 2 need the loads that it starts after its wait.
+  W_DZ_READY0, W_DZ_READY1,
+  W_O_READY0, W_O_READY1,
   W_GATE0, W_GATE1,          // GATED: a block's sums of squares exchanged (4 warps), per half of the tokens
   W_DRAIN,
   W_NUM_BARS
@@ -259,9 +262,9 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           TC_WAIT_TO(producer_done, W_M2_DONE, it & 1, 3);
           load_a(it + 1);
           if (it + 2 < nblk) {
-            TC_WAIT_TO(producer_done, W_DZ_READY, it & 1, 5);
+            TC_WAIT_TO(producer_done, W_DZ_READY0 + (it & 1), (it >> 1) & 1, 5);
             load_b(it + 2);
-            TC_WAIT_TO(producer_done, W_O_READY, it & 1, 2);
+            TC_WAIT_TO(producer_done, W_O_READY0 + (it & 1), (it >> 1) & 1, 2);
             load_c(it + 2);
           }
         }
@@ -313,7 +316,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           umma_group_tsd<false>(tmem + WCOL_R, tmem + WCOL_FH, buf + OB + MNMAJ, HI, ID_KN, 0, go);
           if (split_c) umma_group_tsd<false>(tmem + WCOL_R, tmem + WCOL_FL, buf + OB + MNMAJ, HI, ID_KN, 1, go);
         }
-        umma_commit_if(&sm.bars[W_DZ_READY], go);
+        umma_commit_if(&sm.bars[W_DZ_READY0 + par], go);
         TC_WAIT_WARP_TO(mma_done, W_FULL_C0 + par, (it >> 1) & 1, 15);
         TC_WAIT_WARP_TO(mma_done, W_M4_OK, par, 14);
         tc_fence_after_sync();
@@ -323,7 +326,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           umma_tri4<REV ? 7 : 0, REV>(tmem + WCOL_O, buf + OC, base + OPL, HI, 1, go);
           umma_tri4<REV ? 3 : 4, REV>(tmem + WCOL_O, buf + OC, base + OPL, HI, 1, go);
         }
-        umma_commit_if(&sm.bars[W_O_READY], go);
+        umma_commit_if(&sm.bars[W_O_READY0 + par], go);
         if (it + 1 < nblk) {
           TC_WAIT_WARP_TO(mma_done, W_M1_OK0 + (par ^ 1), ((it + 1) >> 1) & 1, 11);
           tc_fence_after_sync();
@@ -537,7 +540,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       }
       // ---- Z <- Gamma Z + dZ ----
       const float gamma = ex2_approx(-s2 * (float)(it == (REV ? 0 : nblk - 1) ? edge_len : 128));
-      TC_WAIT_WARP(W_DZ_READY, it & 1, 22);  // M2 and M3 of this block are done
+      TC_WAIT_WARP(W_DZ_READY0 + (it & 1), (it >> 1) & 1, 22);  // M2 and M3 of this block are done
       tc_fence_after_sync();
 #pragma unroll
       for (int pc = 0; pc < 2; ++pc) {
@@ -614,7 +617,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           if (2 * x < mine) upair[x] = load_u32_at(up, (uint32_t)args.sT * 4u, x);
         }
       }
-      TC_WAIT_WARP(W_O_READY, it & 1, 25);
+      TC_WAIT_WARP(W_O_READY0 + (it & 1), (it >> 1) & 1, 25);
       tc_fence_after_sync();
       const uint32_t stride = (uint32_t)args.sT * (uint32_t)sizeof(TOut);
       if constexpr (GATED) {

@@ -79,3 +79,54 @@ def test_state_kernel_with_one_barrier_a_stage_would_be_overrun(fc_buffers):
     # (the group that does not own a piece is held back by nothing)
     found = overruns(*state_kernel(7, fc_buffers, STAGES))
     assert ("odd", "full0", 0) in found and ("even", "full1", 0) in found
+
+
+def walk_kernel(blocks, want_final, ready_barriers):
+    """tc_walk_kernel (one warp of workers, one of the output group).  ready_barriers: how many barriers the completions of M3
+    and of M4 go round."""
+    two, k = lambda name, n: name + str(n % 2), ready_barriers
+    dz, o = (lambda n: ("dz%d" % (n % k))), (lambda n: ("o%d" % (n % k)))
+    producer = [("arrive", "m1_0"), ("arrive", "m1_0"), ("arrive", "c0")]
+    if blocks > 1:
+        producer += [("arrive", "m1_1"), ("arrive", "c1")]
+    for n in range(blocks - 1):
+        producer += [("wait", "m2_done", n), ("arrive", two("m1_", n + 1))]
+        if n + 2 < blocks:
+            producer += [("wait", dz(n), n // k), ("arrive", two("m1_", n)), ("wait", o(n), n // k), ("arrive", two("c", n))]
+    mma = [("wait", "m1_0", 0), ("arrive", "s")]
+    workers = [("arrive", "m1_0"), ("arrive", "m2_ok")]
+    if blocks > 1 or want_final:
+        workers.append(("wait", "c0", 0))
+    output = [("arrive", "m2_ok")]
+    for n in range(blocks):
+        more = n + 1 < blocks
+        mma += [("wait", "m2_ok", n), ("arrive", "m2_done")]
+        if more or want_final:
+            mma.append(("wait", "m3_ok", n))
+        mma += [("arrive", dz(n)), ("wait", two("c", n), n // 2), ("wait", "m4_ok", n), ("arrive", o(n))]
+        if more:
+            mma += [("wait", two("m1_", n + 1), (n + 1) // 2), ("arrive", "s")]
+        workers += [("wait", "s", n), ("arrive", "m3_ok"), ("arrive", "m4_ok")]
+        if more:
+            workers.append(("wait", two("c", n + 1), (n + 1) // 2))
+        if more or want_final:
+            workers.append(("wait", dz(n), n // k))
+        if more:
+            workers += [("arrive", two("m1_", n + 1)), ("arrive", "m2_ok")]
+        output += [("wait", "m2_done", n), ("arrive", "m4_ok"), ("wait", o(n), n // k), ("arrive", "m2_ok")]
+    roles = {"producer": producer, "mma": mma, "workers": workers, "output": output}
+    counts = {op[1]: 1 for ops in roles.values() for op in ops}
+    counts.update({"m1_0": 3, "m1_1": 3, "m2_ok": 2, "m4_ok": 2})
+    return roles, counts
+
+
+@pytest.mark.parametrize("want_final", [False, True])
+@pytest.mark.parametrize("blocks", [1, 2, 3, 4, 9])
+def test_walk_kernel_phases_are_never_overrun(blocks, want_final):
+    assert overruns(*walk_kernel(blocks, want_final, 2)) == []
+
+
+def test_walk_kernel_with_one_barrier_for_every_block_would_be_overrun():
+    # (a producer that is a block late)
+    found = overruns(*walk_kernel(6, True, 1))
+    assert ("producer", "dz0", 0) in found and ("producer", "o0", 0) in found
