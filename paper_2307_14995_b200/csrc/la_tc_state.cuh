@@ -128,6 +128,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     for (int i = 0; i < S_NUM_BARS; ++i) mbar_init(&sm.bars[i], (i >= S_FC_READY0 && i < S_FC_FREE0) ? 8 : 1);
     sm.abort = 0;
     fence_mbar_init();
+    tma_prefetch_desc(&map_b);
+    tma_prefetch_desc(&map_c);
   }
   if (warp == 1) {
     tmem_alloc(&sm.tmem_slot, S_TMEM_COLS);
@@ -293,9 +295,15 @@ teardown:
   }
 }
 
-// Splits the work: cluster size and the heads whose segments are shared.  A thread block costs its blocks plus about four
-// more (start, end), sharing about two more; a launch costs its longest thread block or its total over two thread blocks
-// per SM, whichever is larger.
+// Splits the work: cluster size and the heads whose segments are shared, in units of one block (1.3 us).  A thread block
+// costs its blocks plus 4.5 (start, end), in a cluster 7, 7.5 or 10, behind clusters 2 more; a launch costs its longest thread
+// block (a quarter of the time that HBM is busy longer), the total over 200 (two thread blocks on an SM slow one
+// another down), or the blocks read at 100 to a unit (HBM), whichever is the most, and a little of the first two.
+// Measured with the cluster size forced, la_chunk_state, us unshared / 2 / 4 / 8: 32 heads x 777 19 / 18.5 / 16.4 /
+// 22.5; 16 x 32768 38 / 31.5 / 38 / 66; 16 heads of lambda = 1 x 65536 97 / 102 / 117 / 129; the 7B-like shape 81 / 58 / 72 / 132.
+// Segments of more than 32 blocks are shared by two at most.  A chain of products in one accumulator carries a rounding bias,
+// 1.3e-5 of a lambda = 1 state after 57 blocks, and cutting it, which takes that away, moves the results of the 7B-like step:
+// by 6e-6 in the 2-norm shared by two, by 7.4e-6 shared by four and eight (la_chunk_state there: 54 us and 45).
 inline StatePlan make_state_plan(const TcArgs& ta, const DecayTable& tab, bool rev, bool all_segments) {
   StatePlan p{};
   p.nseg_used = all_segments ? ta.nseg : ta.nseg - 1;
@@ -311,21 +319,22 @@ inline StatePlan make_state_plan(const TcArgs& ta, const DecayTable& tab, bool r
   double best = 1e30;
   int best_limit = 0;
   p.cluster = 1;
-  for (int cl = 1; cl <= 8; cl *= 2) {
-    // A long chain of products in one accumulator carries a rounding bias (1.3e-5 of a lambda = 1 state after 57 blocks), so
-    // cutting it decides the last digits of the result: 7e-6 of it there, 3e-6 after 16 blocks.  Segments of more than 32
-    // blocks are left to one thread block (B = 1, H = 32, N = 65536: 83 us, shared by eight 51).
-    if (cl > 1 && blocks > 32) break;
+  for (int cl = 1; cl <= (blocks > 32 ? 2 : 8); cl *= 2) {
+    const double around = cl == 2 ? 7.0 : cl == 4 ? 7.5 : 10.0;
     for (int limit = 2; limit <= 64; limit *= 2) {  // heads that keep more blocks than this are shared
-      double total = 0.0, longest = 0.0;
+      double total = 0.0, longest = 0.0, read = 0.0;
       for (int h = 0; h < ta.H; ++h) {
         const bool sh = cl > 1 && keep[h] > limit;
-        const double t = sh ? (keep[h] + cl - 1) / cl + 6.0 : keep[h] + 4.0;
+        const double t = sh ? (keep[h] + cl - 1) / cl + around : keep[h] + (cl > 1 ? 6.5 : 4.5);
         total += units * t * (sh ? cl : 1);
+        read += units * keep[h];
         if (t > longest) longest = t;
       }
-      const double cost = longest > total / 296.0 ? longest : total / 296.0;
-      if (cost < best * 0.98) {
+      read *= 0.01;
+      longest += 0.25 * (read < longest ? read : longest);
+      const double busy = longest > total / 200.0 ? longest : total / 200.0;
+      const double cost = (busy > read ? busy : read) + 0.1 * busy;
+      if (cost < best * (p.cluster == 1 ? 0.9 : 0.95)) {
         best = cost;
         best_limit = limit;
         p.cluster = cl;
