@@ -714,20 +714,27 @@ cudaError_t launch_simt_prepass(const OpArgs& args, const DecayTable& tab, int D
 // One thread per four consecutive state elements; the pieces are few (ranks of a sequence-parallel group, or the
 // segments of one chunk), so the sequential chain is short and every access is a coalesced 16-byte one.
 __global__ void __launch_bounds__(256) chain_kernel(const ChainArgs args, const DecayTable tab) {
+  // Every piece but the sequence's last is whole: two powers, formed once per thread block, which lies in one state.  (In
+  // double by every thread and for every piece they took longer than the sums: 65536 tokens, 32 heads, 32 segments of
+  // 2048 tokens 107 us with the states, 97 this way; 64 segments 182 and 164.)
+  __shared__ float power[2];
   const long per_head = args.DE / 4;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long)args.BH * per_head) return;
   const int bh = (int)(i / per_head);
   const size_t e0 = (size_t)(i % per_head) * 4;
-  const double s2 = tab.s2[bh % args.H];
+  const long long last = (args.N + args.piece_len - 1) / args.piece_len - 1;
+  if (threadIdx.x < 2)
+    power[threadIdx.x] = decay_pow_d(tab.s2[bh % args.H], (double)(threadIdx.x ? args.N - last * args.piece_len : args.piece_len));
   float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   if (args.z_in) z = *reinterpret_cast<const float4*>(args.z_in + (size_t)bh * args.DE + e0);
+  const float* src = args.src + (size_t)bh * args.stride_bh + e0;
+  __syncthreads();
+  const float g_whole = power[0], g_last = power[1];
   int j = args.first;
+#pragma unroll 4
   for (int n = 0; n < args.count; ++n, j += args.step) {
-    const long long t0 = (long long)j * args.piece_len;
-    const long long t1 = (t0 + args.piece_len < args.N) ? t0 + args.piece_len : args.N;
-    const float g = decay_pow_d(s2, (double)(t1 - t0));
-    const float4 x = *reinterpret_cast<const float4*>(args.src + (size_t)j * args.stride_j + (size_t)bh * args.stride_bh + e0);
+    const float g = j == last ? g_last : g_whole;
+    const float4 x = *reinterpret_cast<const float4*>(src + (size_t)j * args.stride_j);
     z.x = fmaf(g, z.x, x.x);
     z.y = fmaf(g, z.y, x.y);
     z.z = fmaf(g, z.z, x.z);
@@ -737,10 +744,10 @@ __global__ void __launch_bounds__(256) chain_kernel(const ChainArgs args, const 
 }
 
 cudaError_t launch_chain(const ChainArgs& args, const DecayTable& tab, cudaStream_t stream) {
-  if (args.DE % 4 != 0 || args.BH < 1 || args.count < 0 || args.piece_len < 1) return cudaErrorInvalidValue;
+  if (args.DE % 1024 != 0 || args.BH < 1 || args.count < 0 || args.piece_len < 1) return cudaErrorInvalidValue;
   const long threads = (long)args.BH * (args.DE / 4);
   KernelTimer timer(K_SCAN, stream);
-  chain_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(args, tab);
+  chain_kernel<<<(unsigned)(threads / 256), 256, 0, stream>>>(args, tab);
   count_launch();
   return cudaGetLastError();
 }
