@@ -96,8 +96,9 @@ bool tensor_path_available(const la_shape* s) {
   return tc_supported() && s->in_dtype == LA_BF16 && s->d == s->e && (s->d == 128 || s->d == 64);
 }
 
-// `packed`: the plan of a packed batch, whose sequences of different lengths share one segment length.
-la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
+// `packed`: the plan of a packed batch, whose sequences of different lengths share one segment length.  `states_only`: of
+// la_chunk_state, which has no walk to shorten; each further segment is a state to write, read and chain.
+la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states_only = false) {
   p->pk = Packed{nullptr, nullptr, nullptr, 0};
   p->fold = Folded{0, {nullptr, nullptr}};
   p->BH = s->B * s->H;
@@ -123,7 +124,9 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
     // Tensor cores at d = 64: the same waves, at about 2.5 us a block; pre-passes and scans take about 24 us and 0.17 us a
     // state.  Measured: 8 heads x 777 62 us as one segment, 43 with 128-token segments; 8 x 2048 94 with 1024, 54 with 256;
     // 16 x 4096 100 with 1024, 89 with 512; 4 x 16 x 2048 130 with 1024, 161 with 512.
-    // Packed batches: waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.
+    // Packed batches: waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.  On the tensor cores la_chunk_state
+    // takes the same rule: 32 heads x 777 22.5 us with the walk's segments, 16.4 with one; 16 x 2048 20.5 and 16.4; 8 x 8192 20.5
+    // and 16.4; d = 64, 4 x 16 x 2048 20.5 and 14.4.
     auto choose = [&](long most, long unit_limit, auto cost_of) {
       if (most < 1) most = 1;
       if (most > 1024) most = 1024;
@@ -147,13 +150,15 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false) {
     const long limit = std::max(p->BH * best_n, (long)(LA_NOALLOC_SCRATCH_BYTES / (2 * s->d * s->e * sizeof(float))));
     if (!p->tensor && !packed) {
       if (s->N > 256) best_n = choose((s->N + 127) / 128, limit, [&](long, long blocks) { return (double)blocks; });
-    } else if (p->chains && !packed) {
+    } else if (states_only || packed) {
+      // as it stands
+    } else if (p->chains) {
       best_n = choose(s->N / 128, limit, [&](long nseg, long blocks) {
         const double units = (double)p->BH * nseg;
         return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 1.3) +
                (nseg > 1 ? 2.0 * (4.0 + 0.01 * units + 0.6 * nseg) : 0.0);
       });
-    } else if (!packed) {
+    } else {
       best_n = choose((s->N + 127) / 128, limit, [&](long nseg, long blocks) {
         const double units = (double)p->BH * nseg;
         return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 0.67) + (nseg > 1 ? 9.6 + 0.068 * units : 0.0);
@@ -806,7 +811,7 @@ la_status la_fwd_bwd_host(const la_shape* shape, const void* q_host, const void*
 size_t la_chunk_state_workspace_bytes(const la_shape* shape) {
   if (check_shape(shape, true) != LA_OK) return (size_t)-1;
   Plan p;
-  if (make_plan(shape, &p) != LA_OK) return (size_t)-1;
+  if (make_plan(shape, &p, false, true) != LA_OK) return (size_t)-1;
   return state_set_bytes(shape, p);
 }
 
@@ -819,7 +824,7 @@ la_status la_chunk_state(const la_shape* shape, int reverse, const void* b, cons
   DecayTable tab;
   if ((st = make_table(shape, lambda_host, &tab)) != LA_OK) return st;
   Plan p;
-  if ((st = make_plan(shape, &p)) != LA_OK) return st;
+  if ((st = make_plan(shape, &p, false, true)) != LA_OK) return st;
   const size_t need = state_set_bytes(shape, p);
   if (!workspace || workspace_bytes < need) return LA_ERR_WORKSPACE;
   if (reinterpret_cast<uintptr_t>(workspace) & 255u) return LA_ERR_INVALID_ARG;

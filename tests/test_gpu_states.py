@@ -88,3 +88,27 @@ def test_decode_token_counts(d, T, layout):
     for t in range(T):
         assert_close(move(o)[:, :, t:t + 1], ref[t][:, :, None, :], 7.8e-5, "o[%d]" % t)
     assert_close(kv, state, 7.8e-5, "state")
+
+
+@pytest.mark.parametrize("d,B,N,seg_len,lam", [
+    (128, 1, 4300, 0, [1.0, 0.9995, 0.97, 1e-30]),      # the library's own plan: segments shared by clusters, a ragged tail
+    (128, 2, 777, 0, [1.0] * 16),                       # one segment of seven blocks, whose last is short
+    (128, 1, 8500, 4224, [1.0, 0.9995, 0.999, 0.9]),    # 33 blocks: shared by two at most
+    (128, 1, 1211, 128, [1.0, 0.999, 0.5]),             # ten pieces in the chain, the last one shorter
+    (128, 1, 5, 0, [1.0, 0.5]),
+    (64, 1, 1211, 128, [1.0, 0.999, 0.5]),
+])
+def test_chunk_state(d, B, N, seg_len, lam):
+    H = len(lam)
+    gen = torch.Generator().manual_seed(N)
+    q, k, v, do = [torch.randn(B, H, N, d, generator=gen).bfloat16() for _ in range(4)]
+    lam = torch.tensor(lam)
+    shape = la.make_shape(B, H, N, d, d, torch.bfloat16, torch.float32, seg_len)
+    ws = torch.empty(la.chunk_state_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    kv, gin = [torch.empty(B, H, d, d, device="cuda") for _ in range(2)]
+    la.la_chunk_state(shape, 0, k.cuda(), v.cuda(), lam, kv, ws)
+    la.la_chunk_state(shape, 1, q.cuda(), do.cuda(), lam, gin, ws)
+    torch.cuda.synchronize()
+    lam64 = lam.double().numpy()
+    assert_close(kv, orc.fwd_rec(q, k, v, lam64, want_state=True)[1], 3.1e-4, "forward")
+    assert_close(gin, orc.bwd_rec(q, k, v, do, lam64, want_state_grad=True)[3], 3.1e-4, "reverse")
