@@ -137,9 +137,8 @@ la_status la_fwd(const la_shape* shape, const void* q, const void* k, const void
  *   o     [B,H,N,e] out_dtype, the attention output itself, or NULL if it is not wanted (inference); the
  *         backward of this stage (la_gate_bwd) needs it;
  *   rstd  [B,H,N] fp32, sqrt(e) / ||o||_2 per row, or NULL.
- * Everything else as for la_fwd.  At d = e = 128 on the tensor-core path, with bf16 outputs, or without o and with y
- * larger than the L2 cache, the epilogue runs inside the walk kernel; otherwise the attention output is written (to o, or
- * to y if o is NULL) and a row kernel turns it into y.
+ * Everything else as for la_fwd.  At d = e = 128 on the tensor-core path the epilogue runs inside the walk kernel;
+ * otherwise the attention output is written (to o, or to y if o is NULL) and a row kernel turns it into y.
  */
 la_status la_fwd_gated(const la_shape* shape, const void* q, const void* k, const void* v, const void* u,
                        const float* lambda_host, void* y, void* o, float* rstd, const float* kv_in, float* kv_out,

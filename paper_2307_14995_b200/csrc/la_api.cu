@@ -458,12 +458,8 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     LA_TRY_CUDA(run_walk(shape, p, tab, q, k, v, o, from, kv_out, 0, cs));
     return LA_OK;
   }
-  // The d = 128 walk has the output stage as an epilogue, which costs it about 4 us per 128 tokens (four quarters of a row
-  // meet through shared memory).  With fp32 results a row kernel behind the plain walk gives the same and is faster where o
-  // is written anyway (1B-like shape: 137 us against 148) or y still sits in L2 when the row kernel reads it; past that the
-  // epilogue saves a pass over y (7B-like shape 991 us against 1027).  bf16 results: always the epilogue, which rounds once.
-  const double y_bytes = (double)p.BH * shape->N * shape->e * sizeof(float);
-  if (p.chains && (shape->out_dtype == LA_BF16 || (!o && y_bytes > 126e6))) {
+  // the d = 128 walk has the output stage as an epilogue
+  if (p.chains) {
     OpArgs wa = walk_args(shape, p, q, k, v, o, from, kv_out, 0);
     wa.u = u;
     wa.y = y;

@@ -932,14 +932,17 @@ cudaError_t launch_walk128(const OpArgs& args, const OpArgs* second, const Decay
   const bool f32 = (out_dt == DT_F32);
   if (args.u) {  // the gate epilogue exists for the single forward walk
     if (second || args.reverse) return cudaErrorInvalidValue;
-    return f32 ? launch_walk_t<false, float, true>(m0, m1, ta, tab, stream)
-               : launch_walk_t<false, __nv_bfloat16, true>(m0, m1, ta, tab, stream);
+    if (args.out)
+      return f32 ? launch_walk_t<false, float, 2>(m0, m1, ta, tab, stream)
+                 : launch_walk_t<false, __nv_bfloat16, 2>(m0, m1, ta, tab, stream);
+    return f32 ? launch_walk_t<false, float, 1>(m0, m1, ta, tab, stream)
+               : launch_walk_t<false, __nv_bfloat16, 1>(m0, m1, ta, tab, stream);
   }
   if (args.reverse)
-    return f32 ? launch_walk_t<true, float, false>(m0, m1, ta, tab, stream)
-               : launch_walk_t<true, __nv_bfloat16, false>(m0, m1, ta, tab, stream);
-  return f32 ? launch_walk_t<false, float, false>(m0, m1, ta, tab, stream)
-             : launch_walk_t<false, __nv_bfloat16, false>(m0, m1, ta, tab, stream);
+    return f32 ? launch_walk_t<true, float, 0>(m0, m1, ta, tab, stream)
+               : launch_walk_t<true, __nv_bfloat16, 0>(m0, m1, ta, tab, stream);
+  return f32 ? launch_walk_t<false, float, 0>(m0, m1, ta, tab, stream)
+             : launch_walk_t<false, __nv_bfloat16, 0>(m0, m1, ta, tab, stream);
 }
 
 cudaError_t launch_walk64(const OpArgs& args, const OpArgs* second, const DecayTable& tab, int out_dt, int precision,

@@ -41,8 +41,8 @@
 constexpr int W_THREADS = 896;
 constexpr uint32_t WCOL_R = 0, WCOL_O = 128, WCOL_FH = 256, WCOL_FL = 320, WCOL_ZH = 384, WCOL_ZL = 448;
 constexpr int W_REGS_LAUNCH = 72, W_REGS_CTL = 24;
-template <bool GATED>
-struct WRegs {  // (the gate's row sums need more than the plain store)
+template <int GATED>
+struct WRegs {  // (the gate needs more than the plain store; with 80 for both the output group spilled: 727 -> 742 us below)
   static constexpr int W = GATED ? 72 : 96, O = GATED ? 96 : 48;
   static_assert(4 * W_REGS_CTL + 16 * W + 8 * O <= 28 * W_REGS_LAUNCH, "registers of the launch");
 };
@@ -128,6 +128,24 @@ __device__ __forceinline__ void store_at(T* p, uint32_t stride_bytes, int x, flo
   }
 }
 
+// The same if x < end, without a branch.
+template <typename T>
+__device__ __forceinline__ void store_below(T* p, uint32_t stride_bytes, int x, float v, int end) {
+  if (sizeof(T) == 4) {
+    asm volatile(
+        "{\n\t.reg .b64 a;\n\t.reg .pred in;\n\tsetp.gt.s32 in, %4, %1;\n\tmad.wide.u32 a, %0, %1, %2;\n\t"
+        "@in st.global.b32 [a], %3;\n\t}" ::"r"(stride_bytes),
+        "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)), "f"(v), "r"(end)
+        : "memory");
+  } else {
+    asm volatile(
+        "{\n\t.reg .b64 a;\n\t.reg .pred in;\n\tsetp.gt.s32 in, %4, %1;\n\tmad.wide.u32 a, %0, %1, %2;\n\t"
+        "@in st.global.b16 [a], %3;\n\t}" ::"r"(stride_bytes),
+        "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)), "h"(__bfloat16_as_ushort(__float2bfloat16_rn(v))), "r"(end)
+        : "memory");
+  }
+}
+
 // The 32 bits at p + x * stride, likewise.
 __device__ __forceinline__ uint32_t load_u32_at(const void* p, uint32_t stride_bytes, int x) {
   uint32_t r;
@@ -137,10 +155,11 @@ __device__ __forceinline__ uint32_t load_u32_at(const void* p, uint32_t stride_b
   return r;
 }
 
-// Sum over the 32 lanes of each of 16 values per lane; lane l returns the total of value l >> 1.
-__device__ __forceinline__ float lane_sums16(const float (&v)[16], int lane) {
-  float t[8];
-  const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0, b1 = (lane & 2) != 0;
+// Sum over the eight lanes with the same lane % 4 of each of 16 values per lane; the lane returns the totals of values
+// 2 (lane / 4) and 2 (lane / 4) + 1.
+__device__ __forceinline__ float2 octet_sums(const float (&v)[16], int lane) {
+  float t[8], r[4];
+  const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0, b2 = (lane & 4) != 0;
 #pragma unroll
   for (int x = 0; x < 8; ++x) {
     const float keep = b4 ? v[8 + x] : v[x], send = b4 ? v[x] : v[8 + x];
@@ -149,24 +168,18 @@ __device__ __forceinline__ float lane_sums16(const float (&v)[16], int lane) {
 #pragma unroll
   for (int x = 0; x < 4; ++x) {
     const float keep = b3 ? t[4 + x] : t[x], send = b3 ? t[x] : t[4 + x];
-    t[x] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    r[x] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
   }
-#pragma unroll
-  for (int x = 0; x < 2; ++x) {
-    const float keep = b2 ? t[2 + x] : t[x], send = b2 ? t[x] : t[2 + x];
-    t[x] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  const float keep = b1 ? t[1] : t[0], send = b1 ? t[0] : t[1];
-  const float r = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-  return r + __shfl_xor_sync(0xffffffffu, r, 1);
+  const float k0 = b2 ? r[2] : r[0], s0 = b2 ? r[0] : r[2], k1 = b2 ? r[3] : r[1], s1 = b2 ? r[1] : r[3];
+  return make_float2(k0 + __shfl_xor_sync(0xffffffffu, s0, 4), k1 + __shfl_xor_sync(0xffffffffu, s1, 4));
 }
 
 // args.njobs == 2: two walks of the same direction over the same tokens in one launch (the dV and dK walks of the
 // backward pass, which between them read Q, K, V and dO); the thread blocks of the two jobs alternate, so that the two
 // readers of a tile run side by side and the tile comes from HBM once.
 // GATED (forward, single job): the epilogue y = SRMSNorm(out) (.) u of Eq. 3 with Eq. 8 is applied to the rows
-// before they leave (job.u, job.y; job.out and job.rstd optional).
-template <bool REV, typename TOut, bool GATED>
+// before they leave (job.u, job.y; job.rstd optional); 1: y alone, 2: out as well.
+template <bool REV, typename TOut, int GATED>
 __global__ void __launch_bounds__(W_THREADS, 1)
 tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps maps1,
                const __grid_constant__ TcArgs args, const __grid_constant__ DecayTable tab) {
@@ -607,7 +620,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       TOut* dst = out + (size_t)t0 * args.sT;
       // u of this warp's 64 tokens, two value columns to a register: lanes 0..15 hold token 2 x, lanes 16..31 token 2 x + 1
       uint32_t upair[GATED ? 32 : 1];
-      if constexpr (GATED) {
+      if constexpr (GATED != 0) {
         const __nv_bfloat16* up = static_cast<const __nv_bfloat16*>(job.u) + head_off +
                                   (size_t)(t0 + (lane >> 4)) * args.sT + q * 32 + (lane & 15) * 2;
         const int mine = rows - (lane >> 4);
@@ -620,61 +633,80 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
       TC_WAIT_WARP(W_O_READY0 + (it & 1), (it >> 1) & 1, 25);
       tc_fence_after_sync();
       const uint32_t stride = (uint32_t)args.sT * (uint32_t)sizeof(TOut);
-      if constexpr (GATED) {
+      if constexpr (GATED != 0) {
         // Sums of squares of 64 tokens over this quarter's value columns (lanes), exchanged between the four quarters through
-        // shared memory once per block (beside M1 a read takes hundreds of clocks); then each quarter's warp reads its
-        // columns again, scales them and multiplies by u, which was fetched before M4.
-        // (The buffer is a part of the score tile that the forward walk never uses: keys 64.. of rows 0..15.  All warps have
-        // read a block's sums before M2 of the next block can start.)
+        // shared memory.  They are read in the 16 x 256-bit shape, which has four lanes of a token in one thread, so that 14
+        // shuffles add up what 64 would.  The factors come back by a broadcast read, O in pieces of 16 tokens, two of them
+        // ahead, so that M2 of the next block may overwrite it when half is stored, and a token past the end costs a
+        // predicate instead of a branch, which kept the loads and shuffles of different tokens from overlapping.
+        // 7B-like shape, la_fwd_gated: y alone 983 -> 727 us in fp32, 952 -> 695 in bf16; with o 978 (o to memory, then a row
+        // kernel) -> 837 and 987 -> 771; 2 x 16 x 8192 in fp32 145 -> 110, with o 138 -> 129.
+        // (The buffers are a part of the score tile that the forward walk never uses: keys 64.. of rows 0..15 for the sums and
+        // of rows 16..31 for the factors.  A warp has read a block's sums before it arrives for M4 of the next block, which
+        // the others' next sums wait for.)
         float(*const g)[64] = reinterpret_cast<float(*)[64]>(&sm.p_hi[1][0]) + (th >> 6) * 4;
-        float* const mine = g[q];
-#pragma unroll 1
-        for (int pc = 0; pc < 2; ++pc) {
-          uint32_t w[32];
-          tmem_ld_x32(colO + pc * 32, w);
-          tmem_ld_wait();
-          float sq[16], sr[16];
+        float* const factor = reinterpret_cast<float*>(&sm.p_hi[1][16 * 64]) + (warp - 20) * 64;
+        {
+          float s[16];  // tokens 8 i + 2 (lane % 4) + c at 2 i + c
 #pragma unroll
-          for (int x = 0; x < 16; ++x) {
-            sq[x] = __uint_as_float(w[x]) * __uint_as_float(w[x]);
-            sr[x] = __uint_as_float(w[16 + x]) * __uint_as_float(w[16 + x]);
+          for (int half = 0; half < 2; ++half) {
+            uint32_t w[32];
+            tmem_ld_16x256b_x8(colO + ((uint32_t)(half * 16) << 16), w);
+            tmem_ld_wait();
+#pragma unroll
+            for (int x = 0; x < 16; ++x) {
+              const float v0 = __uint_as_float(w[(x >> 1) * 4 + (x & 1)]), v1 = __uint_as_float(w[(x >> 1) * 4 + 2 + (x & 1)]);
+              s[x] = half ? fmaf(v0, v0, fmaf(v1, v1, s[x])) : fmaf(v0, v0, v1 * v1);
+            }
           }
-          const float p0 = lane_sums16(sq, lane), p1 = lane_sums16(sr, lane);
-          // (lane l: token l >> 1 of either half; even lanes store the first, odd lanes the second)
-          mine[pc * 32 + ((lane & 1) << 4) + (lane >> 1)] = (lane & 1) ? p1 : p0;
+          *reinterpret_cast<float2*>(&g[q][2 * lane]) = octet_sums(s, lane);
         }
         WARP_ARRIVE(W_GATE0 + (th >> 6));
+        uint32_t o[32];
+        tmem_ld_x32(colO, o);
         TC_WAIT_WARP(W_GATE0 + (th >> 6), it & 1, 26);
-        float scale[2];  // of tokens lane and 32 + lane
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int t = 32 * k + lane;
-          const float ss = (g[0][t] + g[1][t]) + (g[2][t] + g[3][t]);
-          scale[k] = ss > 0.f ? rsqrtf(ss * (1.f / 128.f)) : 0.f;
-          // rstd has the layout of the token tensors without the feature dimension
-          if (job.rstd && q == 0 && t < rows) job.rstd[(head_off + (size_t)(t0 + t) * args.sT) >> 7] = scale[k];
+        {
+          float2 f;  // of tokens 2 lane, 2 lane + 1
+          const float2 a = *reinterpret_cast<const float2*>(&g[0][2 * lane]), b = *reinterpret_cast<const float2*>(&g[1][2 * lane]);
+          const float2 c = *reinterpret_cast<const float2*>(&g[2][2 * lane]), d = *reinterpret_cast<const float2*>(&g[3][2 * lane]);
+          f.x = (a.x + b.x) + (c.x + d.x);
+          f.y = (a.y + b.y) + (c.y + d.y);
+          f.x = f.x > 0.f ? rsqrtf(f.x * (1.f / 128.f)) : 0.f;
+          f.y = f.y > 0.f ? rsqrtf(f.y * (1.f / 128.f)) : 0.f;
+          *reinterpret_cast<float2*>(&factor[2 * lane]) = f;
+          if (job.rstd && q == 0) {  // rstd has the layout of the token tensors without the feature dimension
+            const size_t at = (head_off + (size_t)(t0 + 2 * lane) * args.sT) >> 7;
+            if (2 * lane < rows) job.rstd[at] = f.x;
+            if (2 * lane + 1 < rows) job.rstd[at + (args.sT >> 7)] = f.y;
+          }
         }
+        __syncwarp();
         TOut* const ydst = static_cast<TOut*>(job.y) + head_off + (size_t)t0 * args.sT + q * 32 + lane;
+        const auto put = [&](int t, uint32_t w, float f) {
+          const uint32_t uw = __shfl_sync(0xffffffffu, upair[t >> 1], ((t & 1) << 4) + (lane >> 1));
+          const float y = __uint_as_float(w) * f * __uint_as_float((lane & 1) ? (uw & 0xffff0000u) : (uw << 16));
+          store_below(ydst, stride, t, y, rows);
+          if (GATED == 2) store_below(dst, stride, t, __uint_as_float(w), rows);
+        };
+        tmem_ld_wait();
 #pragma unroll
-        for (int pc = 0; pc < 4; ++pc) {
-          uint32_t w[16];
-          tmem_ld_x16(colO + pc * 16, w);
-          tmem_ld_wait();
-          if (pc == 3) {
+        for (int p = 0; p < 4; ++p) {  // 16 tokens at a time
+#pragma unroll
+          for (int t4 = 0; t4 < 16; t4 += 4) {
+            const float4 f = *reinterpret_cast<const float4*>(&factor[16 * p + t4]);
+            const int x = 16 * (p % 2) + t4, t = 16 * p + t4;
+            put(t, o[x], f.x);
+            put(t + 1, o[x + 1], f.y);
+            put(t + 2, o[x + 2], f.z);
+            put(t + 3, o[x + 3], f.w);
+          }
+          if (p < 2) {  // the next 16 tokens into the registers of these
+            tmem_ld_x16(colO + 32 + 16 * p, *reinterpret_cast<uint32_t(*)[16]>(&o[16 * p]));
+            tmem_ld_wait();
+          }
+          if (p == 1) {
             tc_fence_before_sync();
             WARP_ARRIVE(W_M2_OK);  // M2 of the next block may overwrite O
-          }
-#pragma unroll
-          for (int x = 0; x < 16; ++x) {
-            const int t = pc * 16 + x;
-            const float v = __uint_as_float(w[x]);
-            const uint32_t uw = __shfl_sync(0xffffffffu, upair[t >> 1], ((t & 1) << 4) + (lane >> 1));
-            const float ug = __uint_as_float((lane & 1) ? (uw & 0xffff0000u) : (uw << 16));
-            const float y = v * __shfl_sync(0xffffffffu, scale[t >> 5], t & 31) * ug;
-            if (t < rows) {
-              store_at(ydst, stride, t, y);
-              if (job.out) store_at(dst, stride, t, v);
-            }
           }
         }
       } else {
@@ -708,7 +740,7 @@ teardown:
   if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-template <bool REV, typename TOut, bool GATED>
+template <bool REV, typename TOut, int GATED>
 cudaError_t launch_walk_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, const DecayTable& tab, cudaStream_t stream) {
   const size_t smem = sizeof(WSmem<REV>) + 1024;
   static_assert(sizeof(WSmem<REV>) + 1024 <= 232448, "shared memory of one SM");

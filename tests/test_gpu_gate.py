@@ -130,6 +130,41 @@ def test_gated_forward_large_without_o():
     check_gated(q, k, v, u, lam, got, TOL_BF16)
 
 
+@pytest.mark.parametrize("out_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("N", [1, 31, 64, 65, 112, 129, 191, 300])
+@pytest.mark.parametrize("layout", [la.LA_LAYOUT_BHND, la.LA_LAYOUT_BNHD])
+def test_gated_epilogue_at_ragged_ends(N, out_dtype, layout):
+    """The epilogue's pieces of 16 tokens and halves of 64 that the sequence's end cuts, with and without o and rstd; nothing
+    past the end is written.  fp32: two-term operands, 2^-17 of |sum| up to 5 RMS, and |y| / RMS(y) up to 4 times as large:
+    1.5e-4; bf16 rounds once."""
+    B, H, d = 2, 3, 128
+    q, k, v, _ = inputs.make_qkvdo(B, H, N, d, d, seed=N, with_do=False)
+    u = draw_gate((B, H, N, d), seed=N + 1)
+    lam = torch.tensor([1.0, 0.97, 0.3])
+    ref_o = orc.fwd_rec(q, k, v, lam.double().numpy())
+    ref_y, ref_rstd = orc.norm_gate_fwd(ref_o, u, want_rstd=True)
+    move = (lambda x: x.transpose(1, 2).contiguous()) if layout == la.LA_LAYOUT_BNHD else (lambda x: x)
+    qg, kg, vg, ug = (move(x).to(DEV) for x in (q, k, v, u))
+    shape = la.make_shape(B, H, N, d, d, torch.bfloat16, out_dtype, layout=layout)
+    n = qg.numel()
+    for want_o in (True, False):
+        ybuf, obuf = (torch.full((n + 64 * d,), float("nan"), dtype=out_dtype, device=DEV) for _ in range(2))
+        y, o = ybuf[:n].view(qg.shape), obuf[:n].view(qg.shape)
+        rstd = torch.full(qg.shape[:3], float("nan"), device=DEV)
+        la.la_fwd_gated(shape, qg, kg, vg, ug, lam, y, o if want_o else None, rstd if want_o else None,
+                        workspace=la.alloc_workspace(la.LA_OP_FWD, shape, DEV))
+        torch.cuda.synchronize()
+        la.device_status()
+        assert torch.isnan(ybuf[n:]).all() and torch.isnan(obuf[n if want_o else 0:]).all()
+        if want_o:
+            r = move(rstd.unsqueeze(-1)).squeeze(-1).double().cpu().numpy()
+            assert np.max(np.abs(r - ref_rstd) / ref_rstd) <= 1.5e-4
+        for got, ref in ((y, ref_y),) + (((o, ref_o),) if want_o else ()):
+            got, ref = move(got).double().cpu().numpy().reshape(B * H, -1), ref.reshape(B * H, -1)
+            rms = np.sqrt(np.mean(ref * ref, axis=1, keepdims=True))
+            assert np.all(np.abs(got - ref) <= 1.5e-4 * rms + (2.0 ** -8 * np.abs(ref) if out_dtype == torch.bfloat16 else 0.0))
+
+
 def test_gated_forward_fp32_path():
     w = inputs.make_workload("pr1_ref")
     u = draw_gate(tuple(w["v"].shape), seed=3, dtype=torch.float32)
