@@ -118,9 +118,12 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
     // launch that makes the states, with what each further state costs to write, read and chain.  Measured, forward plus
     // backward: 3 x 8 heads x 3001 tokens 172 us with 1536-token segments, 141 with 512; 8 heads x 2048 118 with 1024, 92
     // with 512, 126 with 128; 2 x 16 x 8192 289 with 2048, 344 with 1024 (the model: 49.7, 34.5 / 38, 29, 33 / 85, 97).
-    // CUDA-core kernels: one segment up to 256 tokens, else 128-token segments.  Forward plus backward in fp32: 2 heads x 256
-    // tokens, d = 64, 38 us as one segment and 57 in two; 4 x 512 85 and 65; 2 x 2048 205 with 512-token segments, 122 with
-    // 256, 81 with 128; 16 x 2048, d = 128, 946, 652 and 488.
+    // CUDA-core kernels: row tiles up to ROWS_MAX_SEG tokens, whose work grows with the segment's length but which end after
+    // as many tiles; else the walk block by block, one thread block to an SM at d = 128 and up to four at d = 64; and the
+    // pre-passes.  Forward plus backward in fp32, us: 2 heads x 256, d = 64, 38 as one segment and 57 in two; 4 x 512 85
+    // and 65; 2 x 2048 205 with 512-token segments, 122 with 256, 81 with 128; 16 x 2048, d = 128, 946, 652 and 488.  Where the heads
+    // fill the chip a state costs more than it saves: 256 x 512, d = 64, 747 with 128-token segments and 605 as one; 256 x 4096
+    // 7769 with 1024 and 6383 as one; 128 x 2048, d = 128, 6560 with 1024 and 5384 as one.
     // Tensor cores at d = 64: the same waves, at about 2.5 us a block; pre-passes and scans take about 24 us and 0.17 us a
     // state.  Measured: 8 heads x 777 62 us as one segment, 43 with 128-token segments; 8 x 2048 94 with 1024, 54 with 256;
     // 16 x 4096 100 with 1024, 89 with 512; 4 x 16 x 2048 130 with 1024, 161 with 512.
@@ -149,7 +152,19 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
     // (la_fwd_noalloc's scratch holds so many segments' states, 256 at d = 128: shapes that fit it with long segments still do)
     const long limit = std::max(p->BH * best_n, (long)(LA_NOALLOC_SCRATCH_BYTES / (2 * s->d * s->e * sizeof(float))));
     if (!p->tensor && !packed) {
-      if (s->N > 256) best_n = choose((s->N + 127) / 128, limit, [&](long, long blocks) { return (double)blocks; });
+      if (states_only) {
+        if (s->N > 256) best_n = choose((s->N + 127) / 128, limit, [&](long, long blocks) { return (double)blocks; });
+      } else {
+        best_n = choose((s->N + 127) / 128, limit, [&](long nseg, long blocks) {
+          const bool wide = s->d == 128;
+          const double len = nseg > 1 ? 128.0 * blocks : s->N, thousands = 1e-3 * p->BH * s->N, sms = waves(p->BH * nseg);
+          double walks, states = 0.0;  // us, of all walks of a forward and a backward pass and of one pre-pass and scan
+          if (len <= ROWS_MAX_SEG) walks = std::max(4.0 * thousands * (wide ? 2.3 + 0.0005 * len : 0.65 + 0.0008 * len), 0.16 * len);
+          else walks = 4.0 * len * (wide ? 0.66 * sms : std::max(0.31, 0.2 * sms));
+          if (nseg > 1) states = std::max(thousands * (wide ? 1.45 : 0.79), len * (wide ? 0.2 : 0.08)) + 8.0;
+          return walks + 2.5 * states;  // (two pre-passes with the forward pass's states, three without)
+        });
+      }
     } else if (states_only || packed) {
       // as it stands
     } else if (p->chains) {

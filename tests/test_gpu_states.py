@@ -112,3 +112,20 @@ def test_chunk_state(d, B, N, seg_len, lam):
     lam64 = lam.double().numpy()
     assert_close(kv, orc.fwd_rec(q, k, v, lam64, want_state=True)[1], 3.1e-4, "forward")
     assert_close(gin, orc.bwd_rec(q, k, v, do, lam64, want_state_grad=True)[3], 3.1e-4, "reverse")
+
+
+@pytest.mark.parametrize("d,B,H,N", [(64, 8, 24, 640), (64, 1, 4, 512), (64, 1, 2, 513), (128, 5, 16, 333), (128, 1, 2, 1300), (128, 40, 8, 1100)])
+def test_full_precision_plans(d, B, H, N):
+    """The library's own segments for fp32 inputs: few heads and many, one segment of row tiles, several, the walk.  Sums of
+    at most N + d fp32 products: 1428 * 2^-24 of the largest partial sum, itself at most 2 RMS: 1.7e-4."""
+    gen = torch.Generator().manual_seed(N)
+    q, k, v, do = [torch.randn(B, H, N, d, generator=gen) * d ** -0.5 for _ in range(4)]
+    lam = torch.linspace(0.6, 1.0, H)
+    dev = [x.cuda() for x in (q, k, v, do)]
+    o = la.fwd(*dev[:3], lam)
+    grads = la.bwd(*dev, lam)
+    torch.cuda.synchronize()
+    lam64 = lam.double().numpy()
+    ref = (orc.fwd_rec(q, k, v, lam64),) + tuple(orc.bwd_rec(q, k, v, do, lam64))
+    for name, g, r in zip(("o", "dq", "dk", "dv"), (o,) + tuple(grads), ref):
+        assert_close(g, r, 1.7e-4, name)
