@@ -104,7 +104,8 @@ typedef struct {
 /* Bytes of device scratch the given op needs for this shape (0 is possible).
  * Returns (size_t)-1 if the shape is invalid or unsupported.  Linear in
  * B*H*d*e*ceil(N/seg_len); never grows with N^2: sets of [B,H,nseg,d,e] fp32 states,
- * two for the forward pass (0 with a single segment), three for the backward pass. */
+ * two for the forward pass (0 with a single segment) and three for the backward pass;
+ * one and two on the tensor cores at d = e = 128. */
 size_t la_workspace_bytes(int op, const la_shape* shape);
 
 /* The segment length the library will use for this shape (after applying

@@ -149,7 +149,7 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
     };
     auto waves = [](long units) { return (double)((units + 147) / 148); };
     long best_n = choose(s->N / 1024, 1L << 40, [&](long nseg, long blocks) { return waves(p->BH * nseg) * (blocks + 2); });
-    // (la_fwd_noalloc's scratch holds so many segments' states, 256 at d = 128: shapes that fit it with long segments still do)
+    // (at most 256 states at d = 128, 1024 at d = 64: shapes that fit la_fwd_noalloc's scratch with long segments still do)
     const long limit = std::max(p->BH * best_n, (long)(LA_NOALLOC_SCRATCH_BYTES / (2 * s->d * s->e * sizeof(float))));
     if (!p->tensor && !packed) {
       if (states_only) {
@@ -191,6 +191,11 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
 size_t state_set_bytes(const la_shape* s, const Plan& p) {
   return (size_t)p.BH * p.nseg * s->d * s->e * sizeof(float);
 }
+
+// State sets a call keeps in its workspace.  Forward: the segments' states, and without chains their transposes; backward: those
+// of KV^T and of dKV, and without chains the transposes of dKV.
+int fwd_sets(const Plan& p) { return p.nseg == 1 ? 0 : p.chains ? 1 : 2; }
+int bwd_sets(const Plan& p) { return p.chains ? 2 : 3; }
 
 la_status make_table(const la_shape* s, const float* lambda_host, DecayTable* tab) {
   if (!lambda_host) return LA_ERR_INVALID_ARG;
@@ -376,9 +381,7 @@ static size_t scratch_bytes(int op, const la_shape* shape, bool packed) {
   if (op == LA_OP_DECODE) return 0;
   Plan p;
   if (make_plan(shape, &p, packed) != LA_OK) return (size_t)-1;
-  const size_t one = state_set_bytes(shape, p);
-  if (op == LA_OP_FWD) return p.nseg > 1 ? 2 * one : 0;  // the segments' states, and (without chains) their transposes
-  return 3 * one;
+  return (size_t)(op == LA_OP_FWD ? fwd_sets(p) : bwd_sets(p)) * state_set_bytes(shape, p);
 }
 
 size_t la_workspace_bytes(int op, const la_shape* shape) { return scratch_bytes(op, shape, false); }
@@ -450,7 +453,7 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   if (fold) p.fold = *fold;
   p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
-  const size_t need = p.nseg > 1 ? 2 * one : 0;
+  const size_t need = (size_t)fwd_sets(p) * one;
   if (need > 0 && (!workspace || workspace_bytes < need)) return LA_ERR_WORKSPACE;
   if (need > 0 && (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_INVALID_ARG;
   if ((st = check_device()) != LA_OK) return st;
@@ -533,7 +536,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   if (fold) p.fold = *fold;
   p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
-  if (!workspace || workspace_bytes < 3 * one) return LA_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < (size_t)bwd_sets(p) * one) return LA_ERR_WORKSPACE;
   if (fwd_workspace == workspace) return LA_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(workspace) & 255u) return LA_ERR_INVALID_ARG;
   if ((st = check_device()) != LA_OK) return st;
@@ -541,7 +544,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
 
   float* buf_kvt = static_cast<float*>(workspace);                 // KV^T entering each segment
   float* buf_e = buf_kvt + one / sizeof(float);                    // dKV entering each segment (from the right)
-  float* buf_et = buf_e + one / sizeof(float);                     // its transpose
+  float* buf_et = buf_e + one / sizeof(float);                     // its transpose (without chains)
   const bool multi = p.nseg > 1;
 
   // dQ = fwd(a = dO, b = V, c = K); its state is KV^T, so the caller's kv_in (and what la_fwd left) enters transposed.

@@ -129,3 +129,36 @@ def test_full_precision_plans(d, B, H, N):
     ref = (orc.fwd_rec(q, k, v, lam64),) + tuple(orc.bwd_rec(q, k, v, do, lam64))
     for name, g, r in zip(("o", "dq", "dk", "dv"), (o,) + tuple(grads), ref):
         assert_close(g, r, 1.7e-4, name)
+
+
+@pytest.mark.parametrize("d,dtype,sets", [(128, torch.bfloat16, (1, 2)), (64, torch.bfloat16, (2, 3)), (128, torch.float32, (2, 3))])
+@pytest.mark.parametrize("B,N,seg_len", [(1, 1211, 128), (2, 700, 256)])
+def test_workspace_holds_the_sets_that_are_used(d, dtype, sets, B, N, seg_len):
+    """Nothing behind la_workspace_bytes is written, a byte less is refused, and the backward pass from the forward pass's
+    states (with more than six segments at d = 128: running sums, read transposed) agrees with the oracle."""
+    lam = torch.tensor([1.0, 0.999, 0.5])
+    H = len(lam)
+    gen = torch.Generator().manual_seed(N)
+    q, k, v, do = [torch.randn(B, H, N, d, generator=gen).to(dtype) for _ in range(4)]
+    kv_in, gko = [torch.randn(B, H, d, d, generator=gen) * 0.1 for _ in range(2)]
+    shape = la.make_shape(B, H, N, d, d, dtype, torch.float32, seg_len)
+    state = B * H * d * d * 4 * -(-N // seg_len)
+    need = [la.workspace_bytes(op, shape) for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    assert need == [n * state for n in sets]
+    bufs = [torch.full((n + 4096,), 0xA5, dtype=torch.uint8, device="cuda") for n in need]
+    ws_f, ws_b = bufs[0][:need[0]], bufs[1][:need[1]]
+    dev = [x.cuda() for x in (q, k, v, do, kv_in, gko)]
+    o, dq, dk, dv = [torch.empty(B, H, N, d, device="cuda") for _ in range(4)]
+    kv, gin = [torch.empty(B, H, d, d, device="cuda") for _ in range(2)]
+    with pytest.raises(la.LaError):
+        la.la_fwd(shape, *dev[:3], lam, o, dev[4], kv, ws_f[:-1])
+    with pytest.raises(la.LaError):
+        la.la_bwd(shape, *dev[:4], lam, dq, dk, dv, dev[4], dev[5], gin, ws_b[:-1])
+    la.la_fwd(shape, *dev[:3], lam, o, dev[4], kv, ws_f)
+    lam64 = lam.double().numpy()
+    ref = orc.bwd_rec(q, k, v, do, lam64, kv_in=kv_in, grad_kv_out=gko, want_state_grad=True)
+    for reuse in (ws_f, None):
+        la.la_bwd(shape, *dev[:4], lam, dq, dk, dv, dev[4], dev[5], gin, ws_b, fwd_workspace=reuse)
+        for name, g, r in zip(("dq", "dk", "dv", "gin"), (dq, dk, dv, gin), ref):
+            assert_close(g, r, 3.1e-4, name)
+    assert all(bool((b[n:] == 0xA5).all()) for b, n in zip(bufs, need))
