@@ -212,7 +212,8 @@ la_status la_decode_step(const la_shape* shape, const void* q, const void* k, co
  *   kv_in, kv_out, grad_kv_out, grad_kv_in   [2,B,H,d,e] fp32 (cos half, then sin half) or NULL;
  *   other arguments as in la_fwd / la_bwd; requires d == e.
  * Workspace: la_lrpe_workspace_bytes(op, shape), 256-byte aligned: the four feature tensors, fp32 temporaries of
- * the tensors' size (1-2 forward, 5-6 backward), a table of angles and the inner calls' own workspace.
+ * the tensors' size (1-2 forward, 5-6 backward), in the backward pass a table of angles (8 bytes for every 16 tokens
+ * of a head and feature), and the inner calls' own workspace.
  * d_theta is a position-weighted sum whose q and k parts cancel down to the relative-position result; with
  * bf16 features its error grows with the absolute positions (see the tests for the bound that is checked).
  */

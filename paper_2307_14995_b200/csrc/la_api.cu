@@ -50,10 +50,13 @@ struct Packed {
   int total_tokens;
 };
 
-// A folded batch: entries t and t + batches of the shape's B = 2 * batches read the same entry t of the tensors named here.
+// A folded batch: entries t and t + batches of the shape's B = 2 * batches read the same entry t of the tensors named here;
+// of the output `out` the second half goes to out2.
 struct Folded {
   int batches;
   const void* tensors[2];
+  const void* out;
+  void* out2;
   bool has(const void* p) const { return batches && (p == tensors[0] || p == tensors[1]); }
 };
 
@@ -100,7 +103,7 @@ bool tensor_path_available(const la_shape* s) {
 // la_chunk_state, which has no walk to shorten; each further segment is a state to write, read and chain.
 la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states_only = false) {
   p->pk = Packed{nullptr, nullptr, nullptr, 0};
-  p->fold = Folded{0, {nullptr, nullptr}};
+  p->fold = Folded{0, {nullptr, nullptr}, nullptr, nullptr};
   p->BH = s->B * s->H;
   if (s->path == LA_PATH_TENSOR && !tensor_path_available(s)) return LA_ERR_UNSUPPORTED;
   p->tensor = (s->path == LA_PATH_TENSOR) || (s->path == LA_PATH_AUTO && tensor_path_available(s));
@@ -343,6 +346,7 @@ OpArgs walk_args(const la_shape* s, const Plan& p, const void* a, const void* b,
   args.seq_order = p.pk.order;
   args.total_tokens = p.pk.total_tokens;
   args.fold = p.fold.batches;
+  args.out2 = p.fold.batches && out == p.fold.out ? p.fold.out2 : nullptr;
   args.shared = (p.fold.has(a) ? SHARED_A : 0) | (p.fold.has(b) ? SHARED_B : 0) | (p.fold.has(c) ? SHARED_C : 0);
   set_strides(s, p.pk.start ? p.pk.total_tokens : s->N, &args);
   return args;
@@ -599,8 +603,8 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
 }  // namespace la
 
 namespace la {
-// Two runs over one batch as one run over twice the batch: q, k (and what they yield: o, dq, dk, dv and the states) have
-// 2 * half->B entries, v and d_o half->B.  Only where the kernels fold a batch.
+// Two runs over one batch as one run over twice the batch: q, k (and what they yield: dq, dk and the states) have
+// 2 * half->B entries, v and d_o half->B; o and dv come in two tensors of half->B.  Only where the kernels fold a batch.
 static la_shape doubled(const la_shape* half) {
   la_shape s = *half;
   s.B *= 2;
@@ -612,18 +616,18 @@ size_t halves_workspace(int op, const la_shape* half) {
   if (half->B > (1 << 20) || check_shape(&s, true) != LA_OK || make_plan(&s, &p) != LA_OK || !p.chains) return (size_t)-1;
   return la_workspace_bytes(op, &s);
 }
-la_status halves_fwd(const la_shape* half, const void* q, const void* k, const void* v, const float* lambda_host, void* o,
+la_status halves_fwd(const la_shape* half, const void* q, const void* k, const void* v, const float* lambda_host, void* o, void* o2,
                      const float* kv_in, float* kv_out, void* workspace, size_t workspace_bytes, void* stream) {
   const la_shape s = doubled(half);
-  const Folded fold{half->B, {v, v}};
+  const Folded fold{half->B, {v, v}, o, o2};
   return fwd_impl(&s, q, k, v, nullptr, lambda_host, nullptr, o, nullptr, kv_in, kv_out, workspace, workspace_bytes, stream, nullptr,
                   &fold);
 }
 la_status halves_bwd(const la_shape* half, const void* q, const void* k, const void* v, const void* d_o, const float* lambda_host,
-                     void* dq, void* dk, void* dv, const float* kv_in, const float* grad_kv_out, float* grad_kv_in, void* workspace,
-                     size_t workspace_bytes, void* stream) {
+                     void* dq, void* dk, void* dv, void* dv2, const float* kv_in, const float* grad_kv_out, float* grad_kv_in,
+                     void* workspace, size_t workspace_bytes, void* stream) {
   const la_shape s = doubled(half);
-  const Folded fold{half->B, {v, d_o}};
+  const Folded fold{half->B, {v, d_o}, dv, dv2};
   return bwd_impl(&s, q, k, v, d_o, lambda_host, dq, dk, dv, kv_in, grad_kv_out, grad_kv_in, nullptr, workspace, workspace_bytes,
                   stream, nullptr, &fold);
 }

@@ -75,8 +75,10 @@ struct OpArgs {
   const int* seq_len;
   // Folded batch (tensor-core kernels at Da = Ec = 128 only; 0 elsewhere): batch entries t and t + fold read the same
   // entry t of the operands in `shared` (SHARED_* bits), which have `fold` batch entries.
+  // out2: where the entries fold .. 2 fold - 1 of the output go, as entries 0 .. fold - 1 (NULL: behind the others in `out`).
   int fold;
   int shared;
+  void* out2;
   const int* seq_order;  // the order in which thread blocks take the sequences (longest first), or NULL
   int total_tokens;
 };

@@ -23,11 +23,11 @@
 namespace la {
 // Both halves of the features as one run over twice the batch (la_api.cu); the size is (size_t)-1 where that cannot be.
 size_t halves_workspace(int op, const la_shape* half);
-la_status halves_fwd(const la_shape* half, const void* q, const void* k, const void* v, const float* lambda_host, void* o,
+la_status halves_fwd(const la_shape* half, const void* q, const void* k, const void* v, const float* lambda_host, void* o, void* o2,
                      const float* kv_in, float* kv_out, void* workspace, size_t workspace_bytes, void* stream);
 la_status halves_bwd(const la_shape* half, const void* q, const void* k, const void* v, const void* d_o, const float* lambda_host,
-                     void* dq, void* dk, void* dv, const float* kv_in, const float* grad_kv_out, float* grad_kv_in, void* workspace,
-                     size_t workspace_bytes, void* stream);
+                     void* dq, void* dk, void* dv, void* dv2, const float* kv_in, const float* grad_kv_out, float* grad_kv_in,
+                     void* workspace, size_t workspace_bytes, void* stream);
 namespace {
 
 constexpr int RUN = 16;  // consecutive tokens a group of d/4 lanes walks
@@ -358,10 +358,12 @@ struct Carve {
   size_t f32;        // bytes of one fp32 temporary of the tensors' size
   size_t part;       // bytes of one partial-sum array for dtheta
   size_t op;         // workspace of the inner la_fwd / la_bwd
-  size_t angles;     // bytes of the angle table
+  size_t angles;     // bytes of the angle table (forward: 0 where it lies in the temporary, which the runs write after the
+                     // features are made)
   int ntiles;
   // One run over both halves: half the launches, and twice the heads to fill the chip with (1 x 16 heads x 8192, d = 128,
-  // forward plus backward 660 us as two runs, 565 as one).  Its operands lie one after the other, so tensors may not be padded.
+  // forward plus backward 660 us as two runs, 565 as one).  The halves of q and k and of their gradients lie one after the
+  // other, so tensors may not be padded.
   bool one_run;
   int n_f32;         // fp32 temporaries
   size_t total;
@@ -384,10 +386,11 @@ bool carve(int op, const la_shape* s, Carve* c) {
   c->angles = up256(angle_count(s) * sizeof(float2));
   const bool out32 = s->out_dtype == LA_F32;
   if (op == LA_OP_FWD) {
-    c->n_f32 = out32 && !c->one_run ? 1 : 2;                    // the second run's result (and the first's when o is bf16)
+    c->n_f32 = out32 ? 1 : 2;                    // the second half's result (and the first's when o is bf16)
+    if (c->angles <= c->f32) c->angles = 0;
     c->total = 4 * c->feat + c->n_f32 * c->f32 + c->angles + c->op;
   } else {
-    c->n_f32 = 4 + (out32 && !c->one_run ? 1 : 2);              // gradients of the four feature tensors, dv of the runs
+    c->n_f32 = 4 + (out32 ? 1 : 2);              // gradients of the four feature tensors, dv of the halves
     c->total = 4 * c->feat + c->n_f32 * c->f32 + 2 * c->part + c->angles + c->op;
   }
   return true;
@@ -420,7 +423,7 @@ la_status la_lrpe_fwd(const la_shape* shape, const void* q, const void* k, const
   char* w = static_cast<char*>(workspace);
   void* qc = w; void* qs = w + c.feat; void* kc = w + 2 * c.feat; void* ks = w + 3 * c.feat;
   float* tmp = reinterpret_cast<float*>(w + 4 * c.feat);
-  float2* table = reinterpret_cast<float2*>(w + 4 * c.feat + c.n_f32 * c.f32);
+  float2* table = reinterpret_cast<float2*>(c.angles ? w + 4 * c.feat + c.n_f32 * c.f32 : w + 4 * c.feat);
   void* op_ws = w + 4 * c.feat + c.n_f32 * c.f32 + c.angles;
   const bool out32 = shape->out_dtype == LA_F32;
   la_shape inner = *shape;
@@ -429,16 +432,16 @@ la_status la_lrpe_fwd(const la_shape* shape, const void* q, const void* k, const
 
   if (run_angles(shape, theta, table, pos0, cs) != cudaSuccess) return LA_ERR_CUDA;
   if (run_features(shape, q, k, table, qc, qs, kc, ks, cs) != cudaSuccess) return LA_ERR_CUDA;
-  if (c.one_run) {
-    const la_status st = halves_fwd(&inner, qc, kc, v, lambda_host, tmp, kv_in, kv_out, op_ws, c.op, stream);
-    if (st != LA_OK) return st;
-    return run_sum(shape, tmp, tmp + c.f32 / 4, o, cs) == cudaSuccess ? LA_OK : LA_ERR_CUDA;
-  }
   float* first = out32 ? static_cast<float*>(o) : tmp + c.f32 / 4;
-  la_status st = la_fwd(&inner, qc, kc, v, lambda_host, first, kv_in, kv_out, op_ws, c.op, stream);
-  if (st != LA_OK) return st;
-  st = la_fwd(&inner, qs, ks, v, lambda_host, tmp, kv_in ? kv_in + state : nullptr, kv_out ? kv_out + state : nullptr,
-              op_ws, c.op, stream);
+  la_status st;
+  if (c.one_run) {
+    st = halves_fwd(&inner, qc, kc, v, lambda_host, first, tmp, kv_in, kv_out, op_ws, c.op, stream);
+  } else {
+    st = la_fwd(&inner, qc, kc, v, lambda_host, first, kv_in, kv_out, op_ws, c.op, stream);
+    if (st == LA_OK)
+      st = la_fwd(&inner, qs, ks, v, lambda_host, tmp, kv_in ? kv_in + state : nullptr, kv_out ? kv_out + state : nullptr,
+                  op_ws, c.op, stream);
+  }
   if (st != LA_OK) return st;
   if (run_sum(shape, first, tmp, o, cs) != cudaSuccess) return LA_ERR_CUDA;
   return LA_OK;
@@ -467,10 +470,6 @@ la_status la_lrpe_bwd(const la_shape* shape, const void* q, const void* k, const
   float* dv_s = reinterpret_cast<float*>(w + 4 * c.f32);
   const bool out32 = shape->out_dtype == LA_F32;
   float* dv_c = out32 ? static_cast<float*>(dv) : reinterpret_cast<float*>(w + 5 * c.f32);
-  if (c.one_run) {
-    dv_c = dv_s;
-    dv_s = reinterpret_cast<float*>(w + 5 * c.f32);
-  }
   w += c.n_f32 * c.f32;
   float* part_q = reinterpret_cast<float*>(w);
   float* part_k = reinterpret_cast<float*>(w + c.part);
@@ -484,7 +483,7 @@ la_status la_lrpe_bwd(const la_shape* shape, const void* q, const void* k, const
   if (run_features(shape, q, k, table, qc, qs, kc, ks, cs) != cudaSuccess) return LA_ERR_CUDA;
   la_status st;
   if (c.one_run) {
-    st = halves_bwd(&inner, qc, kc, v, d_o, lambda_host, g_qc, g_kc, dv_c, kv_in, grad_kv_out, grad_kv_in, op_ws, c.op, stream);
+    st = halves_bwd(&inner, qc, kc, v, d_o, lambda_host, g_qc, g_kc, dv_c, dv_s, kv_in, grad_kv_out, grad_kv_in, op_ws, c.op, stream);
     if (st != LA_OK) return st;
   } else {
     st = la_bwd(&inner, qc, kc, v, d_o, lambda_host, g_qc, g_kc, dv_c, kv_in, grad_kv_out, grad_kv_in, op_ws, c.op, stream);

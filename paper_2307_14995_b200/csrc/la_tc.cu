@@ -117,6 +117,7 @@ struct TcJob {
   const float* local;
   bool z_in_t, local_t;
   int shared;  // see OpArgs
+  void* out2;
   // gate epilogue of the forward walk (D = 128 only): y = SRMSNorm(out) (.) u
   const void* u;
   void* y;
@@ -901,7 +902,7 @@ bool make_maps(TcMaps* m, const OpArgs& args, int D, const bool* out_f32) {
 }
 
 TcJob make_job(const OpArgs& a) {
-  return TcJob{a.c, a.out, a.entry, a.final_out, a.z_in, a.local, a.z_in_t != 0, a.local_t != 0, a.shared, a.u, a.y, a.rstd};
+  return TcJob{a.c, a.out, a.entry, a.final_out, a.z_in, a.local, a.z_in_t != 0, a.local_t != 0, a.shared, a.out2, a.u, a.y, a.rstd};
 }
 
 TcArgs make_args(const OpArgs& args, const OpArgs* second, int precision) {

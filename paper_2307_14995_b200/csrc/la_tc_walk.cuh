@@ -585,9 +585,11 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     const int q = warp & 3;
     const int th = (warp >= 24) ? 64 : 0;  // first of this warp's 64 tokens
     const uint32_t colO = tmem + ((uint32_t)(q * 32) << 16) + WCOL_O + th;
-    const size_t head_off = (size_t)(args.seq_start ? 0 : bh / args.H) * args.sB + (size_t)(bh % args.H) * args.sH +
+    const int batch = args.seq_start ? 0 : bh / args.H;
+    const bool apart = job.out2 != nullptr && batch >= args.fold;
+    const size_t head_off = (size_t)(apart ? batch - args.fold : batch) * args.sB + (size_t)(bh % args.H) * args.sH +
                             (size_t)tok0 * args.sT;
-    TOut* const out = static_cast<TOut*>(job.out) + head_off + q * 32 + lane;
+    TOut* const out = static_cast<TOut*>(apart ? job.out2 : job.out) + head_off + q * 32 + lane;
     WARP_ARRIVE(W_M2_OK);  // there is no earlier O to read
     for (int it = 0; it < nblk; ++it) {
       // ---- O <- O diag(f_out), between M2 and M4 ----

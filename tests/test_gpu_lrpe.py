@@ -223,3 +223,46 @@ def test_lrpe_rejects_bad_arguments():
         la.la_lrpe_fwd(shape, x, x, x, th, lam, o, -1, None, None, ws)                # negative position
     with pytest.raises(la.LaError):
         la.la_lrpe_fwd(shape, x, x, x, th, torch.tensor([1.0, 1.5]), o, 0, None, None, ws)   # lambda out of range
+
+
+@pytest.mark.parametrize("B,N,seg_len,out_dtype,layout", [
+    (1, 2500, 1024, torch.float32, "BHND"),   # segments of eight blocks shared by clusters, a ragged tail
+    (2, 1100, 0, torch.bfloat16, "BNHD"),
+    (1, 3, 0, torch.float32, "BNHD"),         # a table of angles larger than the temporary
+])
+def test_lrpe_workspace_and_folded_segments(B, N, seg_len, out_dtype, layout):
+    """The two halves' results in two tensors, the table of angles in the temporary: nothing behind
+    la_lrpe_workspace_bytes is written, its fp32 temporaries are one (two with bf16 results) and five (six), and the results
+    are those of the definition."""
+    H, d = 2, 128
+    q, k, v, do = inputs.make_qkvdo(B, H, N, d, d, seed=N)
+    lam = torch.tensor([1.0, 0.99])
+    theta = inputs.make_theta(H, d, seed=3)
+    lam64, th64 = lam.double().numpy(), theta.double().numpy()
+    tm = (lambda x: x.permute(0, 2, 1, 3).contiguous()) if layout == "BNHD" else (lambda x: x)
+    back = (lambda x: x.permute(0, 2, 1, 3)) if layout == "BNHD" else (lambda x: x)
+    shape = la.make_shape(B, H, N, d, d, torch.bfloat16, out_dtype, seg_len,
+                          layout=la.LA_LAYOUT_BNHD if layout == "BNHD" else la.LA_LAYOUT_BHND)
+    inner = la.make_shape(2 * B, H, N, d, d, torch.bfloat16, torch.float32, seg_len, layout=shape.layout)
+    elems, more = B * H * N * d, 1 if out_dtype == torch.float32 else 2
+    table = H * d * 8 * (-(-N // 16) + 1)
+    need = [la.lrpe_workspace_bytes(op, shape) for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    assert need[0] <= 4 * 2 * elems + more * 4 * elems + table * (table > 4 * elems) + \
+        la.workspace_bytes(la.LA_OP_FWD, inner) + 4096
+    assert need[1] <= 4 * 2 * elems + (4 + more) * 4 * elems + table + 2 * B * H * -(-N // 128) * d * 4 + \
+        la.workspace_bytes(la.LA_OP_BWD, inner) + 4096
+    bufs = [torch.full((n + 4096,), 0xA5, dtype=torch.uint8, device=DEV) for n in need]
+    dev = [tm(x).to(DEV) for x in (q, k, v, do)]
+    o, dq, dk, dv = [torch.full(dev[0].shape, float("nan"), dtype=out_dtype, device=DEV) for _ in range(4)]
+    dth = torch.empty(H, d, device=DEV)
+    la.la_lrpe_fwd(shape, *dev[:3], theta.to(DEV), lam, o, workspace=bufs[0][:need[0]])
+    la.la_lrpe_bwd(shape, *dev, theta.to(DEV), lam, dq, dk, dv, dth, workspace=bufs[1][:need[1]])
+    torch.cuda.synchronize()
+    la.device_status()
+    assert all(bool((b[n:] == 0xA5).all()) for b, n in zip(bufs, need))
+    rel = 2.0 ** -8 if out_dtype == torch.float32 else 2.0 ** -7
+    close_with_feature_rounding(back(o), orc.lrpe_fwd_quad(q, k, v, lam64, th64), "o", rel)
+    rq, rk, rv, rth = orc.lrpe_bwd_quad(q, k, v, do, lam64, th64)
+    for g, r, name in ((dq, rq, "dq"), (dk, rk, "dk"), (dv, rv, "dv")):
+        close_with_feature_rounding(back(g), r, name, rel)
+    check_theta(dth, rth, theta_bound(q, k, v, do, lam64, th64))
