@@ -192,9 +192,10 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 def _lam(lam):
-    # a contiguous fp32 CPU tensor is read where it lies (the library copies it before it returns); anything else is
-    # converted, 5 us for 32 heads
-    if type(lam) is torch.Tensor and lam.dtype is torch.float32 and lam.is_cpu and lam.is_contiguous():
+    # a contiguous fp32 CPU vector is read where it lies (the library copies it before it returns); anything else is
+    # converted, 5 us for 32 heads, or refused
+    if (type(lam) is torch.Tensor and lam.dtype is torch.float32 and lam.is_cpu and lam.dim() == 1 and lam.is_contiguous()
+            and not lam.is_neg()):
         return lam.data_ptr()
     vals = [float(x) for x in (lam.tolist() if hasattr(lam, "tolist") else lam)]
     return (ctypes.c_float * len(vals))(*vals)
