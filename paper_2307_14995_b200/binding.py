@@ -201,13 +201,18 @@ def _lam(lam):
     return (ctypes.c_float * len(vals))(*vals)
 
 
+# The raw handle of the current stream, without the Stream object around it (2 us); private functions of torch, which a
+# release may not have.
+_RAW_STREAM = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_CURRENT_DEVICE = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
-    if not torch.cuda.is_initialized():
+    if _RAW_STREAM is None or _CURRENT_DEVICE is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    # the raw handle of the current stream, without the Stream object around it (2 us)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _RAW_STREAM(_CURRENT_DEVICE())
 
 
 def alloc_workspace(op: int, shape: LaShape, device) -> Optional[torch.Tensor]:

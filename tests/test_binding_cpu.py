@@ -29,3 +29,17 @@ def test_decay_rates_reach_the_library_by_value(lam):
 def test_decay_rates_that_are_no_vector_are_refused(lam):
     with pytest.raises(TypeError):
         la._lam(lam)
+
+
+@pytest.mark.parametrize("missing", ["_RAW_STREAM", "_CURRENT_DEVICE"])
+def test_current_stream_without_the_private_functions(monkeypatch, missing):
+    class Stream:
+        cuda_stream = 77
+
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.setattr(la, "_RAW_STREAM", lambda device: 5)
+    monkeypatch.setattr(la, "_CURRENT_DEVICE", lambda: 0)
+    assert la._stream(None) == 5 and la._stream(Stream) == 77
+    monkeypatch.setattr(la, missing, None)
+    assert la._stream(None) == 77
