@@ -31,9 +31,9 @@ decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* _
   constexpr int PASSES = D / RPP;
   static_assert(D == E && D % RPP == 0 && THREADS % LPR == 0, "shape");
 
-  __shared__ float sq[CHUNK][D];
-  __shared__ float sk[CHUNK][D];
-  __shared__ float sv[CHUNK][E];
+  __shared__ alignas(16) float sq[CHUNK][D];  // (written, and sv read, 16 bytes at a time)
+  __shared__ alignas(16) float sk[CHUNK][D];
+  __shared__ alignas(16) float sv[CHUNK][E];
   __shared__ float4 red[2][RPP][LPR];
 
   const int bh = blockIdx.x;
