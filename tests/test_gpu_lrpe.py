@@ -154,6 +154,23 @@ def test_lrpe_zero_angles_equal_the_plain_operator_bitwise():
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("N,seg_len", [(700, 128), (2100, 1024), (2100, 0)])
+def test_lrpe_zero_angles_in_several_segments(N, seg_len):
+    """Equal segments: bit for bit.  The library's own plan sees twice the heads and may choose others: sums that differ in
+    their order, 2^-17 of |sum| up to 5 RMS on either side, twice (o feeds nothing else): 1.5e-4."""
+    B, H, d = 1, 8, 128
+    q, k, v, do = inputs.make_qkvdo(B, H, N, d, d, seed=29)
+    lam = inputs.decay_rates(H, 0.5)
+    got = run_gpu(q, k, v, do, lam, torch.zeros((H, d)), seg_len=seg_len)[:4]
+    dev = [x.to(DEV) for x in (q, k, v, do)]
+    ref = (la.fwd(*dev[:3], lam, seg_len=seg_len),) + tuple(la.bwd(*dev, lam, seg_len=seg_len))
+    for a, b in zip(got, ref):
+        if seg_len:
+            assert torch.equal(a, b)
+        else:
+            assert_close(a, b.double().cpu().numpy(), 1.5e-4)
+
+
 def test_lrpe_fp32_inputs():
     B, H, N, d = 1, 2, 200, 64
     q, k, v, do = inputs.make_qkvdo(B, H, N, d, d, dtype=torch.float32, seed=24)

@@ -162,3 +162,33 @@ def test_workspace_holds_the_sets_that_are_used(d, dtype, sets, B, N, seg_len):
         for name, g, r in zip(("dq", "dk", "dv", "gin"), (dq, dk, dv, gin), ref):
             assert_close(g, r, 3.1e-4, name)
     assert all(bool((b[n:] == 0xA5).all()) for b, n in zip(bufs, need))
+
+
+@pytest.mark.parametrize("lens", [[2600, 700, 1025, 3], [1, 1024, 2048, 2049, 5000]])
+def test_packed_segments_shared_by_clusters(lens):
+    """Packed sequences in segments of eight blocks, which clusters share, with clusters whose segment a shorter sequence does
+    not have, sequences taken longest first, and a tail of one and of three tokens."""
+    H, d, S = 3, 128, len(lens)
+    cu = [sum(lens[:i]) for i in range(S + 1)]
+    T = cu[-1]
+    gen = torch.Generator().manual_seed(T)
+    q, k, v, do = [torch.randn(1, T, H, d, generator=gen).bfloat16() for _ in range(4)]
+    kv_in, gko = [torch.randn(S, H, d, d, generator=gen) * 0.1 for _ in range(2)]
+    lam = torch.tensor([1.0, 0.9995, 0.9])
+    shape = la.make_shape(1, H, T, d, d, torch.bfloat16, torch.float32, 1024, layout=la.LA_LAYOUT_BNHD)
+    dev = [x.cuda() for x in (q, k, v, do, kv_in, gko)]
+    o, dq, dk, dv = [torch.empty(1, T, H, d, device="cuda") for _ in range(4)]
+    kv, gin = [torch.empty(S, H, d, d, device="cuda") for _ in range(2)]
+    ws = [torch.empty(la.varlen_workspace_bytes(op, shape, cu), dtype=torch.uint8, device="cuda") for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    la.la_fwd_varlen(shape, *dev[:3], lam, o, cu, dev[4], kv, ws[0])
+    la.la_bwd_varlen(shape, *dev[:4], lam, dq, dk, dv, cu, dev[4], dev[5], gin, ws[1])
+    torch.cuda.synchronize()
+    lam64 = lam.double().numpy()
+    for i in range(S):
+        part = lambda x: x[:, cu[i]:cu[i + 1]].transpose(1, 2)
+        one = [part(x).contiguous() for x in (q, k, v, do)]
+        ref = orc.fwd_rec(*one[:3], lam64, kv_in=kv_in[i:i + 1], want_state=True)
+        ref += orc.bwd_rec(*one, lam64, kv_in=kv_in[i:i + 1], grad_kv_out=gko[i:i + 1], want_state_grad=True)
+        got = (part(o), kv[i:i + 1], part(dq), part(dk), part(dv), gin[i:i + 1])
+        for name, g, r in zip(("o", "kv", "dq", "dk", "dv", "gin"), got, ref):
+            assert_close(g, r, 3.1e-4, "%s of sequence %d" % (name, i))
