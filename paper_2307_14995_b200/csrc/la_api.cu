@@ -274,7 +274,6 @@ cudaError_t run_scan(const la_shape* s, const Plan& p, const DecayTable& tab, fl
   sa.N = s->N;
   sa.seg_len = p.seg_len;
   sa.nseg = p.nseg;
-  sa.seq_len = p.pk.len;
   sa.Da = s->d;  // d == e in every supported shape, so both orientations are square
   sa.Ec = s->e;
   sa.reverse = reverse;

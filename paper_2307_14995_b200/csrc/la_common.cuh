@@ -89,7 +89,7 @@ struct ScanArgs {
   const float* z_in;   // [BH, Da*Ec] (or [BH, Ec*Da] if z_in_transposed), or NULL = zeros
   int z_in_transposed;
   int BH, H, N, seg_len, nseg, Da, Ec, reverse;
-  const int* seq_len;  // packed batch: DEVICE array of BH / H lengths (N is then the longest), or NULL
+  const int* seq_len;  // launch_prefix, packed batch: DEVICE array of BH / H lengths (N is then the longest), or NULL
 };
 
 // Chain of piece-local states into the state at one boundary (a cut of the sequence):
@@ -175,12 +175,8 @@ struct KernelTimer {
 enum { K_PREPASS = 0, K_SCAN = 1, K_WALK = 2, K_DECODE = 3, K_WALK_PAIR = 4, K_GATE = 5, K_LRPE = 6, K_NUM = 7 };
 
 // ---- small device helpers --------------------------------------------------
-__device__ __forceinline__ float decay_pow(float s2, float n) {
-  // lambda^n for n >= 0; s2 == 0 (lambda == 1) gives exactly 1.
-  return exp2f(-s2 * n);
-}
 __device__ __forceinline__ float decay_pow_d(double s2, double n) {
-  // Same in double, rounded once; used where a handful of factors per block are tabulated.
+  // lambda^n for n >= 0 in double, rounded once; s2 == 0 (lambda == 1) gives exactly 1.
   return (float)exp2(-s2 * n);
 }
 

@@ -300,9 +300,7 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanArgs args, const De
   const int x0 = (blockIdx.y / tiles_y) * 32, y0 = (blockIdx.y % tiles_y) * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   const double s2 = tab.s2[bh % args.H];
-  // this (batch, head)'s own length and segment count (a packed batch has sequences of different lengths)
-  const int n_tok = args.seq_len ? args.seq_len[bh / args.H] : args.N;
-  const int nseg = (n_tok + args.seg_len - 1) / args.seg_len;
+  const int n_tok = args.N, nseg = args.nseg;
   for (int p = threadIdx.x; p < nseg; p += 256) {
     const int L = min(n_tok, (p + 1) * args.seg_len) - p * args.seg_len;
     gamma[p] = decay_pow_d(s2, (double)L);
@@ -360,10 +358,10 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanArgs args, const De
 // the decayed a, or (final state) rows of c with w the decayed b.
 // A walk that carries the state from block to block is bound by that chain where it has few heads: 8 us a block at d = 64
 // with two thread blocks on the chip.  Here the work grows with the square of the segment, but all tiles run at once, and the
-// walks of a launch do too (B = 1, H = 2, N = 256, d = 64 in fp32, forward
-// plus backward: 240 us before, 38 now; with N = 2048 and 128-token segments 1155 and 81).
-// 128 threads and 60 KB at d = 128, so that three thread blocks share an SM; the next tiles are loaded into registers while
-// the present ones are multiplied.
+// walks of a launch do too (B = 1, H = 2, N = 256, d = 64 in fp32, forward plus backward: 240 us before, 38 now; with N = 2048
+// and 128-token segments 1155 and 81).
+// 128 threads; at d = 128 57 KB and 178 registers, which let two thread blocks share an SM; the next tiles are loaded into
+// registers while the present ones are multiplied.
 constexpr int ROWS_THREADS = 128;
 constexpr int ROWS_MAX_JOBS = 3;
 static_assert(ROWS_MAX_SEG % C == 0, "whole tiles");
@@ -380,7 +378,6 @@ struct RowsSmem {
   float b[C][D + 4];
   float t[C][D];       // rows of c or Z
   float w[C][AP];      // w[j][i]
-  float f_out[C];
   float dtab[ROWS_MAX_SEG + 1];  // lambda^n
 };
 

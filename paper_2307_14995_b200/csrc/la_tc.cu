@@ -955,14 +955,10 @@ cudaError_t launch_walk64(const OpArgs& args, const OpArgs* second, const DecayT
   m1 = m0;
   if (second && !make_maps(&m1, *second, 64, &f32)) return cudaErrorInvalidValue;
   const TcArgs ta = make_args(args, second, precision);
-  if (second) {  // only the reverse direction is ever paired
-    if (!args.reverse) return cudaErrorInvalidValue;
+  if ((second != nullptr) != (args.reverse != 0)) return cudaErrorInvalidValue;  // the reverse walks come in pairs, and only they
+  if (second)
     return f32 ? launch_t<true, false, float, 2>(m0, m1, ta, tab, stream)
                : launch_t<true, false, __nv_bfloat16, 2>(m0, m1, ta, tab, stream);
-  }
-  if (args.reverse)
-    return f32 ? launch_t<true, false, float, 1>(m0, m1, ta, tab, stream)
-               : launch_t<true, false, __nv_bfloat16, 1>(m0, m1, ta, tab, stream);
   return f32 ? launch_t<false, false, float, 1>(m0, m1, ta, tab, stream)
              : launch_t<false, false, __nv_bfloat16, 1>(m0, m1, ta, tab, stream);
 }
