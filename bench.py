@@ -65,8 +65,8 @@ def bytes_per_token_head(d: int, out_bytes: int, what: str) -> float:
     return float({"fwd": fwd, "bwd": bwd, "step": fwd + bwd, "walk": walk, "walk_pair": pair}[what])
 
 
-# DRAM traffic of one walk launch per token-head, from the ncu capture summarised in
-# profiles/tc_walk_kernel_small_case.md: 207.7 MB read per 262144 token-heads (the algorithmic
+# DRAM traffic of one walk launch per token-head, from an ncu capture of the forward walk at 2 x 16 heads x 8192
+# tokens: 207.7 MB read per 262144 token-heads (the algorithmic
 # 768 B plus 3.2 % for segment states and re-fetches).  The writes of that small launch (91 MB of the
 # 134 MB of output; the rest was still in L2 when it ended) do not grow in proportion: at full size
 # the 4.3 GB of output cannot stay in the 126 MB L2, so the output is counted in full (512 B).

@@ -263,7 +263,7 @@ la_status la_chain_states(const la_shape* shape, long long total_tokens, long lo
  * cu[num_seqs] = T, strictly increasing) gives the first token of each sequence.  Sequence i runs
  * from the state kv_in[i] (or zero) and leaves kv_out[i]; kv_in, kv_out, grad_kv_out, grad_kv_in are
  * [num_seqs, H, d, e] fp32 or NULL.  Results are those of la_fwd / la_bwd on each sequence alone.
- * bf16 inputs at d = e = 128 with outputs aligned to 32 bytes (and more than one sequence) run as ONE set of
+ * bf16 inputs at d = e = 128 (and more than one sequence) run as ONE set of
  * launches over all sequences: every (sequence, head[, segment]) is a thread block of the tensor-core kernels, which
  * take each sequence's first token and length from a small table the call copies to the head of the workspace
  * (a host-to-device copy on `stream` from pageable memory: such a call cannot be captured into a graph).  Other

@@ -4,7 +4,7 @@
 // A row with ||o||_2 = 0 gives y = 0 and zero gradients (Eq. 8 has no epsilon).
 //
 // The forward kernel is the fallback of la_fwd_gated where the epilogue is not fused into the walk kernel
-// (d = 64, the fp32 path, outputs aligned to 16 bytes only); the backward kernel is la_gate_bwd.  Both are
+// (d = 64, the fp32 path); the backward kernel is la_gate_bwd.  Both are
 // bound by HBM: e / 4 lanes share a row, each lane moves 4 consecutive elements with one vector access per
 // tensor, and the row sums are reduced with shuffles.
 #include "la_common.cuh"
