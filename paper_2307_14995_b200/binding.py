@@ -191,11 +191,13 @@ def _ptr(t: Optional[torch.Tensor]):
     return t.data_ptr()
 
 
+_TENSOR, _F32 = torch.Tensor, torch.float32
+
+
 def _lam(lam):
     # a contiguous fp32 CPU vector is read where it lies (the library copies it before it returns); anything else is
     # converted, 5 us for 32 heads, or refused
-    if (type(lam) is torch.Tensor and lam.dtype is torch.float32 and lam.is_cpu and lam.dim() == 1 and lam.is_contiguous()
-            and not lam.is_neg()):
+    if type(lam) is _TENSOR and lam.dtype is _F32 and lam.is_cpu and lam.stride() == (1,) and not lam.is_neg():
         return lam.data_ptr()
     vals = [float(x) for x in (lam.tolist() if hasattr(lam, "tolist") else lam)]
     return (ctypes.c_float * len(vals))(*vals)
