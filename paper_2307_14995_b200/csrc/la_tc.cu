@@ -117,7 +117,6 @@ struct TcJob {
   const float* local;
   bool z_in_t, local_t;
   int shared;  // see OpArgs
-  void* out2;
   // gate epilogue of the forward walk (D = 128 only): y = SRMSNorm(out) (.) u
   const void* u;
   void* y;
@@ -138,6 +137,7 @@ struct TcArgs {
   int BH, H, N, seg_len, nseg;
   int precision;
   int scanned, fold;  // see OpArgs
+  long long second_half;  // bytes to add to the first job's output for entries fold .. 2 fold - 1 (OpArgs::out2)
   long long sT, sH, sB;  // element offset of token t of (b,h): b*sB + h*sH + t*sT (rows of D contiguous features)
 };
 
@@ -902,7 +902,7 @@ bool make_maps(TcMaps* m, const OpArgs& args, int D, const bool* out_f32) {
 }
 
 TcJob make_job(const OpArgs& a) {
-  return TcJob{a.c, a.out, a.entry, a.final_out, a.z_in, a.local, a.z_in_t != 0, a.local_t != 0, a.shared, a.out2, a.u, a.y, a.rstd};
+  return TcJob{a.c, a.out, a.entry, a.final_out, a.z_in, a.local, a.z_in_t != 0, a.local_t != 0, a.shared, a.u, a.y, a.rstd};
 }
 
 TcArgs make_args(const OpArgs& args, const OpArgs* second, int precision) {
@@ -929,8 +929,11 @@ cudaError_t launch_walk128(const OpArgs& args, const OpArgs* second, const Decay
   if (!make_maps(&m0, args, 128, nullptr)) return cudaErrorInvalidValue;
   m1 = m0;
   if (second && !make_maps(&m1, *second, 128, nullptr)) return cudaErrorInvalidValue;
-  const TcArgs ta = make_args(args, second, precision);
   const bool f32 = (out_dt == DT_F32);
+  TcArgs ta = make_args(args, second, precision);
+  if (second && second->out2) return cudaErrorInvalidValue;
+  if (args.out2)
+    ta.second_half = static_cast<char*>(args.out2) - static_cast<char*>(args.out) - args.fold * args.sB * (f32 ? 4 : 2);
   if (args.u) {  // the gate epilogue exists for the single forward walk
     if (second || args.reverse) return cudaErrorInvalidValue;
     if (args.out)
