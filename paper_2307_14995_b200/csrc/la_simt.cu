@@ -362,57 +362,69 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanArgs args, const De
 // and 128-token segments 1155 and 81).
 // 128 threads; at d = 128 57 KB and 178 registers, which let two thread blocks share an SM; the next tiles are loaded into
 // registers while the present ones are multiplied.
-constexpr int ROWS_THREADS = 128;
+//
+// The tiles that a thread block adds up are shared out over G groups of 128 threads, each with its own pair of tiles in shared
+// memory, whose sums meet at the end: with one group a tile costs 4400 clocks, a warp per scheduler waiting for its own loads.
+// Where thread blocks fill the chip several times over, groups only add their meeting (rows_groups).
+constexpr int ROWS_THREADS = 128;  // of a group
 constexpr int ROWS_MAX_JOBS = 3;
 static_assert(ROWS_MAX_SEG % C == 0, "whole tiles");
 
 struct RowsArgs {
   OpArgs job[ROWS_MAX_JOBS];
   int first_block[ROWS_MAX_JOBS + 1];  // thread blocks of job j: first_block[j] .. first_block[j + 1] - 1
-  int units[ROWS_MAX_JOBS];            // how many of them make rows; the others make the final state
+  int units[ROWS_MAX_JOBS];            // how many of them make rows; the others make states
 };
 
-template <int D>
+template <int D, int G>
 struct RowsSmem {
-  float a[C][D + 4];   // rows of a (final state: unused)
-  float b[C][D + 4];
-  float t[C][D];       // rows of c or Z
-  float w[C][AP];      // w[j][i]
+  float a[C][D + 4];   // rows of a (states: unused)
+  struct Group {
+    float b[C][D + 4];
+    float t[C][D];     // rows of c or Z
+    float w[C][AP];    // w[j][i]
+  } group[G];
   float dtab[ROWS_MAX_SEG + 1];  // lambda^n
 };
 
 // 32 rows of D values into registers, 16 bytes (fp32) at a time; rows past `valid` are zero.
 template <typename TIn, int D>
-__device__ __forceinline__ void fetch_tile(float4 (&x)[D / 16], const TIn* src, long long row_stride, int valid) {
+__device__ __forceinline__ void fetch_tile(float4 (&x)[D / 16], const TIn* src, long long row_stride, int valid, int tid) {
 #pragma unroll
   for (int n = 0; n < D / 16; ++n) {
-    const int idx = threadIdx.x + n * ROWS_THREADS, row = idx / (D / 4), col = idx % (D / 4) * 4;
+    const int idx = tid + n * ROWS_THREADS, row = idx / (D / 4), col = idx % (D / 4) * 4;
     float v[4] = {0.f, 0.f, 0.f, 0.f};
     if (row < valid) Vec4<TIn>::load(src + (size_t)row * row_stride + col, v);
     x[n] = make_float4(v[0], v[1], v[2], v[3]);
   }
 }
 template <int D, int W>
-__device__ __forceinline__ void put_tile(float (*dst)[W], const float4 (&x)[D / 16]) {
+__device__ __forceinline__ void put_tile(float (*dst)[W], const float4 (&x)[D / 16], int tid) {
 #pragma unroll
   for (int n = 0; n < D / 16; ++n) {
-    const int idx = threadIdx.x + n * ROWS_THREADS;
+    const int idx = tid + n * ROWS_THREADS;
     *reinterpret_cast<float4*>(&dst[idx / (D / 4)][idx % (D / 4) * 4]) = x[n];
   }
 }
+template <int G>
+__device__ __forceinline__ void group_sync(int grp) {
+  if (G == 1) __syncthreads();
+  else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(ROWS_THREADS) : "memory");
+}
 
-template <typename TIn, typename TOut, int D>
-__global__ void __launch_bounds__(ROWS_THREADS)
+template <typename TIn, typename TOut, int D, int G>
+__global__ void __launch_bounds__(ROWS_THREADS * G)
 simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ DecayTable tab) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  RowsSmem<D>& sm = *reinterpret_cast<RowsSmem<D>*>(smem_raw);
-  const int tid = threadIdx.x;
+  RowsSmem<D, G>& sm = *reinterpret_cast<RowsSmem<D, G>*>(smem_raw);
+  const int grp = threadIdx.x / ROWS_THREADS, tid = threadIdx.x % ROWS_THREADS;
+  typename RowsSmem<D, G>::Group& gm = sm.group[grp];
   int jb = 0;
   while (jb + 1 < ROWS_MAX_JOBS && (int)blockIdx.x >= all.first_block[jb + 1]) ++jb;
   const OpArgs& args = all.job[jb];
   int unit = (int)blockIdx.x - all.first_block[jb];
   const bool rev = args.reverse != 0;
-  const bool state = unit >= all.units[jb];
+  const bool state = unit >= all.units[jb];  // the state leaving the sequence, or (local_out) every segment's local state
   const int per_seg = (args.seg_len + C - 1) / C;
   int bh, seg, tile;
   if (state) {
@@ -420,6 +432,10 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
     tile = unit % (D / C);
     bh = unit / (D / C);
     seg = rev ? 0 : args.nseg - 1;
+    if (args.local_out) {
+      seg = bh % args.nseg;
+      bh /= args.nseg;
+    }
   } else {
     // the row tiles with the most tiles to add up first
     tile = unit / (args.BH * args.nseg);
@@ -434,7 +450,6 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
 
   const size_t head_off = (size_t)(bh / args.H) * args.sB + (size_t)(bh % args.H) * args.sH + (size_t)seg_t0 * args.sT;
   const long long sT = args.sT;
-  const TIn* a = static_cast<const TIn*>(args.a) + head_off;
   const TIn* b = static_cast<const TIn*>(args.b) + head_off;
   const TIn* c = static_cast<const TIn*>(args.c) + head_off;
   const float* Z = args.entry ? args.entry + ((size_t)bh * args.nseg + seg) * D * D : nullptr;
@@ -448,15 +463,34 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
   const int dir = state ? (rev ? -1 : 1) : step;
 
   float4 nb[D / 16], nc[D / 16];
-  fetch_tile<TIn, D>(nb, b + (size_t)first * C * sT, sT, L - first * C);
-  fetch_tile<TIn, D>(nc, c + (size_t)first * C * sT, sT, L - first * C);
-  if (!state) {
+  const auto fetch_pair = [&](int n) {
+    const int t0 = (first + n * dir) * C;
+    fetch_tile<TIn, D>(nb, b + (size_t)t0 * sT, sT, L - t0, tid);
+    fetch_tile<TIn, D>(nc, c + (size_t)t0 * sT, sT, L - t0, tid);
+  };
+  if (grp < count) fetch_pair(grp);
+  if (!state && grp == G - 1) {
     float4 na[D / 16];
-    fetch_tile<TIn, D>(na, a + (size_t)tile * C * sT, sT, L - tile * C);
-    put_tile<D, D + 4>(sm.a, na);
+    const TIn* a = static_cast<const TIn*>(args.a) + head_off;
+    fetch_tile<TIn, D>(na, a + (size_t)tile * C * sT, sT, L - tile * C, tid);
+    put_tile<D, D + 4>(sm.a, na, tid);
   }
-  for (int n = tid; n <= L; n += ROWS_THREADS) sm.dtab[n] = decay_pow_d(s2, (double)n);
+  for (int n = threadIdx.x; n <= L; n += ROWS_THREADS * G) sm.dtab[n] = decay_pow_d(s2, (double)n);
   __syncthreads();
+
+  int items = count;
+  if (!state) {
+    // leave out the tiles whose every weight is zero in fp32, and add those of the entry state
+    items = 1;
+    while (items < count && sm.dtab[(items - 1) * C + 1] != 0.f) ++items;
+    count = items;
+    if (Z && sm.dtab[rev ? max(L - tile * C - C, 0) : tile * C + 1] != 0.f) items += D / C;
+  }
+  const auto fetch = [&](int n) {
+    if (n < count) fetch_pair(n);
+    else fetch_tile<float, D>(nc, Z + (size_t)(n - count) * C * D, D, C, tid);
+  };
+  if (grp >= count && grp < items) fetch(grp);
 
   constexpr int EM = D / 16;  // value columns of a thread
   const int i4 = (tid / 16) * 4, e0 = (tid % 16) * 4;
@@ -465,43 +499,25 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int m = 0; m < EM; ++m) acc[r][m] = 0.f;
-  // acc += w^T t over 32 rows; a thread has rows i4 .. i4 + 3 and columns e0 .. e0 + 3 (d = 128: and 64 + those)
-  const auto accumulate = [&]() {
-#pragma unroll 4
-    for (int j = 0; j < C; ++j) {
-      const float4 w = *reinterpret_cast<const float4*>(&sm.w[j][i4]);
-      const float wr[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int g = 0; g < EM / 4; ++g) {
-        const float4 t = *reinterpret_cast<const float4*>(&sm.t[j][e0 + 64 * g]);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          acc[r][4 * g + 0] = fmaf(wr[r], t.x, acc[r][4 * g + 0]);
-          acc[r][4 * g + 1] = fmaf(wr[r], t.y, acc[r][4 * g + 1]);
-          acc[r][4 * g + 2] = fmaf(wr[r], t.z, acc[r][4 * g + 2]);
-          acc[r][4 * g + 3] = fmaf(wr[r], t.w, acc[r][4 * g + 3]);
-        }
-      }
-    }
-  };
 
-  for (int n = 0; n < count; ++n) {
+  for (int n = grp; n < items; n += G) {
+    const bool pair = n < count;  // else 32 rows of the entry state
     const int jt = first + n * dir;
-    put_tile<D, D + 4>(sm.b, nb);
-    put_tile<D, D>(sm.t, nc);
-    __syncthreads();
-    // the next tile, unless every weight past this one is zero in fp32
-    bool more = n + 1 < count;
-    if (!state && more) more = sm.dtab[n * C + 1] != 0.f;
-    if (more) {
-      const int nt = jt + dir;
-      fetch_tile<TIn, D>(nb, b + (size_t)nt * C * sT, sT, L - nt * C);
-      fetch_tile<TIn, D>(nc, c + (size_t)nt * C * sT, sT, L - nt * C);
-    }
-    if (state) {
+    if (pair) put_tile<D, D + 4>(gm.b, nb, tid);
+    put_tile<D, D>(gm.t, nc, tid);
+    group_sync<G>(grp);
+    if (n + G < items) fetch(n + G);
+    if (!pair) {
+      const int k0 = (n - count) * C;
+      for (int x = tid; x < C * C; x += ROWS_THREADS) {
+        const int k = x / C, i = x % C;
+        const int dist = rev ? L - 1 - (tile * C + i) : tile * C + i + 1;
+        gm.w[k][i] = dist >= 0 && dist <= L ? sm.a[i][k0 + k] * sm.dtab[dist] : 0.f;
+      }
+    } else if (state) {
       for (int x = tid; x < C * C; x += ROWS_THREADS) {
         const int j = x / C, i = x % C, t = jt * C + j;
-        sm.w[j][i] = t < L ? sm.b[j][tile * C + i] * sm.dtab[rev ? t + 1 : L - 1 - t] : 0.f;
+        gm.w[j][i] = t < L ? gm.b[j][tile * C + i] * sm.dtab[rev ? t + 1 : L - 1 - t] : 0.f;
       }
     } else {
       // scores: a thread has rows i2, i2 + 1 and columns jc + 8 x
@@ -517,7 +533,7 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
 #pragma unroll
         for (int r = 0; r < 2; ++r) av[r] = *reinterpret_cast<const float4*>(&sm.a[i2 + r][k]);
 #pragma unroll
-        for (int x = 0; x < 4; ++x) bv[x] = *reinterpret_cast<const float4*>(&sm.b[jc + 8 * x][k]);
+        for (int x = 0; x < 4; ++x) bv[x] = *reinterpret_cast<const float4*>(&gm.b[jc + 8 * x][k]);
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -535,48 +551,64 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
           const int i = i2 + r, j = jc + 8 * x;
           const int dist = rev ? (jt - tile) * C + j - i : (tile - jt) * C + i - j;
           // a select, not a multiply by zero: masked-out tokens can never leak
-          sm.w[j][i] = dist >= 0 && jt * C + j < L ? s[r][x] * sm.dtab[min(dist, L)] : 0.f;
+          gm.w[j][i] = dist >= 0 && jt * C + j < L ? s[r][x] * sm.dtab[min(dist, L)] : 0.f;
         }
     }
+    group_sync<G>(grp);
+    // acc += w^T t over 32 rows; a thread has rows i4 .. i4 + 3 and columns e0 .. e0 + 3 (d = 128: and 64 + those)
+#pragma unroll 4
+    for (int j = 0; j < C; ++j) {
+      const float4 w = *reinterpret_cast<const float4*>(&gm.w[j][i4]);
+      const float wr[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int g = 0; g < EM / 4; ++g) {
+        const float4 t = *reinterpret_cast<const float4*>(&gm.t[j][e0 + 64 * g]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          acc[r][4 * g + 0] = fmaf(wr[r], t.x, acc[r][4 * g + 0]);
+          acc[r][4 * g + 1] = fmaf(wr[r], t.y, acc[r][4 * g + 1]);
+          acc[r][4 * g + 2] = fmaf(wr[r], t.z, acc[r][4 * g + 2]);
+          acc[r][4 * g + 3] = fmaf(wr[r], t.w, acc[r][4 * g + 3]);
+        }
+      }
+    }
+    group_sync<G>(grp);
+  }
+  if (G > 1) {
+    // the groups' sums, in order, through their own tiles
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int g = 0; g < EM / 4; ++g)
+        if (grp > 0)
+          *reinterpret_cast<float4*>(&gm.t[i4 + r][e0 + 64 * g]) = make_float4(acc[r][4 * g], acc[r][4 * g + 1], acc[r][4 * g + 2], acc[r][4 * g + 3]);
     __syncthreads();
-    accumulate();
-    __syncthreads();
-    if (!more) break;
+    if (grp > 0) return;
+    for (int x = 1; x < G && x < items; ++x)
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int g = 0; g < EM / 4; ++g) {
+          const float4 v = *reinterpret_cast<const float4*>(&sm.group[x].t[i4 + r][e0 + 64 * g]);
+          acc[r][4 * g + 0] += v.x; acc[r][4 * g + 1] += v.y; acc[r][4 * g + 2] += v.z; acc[r][4 * g + 3] += v.w;
+        }
   }
 
   if (state) {
     // state leaving the last segment: lambda^L Z + sum
-    float* dst = args.final_out + (size_t)bh * D * D + (size_t)tile * C * D;
-    const float g = sm.dtab[L];
+    const bool local = args.local_out != nullptr;
+    float* dst = (local ? args.local_out + ((size_t)bh * args.nseg + seg) * D * D : args.final_out + (size_t)bh * D * D) + (size_t)tile * C * D;
+    const float gam = sm.dtab[L];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int gq = 0; gq < EM / 4; ++gq) {
         const size_t at = (size_t)(i4 + r) * D + e0 + 64 * gq;
         float4 z = Z ? *reinterpret_cast<const float4*>(Z + (size_t)tile * C * D + at) : make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(dst + at) = make_float4(fmaf(g, z.x, acc[r][4 * gq]), fmaf(g, z.y, acc[r][4 * gq + 1]),
-                                                           fmaf(g, z.z, acc[r][4 * gq + 2]), fmaf(g, z.w, acc[r][4 * gq + 3]));
+        *reinterpret_cast<float4*>(dst + at) = make_float4(fmaf(gam, z.x, acc[r][4 * gq]), fmaf(gam, z.y, acc[r][4 * gq + 1]),
+                                                           fmaf(gam, z.z, acc[r][4 * gq + 2]), fmaf(gam, z.w, acc[r][4 * gq + 3]));
       }
     return;
-  }
-  if (Z) {
-    const int at = tile * C;  // decay of row i to the entry state
-    const float lead = sm.dtab[rev ? max(L - at - C, 0) : at + 1];
-    if (lead != 0.f) {
-      for (int k0 = 0; k0 < D; k0 += C) {
-        float4 nz[D / 16];
-        fetch_tile<float, D>(nz, Z + (size_t)k0 * D, D, C);
-        put_tile<D, D>(sm.t, nz);
-        for (int x = tid; x < C * C; x += ROWS_THREADS) {
-          const int k = x / C, i = x % C;
-          const int dist = rev ? L - 1 - (at + i) : at + i + 1;
-          sm.w[k][i] = dist >= 0 && dist <= L ? sm.a[i][k0 + k] * sm.dtab[dist] : 0.f;
-        }
-        __syncthreads();
-        accumulate();
-        __syncthreads();
-      }
-    }
   }
   TOut* out = static_cast<TOut*>(args.out) + head_off;
 #pragma unroll
@@ -591,16 +623,24 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
   }
 }
 
-template <typename TIn, typename TOut, int D>
-cudaError_t launch_rows_t(const RowsArgs& ra, const DecayTable& tab, cudaStream_t stream) {
-  const size_t smem = sizeof(RowsSmem<D>);
-  auto kern = simt_rows_kernel<TIn, TOut, D>;
+template <typename TIn, typename TOut, int D, int G>
+cudaError_t launch_rows_g(const RowsArgs& ra, const DecayTable& tab, cudaStream_t stream) {
+  const size_t smem = sizeof(RowsSmem<D, G>);
+  auto kern = simt_rows_kernel<TIn, TOut, D, G>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  KernelTimer timer(K_WALK, stream);
-  kern<<<(unsigned)ra.first_block[ROWS_MAX_JOBS], ROWS_THREADS, smem, stream>>>(ra, tab);
+  KernelTimer timer(ra.units[0] ? K_WALK : K_PREPASS, stream);
+  kern<<<(unsigned)ra.first_block[ROWS_MAX_JOBS], ROWS_THREADS * G, smem, stream>>>(ra, tab);
   count_launch();
   return cudaGetLastError();
+}
+// Thread blocks up to which their tiles are shared out over groups: as many as run at once, two or four to a multiprocessor.
+constexpr int rows_groups_limit(int d) { return d == 64 ? 592 : 296; }
+template <typename TIn, typename TOut, int D>
+cudaError_t launch_rows_t(const RowsArgs& ra, const DecayTable& tab, cudaStream_t stream) {
+  constexpr int MANY = D == 64 ? 4 : 2;
+  return ra.first_block[ROWS_MAX_JOBS] <= rows_groups_limit(D) ? launch_rows_g<TIn, TOut, D, MANY>(ra, tab, stream)
+                                                               : launch_rows_g<TIn, TOut, D, 1>(ra, tab, stream);
 }
 template <int D>
 cudaError_t launch_rows_dims(const RowsArgs& ra, const DecayTable& tab, int in_dt, int out_dt, cudaStream_t stream) {
@@ -672,7 +712,7 @@ cudaError_t launch_simt_walk(const OpArgs& args, const DecayTable& tab, int Da, 
   return cudaErrorInvalidValue;
 }
 
-// Up to three independent walks (one launch) whose segments have at most ROWS_MAX_SEG tokens.
+// Up to three independent walks, or the local states of one (local_out), in one launch; segments of at most ROWS_MAX_SEG tokens.
 cudaError_t launch_simt_rows(const OpArgs* jobs, int njobs, const DecayTable& tab, int D, int in_dt, int out_dt,
                              cudaStream_t stream) {
   if (njobs < 1 || njobs > ROWS_MAX_JOBS || (D != 64 && D != 128)) return cudaErrorInvalidValue;
@@ -684,7 +724,8 @@ cudaError_t launch_simt_rows(const OpArgs* jobs, int njobs, const DecayTable& ta
     const OpArgs& a = jobs[j];
     if (a.seg_len > ROWS_MAX_SEG) return cudaErrorInvalidValue;
     const long tiles = (std::min(a.seg_len, a.N) + C - 1) / C;
-    const long rows = (long)a.BH * a.nseg * tiles, states = a.final_out ? (long)a.BH * (D / C) : 0;
+    const long rows = a.local_out ? 0 : (long)a.BH * a.nseg * tiles;
+    const long states = a.local_out ? (long)a.BH * a.nseg * (D / C) : a.final_out ? (long)a.BH * (D / C) : 0;
     ra.job[j] = a;
     ra.job[j].seg_len = (int)std::min((long)a.seg_len, tiles * C);
     ra.units[j] = (int)rows;
@@ -697,6 +738,7 @@ cudaError_t launch_simt_rows(const OpArgs* jobs, int njobs, const DecayTable& ta
 
 cudaError_t launch_simt_prepass(const OpArgs& args, const DecayTable& tab, int Da, int Ec, int in_dt,
                                 cudaStream_t stream) {
+  if (args.seg_len <= ROWS_MAX_SEG) return launch_simt_rows(&args, 1, tab, Da, in_dt, DT_F32, stream);
   if (Da == 64 && Ec == 64) {
     return in_dt == DT_F32 ? launch_prepass_t<float, 64, 64>(args, tab, stream)
                            : launch_prepass_t<__nv_bfloat16, 64, 64>(args, tab, stream);

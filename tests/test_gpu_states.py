@@ -192,3 +192,20 @@ def test_packed_segments_shared_by_clusters(lens):
         got = (part(o), kv[i:i + 1], part(dq), part(dk), part(dv), gin[i:i + 1])
         for name, g, r in zip(("o", "kv", "dq", "dk", "dv", "gin"), got, ref):
             assert_close(g, r, 3.1e-4, "%s of sequence %d" % (name, i))
+
+
+@pytest.mark.parametrize("B,H,N,d", [(8, 16, 200, 64), (8, 8, 200, 128), (1, 1, 31, 64), (1, 1, 480, 128), (1, 5, 1100, 64)])
+def test_full_precision_tiles_shared_by_groups_or_not(B, H, N, d):
+    """Few thread blocks share their tiles out over groups of threads, many do not.  Sums of at most N + d products: (N + d) *
+    2^-24 of the largest partial sum, at most 5 RMS: 3.6e-4."""
+    gen = torch.Generator().manual_seed(N)
+    q, k, v, do = [torch.randn(B, H, N, d, generator=gen) * d ** -0.5 for _ in range(4)]
+    lam = torch.linspace(0.3, 1.0, H)
+    dev = [x.cuda() for x in (q, k, v, do)]
+    o, kv = la.fwd(*dev[:3], lam, want_state=True)
+    grads = la.bwd(*dev, lam)
+    torch.cuda.synchronize()
+    lam64 = lam.double().numpy()
+    ref = tuple(orc.fwd_rec(q, k, v, lam64, want_state=True)) + tuple(orc.bwd_rec(q, k, v, do, lam64))
+    for name, g, r in zip(("o", "kv", "dq", "dk", "dv"), (o, kv) + tuple(grads), ref):
+        assert_close(g, r, 3.6e-4, name)
