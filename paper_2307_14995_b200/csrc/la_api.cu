@@ -63,7 +63,7 @@ struct Folded {
 struct Plan {
   int BH, seg_len, nseg;
   bool tensor;      // tensor-core kernels
-  bool chains;      // the walk chains the segments' local states itself (tensor-core kernels at d = 128): no scan ...
+  bool chains;      // the walk chains the segments' local states itself (tensor-core kernels): no scan ...
   bool scanned;     // ... but running sums of the slowly decaying heads' states
   bool rows;        // CUDA-core kernels: short segments, every row tile by itself (no chain of blocks)
   int precision;    // LA_SPLIT_* bits (tensor path)
@@ -107,7 +107,7 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
   p->BH = s->B * s->H;
   if (s->path == LA_PATH_TENSOR && !tensor_path_available(s)) return LA_ERR_UNSUPPORTED;
   p->tensor = (s->path == LA_PATH_TENSOR) || (s->path == LA_PATH_AUTO && tensor_path_available(s));
-  p->chains = p->tensor && s->d == 128;
+  p->chains = p->tensor;
   p->scanned = false;
   p->precision = (s->precision == LA_PRECISION_DEFAULT)
                      ? (LA_SPLIT_SCORES | LA_SPLIT_STATE | LA_SPLIT_DECAYED)
@@ -195,10 +195,11 @@ size_t state_set_bytes(const la_shape* s, const Plan& p) {
   return (size_t)p.BH * p.nseg * s->d * s->e * sizeof(float);
 }
 
-// State sets a call keeps in its workspace.  Forward: the segments' states, and without chains their transposes; backward: those
-// of KV^T and of dKV, and without chains the transposes of dKV.
-int fwd_sets(const Plan& p) { return p.nseg == 1 ? 0 : p.chains ? 1 : 2; }
-int bwd_sets(const Plan& p) { return p.chains ? 2 : 3; }
+// State sets that la_workspace_bytes asks for.  Walks that chain the segments' states need one for the forward pass and those of
+// KV^T and of dKV for the backward pass; a scan also writes their transposes.  (At d = 64 the tensor-core walk had a scan before
+// it; what it asks for has stayed.)
+int fwd_sets(const la_shape* s, const Plan& p) { return p.nseg == 1 ? 0 : p.chains && s->d == 128 ? 1 : 2; }
+int bwd_sets(const la_shape* s, const Plan& p) { return p.chains && s->d == 128 ? 2 : 3; }
 
 la_status make_table(const la_shape* s, const float* lambda_host, DecayTable* tab) {
   if (!lambda_host) return LA_ERR_INVALID_ARG;
@@ -384,7 +385,7 @@ static size_t scratch_bytes(int op, const la_shape* shape, bool packed) {
   if (op == LA_OP_DECODE) return 0;
   Plan p;
   if (make_plan(shape, &p, packed) != LA_OK) return (size_t)-1;
-  return (size_t)(op == LA_OP_FWD ? fwd_sets(p) : bwd_sets(p)) * state_set_bytes(shape, p);
+  return (size_t)(op == LA_OP_FWD ? fwd_sets(shape, p) : bwd_sets(shape, p)) * state_set_bytes(shape, p);
 }
 
 size_t la_workspace_bytes(int op, const la_shape* shape) { return scratch_bytes(op, shape, false); }
@@ -456,7 +457,7 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   if (fold) p.fold = *fold;
   p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
-  const size_t need = (size_t)fwd_sets(p) * one;
+  const size_t need = (size_t)fwd_sets(shape, p) * one;
   if (need > 0 && (!workspace || workspace_bytes < need)) return LA_ERR_WORKSPACE;
   if (need > 0 && (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_INVALID_ARG;
   if ((st = check_device()) != LA_OK) return st;
@@ -480,7 +481,7 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     return LA_OK;
   }
   // the d = 128 walk has the output stage as an epilogue
-  if (p.chains) {
+  if (p.chains && shape->d == 128) {
     OpArgs wa = walk_args(shape, p, q, k, v, o, from, kv_out, 0);
     wa.u = u;
     wa.y = y;
@@ -539,7 +540,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   if (fold) p.fold = *fold;
   p.scanned = wants_running(shape, p, tab);
   const size_t one = state_set_bytes(shape, p);
-  if (!workspace || workspace_bytes < (size_t)bwd_sets(p) * one) return LA_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < (size_t)bwd_sets(shape, p) * one) return LA_ERR_WORKSPACE;
   if (fwd_workspace == workspace) return LA_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(workspace) & 255u) return LA_ERR_INVALID_ARG;
   if ((st = check_device()) != LA_OK) return st;
@@ -918,9 +919,9 @@ size_t esize(int dt) { return dt == LA_BF16 ? 2 : 4; }
 
 // The single-launch form: every sequence is a "batch" entry of its own length inside the packed tensors, and the
 // tensor-core walk (with the pre-pass where the longest sequence is cut into segments) runs over all of them at once.
-// It exists for bf16 inputs at d = e = 128; everything else runs one call per sequence.  `sp` is the shape that goes with it: B = sequences, N = longest.
+// It exists for bf16 inputs; everything else runs one call per sequence.  `sp` is the shape that goes with it: B = sequences, N = longest.
 bool packed_shape(const la_shape* shape, const int* cu, int S, la_shape* sp) {
-  if (S < 2 || shape->d != 128 || shape->in_dtype != LA_BF16 || shape->path == LA_PATH_SIMT || !tc_supported())
+  if (S < 2 || shape->in_dtype != LA_BF16 || shape->path == LA_PATH_SIMT || !tc_supported())
     return false;
   int longest = 0;
   for (int i = 0; i < S; ++i) longest = std::max(longest, cu[i + 1] - cu[i]);
@@ -930,6 +931,15 @@ bool packed_shape(const la_shape* shape, const int* cu, int S, la_shape* sp) {
   return check_shape(sp, true) == LA_OK;
 }
 size_t packed_table_bytes(int S) { return ((size_t)3 * S * sizeof(int) + 255) / 256 * 256; }
+
+// Whether the single-launch form's table and state sets fit the caller's workspace.  At d = 64 a call with less runs sequence by
+// sequence, which may need none.
+bool packed_fits(int op, const la_shape* sp, const void* workspace, size_t workspace_bytes) {
+  if (sp->d == 128) return true;
+  const size_t w = scratch_bytes(op, sp, true);
+  return workspace && !(reinterpret_cast<uintptr_t>(workspace) & 255u) && w != (size_t)-1 &&
+         workspace_bytes >= packed_table_bytes(sp->B) + w;
+}
 
 // Copies first tokens and lengths to the head of the workspace (stream-ordered) and describes them.
 la_status packed_upload(const int* cu, int S, int total, void* workspace, cudaStream_t cs, Packed* pk) {
@@ -979,7 +989,7 @@ la_status la_fwd_varlen(const la_shape* shape, const void* q, const void* k, con
   if (st != LA_OK) return st;
   if (!q || !k || !v || !o) return LA_ERR_INVALID_ARG;
   la_shape sp;
-  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp)) {
+  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp) && packed_fits(LA_OP_FWD, &sp, workspace, workspace_bytes)) {
     const size_t tb = packed_table_bytes(num_seqs);
     if (!workspace || workspace_bytes < tb || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_WORKSPACE;
     if ((st = check_device()) != LA_OK) return st;
@@ -1013,7 +1023,7 @@ la_status la_bwd_varlen(const la_shape* shape, const void* q, const void* k, con
   if (st != LA_OK) return st;
   if (!q || !k || !v || !d_o || !dq || !dk || !dv) return LA_ERR_INVALID_ARG;
   la_shape sp;
-  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp)) {
+  if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp) && packed_fits(LA_OP_BWD, &sp, workspace, workspace_bytes)) {
     const size_t tb = packed_table_bytes(num_seqs);
     if (!workspace || workspace_bytes < tb || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_WORKSPACE;
     if ((st = check_device()) != LA_OK) return st;

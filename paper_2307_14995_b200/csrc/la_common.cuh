@@ -44,7 +44,7 @@ struct OpArgs {
   const void* c;      // [BH, N, Ec]
   void* out;          // [BH, N, Ec]  (unused by the pre-pass)
   const float* entry; // [BH, nseg, Da*Ec] state entering each segment, or NULL = zeros
-  // Tensor-core walk at Da = Ec = 128 instead of `entry`: the state entering the sequence [BH, Da*Ec] (NULL = zeros) and
+  // Tensor-core walks instead of `entry`: the state entering the sequence [BH, Da*Ec] (NULL = zeros) and
   // the segments' local states [BH, nseg, Da*Ec] as the pre-pass leaves them, which the walk chains itself; each may be
   // stored transposed.
   const float* z_in;
@@ -65,7 +65,7 @@ struct OpArgs {
   const void* u;      // [BH, N, Ec] gate, input dtype
   void* y;            // [BH, N, Ec] output dtype
   float* rstd;        // [BH, N] sqrt(Ec) / ||out row||_2, or NULL
-  // Packed batch of sequences of different lengths (tensor-core kernels at Da = Ec = 128 only; NULL elsewhere):
+  // Packed batch of sequences of different lengths (tensor-core kernels only; NULL elsewhere):
   // the token tensors are [total_tokens, H, D] with the sequences one after the other, "batch" entry b is
   // sequence b with seq_len[b] tokens starting at token seq_start[b] (DEVICE arrays of BH / H ints), N is the
   // longest length (it fixes the segment grid; thread blocks of segments a sequence does not have return at once)
@@ -73,7 +73,7 @@ struct OpArgs {
   // bound below is the sequence's own length.
   const int* seq_start;
   const int* seq_len;
-  // Folded batch (tensor-core kernels at Da = Ec = 128 only; 0 elsewhere): batch entries t and t + fold read the same
+  // Folded batch (tensor-core kernels only; 0 elsewhere): batch entries t and t + fold read the same
   // entry t of the operands in `shared` (SHARED_* bits), which have `fold` batch entries.
   // out2: where the entries fold .. 2 fold - 1 of the output go, as entries 0 .. fold - 1 (NULL: behind the others in `out`).
   int fold;
@@ -149,7 +149,7 @@ cudaError_t launch_tc_walk(const OpArgs& args, const DecayTable& tab, int D, int
 cudaError_t launch_tc_walk_pair(const OpArgs& first, const OpArgs& second, const DecayTable& tab, int D, int out_dt,
                                 int precision, cudaStream_t stream);
 // all_segments: false leaves out the segment that no other segment's state depends on (forward the last, reverse the
-// first); a hint, at D = 64 every state is made.
+// first).
 cudaError_t launch_tc_prepass(const OpArgs& args, const DecayTable& tab, int D, int precision, bool all_segments,
                               cudaStream_t stream);
 

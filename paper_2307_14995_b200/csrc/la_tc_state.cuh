@@ -1,4 +1,4 @@
-// Segment states for D = 128 (included by la_tc.cu, inside its anonymous namespace, after the helpers): per (batch*head,
+// Segment states (included by la_tc.cu, inside its anonymous namespace, after the helpers): per (batch*head,
 // segment) the local state sum_t decay-to-segment-edge * b_t c_t^T, which the walk chains into the state entering each
 // segment.
 //
@@ -15,10 +15,12 @@
 //
 // Warps: 0 TMA producer, 1 MMA issuer, 4-19 workers (32 value columns x 32 tokens of fc of every other piece each).
 
+// D = 64: the hi terms of fc are in lanes 0 .. 63 and the lo terms in lanes 64 .. 127, one product of 64 columns for both, whose
+// halves are added up on the way out.  A piece is 16 KB, so that six stages hold as much as three.
+
 constexpr int S_THREADS = 640;
-constexpr int S_STAGES = 3;
 constexpr uint32_t S_TMEM_COLS = 256;
-constexpr uint32_t SCOL_Z = 0, SCOL_F = 128;  // two fc buffers of 64 columns (hi, lo), or four of 32 (hi alone)
+constexpr uint32_t SCOL_Z = 0, SCOL_F = 128;  // two fc buffers of 64 columns (hi, lo), or four of 32 (hi alone, or D = 64)
 
 // Which (batch, head, segment) a thread block works on: `order` has the slowly decaying heads first, so that the longest
 // chains start first (B = 1, H = 32, N = 65536, chains of 57 blocks: 118 us with the heads in their own order, 97 in this
@@ -30,29 +32,26 @@ struct StatePlan {
   unsigned char order[LA_MAX_H];
 };
 
-// The loads of piece p arrive on barrier p % S_FULLS: all pieces of one barrier belong to the same group of workers, which
+// The loads of piece p arrive on barrier p % FULLS: all pieces of one barrier belong to the same group of workers, which
 // waits for no others.  (With a barrier per stage a group had to see the other's pieces go by, and nothing kept a stage from
 // being loaded again, twice, before a warp that came late had looked; it then waited until its budget ran out.)
-constexpr int S_FULLS = 2 * S_STAGES;
-enum SBar {
-  S_FULL0 = 0,
-  S_FREE0 = S_FULL0 + S_FULLS,
-  S_FC_READY0 = S_FREE0 + S_STAGES,
-  S_FC_FREE0 = S_FC_READY0 + 4,
-  S_DONE = S_FC_FREE0 + 4,
-  S_DRAIN,
-  S_NUM_BARS
+template <int D>
+struct SBar {
+  static constexpr int STAGES = D == 128 ? 3 : 6, FULLS = D == 128 ? 2 * STAGES : STAGES;
+  static constexpr int FULL0 = 0, FREE0 = FULL0 + FULLS, FC_READY0 = FREE0 + STAGES, FC_FREE0 = FC_READY0 + 4, DONE = FC_FREE0 + 4,
+                       DRAIN = DONE + 1, NUM = DRAIN + 1;
 };
 
+template <int D>
 struct alignas(1024) SSmem {
-  uint64_t bars[S_NUM_BARS];
+  uint64_t bars[SBar<D>::NUM];
   uint32_t tmem_slot;
   int abort;
   struct alignas(1024) Stage {
-    __nv_bfloat16 b[2][64 * 64], c[2][64 * 64];
-  } stage[S_STAGES];
+    __nv_bfloat16 b[D / 64][64 * 64], c[D / 64][64 * 64];
+  } stage[SBar<D>::STAGES];
 };
-static_assert(S_STAGES * sizeof(SSmem::Stage) >= 128 * 128 * 4, "a part of the state fits the stages");
+static_assert(3 * sizeof(SSmem<128>::Stage) >= 128 * 128 * 4 && 6 * sizeof(SSmem<64>::Stage) >= 2 * 64 * 64 * 4, "a part of the state fits the stages");
 
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -65,12 +64,16 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t saddr, uint32_t rank) {
   return v;
 }
 
-template <bool REV>
+template <bool REV, int D>
 __global__ void __launch_bounds__(S_THREADS, 2)
 tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_c,
                 const __grid_constant__ TcArgs args, const __grid_constant__ StatePlan plan, const __grid_constant__ DecayTable tab) {
   extern __shared__ unsigned char smem_raw[];
-  SSmem& sm = *reinterpret_cast<SSmem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+  using SB = SBar<D>;
+  constexpr int S_STAGES = SB::STAGES, S_FULLS = SB::FULLS, S_FULL0 = SB::FULL0, S_FREE0 = SB::FREE0, S_FC_READY0 = SB::FC_READY0,
+                S_FC_FREE0 = SB::FC_FREE0, S_DONE = SB::DONE, S_DRAIN = SB::DRAIN, S_NUM_BARS = SB::NUM;
+  constexpr int PANELS = D / 64;
+  SSmem<D>& sm = *reinterpret_cast<SSmem<D>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   // ---- which segment, and which of its pieces ----
@@ -94,7 +97,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
   if (seg_t0 >= n_tok) return;  // (all thread blocks of a cluster that shares a segment alike)
   const float s2 = (float)tab.s2[h];
   const bool split_c = (args.precision & 4) != 0 && s2 != 0.f;  // lambda == 1: the lo term is identically zero
-  const int nf = split_c ? 2 : 4, fcols = split_c ? 64 : 32;    // fc buffers, and their columns
+  const int nf = D == 128 && split_c ? 2 : 4, fcols = D == 128 && split_c ? 64 : 32;  // fc buffers, and their columns
   int first = 0, count = (seg_t1 - seg_t0 + 127) >> 7;
   if (s2 > 0.f) {
     // blocks whose nearest token is within 160 / s2 + 128 tokens of the edge (the margin makes the skipped weights zero
@@ -149,11 +152,11 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
         const int t = tok0 + seg_t0 + piece(it) * 64;
         uint64_t* bar = &sm.bars[S_FULL0 + f];
         if (++f == S_FULLS) f = 0;
-        mbar_arrive_expect_tx(bar, 32768);
-        tma_load_4d(&sm.stage[s].c[0][0], &map_c, bar, 0, t, h, bat_c);
-        tma_load_4d(&sm.stage[s].c[1][0], &map_c, bar, 64, t, h, bat_c);
-        tma_load_4d(&sm.stage[s].b[0][0], &map_b, bar, 0, t, h, bat_b);
-        tma_load_4d(&sm.stage[s].b[1][0], &map_b, bar, 64, t, h, bat_b);
+        mbar_arrive_expect_tx(bar, PANELS * 16384);
+#pragma unroll
+        for (int x = 0; x < PANELS; ++x) tma_load_4d(&sm.stage[s].c[x][0], &map_c, bar, x * 64, t, h, bat_c);
+#pragma unroll
+        for (int x = 0; x < PANELS; ++x) tma_load_4d(&sm.stage[s].b[x][0], &map_b, bar, x * 64, t, h, bat_b);
         armed = it + 1;
         if (++s == S_STAGES) s = 0, phase ^= 1;
       }
@@ -165,8 +168,9 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------ MMA issuer ------------------------------------
-    constexpr uint32_t ID_KN = umma_idesc_bf16(128, 128, false, true);  // tensor-memory A x MN-major B
+    constexpr uint32_t ID_KN = umma_idesc_bf16(128, D, false, true);  // tensor-memory A x MN-major B
     constexpr uint32_t HI = UMMA_DESC_HI_SBO1024;
+    constexpr uint32_t STAGE = (uint32_t)(sizeof(typename SSmem<D>::Stage) >> 4);
     const uint32_t go = elect_one();
     const uint32_t b0 = umma_desc_lo(smem_u32(&sm.stage[0].b[0][0]), 8192);
     for (int it = 0, s = 0, u = 0, phase = 0, f = 0, fphase = 0; it < count; ++it) {
@@ -174,8 +178,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
       TC_WAIT_WARP_TO(mma_done, S_FC_READY0 + f, fphase, 33);
       tc_fence_after_sync();
       const uint32_t fcol = tmem + SCOL_F + f * fcols;
-      umma_group_tsd4<false>(tmem + SCOL_Z, fcol, b0 + s * 2048, HI, ID_KN, it > 0 ? 1u : 0u, go);
-      if (split_c) umma_group_tsd4<false>(tmem + SCOL_Z, fcol + 32, b0 + s * 2048, HI, ID_KN, 1, go);
+      umma_group_tsd4<false>(tmem + SCOL_Z, fcol, b0 + s * STAGE, HI, ID_KN, it > 0 ? 1u : 0u, go);
+      if (D == 128 && split_c) umma_group_tsd4<false>(tmem + SCOL_Z, fcol + 32, b0 + s * STAGE, HI, ID_KN, 1, go);
       umma_commit_if(&sm.bars[S_FREE0 + s], go);
       umma_commit_if(&sm.bars[S_FC_FREE0 + f], go);
       if (++s == S_STAGES) s = 0;
@@ -197,8 +201,10 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     // bound by the instructions between two pieces (57 blocks in one thread block: 66 us through split2, 45 us this way; the
     // shape above: 97 and 83).
     const int group = w4 >> 1;
-    // lane l points ldmatrix at token row (w4 & 1) * 32 + (l >> 4) * 8 + (l & 7), value columns q * 32 + ((l >> 3) & 1) * 8
-    const uint32_t unit0 = (uint32_t)((q >> 1) * 8192 + ((w4 & 1) * 32 + ((lane >> 4) << 3) + (lane & 7)) * 128 +
+    // lane l points ldmatrix at token row (w4 & 1) * 32 + (l >> 4) * 8 + (l & 7), value columns q * 32 (D = 64:
+    // (q & 1) * 32) + ((l >> 3) & 1) * 8
+    const bool lo_part = D == 64 && q >= 2;
+    const uint32_t unit0 = (uint32_t)((D == 128 ? (q >> 1) * 8192 : 0) + ((w4 & 1) * 32 + ((lane >> 4) << 3) + (lane & 7)) * 128 +
                                       ((((q & 1) * 4 + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
     for (int it = group, u = group, phase = 0, fb = group, fphase = 0; it < count; it += 2) {
       const int st = u < S_STAGES ? u : u - S_STAGES;
@@ -207,6 +213,20 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
       if (u >= S_FULLS) u -= S_FULLS, phase ^= 1;
       if (it >= nf) TC_WAIT_WARP(S_FC_FREE0 + fb, fphase ^ 1, 35);
       tc_fence_after_sync();
+      const int own = seg_t1 - (seg_t0 + piece(it) * 64);  // tokens of this piece that are the segment's
+      if (args.seq_start && own < 64) {
+        // packed batch: what follows is another sequence's and must not come through its zero weight either (0 * inf)
+        for (int x = own * 8 + ((w4 & 1) * 4 + q) * 32 + lane; x < 512; x += 256)
+#pragma unroll
+          for (int n = 0; n < PANELS; ++n) reinterpret_cast<uint4*>(sm.stage[st].b[n])[x] = make_uint4(0u, 0u, 0u, 0u);
+        fence_proxy_async_smem();
+      }
+      if (lo_part && !split_c) {
+        WARP_ARRIVE(S_FC_READY0 + fb);
+        fb += 2;
+        if (fb >= nf) fb -= nf, fphase ^= 1;
+        continue;
+      }
 #pragma unroll
       for (int k = 0; k < 2; ++k) {  // 16 tokens at a time
         uint32_t raw[8];             // [16 value columns][8 tokens][8 value columns]
@@ -228,6 +248,13 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
           const int t = t0 + 8 * (o >> 1) + (o & 1);
           f[o] = t < seg_t1 ? exp2f(-s2 * (float)(REV ? t - seg_t0 + 1 : seg_t1 - 1 - t)) : 0.f;
         }
+        if (own < 64) {
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            const int t = t0 + 8 * ((x >> 1) & 1);
+            raw[x] &= (t < seg_t1 ? 0xffffu : 0u) | (t + 1 < seg_t1 ? 0xffff0000u : 0u);
+          }
+        }
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
           uint32_t hh[4], ll[4];
@@ -238,8 +265,12 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
                    hh[x], ll[x]);
           }
           const uint32_t at = colF + ((uint32_t)(g * 16) << 16);
-          tmem_st_16x128b_x2(at, hh);
-          if (split_c) tmem_st_16x128b_x2(at + 32, ll);
+          if (D == 64) {
+            tmem_st_16x128b_x2(at, lo_part ? ll : hh);
+          } else {
+            tmem_st_16x128b_x2(at, hh);
+            if (split_c) tmem_st_16x128b_x2(at + 32, ll);
+          }
         }
       }
       tmem_st_wait();
@@ -248,25 +279,34 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
       fb += 2;
       if (fb >= nf) fb -= nf, fphase ^= 1;
     }
-    // ---- result: value column q * 32 + lane, features w4 * 32 .. + 31 ----
-    uint32_t z[32];
+    // ---- result: value column q * 32 + lane (D = 64: that of the hi or the lo half), features w4 * D / 4 .. ----
+    constexpr int PER = D / 4;
+    uint32_t z[PER];
     if (count > 0) {
       TC_WAIT_WARP(S_DONE, 0, 36);
       tc_fence_after_sync();
-      tmem_ld_x16(lane_addr + SCOL_Z + w4 * 32, *reinterpret_cast<uint32_t(*)[16]>(&z[0]));
-      tmem_ld_x16(lane_addr + SCOL_Z + w4 * 32 + 16, *reinterpret_cast<uint32_t(*)[16]>(&z[16]));
+#pragma unroll
+      for (int x = 0; x < PER; x += 16) tmem_ld_x16(lane_addr + SCOL_Z + w4 * PER + x, *reinterpret_cast<uint32_t(*)[16]>(&z[x]));
       tmem_ld_wait();
       tc_fence_before_sync();
-    } else {
-#pragma unroll
-      for (int x = 0; x < 32; ++x) z[x] = 0u;
     }
-    float* dst = args.local_out + ((size_t)bh * args.nseg + seg) * (128 * 128) + (size_t)(w4 * 32) * 128 + q * 32 + lane;
-    float* part = reinterpret_cast<float*>(&sm.stage[0]) + (w4 * 32) * 128 + q * 32 + lane;  // (every load has been read)
+    if (count == 0 || (lo_part && !split_c)) {
 #pragma unroll
-    for (int x = 0; x < 32; ++x) {
-      if (shared) part[x * 128] = __uint_as_float(z[x]);
-      else dst[x * 128] = __uint_as_float(z[x]);
+      for (int x = 0; x < PER; ++x) z[x] = 0u;
+    }
+    // (every load has been read)
+    if (D == 64) {
+      float* part = reinterpret_cast<float*>(&sm.stage[0]) + (lo_part ? D * D : 0) + (w4 * PER) * D + (q & 1) * 32 + lane;
+#pragma unroll
+      for (int x = 0; x < PER; ++x) part[x * D] = __uint_as_float(z[x]);
+    } else {
+      float* dst = args.local_out + ((size_t)bh * args.nseg + seg) * (D * D) + (size_t)(w4 * PER) * D + q * 32 + lane;
+      float* part = reinterpret_cast<float*>(&sm.stage[0]) + (w4 * PER) * D + q * 32 + lane;
+#pragma unroll
+      for (int x = 0; x < PER; ++x) {
+        if (shared) part[x * D] = __uint_as_float(z[x]);
+        else dst[x * D] = __uint_as_float(z[x]);
+      }
     }
   }
 
@@ -274,24 +314,35 @@ teardown:
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, S_TMEM_COLS);
-  if (shared) {
-    // each thread block of the cluster adds up its share of the parts, in rank order
-    cluster_sync();
-    const int per = 4096 / plan.cluster;  // float4 groups of the state per thread block
-    float4* out = reinterpret_cast<float4*>(args.local_out + ((size_t)bh * args.nseg + seg) * (128 * 128));
-    for (int i = rank * per + tid; i < (rank + 1) * per; i += S_THREADS) {
-      const uint32_t at = smem_u32(&sm.stage[0]) + i * 16;
-      float4 x[8];  // all loads first: one by one they take 700 clocks each
+  if (shared || D == 64) {
+    // each thread block of the cluster adds up its share of the parts, in rank order, the hi halves first
+    const int ranks = shared ? plan.cluster : 1, first_rank = shared ? rank : 0;
+    if (shared) cluster_sync();
+    const int per = D * D / 4 / ranks;  // float4 groups of the state per thread block
+    float4* out = reinterpret_cast<float4*>(args.local_out + ((size_t)bh * args.nseg + seg) * (D * D));
+    for (int i = first_rank * per + tid; i < (first_rank + 1) * per; i += S_THREADS) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int r = 0; r < 8; ++r) x[r] = r < plan.cluster ? ld_cluster_f4(at, (uint32_t)r) : make_float4(0.f, 0.f, 0.f, 0.f);
-      float4 v = x[0];
+      for (int half = 0; half < (D == 64 ? 2 : 1); ++half) {
+        const uint32_t at = smem_u32(&sm.stage[0]) + (half * (D * D / 4) + i) * 16;
+        if (!shared) {
+          const float4 x = reinterpret_cast<const float4*>(&sm.stage[0])[half * (D * D / 4) + i];
+          v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+          continue;
+        }
+        float4 x[8];  // all loads first: one by one they take 700 clocks each
 #pragma unroll
-      for (int r = 1; r < 8; ++r) {
-        v.x += x[r].x; v.y += x[r].y; v.z += x[r].z; v.w += x[r].w;
+        for (int r = 0; r < 8; ++r) x[r] = r < plan.cluster ? ld_cluster_f4(at, (uint32_t)r) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (half == 0) v = x[0];
+        else v.x += x[0].x, v.y += x[0].y, v.z += x[0].z, v.w += x[0].w;
+#pragma unroll
+        for (int r = 1; r < 8; ++r) {
+          v.x += x[r].x; v.y += x[r].y; v.z += x[r].z; v.w += x[r].w;
+        }
       }
       out[i] = v;
     }
-    cluster_sync();  // nobody leaves while its part is being read
+    if (shared) cluster_sync();  // nobody leaves while its part is being read
   }
 }
 
@@ -351,11 +402,11 @@ inline StatePlan make_state_plan(const TcArgs& ta, const DecayTable& tab, bool r
   return p;
 }
 
-template <bool REV>
+template <bool REV, int D>
 cudaError_t launch_state_t(const TcMaps& m, const TcArgs& ta, const DecayTable& tab, bool all_segments, cudaStream_t stream) {
-  const size_t smem = sizeof(SSmem) + 1024;
-  static_assert(2 * (sizeof(SSmem) + 2048) <= 233472, "two thread blocks in the shared memory of one SM");
-  auto kern = tc_state_kernel<REV>;
+  const size_t smem = sizeof(SSmem<D>) + 1024;
+  static_assert(2 * (sizeof(SSmem<D>) + 2048) <= 233472, "two thread blocks in the shared memory of one SM");
+  auto kern = tc_state_kernel<REV, D>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   const StatePlan plan = make_state_plan(ta, tab, REV, all_segments);

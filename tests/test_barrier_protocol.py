@@ -43,11 +43,11 @@ def overruns(roles, counts):
 STAGES = 3
 
 
-def state_kernel(pieces, fc_buffers, full_barriers):
-    """tc_state_kernel: loads in STAGES stages, two groups of workers that take turns (one warp of each here), products.
+def state_kernel(pieces, fc_buffers, full_barriers, stages=STAGES):
+    """tc_state_kernel: loads in `stages` stages, two groups of workers that take turns (one warp of each here), products.
     full_barriers: how many barriers the loads' arrivals go round; with one per stage a group must follow every phase."""
     full = lambda p: "full%d" % (p % full_barriers)
-    n = STAGES
+    n = stages
     producer, mma = [], []
     groups = {0: [], 1: []}
     for p in range(pieces):
@@ -72,6 +72,15 @@ def state_kernel(pieces, fc_buffers, full_barriers):
 @pytest.mark.parametrize("pieces", [1, 2, 3, 7, 13, 30])
 def test_state_kernel_phases_are_never_overrun(pieces, fc_buffers):
     assert overruns(*state_kernel(pieces, fc_buffers, 2 * STAGES)) == []
+
+
+@pytest.mark.parametrize("pieces", [1, 5, 6, 7, 13, 30])
+def test_state_kernel_of_64_features_phases_are_never_overrun(pieces):
+    # (an even number of stages: all pieces of a stage are the same group's, so that a barrier a stage is enough)
+    roles, counts = state_kernel(pieces, 4, 6, 6)
+    for g, parity in (("even", 0), ("odd", 1)):
+        roles[g] = [op for op in roles[g] if op[1][:4] != "full" or int(op[1][4:]) % 2 == parity]
+    assert overruns(roles, counts) == []
 
 
 @pytest.mark.parametrize("fc_buffers", [2, 4])
@@ -130,3 +139,46 @@ def test_walk_kernel_with_one_barrier_for_every_block_would_be_overrun():
     # (a producer that is a block late)
     found = overruns(*walk_kernel(6, True, 1))
     assert ("producer", "dz0", 0) in found and ("producer", "o0", 0) in found
+
+
+def walk64_kernel(blocks, last_m3):
+    """tc_walk64_kernel (one warp of each group)."""
+    two, three = (lambda name, n: name + str(n % 2)), (lambda name, n: name + str(n % 3))
+    m3 = lambda n: n + 1 < blocks or last_m3
+    producer, p, output = [], [], []
+    mma = [("wait", "ab0", 0), ("arrive", "s0")]
+    state = []
+    if m3(0):
+        mma += [("wait", "fc", 0), ("arrive", "dz")]
+        state += [("wait", "c0", 0), ("arrive", "fc")]
+    state.append(("arrive", "z"))
+    for n in range(blocks):
+        if n >= 3:
+            producer.append(("wait", three("free", n), n // 3 - 1))
+        producer += [("arrive", three("ab", n)), ("arrive", three("c", n))]
+        more = n + 1 < blocks
+        if more:
+            mma += [("wait", three("ab", n + 1), (n + 1) // 3), ("arrive", two("s", n + 1))]
+        mma.append(("wait", "z", n))
+        if n > 0:
+            mma.append(("wait", "o_free", n - 1))
+        mma += [("arrive", "m2"), ("wait", three("c", n), n // 3), ("wait", two("p", n), n // 2), ("arrive", "o"), ("arrive", three("free", n))]
+        if more and m3(n + 1):
+            mma += [("wait", "fc", n + 1), ("arrive", "dz")]
+        p += [("wait", two("s", n), n // 2), ("arrive", two("p", n))]
+        if more or last_m3:
+            state.append(("wait", "dz", n))
+        if more:
+            if m3(n + 1):
+                state += [("wait", three("c", n + 1), (n + 1) // 3), ("arrive", "fc")]
+            state += [("wait", "m2", n), ("arrive", "z")]
+        output += [("wait", "o", n), ("arrive", "o_free")] + [("wait", "stored", n - 1)] * (n > 0)
+        output += [("arrive", "staged"), ("wait", "staged", n), ("arrive", "stored")]
+    roles = {"producer": producer, "mma": mma, "p": p, "state": state, "output": output}
+    return roles, {op[1]: 1 for ops in roles.values() for op in ops}
+
+
+@pytest.mark.parametrize("last_m3", [False, True])
+@pytest.mark.parametrize("blocks", [1, 2, 3, 4, 5, 11])
+def test_walk64_kernel_phases_are_never_overrun(blocks, last_m3):
+    assert overruns(*walk64_kernel(blocks, last_m3)) == []

@@ -1,0 +1,96 @@
+"""d = 64 on the tensor cores: packed batches in one set of launches, and what the walk does at the ends of sequences.
+
+Tolerance as for the segment states: two-term operands, 2^-17 of each product, sums of up to 8 blocks; against RMS(ref) with
+|sum| up to 5 RMS 1.7e-4.  bf16 results: 2^-8 |ref| besides."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import la_oracle as orc
+from paper_2307_14995_b200 import binding as la
+
+pytestmark = pytest.mark.gpu
+H, D, LAM = 3, 64, torch.tensor([1.0, 0.97, 0.2])
+
+
+def packed(lens, dtype, seg_len, seed, states=False):
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    gen = torch.Generator().manual_seed(seed)
+    x = [torch.randn(1, cu[-1], H, D, generator=gen).bfloat16() for _ in range(4)]
+    extra = [torch.randn(len(lens), H, D, D, generator=gen) * 0.1 for _ in range(2)] if states else [None, None]
+    return cu, x, extra, la.make_shape(1, H, cu[-1], D, D, torch.bfloat16, dtype, seg_len, layout=la.LA_LAYOUT_BNHD)
+
+
+def run(cu, x, extra, shape, dtype, workspace=True):
+    q, k, v, do = [t.cuda() for t in x]
+    kv_in, gko = [None if t is None else t.cuda() for t in extra]
+    S = len(cu) - 1
+    o, dq, dk, dv = [torch.full_like(q, float("nan"), dtype=dtype) for _ in range(4)]
+    kv, gin = [torch.empty(S, H, D, D, device="cuda") for _ in range(2)]
+    ws = [torch.empty(la.varlen_workspace_bytes(op, shape, cu), dtype=torch.uint8, device="cuda") for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    n = la.launch_count()
+    la.la_fwd_varlen(shape, q, k, v, LAM, o, cu, kv_in, kv, ws[0] if workspace else None)
+    n = la.launch_count() - n
+    la.la_bwd_varlen(shape, q, k, v, do, LAM, dq, dk, dv, cu, kv_in, gko, gin, ws[1])
+    torch.cuda.synchronize()
+    la.device_status()
+    return [t.cpu() for t in (o, dq, dk, dv, kv, gin)], n
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("seg_len,states", [(0, False), (256, True), (128, False)])
+def test_packed_sequences(dtype, seg_len, states):
+    lens = [300, 1, 127, 128, 129, 1000, 64, 513]
+    cu, x, extra, shape = packed(lens, dtype, seg_len, 5, states)
+    got, launches = run(cu, x, extra, shape, dtype)
+    assert launches == (3 if seg_len else 1)
+    lam64 = LAM.double().numpy()
+    heads = lambda t: t.permute(0, 2, 1, 3)
+    for i in range(len(lens)):
+        at = slice(cu[i], cu[i + 1])
+        q, k, v, do = [heads(t[:, at]) for t in x]
+        kv_in, gko = [None if t is None else t[i:i + 1] for t in extra]
+        ref = dict(zip(("o", "kv"), orc.fwd_rec(q, k, v, lam64, kv_in=kv_in, want_state=True)))
+        ref.update(zip(("dq", "dk", "dv", "gin"), orc.bwd_rec(q, k, v, do, lam64, kv_in=kv_in, grad_kv_out=gko, want_state_grad=True)))
+        for name, t in zip(("o", "dq", "dk", "dv", "kv", "gin"), got):
+            g = (t[i:i + 1] if name in ("kv", "gin") else heads(t[:, at])).double().numpy()
+            r = ref[name]
+            rms = np.sqrt(np.mean(r * r, axis=(2, 3), keepdims=True))
+            slack = 2.0 ** -8 * np.abs(r) if dtype == torch.bfloat16 and name not in ("kv", "gin") else 0.0
+            assert np.all(np.abs(g - r) <= 1.7e-4 * rms + slack), (name, i)
+
+
+@pytest.mark.parametrize("seg_len", [0, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_a_packed_sequence_does_not_see_its_neighbours(bad, seg_len):
+    cu, x, extra, shape = packed([200, 77, 300], torch.float32, seg_len, 6)
+    clean, _ = run(cu, x, extra, shape, torch.float32)
+    for t in x:
+        t[:, cu[1]:cu[2]] = bad
+    dirty, _ = run(cu, x, extra, shape, torch.float32)
+    for name, a, b in zip(("o", "dq", "dk", "dv", "kv", "gin"), clean, dirty):
+        for i in (0, 2):
+            at = (slice(i, i + 1),) if name in ("kv", "gin") else (slice(None), slice(cu[i], cu[i + 1]))
+            assert torch.equal(a[at], b[at]), (name, i)
+
+
+def test_packed_sequences_without_a_workspace_run_one_by_one():
+    cu, x, extra, shape = packed([100, 60, 128], torch.float32, 0, 7)
+    with_ws, one = run(cu, x, extra, shape, torch.float32)
+    without, each = run(cu, x, extra, shape, torch.float32, workspace=False)
+    assert (one, each) == (1, 3) and torch.equal(with_ws[0], without[0]) and torch.equal(with_ws[4], without[4])
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2, 4, 7])
+@pytest.mark.parametrize("N", [1, 128, 129, 500])
+def test_state_after_the_last_block(N, precision):
+    """The two halves that the state is kept in, with and without lo terms: single terms round to 2^-9 of each product."""
+    gen = torch.Generator().manual_seed(N)
+    q, k, v = [torch.randn(2, H, N, D, generator=gen).bfloat16() for _ in range(3)]
+    o, kv = la.fwd(q.cuda(), k.cuda(), v.cuda(), LAM, want_state=True, precision=precision)
+    torch.cuda.synchronize()
+    ref = orc.fwd_rec(q, k, v, LAM.double().numpy(), want_state=True)
+    tol = 1.7e-4 if precision == 7 else 5 * 2.0 ** -8
+    for g, r in zip((o, kv), ref):
+        rms = np.sqrt(np.mean(r * r, axis=(2, 3), keepdims=True))
+        assert np.all(np.abs(g.cpu().double().numpy() - r) <= tol * rms + 2 * tol * np.abs(r))
