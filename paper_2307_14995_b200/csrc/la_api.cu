@@ -311,6 +311,7 @@ struct Carried {
   const float* z_in = nullptr;
   const float* local = nullptr;
   bool z_in_t = false, local_t = false;
+  Follows follows = FOLLOWS_ANY;  // the launch before the walk (tensor-core kernels)
 };
 Carried chained(const float* z_in, bool z_in_t, const float* local, bool local_t) {
   Carried c;
@@ -334,6 +335,7 @@ OpArgs walk_args(const la_shape* s, const Plan& p, const void* a, const void* b,
   args.z_in_t = from.z_in_t;
   args.local_t = from.local_t;
   args.scanned = p.scanned;
+  args.follows = from.follows;
   args.final_out = final_out;
   args.BH = p.BH;
   args.H = s->H;
@@ -476,6 +478,7 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   } else {
     from.entry = kv_in;  // single segment: the caller's state is the entry state
   }
+  from.follows = p.chains && p.nseg > 1 ? FOLLOWS_STATES : FOLLOWS_ANY;
   if (!u) {
     LA_TRY_CUDA(run_walk(shape, p, tab, q, k, v, o, from, kv_out, 0, cs));
     return LA_OK;
@@ -567,7 +570,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     LA_TRY_CUDA(run_scan(shape, p, tab, buf_kvt, nullptr, kv_in, true, 0, cs));
     from_q.entry = buf_kvt;
   }
-  if (!p.rows) LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
+  if (!p.rows && !p.chains) LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
 
   // dV = rev(a = K, b = Q, c = dO) carries dKV; dK = rev(a = V, b = dO, c = Q) carries dKV^T.
   Carried from_v, from_k;
@@ -576,6 +579,11 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf_e, 1, cs));
     from_v = chained(grad_kv_out, false, buf_e, false);
     from_k = chained(grad_kv_out, true, buf_e, true);
+    // The states of both directions come before all walks: the dQ walk begins while they end and the other two while it ends,
+    // so that the thread blocks of a launch fill the multiprocessors that the last ones of the launch before leave idle.
+    from_q.follows = multi ? FOLLOWS_STATES : FOLLOWS_ANY;
+    from_v.follows = from_k.follows = FOLLOWS_WALK;
+    LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
   } else if (multi || grad_kv_out) {
     LA_TRY_CUDA(run_scan(shape, p, tab, buf_e, buf_et, grad_kv_out, false, 1, cs));
     from_v.entry = buf_e;

@@ -27,6 +27,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <utility>
+
 #define LA_MAX_H 256
 
 namespace la {
@@ -56,6 +58,7 @@ struct OpArgs {
   int BH, H, N;
   int seg_len, nseg;  // seg_len is a multiple of 128
   int reverse;        // 0 forward, 1 reverse
+  int follows;        // tensor-core walk: Follows
   // Where token t of (batch b, head h) sits in a, b, c, out, u, y: element offset b*sB + h*sH + t*sT of a row of
   // Da / Ec contiguous features.  [B,H,N,D]: sT = D, sH = N*D, sB = H*N*D; [B,N,H,D]: sT = H*D, sH = D, sB = N*H*D
   // (D = Da = Ec in every supported shape).
@@ -161,6 +164,36 @@ cudaError_t launch_bounded_wait_selftest(long long budget_clocks, cudaStream_t s
 unsigned int tc_read_status(bool clear);
 
 void count_launch(int n = 1);
+
+// Launches that may begin while the launch before them on the stream drains (programmatic dependent launch).  A kernel lets its
+// successor begin (grid_dep_launch) only after its own wait for its predecessor (grid_dep_wait), so whatever came before the
+// predecessor is complete when a kernel begins; what the predecessor itself writes needs the wait.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, Args&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2]{};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// What a walk needs of the launch before it on the stream.
+enum Follows {
+  FOLLOWS_ANY = 0,     // the first launch of a call: everything
+  FOLLOWS_STATES = 1,  // the states that it chains; its other inputs were complete before that launch began
+  FOLLOWS_WALK = 2,    // nothing: a walk of the same call, which began when the states of both were complete
+};
 
 // Brackets one kernel launch with CUDA events when benchmark profiling is enabled
 // (la_profile_enable); otherwise does nothing.  kind is one of LA_KERNEL_*.

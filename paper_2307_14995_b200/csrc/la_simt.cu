@@ -793,6 +793,8 @@ cudaError_t launch_chain(const ChainArgs& args, const DecayTable& tab, cudaStrea
 
 // One thread per four state elements; the next segment's state is fetched one step ahead.
 __global__ void __launch_bounds__(256) prefix_kernel(const ScanArgs args, const DecayTable tab) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int bh = blockIdx.y;
   const double s2 = tab.s2[bh % args.H];
   if (!slow_head((float)s2, args.seg_len)) return;
@@ -820,9 +822,10 @@ __global__ void __launch_bounds__(256) prefix_kernel(const ScanArgs args, const 
 cudaError_t launch_prefix(const ScanArgs& args, const DecayTable& tab, cudaStream_t stream) {
   if ((args.Da * args.Ec) % 1024 != 0 || args.BH > 65535) return cudaErrorInvalidValue;
   KernelTimer timer(K_SCAN, stream);
-  prefix_kernel<<<dim3((unsigned)(args.Da * args.Ec / 1024), (unsigned)args.BH), 256, 0, stream>>>(args, tab);
+  const cudaError_t err =
+      launch_early(prefix_kernel, dim3((unsigned)(args.Da * args.Ec / 1024), (unsigned)args.BH), dim3(256), 0, stream, 1, args, tab);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 cudaError_t launch_scan(const ScanArgs& args, const DecayTable& tab, cudaStream_t stream) {

@@ -55,7 +55,7 @@ struct TcArgs {
   int njobs;
   int BH, H, N, seg_len, nseg;
   int precision;
-  int scanned, fold;  // see OpArgs
+  int scanned, fold, follows;  // see OpArgs
   // D = 128: bytes to add to the first job's output for entries fold .. 2 fold - 1 (OpArgs::out2); D = 64: whether there is one
   long long second_half;
   long long sT, sH, sB;  // element offset of token t of (b,h): b*sB + h*sH + t*sT (rows of D contiguous features)
@@ -187,6 +187,7 @@ TcArgs make_args(const OpArgs& args, const OpArgs* second, int precision) {
   ta.precision = precision;
   ta.scanned = args.scanned;
   ta.fold = args.fold;
+  ta.follows = args.follows;
   ta.sT = args.sT; ta.sH = args.sH; ta.sB = args.sB;
   ta.seq_start = args.seq_start;
   ta.seq_len = args.seq_len;

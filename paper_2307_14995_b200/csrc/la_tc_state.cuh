@@ -75,6 +75,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
   constexpr int PANELS = D / 64;
   SSmem<D>& sm = *reinterpret_cast<SSmem<D>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (args.seq_start) grid_dep_wait();  // the tables of a packed batch
 
   // ---- which segment, and which of its pieces ----
   const int cid = blockIdx.x / plan.cluster, rank = blockIdx.x % plan.cluster;
@@ -142,6 +143,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = sm.tmem_slot;
+  grid_dep_wait();
+  grid_dep_launch();
 
   if (warp == 0) {
     // ------------------------------------ TMA producer ------------------------------------
@@ -413,19 +416,8 @@ cudaError_t launch_state_t(const TcMaps& m, const TcArgs& ta, const DecayTable& 
   const long shared_units = (long)plan.n_shared * (ta.BH / ta.H) * plan.nseg_used;
   const long other_units = (long)(ta.H - plan.n_shared) * (ta.BH / ta.H) * plan.nseg_used;
   const long clusters = shared_units + (other_units + plan.cluster - 1) / plan.cluster;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(clusters * plan.cluster));
-  cfg.blockDim = dim3(S_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned)plan.cluster;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
   KernelTimer timer(K_PREPASS, stream);
-  err = cudaLaunchKernelEx(&cfg, kern, m.b, m.c, ta, plan, tab);
+  err = launch_early(kern, dim3((unsigned)(clusters * plan.cluster)), dim3(S_THREADS), smem, stream, plan.cluster, m.b, m.c, ta, plan, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }

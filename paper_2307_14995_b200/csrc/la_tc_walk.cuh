@@ -187,6 +187,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   WSmem<REV>& sm = *reinterpret_cast<WSmem<REV>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (args.follows == FOLLOWS_ANY && args.seq_start) grid_dep_wait();  // the tables of a packed batch
   const int jobid = (args.njobs == 2) ? (int)(blockIdx.x & 1) : 0;
   const int bidx = (args.njobs == 2) ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const TcJob& job = args.job[jobid];
@@ -243,6 +244,10 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = sm.tmem_slot;
+  if (args.follows == FOLLOWS_ANY) {
+    grid_dep_wait();
+    grid_dep_launch();
+  }
   if (warp < 4) {
     set_regs<W_REGS_CTL, W_REGS_LAUNCH>();
     if (warp == 0) {
@@ -456,6 +461,10 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], __ldg(r1 + x * 128));
         }
       };
+      if (args.follows == FOLLOWS_STATES) {
+        grid_dep_wait();
+        grid_dep_launch();
+      }
       const float reach = state_reach(s2, args.seg_len);
       const bool running = args.scanned && slow_head(s2, args.seg_len) && before > 0;
       const int near = running ? 1 : ((float)before <= reach ? before : (int)reach + 1);
@@ -737,6 +746,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   }
 
 teardown:
+  if (args.follows != FOLLOWS_ANY) grid_dep_wait();  // (a launch is complete only when those before it are)
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
@@ -750,7 +760,7 @@ cudaError_t launch_walk_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, 
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ta.njobs == 2 ? K_WALK_PAIR : K_WALK, stream);
-  kern<<<(unsigned)(ta.BH * ta.nseg * ta.njobs), W_THREADS, smem, stream>>>(m0, m1, ta, tab);
+  err = launch_early(kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(W_THREADS), smem, stream, 1, m0, m1, ta, tab);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }

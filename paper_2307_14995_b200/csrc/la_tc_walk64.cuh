@@ -80,6 +80,7 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
   Sm& sm = *reinterpret_cast<Sm*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (args.follows == FOLLOWS_ANY && args.seq_start) grid_dep_wait();  // the tables of a packed batch
   const int jobid = (args.njobs == 2) ? (int)(blockIdx.x & 1) : 0;
   const int bidx = (args.njobs == 2) ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const TcJob& job = args.job[jobid];
@@ -129,6 +130,10 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = sm.tmem_slot;
+  if (args.follows == FOLLOWS_ANY) {
+    grid_dep_wait();
+    grid_dep_launch();
+  }
 
   if (warp < 4) {
     set_regs<V_REGS_CTL, V_REGS_LAUNCH>();
@@ -409,6 +414,10 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
           for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], __ldg(r1 + x * 64));
         }
       };
+      if (args.follows == FOLLOWS_STATES) {
+        grid_dep_wait();
+        grid_dep_launch();
+      }
       if (!lo_part) {
         const float reach = state_reach(s2, args.seg_len);
         const bool running = args.scanned && slow_head(s2, args.seg_len) && before > 0;
@@ -558,6 +567,7 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
   }
 
 teardown:
+  if (args.follows != FOLLOWS_ANY) grid_dep_wait();  // (a launch is complete only when those before it are)
   // (the bulk stores' sources were read before V_STORED; their writes complete before the kernel does)
   tc_fence_before_sync();
   __syncthreads();
@@ -572,7 +582,7 @@ cudaError_t launch_walk64_t(const TcMaps& m0, const TcMaps& m1, const VOutMaps& 
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ta.njobs == 2 ? K_WALK_PAIR : K_WALK, stream);
-  kern<<<(unsigned)(ta.BH * ta.nseg * ta.njobs), V_THREADS, smem, stream>>>(m0, m1, out, ta, tab);
+  err = launch_early(kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(V_THREADS), smem, stream, 1, m0, m1, out, ta, tab);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
