@@ -201,12 +201,24 @@ size_t state_set_bytes(const la_shape* s, const Plan& p) {
 int fwd_sets(const la_shape* s, const Plan& p) { return p.nseg == 1 ? 0 : p.chains && s->d == 128 ? 1 : 2; }
 int bwd_sets(const la_shape* s, const Plan& p) { return p.chains && s->d == 128 ? 2 : 3; }
 
-la_status make_table(const la_shape* s, const float* lambda_host, DecayTable* tab) {
+// (logarithms and a table twice as large are half a microsecond of a decode step: it takes the rates as they are)
+la_status make_rates(const la_shape* s, const float* lambda_host, RateTable* rates) {
   if (!lambda_host) return LA_ERR_INVALID_ARG;
   for (int h = 0; h < s->H; ++h) {
     const float lam = lambda_host[h];
     if (!(std::isfinite(lam) && lam > 0.f && lam <= 1.f)) return LA_ERR_INVALID_ARG;
-    const double s2 = -std::log2((double)lam);
+    rates->lam[h] = lam;
+  }
+  for (int h = s->H; h < LA_MAX_H; ++h) rates->lam[h] = 0.f;
+  return LA_OK;
+}
+
+la_status make_table(const la_shape* s, const float* lambda_host, DecayTable* tab) {
+  RateTable rates;
+  const la_status st = make_rates(s, lambda_host, &rates);
+  if (st != LA_OK) return st;
+  for (int h = 0; h < s->H; ++h) {
+    const double s2 = -std::log2((double)rates.lam[h]);
     tab->s2[h] = (s2 > 0.0) ? s2 : 0.0;  // lambda == 1 gives exactly 0 (never -0)
   }
   for (int h = s->H; h < LA_MAX_H; ++h) tab->s2[h] = 0.0;
@@ -665,13 +677,13 @@ la_status decode_impl(const la_shape* shape, int T, const void* q, const void* k
   if (!q || !k || !v || !kv || !o) return LA_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(kv) || !aligned16(o))
     return LA_ERR_INVALID_ARG;
-  DecayTable tab;
-  if ((st = make_table(shape, lambda_host, &tab)) != LA_OK) return st;
+  RateTable rates;
+  if ((st = make_rates(shape, lambda_host, &rates)) != LA_OK) return st;
   if ((st = check_device()) != LA_OK) return st;
   OpArgs strides{};
   set_strides(shape, T, &strides);
   LA_TRY_CUDA(launch_decode(q, k, v, kv, o, shape->B * shape->H, shape->H, T, shape->d, shape->e,
-                            (int)shape->in_dtype, (int)shape->out_dtype, strides.sT, strides.sH, strides.sB, tab,
+                            (int)shape->in_dtype, (int)shape->out_dtype, strides.sT, strides.sH, strides.sB, rates,
                             static_cast<cudaStream_t>(stream)));
   return LA_OK;
 }

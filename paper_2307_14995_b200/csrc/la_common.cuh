@@ -131,10 +131,14 @@ cudaError_t launch_prefix(const ScanArgs& args, const DecayTable& tab, cudaStrea
 __host__ __device__ inline float state_reach(float s2, int seg_len) { return s2 > 0.f ? 160.f / (s2 * (float)seg_len) : 3.0e38f; }
 __host__ __device__ inline bool slow_head(float s2, int seg_len) { return state_reach(s2, seg_len) >= 2.f; }
 cudaError_t launch_chain(const ChainArgs& args, const DecayTable& tab, cudaStream_t stream);
+// The decay rates themselves, where a single power is all that is needed.
+struct RateTable {
+  float lam[LA_MAX_H];
+};
 // T >= 1 consecutive tokens per (batch, head); token t of (b,h) is the row at element offset b*sB + h*sH + t*sT.
 cudaError_t launch_decode(const void* q, const void* k, const void* v, float* kv, void* o, int BH,
                           int H, int T, int d, int e, int in_dt, int out_dt, long long sT, long long sH, long long sB,
-                          const DecayTable& tab, cudaStream_t stream);
+                          const RateTable& rates, cudaStream_t stream);
 
 // SimpleRMSNorm followed by the gate as stand-alone row kernels (la_gate.cu): y = SRMSNorm(o) (.) u (o and y may be
 // the same buffer), and the gradients of <y, dy> with respect to o (written in the input dtype) and u.
@@ -165,9 +169,9 @@ unsigned int tc_read_status(bool clear);
 
 void count_launch(int n = 1);
 
-// Launches that may begin while the launch before them on the stream drains (programmatic dependent launch).  A kernel lets its
-// successor begin (grid_dep_launch) only after its own wait for its predecessor (grid_dep_wait), so whatever came before the
-// predecessor is complete when a kernel begins; what the predecessor itself writes needs the wait.
+// Launches that may begin while the launch before them on the stream ends (programmatic dependent launch).  A kernel lets its
+// successor begin (grid_dep_launch) only after its own wait for its predecessor (grid_dep_wait), so whatever came before the predecessor is complete when a kernel begins; what the predecessor itself writes
+// needs the wait.  Kernels that do not say otherwise (Follows) wait before their first access to memory.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, Args&&... args) {
   cudaLaunchConfig_t cfg{};

@@ -25,7 +25,7 @@ template <typename TIn, typename TOut, int D, int E>
 __global__ void __launch_bounds__(THREADS)
 decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v,
               float* __restrict__ kv, TOut* __restrict__ o, int H, int T, long long sT, long long sH, long long sB,
-              const DecayTable tab) {
+              const __grid_constant__ RateTable rates) {
   constexpr int LPR = E / 4;              // lanes per state row (float4 each)
   constexpr int RPP = THREADS / LPR;      // rows per pass
   constexpr int PASSES = D / RPP;
@@ -36,9 +36,11 @@ decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* _
   __shared__ alignas(16) float sv[CHUNK][E];
   __shared__ float4 red[2][RPP][LPR];
 
+  grid_dep_wait();
+  grid_dep_launch();
   const int bh = blockIdx.x;
   const int tid = threadIdx.x;
-  const float lam = (float)exp2(-tab.s2[bh % H]);
+  const float lam = rates.lam[bh % H];
   const int col4 = tid % LPR;
   const int row0 = tid / LPR;
 
@@ -105,25 +107,25 @@ decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* _
 
 template <typename TIn, typename TOut, int D, int E>
 cudaError_t launch_t(const void* q, const void* k, const void* v, float* kv, void* o, int BH, int H, int T,
-                     long long sT, long long sH, long long sB, const DecayTable& tab, cudaStream_t stream) {
+                     long long sT, long long sH, long long sB, const RateTable& rates, cudaStream_t stream) {
   KernelTimer timer(K_DECODE, stream);
-  decode_kernel<TIn, TOut, D, E><<<BH, THREADS, 0, stream>>>(
-      static_cast<const TIn*>(q), static_cast<const TIn*>(k), static_cast<const TIn*>(v), kv,
-      static_cast<TOut*>(o), H, T, sT, sH, sB, tab);
+  const cudaError_t err = launch_early(decode_kernel<TIn, TOut, D, E>, dim3((unsigned)BH), dim3(THREADS), 0, stream, 1,
+                                       static_cast<const TIn*>(q), static_cast<const TIn*>(k), static_cast<const TIn*>(v), kv,
+                                       static_cast<TOut*>(o), H, T, sT, sH, sB, rates);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 template <int D, int E>
 cudaError_t launch_dims(const void* q, const void* k, const void* v, float* kv, void* o, int BH, int H, int T,
-                        int in_dt, int out_dt, long long sT, long long sH, long long sB, const DecayTable& tab,
+                        int in_dt, int out_dt, long long sT, long long sH, long long sB, const RateTable& rates,
                         cudaStream_t stream) {
   if (in_dt == DT_F32 && out_dt == DT_F32)
-    return launch_t<float, float, D, E>(q, k, v, kv, o, BH, H, T, sT, sH, sB, tab, stream);
+    return launch_t<float, float, D, E>(q, k, v, kv, o, BH, H, T, sT, sH, sB, rates, stream);
   if (in_dt == DT_BF16 && out_dt == DT_F32)
-    return launch_t<__nv_bfloat16, float, D, E>(q, k, v, kv, o, BH, H, T, sT, sH, sB, tab, stream);
+    return launch_t<__nv_bfloat16, float, D, E>(q, k, v, kv, o, BH, H, T, sT, sH, sB, rates, stream);
   if (in_dt == DT_BF16 && out_dt == DT_BF16)
-    return launch_t<__nv_bfloat16, __nv_bfloat16, D, E>(q, k, v, kv, o, BH, H, T, sT, sH, sB, tab, stream);
+    return launch_t<__nv_bfloat16, __nv_bfloat16, D, E>(q, k, v, kv, o, BH, H, T, sT, sH, sB, rates, stream);
   return cudaErrorInvalidValue;
 }
 
@@ -131,11 +133,11 @@ cudaError_t launch_dims(const void* q, const void* k, const void* v, float* kv, 
 
 cudaError_t launch_decode(const void* q, const void* k, const void* v, float* kv, void* o, int BH,
                           int H, int T, int d, int e, int in_dt, int out_dt, long long sT, long long sH, long long sB,
-                          const DecayTable& tab, cudaStream_t stream) {
+                          const RateTable& rates, cudaStream_t stream) {
   if (T < 1) return cudaErrorInvalidValue;
-  if (d == 64 && e == 64) return launch_dims<64, 64>(q, k, v, kv, o, BH, H, T, in_dt, out_dt, sT, sH, sB, tab, stream);
+  if (d == 64 && e == 64) return launch_dims<64, 64>(q, k, v, kv, o, BH, H, T, in_dt, out_dt, sT, sH, sB, rates, stream);
   if (d == 128 && e == 128)
-    return launch_dims<128, 128>(q, k, v, kv, o, BH, H, T, in_dt, out_dt, sT, sH, sB, tab, stream);
+    return launch_dims<128, 128>(q, k, v, kv, o, BH, H, T, in_dt, out_dt, sT, sH, sB, rates, stream);
   return cudaErrorInvalidValue;
 }
 

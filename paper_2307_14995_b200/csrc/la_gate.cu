@@ -22,6 +22,8 @@ __device__ __forceinline__ float row_sum(float x, int lanes) {
 template <typename TO, typename TU>
 __global__ void __launch_bounds__(256) norm_gate_fwd_kernel(const TO* o, const TU* __restrict__ u, TO* y,
                                                             float* __restrict__ rstd, long rows, int e) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int lanes = e >> 2;  // lanes per row: 16 or 32
   const long gthread = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long nthreads = (long)gridDim.x * blockDim.x;
@@ -50,6 +52,8 @@ template <typename TO, typename TU>
 __global__ void __launch_bounds__(256) norm_gate_bwd_kernel(const TO* __restrict__ o, const TU* __restrict__ u,
                                                             const TU* __restrict__ dy, TU* __restrict__ d_o,
                                                             TO* __restrict__ d_u, long rows, int e) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int lanes = e >> 2;
   const long gthread = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long nthreads = (long)gridDim.x * blockDim.x;
@@ -103,18 +107,20 @@ cudaError_t launch_norm_gate_fwd(const void* o, const void* u, void* y, float* r
   if ((e != 64 && e != 128) || rows < 1) return cudaErrorInvalidValue;
   KernelTimer timer(K_GATE, stream);
   const unsigned grid = grid_for(rows, e);
+  cudaError_t err = cudaSuccess;
   if (out_dt == DT_F32 && in_dt == DT_F32)
-    norm_gate_fwd_kernel<float, float><<<grid, 256, 0, stream>>>((const float*)o, (const float*)u, (float*)y, rstd, rows, e);
+    err = launch_early(norm_gate_fwd_kernel<float, float>, dim3(grid), dim3(256), 0, stream, 1, (const float*)o, (const float*)u, (float*)y, rstd,
+                       rows, e);
   else if (out_dt == DT_F32)
-    norm_gate_fwd_kernel<float, __nv_bfloat16><<<grid, 256, 0, stream>>>((const float*)o, (const __nv_bfloat16*)u, (float*)y,
-                                                                        rstd, rows, e);
+    err = launch_early(norm_gate_fwd_kernel<float, __nv_bfloat16>, dim3(grid), dim3(256), 0, stream, 1, (const float*)o,
+                       (const __nv_bfloat16*)u, (float*)y, rstd, rows, e);
   else if (in_dt == DT_BF16)
-    norm_gate_fwd_kernel<__nv_bfloat16, __nv_bfloat16><<<grid, 256, 0, stream>>>(
-        (const __nv_bfloat16*)o, (const __nv_bfloat16*)u, (__nv_bfloat16*)y, rstd, rows, e);
+    err = launch_early(norm_gate_fwd_kernel<__nv_bfloat16, __nv_bfloat16>, dim3(grid), dim3(256), 0, stream, 1, (const __nv_bfloat16*)o,
+                       (const __nv_bfloat16*)u, (__nv_bfloat16*)y, rstd, rows, e);
   else
     return cudaErrorInvalidValue;
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 cudaError_t launch_norm_gate_bwd(const void* o, const void* u, const void* dy, void* d_o, void* d_u, long rows, int e,
@@ -122,20 +128,20 @@ cudaError_t launch_norm_gate_bwd(const void* o, const void* u, const void* dy, v
   if ((e != 64 && e != 128) || rows < 1) return cudaErrorInvalidValue;
   KernelTimer timer(K_GATE, stream);
   const unsigned grid = grid_for(rows, e);
+  cudaError_t err = cudaSuccess;
   if (out_dt == DT_F32 && in_dt == DT_F32)
-    norm_gate_bwd_kernel<float, float><<<grid, 256, 0, stream>>>((const float*)o, (const float*)u, (const float*)dy,
-                                                                 (float*)d_o, (float*)d_u, rows, e);
+    err = launch_early(norm_gate_bwd_kernel<float, float>, dim3(grid), dim3(256), 0, stream, 1, (const float*)o, (const float*)u,
+                       (const float*)dy, (float*)d_o, (float*)d_u, rows, e);
   else if (out_dt == DT_F32)
-    norm_gate_bwd_kernel<float, __nv_bfloat16><<<grid, 256, 0, stream>>>(
-        (const float*)o, (const __nv_bfloat16*)u, (const __nv_bfloat16*)dy, (__nv_bfloat16*)d_o, (float*)d_u, rows, e);
+    err = launch_early(norm_gate_bwd_kernel<float, __nv_bfloat16>, dim3(grid), dim3(256), 0, stream, 1, (const float*)o,
+                       (const __nv_bfloat16*)u, (const __nv_bfloat16*)dy, (__nv_bfloat16*)d_o, (float*)d_u, rows, e);
   else if (in_dt == DT_BF16)
-    norm_gate_bwd_kernel<__nv_bfloat16, __nv_bfloat16><<<grid, 256, 0, stream>>>(
-        (const __nv_bfloat16*)o, (const __nv_bfloat16*)u, (const __nv_bfloat16*)dy, (__nv_bfloat16*)d_o,
-        (__nv_bfloat16*)d_u, rows, e);
+    err = launch_early(norm_gate_bwd_kernel<__nv_bfloat16, __nv_bfloat16>, dim3(grid), dim3(256), 0, stream, 1, (const __nv_bfloat16*)o,
+                       (const __nv_bfloat16*)u, (const __nv_bfloat16*)dy, (__nv_bfloat16*)d_o, (__nv_bfloat16*)d_u, rows, e);
   else
     return cudaErrorInvalidValue;
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 }  // namespace la

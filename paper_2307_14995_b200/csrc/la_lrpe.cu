@@ -52,6 +52,8 @@ struct Geometry {   // where token t of (b,h) lives: element offset b*sB + h*sH 
 // a warp spent most of its 2100 instructions on them with nothing in flight (this kernel: 7 us at 16 heads x 8192 tokens).
 __global__ void __launch_bounds__(256) lrpe_angle_kernel(const float* __restrict__ theta, float2* __restrict__ table, int H, int d,
                                                          int runs, long long pos0) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int hd = H * d, chunks = (hd + 255) / 256;
   const int run = blockIdx.x / chunks, i = blockIdx.x % chunks * 256 + threadIdx.x;  // run == runs: the step angles
   if (i >= hd) return;
@@ -101,6 +103,8 @@ __device__ __forceinline__ void store_features(const FeatureArgs<T>& io, size_t 
 
 template <typename T>
 __global__ void __launch_bounds__(256, 4) lrpe_feature_kernel(const FeatureArgs<T> io, const float2* __restrict__ table, Geometry g) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int lanes = g.d >> 2;
   const int groups = 256 / lanes;
   const int lane = threadIdx.x % lanes, grp = threadIdx.x / lanes;
@@ -141,6 +145,8 @@ __global__ void __launch_bounds__(256, 4) lrpe_feature_kernel(const FeatureArgs<
 // dst = a + b (fp32 operands; dst may be a itself), four elements per thread.
 template <typename TOut>
 __global__ void __launch_bounds__(256) lrpe_sum_kernel(const float* a, const float* __restrict__ b, TOut* dst, long n4) {
+  grid_dep_wait();
+  grid_dep_launch();
   const long nthreads = (long)gridDim.x * blockDim.x;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += nthreads) {
     float x[4], y[4];
@@ -171,6 +177,8 @@ template <typename TIn, typename TOut>
 __global__ void __launch_bounds__(256) lrpe_grad_kernel(const GradArgs<TIn, TOut> io, const float2* __restrict__ table, Geometry g,
                                                            long long pos0, int ntiles) {
   __shared__ float red[2048];  // [tokens per pass][d]: 8 x 128 or 16 x 64
+  grid_dep_wait();
+  grid_dep_launch();
   const bool second = blockIdx.y != 0;
   const TIn* __restrict__ const x = second ? io.x[1] : io.x[0];
   const float* __restrict__ const gc = second ? io.gc[1] : io.gc[0];
@@ -224,6 +232,8 @@ __global__ void __launch_bounds__(256) lrpe_grad_kernel(const GradArgs<TIn, TOut
 __global__ void __launch_bounds__(256) lrpe_theta_reduce_kernel(const float* __restrict__ part_q,
                                                                 const float* __restrict__ part_k,
                                                                 float* __restrict__ dtheta, int B, int H, int ntiles, int d) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int slice = threadIdx.x >> 3, fi = threadIdx.x & 7;
   const int idx = blockIdx.x * 8 + fi;  // feature index in [0, H*d)
   __shared__ double red[32][8];
@@ -270,9 +280,9 @@ cudaError_t run_angles(const la_shape* s, const float* theta, float2* table, lon
   const int runs = (s->N + RUN - 1) / RUN;
   const long blocks = (runs + 1L) * ((s->H * s->d + 255) / 256);
   if (blocks > 2147483647L) return cudaErrorInvalidValue;
-  lrpe_angle_kernel<<<(unsigned)blocks, 256, 0, st>>>(theta, table, s->H, s->d, runs, pos0);
+  const cudaError_t err = launch_early(lrpe_angle_kernel, dim3((unsigned)blocks), dim3(256), 0, st, 1, theta, table, s->H, s->d, runs, pos0);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 template <typename T>
@@ -284,9 +294,9 @@ cudaError_t run_features_t(const la_shape* s, const void* q, const void* k, cons
   io.c[0] = static_cast<T*>(qc); io.c[1] = static_cast<T*>(kc);
   io.s[0] = static_cast<T*>(qs); io.s[1] = static_cast<T*>(ks);
   const unsigned grid = grid_for((long)s->B * s->H * ((s->N + RUN - 1) / RUN) * (s->d / 4));
-  lrpe_feature_kernel<T><<<grid, 256, 0, st>>>(io, table, geometry(s));
+  const cudaError_t err = launch_early(lrpe_feature_kernel<T>, dim3(grid), dim3(256), 0, st, 1, io, table, geometry(s));
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 cudaError_t run_features(const la_shape* s, const void* q, const void* k, const float2* table, void* qc, void* qs, void* kc,
                          void* ks, cudaStream_t st) {
@@ -298,12 +308,12 @@ cudaError_t run_sum(const la_shape* s, const float* a, const float* b, void* dst
   KernelTimer timer(K_LRPE, st);
   const long n4 = (long)s->B * s->H * s->N * s->e / 4;
   const unsigned grid = grid_for(n4);
-  if (s->out_dtype == LA_BF16)
-    lrpe_sum_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(a, b, (__nv_bfloat16*)dst, n4);
-  else
-    lrpe_sum_kernel<float><<<grid, 256, 0, st>>>(a, b, (float*)dst, n4);
+  const cudaError_t err =
+      s->out_dtype == LA_BF16
+          ? launch_early(lrpe_sum_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, st, 1, a, b, (__nv_bfloat16*)dst, n4)
+          : launch_early(lrpe_sum_kernel<float>, dim3(grid), dim3(256), 0, st, 1, a, b, (float*)dst, n4);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 // The tensors of GradArgs for q and k, untyped.
@@ -327,9 +337,9 @@ cudaError_t run_grad_t(const la_shape* s, const GradSet& q, const GradSet& k, co
     io.dx[w] = static_cast<TOut*>(one.dx);
     io.part[w] = one.part;
   }
-  lrpe_grad_kernel<TIn, TOut><<<dim3((unsigned)((long)s->B * s->H * ntiles), 2), 256, 0, st>>>(io, table, geometry(s), pos0, ntiles);
+  const cudaError_t err = launch_early((lrpe_grad_kernel<TIn, TOut>), dim3((unsigned)((long)s->B * s->H * ntiles), 2), dim3(256), 0, st, 1, io, table, geometry(s), pos0, ntiles);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 cudaError_t run_grad(const la_shape* s, const GradSet& q, const GradSet& k, const float2* table, long long pos0, int ntiles,
                      cudaStream_t st) {
@@ -499,9 +509,10 @@ la_status la_lrpe_bwd(const la_shape* shape, const void* q, const void* k, const
   {
     KernelTimer timer(K_LRPE, cs);
     const int n = shape->H * shape->d;
-    lrpe_theta_reduce_kernel<<<(n + 7) / 8, 256, 0, cs>>>(part_q, part_k, d_theta, shape->B, shape->H, c.ntiles, shape->d);
+    const cudaError_t err = launch_early(lrpe_theta_reduce_kernel, dim3((unsigned)((n + 7) / 8)), dim3(256), 0, cs, 1, part_q, part_k, d_theta,
+                                         shape->B, shape->H, c.ntiles, shape->d);
     count_launch();
-    if (cudaGetLastError() != cudaSuccess) return LA_ERR_CUDA;
+    if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return LA_ERR_CUDA;
   }
   return LA_OK;
 }

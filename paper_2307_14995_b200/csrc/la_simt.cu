@@ -294,6 +294,8 @@ constexpr int SCAN_MAX_SEG = 1024;
 __global__ void __launch_bounds__(256) scan_kernel(const ScanArgs args, const DecayTable tab) {
   __shared__ float gamma[SCAN_MAX_SEG];
   __shared__ float tile[32][33];
+  grid_dep_wait();
+  grid_dep_launch();
   const int Da = args.Da, Ec = args.Ec, DE = Da * Ec;
   const int bh = blockIdx.x;
   const int tiles_y = Ec / 32;
@@ -417,6 +419,8 @@ __global__ void __launch_bounds__(ROWS_THREADS * G)
 simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ DecayTable tab) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RowsSmem<D, G>& sm = *reinterpret_cast<RowsSmem<D, G>*>(smem_raw);
+  grid_dep_wait();
+  grid_dep_launch();
   const int grp = threadIdx.x / ROWS_THREADS, tid = threadIdx.x % ROWS_THREADS;
   typename RowsSmem<D, G>::Group& gm = sm.group[grp];
   int jb = 0;
@@ -630,9 +634,9 @@ cudaError_t launch_rows_g(const RowsArgs& ra, const DecayTable& tab, cudaStream_
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ra.units[0] ? K_WALK : K_PREPASS, stream);
-  kern<<<(unsigned)ra.first_block[ROWS_MAX_JOBS], ROWS_THREADS * G, smem, stream>>>(ra, tab);
+  err = launch_early(kern, dim3((unsigned)ra.first_block[ROWS_MAX_JOBS]), dim3(ROWS_THREADS * G), smem, stream, 1, ra, tab);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 // Thread blocks up to which their tiles are shared out over groups: as many as run at once, two or four to a multiprocessor.
 constexpr int rows_groups_limit(int d) { return d == 64 ? 592 : 296; }
@@ -757,6 +761,8 @@ __global__ void __launch_bounds__(256) chain_kernel(const ChainArgs args, const 
   // double by every thread and for every piece they took longer than the sums: 65536 tokens, 32 heads, 32 segments of
   // 2048 tokens 107 us with the states, 97 this way; 64 segments 182 and 164.)
   __shared__ float power[2];
+  grid_dep_wait();
+  grid_dep_launch();
   const long per_head = args.DE / 4;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const int bh = (int)(i / per_head);
@@ -786,9 +792,9 @@ cudaError_t launch_chain(const ChainArgs& args, const DecayTable& tab, cudaStrea
   if (args.DE % 1024 != 0 || args.BH < 1 || args.count < 0 || args.piece_len < 1) return cudaErrorInvalidValue;
   const long threads = (long)args.BH * (args.DE / 4);
   KernelTimer timer(K_SCAN, stream);
-  chain_kernel<<<(unsigned)(threads / 256), 256, 0, stream>>>(args, tab);
+  const cudaError_t err = launch_early(chain_kernel, dim3((unsigned)(threads / 256)), dim3(256), 0, stream, 1, args, tab);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 // One thread per four state elements; the next segment's state is fetched one step ahead.
@@ -832,9 +838,9 @@ cudaError_t launch_scan(const ScanArgs& args, const DecayTable& tab, cudaStream_
   if (args.nseg > SCAN_MAX_SEG || (args.Da % 32) != 0 || (args.Ec % 32) != 0) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)args.BH, (unsigned)((args.Da / 32) * (args.Ec / 32)));
   KernelTimer timer(K_SCAN, stream);
-  scan_kernel<<<grid, 256, 0, stream>>>(args, tab);
+  const cudaError_t err = launch_early(scan_kernel, grid, dim3(256), 0, stream, 1, args, tab);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 }  // namespace la
