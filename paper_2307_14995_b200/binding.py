@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C ABI in ``include/la.h``.
+"""Thin binding of the C ABI in ``include/la.h``: calls on device tensors through the extension module `_la_call`, the others through
+ctypes.
 
 Argument marshalling only: every step of the attention path runs in the CUDA
 kernels behind ``libla_b200.so``.  PyTorch is used for device memory and streams.
@@ -46,6 +47,7 @@ class LaError(RuntimeError):
 
 
 _lib = None
+_call, _address = None, {}  # _la_call.call, and where the C functions are
 
 
 def load():
@@ -118,8 +120,27 @@ def load():
         lib.la_profile_collect.argtypes = [ctypes.POINTER(ctypes.c_double),
                                            ctypes.POINTER(ctypes.c_ulonglong)]
         lib.la_profile_collect.restype = I
+        try:
+            from . import _la_call
+        except ImportError as e:
+            raise RuntimeError("extension module _la_call is missing; run `python -m paper_2307_14995_b200.build`") from e
+        global _call
+        _address.update((name, ctypes.cast(getattr(lib, name), ctypes.c_void_p).value) for name in EXPORTS)
+        _la_call.bind(LaShape, lambda stream: _stream(stream))
+        _address["la_bwd"] = _address["la_bwd_reuse"]  # (the same with a NULL fwd_workspace)
+        _call = _la_call.call
         _lib = lib
     return _lib
+
+
+def _enter(name: str, kinds: str, *args) -> None:
+    """Calls a C function; kinds has a letter for each argument (s: shape, t: tensor or None, i: integer,
+    h: host memory, r: stream)."""
+    if _call is None:
+        load()
+    rc = _call(_address[name], kinds, *args)
+    if rc != 0:
+        raise LaError(rc, name)
 
 
 def status_string(code: int) -> str:
@@ -224,34 +245,27 @@ def alloc_workspace(op: int, shape: LaShape, device) -> Optional[torch.Tensor]:
     return torch.empty(n, dtype=torch.uint8, device=device)  # torch allocations are >= 256-byte aligned
 
 
+def _bytes(workspace) -> int:
+    return 0 if workspace is None else workspace.numel() * workspace.element_size()
+
+
 def la_fwd(shape: LaShape, q, k, v, lam, o, kv_in=None, kv_out=None, workspace=None, stream=None):
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().la_fwd(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _lam(lam), _ptr(o), _ptr(kv_in),
-                       _ptr(kv_out), _ptr(workspace), ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_fwd")
+    _enter("la_fwd", "sttthttttir", shape, q, k, v, _lam(lam), o, kv_in, kv_out, workspace, _bytes(workspace), stream)
 
 
 def la_fwd_gated(shape: LaShape, q, k, v, u, lam, y, o=None, rstd=None, kv_in=None, kv_out=None, workspace=None,
                  stream=None):
     """la_fwd with y = SRMSNorm(o) (.) u as its output stage; o and rstd are optional outputs."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().la_fwd_gated(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(u), _lam(lam), _ptr(y), _ptr(o),
-                             _ptr(rstd), _ptr(kv_in), _ptr(kv_out), _ptr(workspace), ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_fwd_gated")
+    _enter("la_fwd_gated", "stttthttttttir", shape, q, k, v, u, _lam(lam), y, o, rstd, kv_in, kv_out, workspace, _bytes(workspace),
+           stream)
 
 
 def la_gate_fwd(shape: LaShape, o, u, y, rstd=None, stream=None):
-    rc = load().la_gate_fwd(ctypes.byref(shape), _ptr(o), _ptr(u), _ptr(y), _ptr(rstd), _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_gate_fwd")
+    _enter("la_gate_fwd", "sttttr", shape, o, u, y, rstd, stream)
 
 
 def la_gate_bwd(shape: LaShape, o, u, dy, d_o, d_u, stream=None):
-    rc = load().la_gate_bwd(ctypes.byref(shape), _ptr(o), _ptr(u), _ptr(dy), _ptr(d_o), _ptr(d_u), _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_gate_bwd")
+    _enter("la_gate_bwd", "stttttr", shape, o, u, dy, d_o, d_u, stream)
 
 
 def la_fwd_noalloc(shape: LaShape, q, k, v, lam, o, kv_in=None, kv_out=None, stream=None):
@@ -259,42 +273,24 @@ def la_fwd_noalloc(shape: LaShape, q, k, v, lam, o, kv_in=None, kv_out=None, str
     memory when they call (everything was handed to a pool at start-up, no allocator is available,
     or an allocation's device-wide synchronisation is unacceptable).  Calls on different streams
     must not overlap; shapes needing more than LA_NOALLOC_SCRATCH_BYTES raise LaError (status 7)."""
-    rc = load().la_fwd_noalloc(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _lam(lam), _ptr(o), _ptr(kv_in),
-                               _ptr(kv_out), _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_fwd_noalloc")
+    _enter("la_fwd_noalloc", "sttthtttr", shape, q, k, v, _lam(lam), o, kv_in, kv_out, stream)
 
 
 def la_bwd(shape: LaShape, q, k, v, do, lam, dq, dk, dv, kv_in=None, grad_kv_out=None, grad_kv_in=None,
            workspace=None, stream=None, fwd_workspace=None):
     """fwd_workspace: the workspace of the matching la_fwd call (same shape, inputs, kv_in), to reuse its
     segment states (la_bwd_reuse); None recomputes them (la_bwd)."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    if fwd_workspace is None:
-        rc = load().la_bwd(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(do), _lam(lam), _ptr(dq),
-                           _ptr(dk), _ptr(dv), _ptr(kv_in), _ptr(grad_kv_out), _ptr(grad_kv_in),
-                           _ptr(workspace), ws_bytes, _stream(stream))
-    else:
-        rc = load().la_bwd_reuse(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(do), _lam(lam), _ptr(dq),
-                                 _ptr(dk), _ptr(dv), _ptr(kv_in), _ptr(grad_kv_out), _ptr(grad_kv_in),
-                                 _ptr(fwd_workspace), _ptr(workspace), ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_bwd")
+    _enter("la_bwd", "stttthttttttttir", shape, q, k, v, do, _lam(lam), dq, dk, dv, kv_in, grad_kv_out, grad_kv_in, fwd_workspace,
+           workspace, _bytes(workspace), stream)
 
 
 def la_decode_step(shape: LaShape, q, k, v, lam, kv, o, stream=None):
-    rc = load().la_decode_step(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _lam(lam), _ptr(kv),
-                               _ptr(o), _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_decode_step")
+    _enter("la_decode_step", "sttthttr", shape, q, k, v, _lam(lam), kv, o, stream)
 
 
 def la_decode_steps(shape: LaShape, q, k, v, lam, kv, o, stream=None):
     """shape.N consecutive tokens per call: q, k [B,H,N,d], v, o [B,H,N,e]; kv updated in place once."""
-    rc = load().la_decode_steps(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _lam(lam), _ptr(kv),
-                                _ptr(o), _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_decode_steps")
+    _enter("la_decode_steps", "sttthttr", shape, q, k, v, _lam(lam), kv, o, stream)
 
 
 def _cu(cu_seqlens):
@@ -313,22 +309,15 @@ def varlen_workspace_bytes(op: int, shape: LaShape, cu_seqlens) -> int:
 def la_fwd_varlen(shape: LaShape, q, k, v, lam, o, cu_seqlens, kv_in=None, kv_out=None, workspace=None, stream=None):
     """Packed [T,H,d] tensors (shape: B=1, N=T, layout BNHD); cu_seqlens: host ints, first token of each sequence."""
     cu, S = _cu(cu_seqlens)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().la_fwd_varlen(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _lam(lam), _ptr(o), cu, S, _ptr(kv_in),
-                              _ptr(kv_out), _ptr(workspace), ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_fwd_varlen")
+    _enter("la_fwd_varlen", "sttththitttir", shape, q, k, v, _lam(lam), o, cu, S, kv_in, kv_out, workspace, _bytes(workspace),
+           stream)
 
 
 def la_bwd_varlen(shape: LaShape, q, k, v, do, lam, dq, dk, dv, cu_seqlens, kv_in=None, grad_kv_out=None,
                   grad_kv_in=None, workspace=None, stream=None):
     cu, S = _cu(cu_seqlens)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().la_bwd_varlen(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(do), _lam(lam), _ptr(dq), _ptr(dk),
-                              _ptr(dv), cu, S, _ptr(kv_in), _ptr(grad_kv_out), _ptr(grad_kv_in), _ptr(workspace),
-                              ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_bwd_varlen")
+    _enter("la_bwd_varlen", "stttthttthittttir", shape, q, k, v, do, _lam(lam), dq, dk, dv, cu, S, kv_in, grad_kv_out, grad_kv_in,
+           workspace, _bytes(workspace), stream)
 
 
 def chunk_state_workspace_bytes(shape: LaShape) -> int:
@@ -340,20 +329,14 @@ def chunk_state_workspace_bytes(shape: LaShape) -> int:
 
 def la_chunk_state(shape: LaShape, reverse: int, b, c, lam, state_out, workspace, stream=None):
     """A chunk's own state contribution: reverse=0 (b=k, c=v) or reverse=1 (b=q, c=dO)."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().la_chunk_state(ctypes.byref(shape), int(reverse), _ptr(b), _ptr(c), _lam(lam), _ptr(state_out),
-                               _ptr(workspace), ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_chunk_state")
+    _enter("la_chunk_state", "sitthttir", shape, int(reverse), b, c, _lam(lam), state_out, workspace, _bytes(workspace), stream)
 
 
 def la_chain_states(shape: LaShape, total_tokens: int, chunk_tokens: int, reverse: int, states, num_chunks: int,
                     chunk: int, boundary, lam, state_out, stream=None):
     """The state at a cut from the gathered per-chunk contributions [num_chunks,B,H,d,e]."""
-    rc = load().la_chain_states(ctypes.byref(shape), int(total_tokens), int(chunk_tokens), int(reverse), _ptr(states),
-                                int(num_chunks), int(chunk), _ptr(boundary), _lam(lam), _ptr(state_out), _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_chain_states")
+    _enter("la_chain_states", "siiitiithtr", shape, int(total_tokens), int(chunk_tokens), int(reverse), states, int(num_chunks),
+           int(chunk), boundary, _lam(lam), state_out, stream)
 
 
 def lrpe_workspace_bytes(op: int, shape: LaShape) -> int:
@@ -365,21 +348,14 @@ def lrpe_workspace_bytes(op: int, shape: LaShape) -> int:
 
 def la_lrpe_fwd(shape: LaShape, q, k, v, theta, lam, o, pos0=0, kv_in=None, kv_out=None, workspace=None, stream=None):
     """LRPE-d forward (Eq. 1); theta: device fp32 [H,d]; states [2,B,H,d,e]."""
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().la_lrpe_fwd(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(theta), _lam(lam), int(pos0), _ptr(o),
-                            _ptr(kv_in), _ptr(kv_out), _ptr(workspace), ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_lrpe_fwd")
+    _enter("la_lrpe_fwd", "stttthittttir", shape, q, k, v, theta, _lam(lam), int(pos0), o, kv_in, kv_out, workspace, _bytes(workspace),
+           stream)
 
 
 def la_lrpe_bwd(shape: LaShape, q, k, v, do, theta, lam, dq, dk, dv, dtheta, pos0=0, kv_in=None, grad_kv_out=None,
                 grad_kv_in=None, workspace=None, stream=None):
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().la_lrpe_bwd(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(do), _ptr(theta), _lam(lam), int(pos0),
-                            _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dtheta), _ptr(kv_in), _ptr(grad_kv_out),
-                            _ptr(grad_kv_in), _ptr(workspace), ws_bytes, _stream(stream))
-    if rc != 0:
-        raise LaError(rc, "la_lrpe_bwd")
+    _enter("la_lrpe_bwd", "sttttthittttttttir", shape, q, k, v, do, theta, _lam(lam), int(pos0), dq, dk, dv, dtheta, kv_in, grad_kv_out,
+           grad_kv_in, workspace, _bytes(workspace), stream)
 
 
 def host_arena_bytes(shape: LaShape) -> int:

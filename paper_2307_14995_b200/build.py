@@ -1,19 +1,21 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a.
+"""Builds the CUDA library in-tree with nvcc for sm_100a, and the extension module that calls it.
 
     python -m paper_2307_14995_b200.build [--force] [--verbose]
 
 Produces ``paper_2307_14995_b200/libla_b200.so`` (C ABI declared in
-``include/la.h``).  nvcc cross-compiles without a GPU.
+``include/la.h``) and ``paper_2307_14995_b200/_la_call.so``.  nvcc cross-compiles without a GPU.
 """
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libla_b200.so")
+CALL = os.path.join(HERE, "_la_call.so")
 SOURCES = ["la_api.cu", "la_simt.cu", "la_decode.cu", "la_tc.cu", "la_noalloc.cu", "la_gate.cu", "la_lrpe.cu"]
 HEADERS = ["la_common.cuh", os.path.join("..", "..", "include", "la.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -56,6 +58,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd = [_nvcc(), "-shared", "-o", tmp] + objs + ["-lcudart"]
         subprocess.check_call(cmd)
         os.replace(tmp, LIB)
+    src = os.path.join(CSRC, "la_call.c")
+    if force or _stale(CALL, [src]):
+        tmp = CALL + ".tmp%d" % os.getpid()
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
+                               src, "-o", tmp])
+        os.replace(tmp, CALL)
     return LIB
 
 
