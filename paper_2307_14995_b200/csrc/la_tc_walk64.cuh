@@ -250,10 +250,10 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
       for (int pi = 0; pi < 4; ++pi) {
         const int j0 = half * 64 + pi * 16;
         const int off = REV ? q - (j0 >> 5) : (j0 >> 5) - q;  // > 0: outside the band
-        uint32_t h8[8], l8[8];
+        uint32_t hl[16];  // 8 columns of hi pairs, 8 of lo pairs
         if (off > 0) {
 #pragma unroll
-          for (int x = 0; x < 8; ++x) h8[x] = l8[x] = 0u;
+          for (int x = 0; x < 16; ++x) hl[x] = 0u;
         } else {
           uint32_t sreg[16];
           tmem_ld_x16(colS + j0, sreg);
@@ -287,11 +287,9 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
             }
           }
 #pragma unroll
-          for (int x = 0; x < 8; ++x) split2(f2_pack(d[2 * x], d[2 * x + 1]), h8[x], l8[x]);
+          for (int x = 0; x < 8; ++x) split2(f2_pack(d[2 * x], d[2 * x + 1]), hl[x], hl[8 + x]);
         }
-        // the 16 fp32 columns just read become 8 columns of hi pairs and 8 of lo pairs
-        tmem_st_x8(colS + j0, h8);
-        if (split_p) tmem_st_x8(colS + j0 + 8, l8);
+        tmem_st_x16(colS + j0, hl);  // in the place of the 16 fp32 columns just read
       }
       tmem_st_wait();
       tc_fence_before_sync();
@@ -324,12 +322,13 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
       }
       fence_proxy_async_smem();
     };
-    uint32_t raw[32];  // c of the next block: [16 tokens][16 value columns][8 tokens][8 value columns]
+    uint32_t raw[2][16];  // c of the next block, then its fc: [16 value columns][16 tokens][8 tokens][8 value columns]
     auto fetch_c = [&](int it) {
       const uint32_t ctile = smem_u32(sm.st[it % V_STAGES].c) + unit0;
 #pragma unroll
       for (int g = 0; g < 8; ++g)  // 16 tokens (g >> 1), 16 value columns (g & 1)
-        ldmatrix_x4_trans((ctile ^ ((g & 1) << 5)) + (g >> 1) * 2048, raw[4 * g], raw[4 * g + 1], raw[4 * g + 2], raw[4 * g + 3]);
+        ldmatrix_x4_trans((ctile ^ ((g & 1) << 5)) + (g >> 1) * 2048, raw[g & 1][(g >> 1) * 4], raw[g & 1][(g >> 1) * 4 + 1],
+                          raw[g & 1][(g >> 1) * 4 + 2], raw[g & 1][(g >> 1) * 4 + 3]);
     };
     const float lam16 = ex2_approx(-s2 * 16.f);
     auto write_fc = [&](int it) {
@@ -354,27 +353,28 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
 #pragma unroll
             for (int x = 0; x < 8; ++x) {
               const int j = j0 + 8 * ((x >> 1) & 1);
-              raw[g * 8 + x] &= (j < Cr ? 0xffffu : 0u) | (j + 1 < Cr ? 0xffff0000u : 0u);
+              raw[x >> 2][g * 4 + (x & 3)] &= (j < Cr ? 0xffffu : 0u) | (j + 1 < Cr ? 0xffff0000u : 0u);
             }
           }
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
-            uint32_t w4[4];
 #pragma unroll
             for (int x = 0; x < 4; ++x) {  // octet x >> 1, value columns (x & 1) * 8
-              const uint32_t w = raw[g * 8 + half * 4 + x];
+              const uint32_t w = raw[half][g * 4 + x];
               const float x0 = __uint_as_float(w << 16) * f[(x >> 1) * 2], x1 = __uint_as_float(w & 0xffff0000u) * f[(x >> 1) * 2 + 1];
               const __nv_bfloat162 hp = __floats2bfloat162_rn(x0, x1);
-              w4[x] = *reinterpret_cast<const uint32_t*>(&hp);
+              uint32_t r = *reinterpret_cast<const uint32_t*>(&hp);
               if (lo_part) {
-                const __nv_bfloat162 lp =
-                    __floats2bfloat162_rn(x0 - __uint_as_float(w4[x] << 16), x1 - __uint_as_float(w4[x] & 0xffff0000u));
-                w4[x] = *reinterpret_cast<const uint32_t*>(&lp);
+                const __nv_bfloat162 lp = __floats2bfloat162_rn(x0 - __uint_as_float(r << 16), x1 - __uint_as_float(r & 0xffff0000u));
+                r = *reinterpret_cast<const uint32_t*>(&lp);
               }
+              raw[half][g * 4 + x] = r;
             }
-            tmem_st_16x128b_x2(colF + ((uint32_t)(half * 16) << 16) + g * 8, w4);
           }
         }
+        // (one wide store each: a store waits its turn behind the products' accumulators, 280 clocks, whatever its width)
+        tmem_st_16x128b_x8(colF, raw[0]);
+        tmem_st_16x128b_x8(colF + (16u << 16), raw[1]);
         tmem_st_wait();
       }
       if (shared_tail && Cr < 128) {
@@ -436,19 +436,27 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
         }
       }
     }
-    if (nblk > 1 || last_m3) {
+    const auto has_m3 = [&](int it) { return it + 1 < nblk || (it < nblk && last_m3); };
+    if (has_m3(0)) {
       TC_WAIT_WARP(V_FULL_C0, 0, 20);
       fetch_c(0);
       if (!write_fc(0)) goto teardown;
+    }
+    // The value rows of the next block are fetched a block ahead, since behind the operands that the products fetch this takes 800
+    // clocks (1 x 32 x 16384, bf16 results: 96 -> 92 us, dV and dK 245 -> 238) ... except where the results are twice as long and
+    // use the shared memory then (fp32: 241 -> 247).
+    constexpr bool AHEAD = sizeof(TOut) == 2;
+    if (AHEAD && has_m3(1)) {
+      TC_WAIT_WARP(V_FULL_C0 + 1, 0, 20);
+      fetch_c(1);
     }
     if (has_entry) write_state_operand();
     WARP_ARRIVE(V_Z_READY);
     for (int it = 0; it < nblk; ++it) {
       const bool more = it + 1 < nblk;
       if (!more && !last_m3) break;
-      const bool next_fc = it + 2 < nblk || (more && last_m3);
       const float gamma = ex2_approx(-s2 * (float)(it == (REV ? 0 : nblk - 1) ? edge_len : 128));
-      if (next_fc) {
+      if (!AHEAD && has_m3(it + 1)) {
         TC_WAIT_WARP(V_FULL_C0 + (it + 1) % V_STAGES, ((it + 1) / V_STAGES) & 1, 20);
         fetch_c(it + 1);
       }
@@ -466,7 +474,11 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
       }
       tc_fence_before_sync();
       if (!more) break;
-      if (next_fc && !write_fc(it + 1)) goto teardown;
+      if (has_m3(it + 1) && !write_fc(it + 1)) goto teardown;
+      if (AHEAD && has_m3(it + 2)) {
+        TC_WAIT_WARP(V_FULL_C0 + (it + 2) % V_STAGES, ((it + 2) / V_STAGES) & 1, 20);
+        fetch_c(it + 2);
+      }
       TC_WAIT_WARP(V_M2_DONE, it & 1, 23);  // the state operand has been read
       write_state_operand();
       WARP_ARRIVE(V_Z_READY);

@@ -141,8 +141,8 @@ def test_walk_kernel_with_one_barrier_for_every_block_would_be_overrun():
     assert ("producer", "dz0", 0) in found and ("producer", "o0", 0) in found
 
 
-def walk64_kernel(blocks, last_m3):
-    """tc_walk64_kernel (one warp of each group)."""
+def walk64_kernel(blocks, last_m3, ahead):
+    """tc_walk64_kernel (one warp of each group).  ahead: the state group fetches its value rows a block ahead."""
     two, three = (lambda name, n: name + str(n % 2)), (lambda name, n: name + str(n % 3))
     m3 = lambda n: n + 1 < blocks or last_m3
     producer, p, output = [], [], []
@@ -151,6 +151,8 @@ def walk64_kernel(blocks, last_m3):
     if m3(0):
         mma += [("wait", "fc", 0), ("arrive", "dz")]
         state += [("wait", "c0", 0), ("arrive", "fc")]
+    if ahead and m3(1) and blocks > 1:
+        state.append(("wait", "c1", 0))
     state.append(("arrive", "z"))
     for n in range(blocks):
         if n >= 3:
@@ -166,11 +168,15 @@ def walk64_kernel(blocks, last_m3):
         if more and m3(n + 1):
             mma += [("wait", "fc", n + 1), ("arrive", "dz")]
         p += [("wait", two("s", n), n // 2), ("arrive", two("p", n))]
+        if not ahead and more and m3(n + 1):
+            state.append(("wait", three("c", n + 1), (n + 1) // 3))
         if more or last_m3:
             state.append(("wait", "dz", n))
         if more:
             if m3(n + 1):
-                state += [("wait", three("c", n + 1), (n + 1) // 3), ("arrive", "fc")]
+                state.append(("arrive", "fc"))
+            if ahead and n + 2 < blocks and m3(n + 2):
+                state.append(("wait", three("c", n + 2), (n + 2) // 3))
             state += [("wait", "m2", n), ("arrive", "z")]
         output += [("wait", "o", n), ("arrive", "o_free")] + [("wait", "stored", n - 1)] * (n > 0)
         output += [("arrive", "staged"), ("wait", "staged", n), ("arrive", "stored")]
@@ -178,7 +184,8 @@ def walk64_kernel(blocks, last_m3):
     return roles, {op[1]: 1 for ops in roles.values() for op in ops}
 
 
+@pytest.mark.parametrize("ahead", [False, True])
 @pytest.mark.parametrize("last_m3", [False, True])
 @pytest.mark.parametrize("blocks", [1, 2, 3, 4, 5, 11])
-def test_walk64_kernel_phases_are_never_overrun(blocks, last_m3):
-    assert overruns(*walk64_kernel(blocks, last_m3)) == []
+def test_walk64_kernel_phases_are_never_overrun(blocks, last_m3, ahead):
+    assert overruns(*walk64_kernel(blocks, last_m3, ahead)) == []
