@@ -115,12 +115,14 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
   long seg_len = s->seg_len;
   if (seg_len == 0) {
     // One thread block per (batch*head, segment) and one block per SM at a time: pick the segment count with the least
-    // cost, in units of one 128-token block (about 3 us).  Depends on the shape only.
-    // Where the walk chains the segment states itself: forward walk and dQ walk, the dV and dK walks in one launch (twice
-    // the thread blocks), each in waves over the 148 SMs of (blocks of a segment + start and end), and per direction the
-    // launch that makes the states, with what each further state costs to write, read and chain.  Measured, forward plus
-    // backward: 3 x 8 heads x 3001 tokens 172 us with 1536-token segments, 141 with 512; 8 heads x 2048 118 with 1024, 92
-    // with 512, 126 with 128; 2 x 16 x 8192 289 with 2048, 344 with 1024 (the model: 49.7, 34.5 / 38, 29, 33 / 85, 97).
+    // cost.  Depends on the shape only.
+    // Where the walk chains the segment states itself, in us: forward walk and dQ walk, the dV and dK walks in one launch (twice
+    // the thread blocks), each in waves over the 148 SMs of (blocks of a segment + start and end), and the launches that make the
+    // states, with what each further state costs to write, read and chain, as far as they are not hidden behind the launches
+    // around them.  Segments of one block leave nothing to hide them behind.  Measured, forward and backward: 32 heads x 777 as one
+    // segment 23.8 + 46.1, 256 tokens 20.8 + 48.1, 128 34.1 + 76.7; 8 x 512 14.8 + 27.3, 19.8 + 26.7 and 19.4 + 23.4; 24 x 2048 with
+    // 768 tokens 34.0 + 70.0, 384 26.1 + 66.4, 256 43.3 + 100.9; 8 x 8192 with 1024 43.7 + 84.6, 512 34.6 + 82.2, 256 49.6 + 123.9;
+    // 64 x 1500 as one segment 40.9 + 84.3, two 40.0 + 96.9; 2 x 16 x 8192 with 2048 72.5 + 197.9, 1024 96.4 + 256.4.
     // CUDA-core kernels: row tiles up to ROWS_MAX_SEG tokens, whose work grows with the segment's length but which end after
     // as many tiles; else the walk block by block, one thread block to an SM at d = 128 and up to four at d = 64; and the
     // pre-passes.  Forward plus backward in fp32, us: 2 heads x 256, d = 64, 38 as one segment and 57 in two; 4 x 512 85
@@ -171,10 +173,9 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
     } else if (states_only || packed) {
       // as it stands
     } else if (p->chains) {
-      best_n = choose(s->N / 128, limit, [&](long nseg, long blocks) {
-        const double units = (double)p->BH * nseg;
-        return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 1.3) +
-               (nseg > 1 ? 2.0 * (4.0 + 0.01 * units + 0.6 * nseg) : 0.0);
+      best_n = choose((s->N + 255) / 256, limit, [&](long nseg, long blocks) {
+        return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (3.0 * blocks + 2.0) +
+               (nseg > 1 ? 17.0 + 0.75 * nseg + 0.11 * p->BH * nseg + 1e-4 * p->BH * s->N : 0.0);
       });
     } else {
       best_n = choose((s->N + 127) / 128, limit, [&](long nseg, long blocks) {
@@ -582,7 +583,11 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     LA_TRY_CUDA(run_scan(shape, p, tab, buf_kvt, nullptr, kv_in, true, 0, cs));
     from_q.entry = buf_kvt;
   }
-  if (!p.rows && !p.chains) LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
+  // Where launches begin early the states of both directions come before all walks: the dQ walk begins while they end and the other
+  // two while it ends, so that the thread blocks of a launch fill the multiprocessors that the last ones of the launch before leave
+  // idle.
+  const bool together = p.chains && early_walks(p.BH, p.nseg);
+  if (!p.rows && !together) LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
 
   // dV = rev(a = K, b = Q, c = dO) carries dKV; dK = rev(a = V, b = dO, c = Q) carries dKV^T.
   Carried from_v, from_k;
@@ -591,11 +596,11 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
     if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf_e, 1, cs));
     from_v = chained(grad_kv_out, false, buf_e, false);
     from_k = chained(grad_kv_out, true, buf_e, true);
-    // The states of both directions come before all walks: the dQ walk begins while they end and the other two while it ends,
-    // so that the thread blocks of a launch fill the multiprocessors that the last ones of the launch before leave idle.
-    from_q.follows = multi ? FOLLOWS_STATES : FOLLOWS_ANY;
-    from_v.follows = from_k.follows = FOLLOWS_WALK;
-    LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
+    if (together) {
+      from_q.follows = multi ? FOLLOWS_STATES : FOLLOWS_ANY;
+      from_v.follows = from_k.follows = FOLLOWS_WALK;
+      LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
+    }
   } else if (multi || grad_kv_out) {
     LA_TRY_CUDA(run_scan(shape, p, tab, buf_e, buf_et, grad_kv_out, false, 1, cs));
     from_v.entry = buf_e;

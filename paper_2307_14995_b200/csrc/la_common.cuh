@@ -173,7 +173,8 @@ void count_launch(int n = 1);
 // successor begin (grid_dep_launch) only after its own wait for its predecessor (grid_dep_wait), so whatever came before the predecessor is complete when a kernel begins; what the predecessor itself writes
 // needs the wait.  Kernels that do not say otherwise (Follows) wait before their first access to memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, Args&&... args) {
+cudaError_t launch_kernel(bool early, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster,
+                          Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -181,7 +182,7 @@ cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
   cfg.stream = stream;
   cudaLaunchAttribute attr[2]{};
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = early;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = (unsigned)cluster;
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
@@ -189,6 +190,14 @@ cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
   cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
+template <typename... KArgs, typename... Args>
+cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, Args&&... args) {
+  return launch_kernel(true, kern, grid, block, smem, stream, cluster, std::forward<Args>(args)...);
+}
+// Tensor-core walks and their states begin early where the thread blocks of one walk run all at once.  Where they come in several
+// waves a launch's end matters less, and held at the power limit the step is slower for it: 1 x 32 heads x 65536, 288 thread blocks
+// a walk, 2333 us with launches one after the other and 2368 with early ones; 2 x 16 x 8192, 128 thread blocks, 333 and 320.
+inline bool early_walks(int bh, int nseg) { return (long)bh * nseg <= 148; }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

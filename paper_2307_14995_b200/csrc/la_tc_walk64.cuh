@@ -7,16 +7,19 @@
 //   M3  dZ^T    [(e, e), d] = [fc_hi | fc_lo]^T b  A in tensor memory, K = 128     (fc = diag(f_state) c)
 //   M4  O_intra [i, e] = P_hi c (+ P_lo c)        A = P in tensor memory, in the place of S, K = 128
 // and the CUDA cores form P = S (.) D, out = O_intra + diag(f_out) O_inter and Z <- Gamma Z + dZ.
-// An instruction has 128 rows whatever D is, so M3 puts the hi terms of fc in lanes 0 .. 63 and the lo terms in lanes 64 .. 127:
-// one product of half the columns for both.  Its two halves stay apart: Z is the state that the hi terms add up to, Y the one of
+// An instruction has 128 rows whatever D is, so M3 puts the hi terms of fc in one half of the lanes and the lo terms in the
+// other: one product of half the columns for both.  Its two halves stay apart: Z is the state that the hi terms add up to, Y the one of
 // the lo terms, 2^-9 of it, for which one bf16 operand is as good as two for Z.  They meet in M2, and in the state that is handed
 // out.
 //
-// The only chain between blocks is Z in registers.  What bounded the walk before this one (products of zero-padded rows, fc made
-// between dZ and the next state operand by the same warps, each waiting for the other: 2.5 us a block) is taken apart: the
-// products of iteration n are M1(n+1) M2(n) M4(n) M3(n+1), about 1600 clocks, and each operand has had at least 1000 of them to
-// be made in: S(n+1) until M4 of the next iteration, dZ(n) and fc(n+1) during M1, M2, M4, the accumulators of M4(n) are read
-// during M3(n+1) and M1(n+2), the state operand is written after M2(n).
+// The only chain between blocks is Z in registers.  The walk before this one (products of zero-padded rows, fc made between dZ and
+// the next state operand by the same warps, each waiting for the other) took 2.5 us a block.  The products of iteration n are M1(n+1)
+// M2(n) M4(n) M3(n+1), 1900 clocks, and each operand is made while others run: S(n+1) has until M4 of the next iteration, dZ(n) and
+// fc(n+1) have M1, M2 and M4, the accumulators of M4(n) are read during M3(n+1) and M1(n+2), the state operand is written after M2(n).
+// A block takes 4000 to 4400 clocks where memory is not the bound (one thread block per SM, HBM: 3500 at fp32 results): the state
+// group's dZ (350), fc (2000, sharing the schedulers with scores and output) and operand (500), and M3, come one after the other.
+// Measured, us, before and after: 2 x 16 heads x 8192, fp32 results, forward 68 and 50, backward 162 and 130; 1 x 32 x 16384 117 and 92,
+// 285 and 241.
 //
 // Tensor memory (512 columns): S/P 2 x 128, O_inter 64, O_intra 64, dZ 64, fc 64.
 // Shared memory: three stages of a, b, c (48 KB each), the state operand (Z hi, Z lo, Y: 8 KB each), the output on its way to
@@ -594,7 +597,8 @@ cudaError_t launch_walk64_t(const TcMaps& m0, const TcMaps& m1, const VOutMaps& 
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ta.njobs == 2 ? K_WALK_PAIR : K_WALK, stream);
-  err = launch_early(kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(V_THREADS), smem, stream, 1, m0, m1, out, ta, tab);
+  err = launch_kernel(early_walks(ta.BH, ta.nseg), kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(V_THREADS), smem, stream, 1, m0, m1,
+                      out, ta, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }
