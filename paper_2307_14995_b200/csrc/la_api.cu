@@ -586,7 +586,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   // Where launches begin early the states of both directions come before all walks: the dQ walk begins while they end and the other
   // two while it ends, so that the thread blocks of a launch fill the multiprocessors that the last ones of the launch before leave
   // idle.
-  const bool together = p.chains && early_walks(p.BH, p.nseg);
+  const bool together = p.chains && early_walks(p.BH, p.nseg, p.seg_len);
   if (!p.rows && !together) LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
 
   // dV = rev(a = K, b = Q, c = dO) carries dKV; dK = rev(a = V, b = dO, c = Q) carries dKV^T.

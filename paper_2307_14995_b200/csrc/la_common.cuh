@@ -194,10 +194,12 @@ template <typename... KArgs, typename... Args>
 cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, Args&&... args) {
   return launch_kernel(true, kern, grid, block, smem, stream, cluster, std::forward<Args>(args)...);
 }
-// Tensor-core walks and their states begin early where the thread blocks of one walk run all at once.  Where they come in several
-// waves a launch's end matters less, and held at the power limit the step is slower for it: 1 x 32 heads x 65536, 288 thread blocks
-// a walk, 2333 us with launches one after the other and 2368 with early ones; 2 x 16 x 8192, 128 thread blocks, 333 and 320.
-inline bool early_walks(int bh, int nseg) { return (long)bh * nseg <= 148; }
+// Tensor-core walks and their states begin early where the thread blocks of one walk run all at once and are not long.  Where they
+// come in several waves or run for long a launch's end matters less, and held at the power limit the step is slower for it: 1 x 32
+// heads x 65536, 288 thread blocks a walk, 2333 us with launches one after the other and 2368 with early ones; 1 x 16 x 51521, 144
+// thread blocks of 45 blocks, 920 and 932; 128 thread blocks: 1 x 32 x 16384, 32 blocks each, 639 and 634; 2 x 16 x 8192, 16 blocks,
+// 333 and 320.
+inline bool early_walks(int bh, int nseg, int seg_len) { return (long)bh * nseg <= 148 && seg_len <= 4096; }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -829,7 +829,7 @@ cudaError_t launch_prefix(const ScanArgs& args, const DecayTable& tab, cudaStrea
   if ((args.Da * args.Ec) % 1024 != 0 || args.BH > 65535) return cudaErrorInvalidValue;
   KernelTimer timer(K_SCAN, stream);
   const cudaError_t err =
-      launch_kernel(early_walks(args.BH, args.nseg), prefix_kernel, dim3((unsigned)(args.Da * args.Ec / 1024), (unsigned)args.BH),
+      launch_kernel(early_walks(args.BH, args.nseg, args.seg_len), prefix_kernel, dim3((unsigned)(args.Da * args.Ec / 1024), (unsigned)args.BH),
                     dim3(256), 0, stream, 1, args, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();

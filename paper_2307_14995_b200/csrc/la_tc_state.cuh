@@ -417,7 +417,7 @@ cudaError_t launch_state_t(const TcMaps& m, const TcArgs& ta, const DecayTable& 
   const long other_units = (long)(ta.H - plan.n_shared) * (ta.BH / ta.H) * plan.nseg_used;
   const long clusters = shared_units + (other_units + plan.cluster - 1) / plan.cluster;
   KernelTimer timer(K_PREPASS, stream);
-  err = launch_kernel(early_walks(ta.BH, ta.nseg), kern, dim3((unsigned)(clusters * plan.cluster)), dim3(S_THREADS), smem, stream, plan.cluster,
+  err = launch_kernel(early_walks(ta.BH, ta.nseg, ta.seg_len), kern, dim3((unsigned)(clusters * plan.cluster)), dim3(S_THREADS), smem, stream, plan.cluster,
                       m.b, m.c, ta, plan, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();

@@ -179,7 +179,8 @@ __device__ __forceinline__ float2 octet_sums(const float (&v)[16], int lane) {
 // readers of a tile run side by side and the tile comes from HBM once.
 // GATED (forward, single job): the epilogue y = SRMSNorm(out) (.) u of Eq. 3 with Eq. 8 is applied to the rows
 // before they leave (job.u, job.y; job.rstd optional); 1: y alone, 2: out as well.
-template <bool REV, typename TOut, int GATED>
+// EARLY: launched while the launch before it ends (see Follows).
+template <bool REV, typename TOut, int GATED, bool EARLY>
 __global__ void __launch_bounds__(W_THREADS, 1)
 tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcMaps maps1,
                const __grid_constant__ TcArgs args, const __grid_constant__ DecayTable tab) {
@@ -187,7 +188,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   WSmem<REV>& sm = *reinterpret_cast<WSmem<REV>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (args.follows == FOLLOWS_ANY && args.seq_start) grid_dep_wait();  // the tables of a packed batch
+  if (EARLY && args.follows == FOLLOWS_ANY && args.seq_start) grid_dep_wait();  // the tables of a packed batch
   const int jobid = (args.njobs == 2) ? (int)(blockIdx.x & 1) : 0;
   const int bidx = (args.njobs == 2) ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const TcJob& job = args.job[jobid];
@@ -244,7 +245,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = sm.tmem_slot;
-  if (args.follows == FOLLOWS_ANY) {
+  if (EARLY && args.follows == FOLLOWS_ANY) {
     grid_dep_wait();
     grid_dep_launch();
   }
@@ -461,7 +462,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], __ldg(r1 + x * 128));
         }
       };
-      if (args.follows == FOLLOWS_STATES) {
+      if (EARLY && args.follows == FOLLOWS_STATES) {
         grid_dep_wait();
         grid_dep_launch();
       }
@@ -746,7 +747,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
   }
 
 teardown:
-  if (args.follows != FOLLOWS_ANY) grid_dep_wait();  // (a launch is complete only when those before it are)
+  if (EARLY && args.follows != FOLLOWS_ANY) grid_dep_wait();  // (a launch is complete only when those before it are)
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
@@ -756,12 +757,12 @@ template <bool REV, typename TOut, int GATED>
 cudaError_t launch_walk_t(const TcMaps& m0, const TcMaps& m1, const TcArgs& ta, const DecayTable& tab, cudaStream_t stream) {
   const size_t smem = sizeof(WSmem<REV>) + 1024;
   static_assert(sizeof(WSmem<REV>) + 1024 <= 232448, "shared memory of one SM");
-  auto kern = tc_walk_kernel<REV, TOut, GATED>;
+  const bool early = early_walks(ta.BH, ta.nseg, ta.seg_len);
+  auto kern = early ? tc_walk_kernel<REV, TOut, GATED, true> : tc_walk_kernel<REV, TOut, GATED, false>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ta.njobs == 2 ? K_WALK_PAIR : K_WALK, stream);
-  err = launch_kernel(early_walks(ta.BH, ta.nseg), kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(W_THREADS), smem, stream, 1, m0, m1,
-                      ta, tab);
+  err = launch_kernel(early, kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(W_THREADS), smem, stream, 1, m0, m1, ta, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }

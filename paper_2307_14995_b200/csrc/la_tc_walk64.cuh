@@ -597,7 +597,7 @@ cudaError_t launch_walk64_t(const TcMaps& m0, const TcMaps& m1, const VOutMaps& 
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ta.njobs == 2 ? K_WALK_PAIR : K_WALK, stream);
-  err = launch_kernel(early_walks(ta.BH, ta.nseg), kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(V_THREADS), smem, stream, 1, m0, m1,
+  err = launch_kernel(early_walks(ta.BH, ta.nseg, ta.seg_len), kern, dim3((unsigned)(ta.BH * ta.nseg * ta.njobs)), dim3(V_THREADS), smem, stream, 1, m0, m1,
                       out, ta, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
