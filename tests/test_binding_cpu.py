@@ -43,3 +43,51 @@ def test_current_stream_without_the_private_functions(monkeypatch, missing):
     assert la._stream(None) == 5 and la._stream(Stream) == 77
     monkeypatch.setattr(la, missing, None)
     assert la._stream(None) == 77
+
+
+def test_argument_kinds_are_those_of_the_header(monkeypatch):
+    """Every call on device tensors names its arguments as the C prototype has them."""
+    import inspect
+    import os
+    import re
+    header = open(os.path.join(os.path.dirname(la.LIB_PATH), "..", "include", "la.h")).read()
+    header = re.sub(r"/\*.*?\*/|//[^\n]*", "", header, flags=re.S)
+    want = {}
+    for name, args in re.findall(r"la_status\s+(la_\w+)\(([^;]*?)\);", header, re.S):
+        kinds = ""
+        for a in (" ".join(x.split()) for x in args.split(",")):
+            if "la_shape" in a:
+                kinds += "s"
+            elif a == "void* stream":
+                kinds += "r"
+            elif a.endswith("_host"):
+                kinds += "h"
+            else:
+                kinds += "t" if "*" in a else "i"
+        want[name] = kinds
+    want["la_bwd"] = want["la_bwd_reuse"]
+    got = []
+    monkeypatch.setattr(la, "_enter", lambda name, kinds, *args: got.append((name, kinds, len(args))))
+    lam, cu = [1.0], [0, 1]
+    for name in ("la_fwd", "la_fwd_gated", "la_gate_fwd", "la_gate_bwd", "la_fwd_noalloc", "la_bwd", "la_decode_step", "la_decode_steps",
+                 "la_fwd_varlen", "la_bwd_varlen", "la_chunk_state", "la_chain_states", "la_lrpe_fwd", "la_lrpe_bwd"):
+        f = getattr(la, name)
+        given = {p: lam if p == "lam" else cu if p == "cu_seqlens" else
+                 0 if p in ("reverse", "total_tokens", "chunk_tokens", "num_chunks", "chunk", "pos0") else None
+                 for p in inspect.signature(f).parameters}
+        f(**given)
+        assert got[-1] == (name, want[name], len(want[name]))
+
+
+@pytest.mark.parametrize("args,error", [
+    (("shape", torch.zeros(4)), ValueError),          # a tensor that is not on a GPU
+    (("shape", 5), AttributeError),                   # an address instead of a tensor
+    (("shape", b"abc"), AttributeError),
+    ((5, None), TypeError),                           # an address instead of a shape
+    ((None, None), TypeError),
+])
+def test_arguments_that_are_refused(args, error):
+    shape = la.make_shape(1, 1, 1, 64, 64, torch.bfloat16, torch.float32)
+    first, q = args
+    with pytest.raises(error):
+        la.la_decode_step(shape if first == "shape" else first, q, None, None, [1.0], None, None)
