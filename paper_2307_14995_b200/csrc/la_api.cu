@@ -129,9 +129,9 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
     // and 65; 2 x 2048 205 with 512-token segments, 122 with 256, 81 with 128; 16 x 2048, d = 128, 946, 652 and 488.  Where the heads
     // fill the chip a state costs more than it saves: 256 x 512, d = 64, 747 with 128-token segments and 605 as one; 256 x 4096
     // 7769 with 1024 and 6383 as one; 128 x 2048, d = 128, 6560 with 1024 and 5384 as one.
-    // Tensor cores at d = 64: the same waves, at about 2.5 us a block; pre-passes and scans take about 24 us and 0.17 us a
-    // state.  Measured: 8 heads x 777 62 us as one segment, 43 with 128-token segments; 8 x 2048 94 with 1024, 54 with 256;
-    // 16 x 4096 100 with 1024, 89 with 512; 4 x 16 x 2048 130 with 1024, 161 with 512.
+    // Tensor cores at d = 64: waves of blocks too, in units of one block (about 2.2 us).  Measured, forward and backward: 8 heads x 777
+    // as one segment 18.4 + 32.3 us, 256 tokens 12.6 + 18.6, 128 13.7 + 20.0; 4 x 16 x 2048 40.9 + 84.6, with 1024 tokens 32.7 + 80.1,
+    // 512 37.5 + 96.6; 16 x 8192 with 2048 48.0 + 93.6, 1024 36.0 + 87.2, 512 44.0 + 104.4.
     // Packed batches: waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.  On the tensor cores la_chunk_state
     // takes the same rule: 32 heads x 777 22.5 us with the walk's segments, 16.4 with one; 16 x 2048 20.5 and 16.4; 8 x 8192 20.5
     // and 16.4; d = 64, 4 x 16 x 2048 20.5 and 14.4.

@@ -17,8 +17,8 @@
 // the one array, so two calls that may overlap on the GPU (different streams) race on it; calls
 // on one stream are safe.  The array keeps whatever the previous call left, which is harmless:
 // the forward pass writes every scratch element it later reads (the pre-pass fills the segment-local
-// states before a scan or a walk reads them; at d = 128 the last segment's, which nothing reads, is left
-// out), so nothing has to start at zero.
+// states before a scan or a walk reads them; on the tensor cores the last segment's, which nothing reads, is
+// left out), so nothing has to start at zero.
 //
 // This file makes no cudaMalloc / cudaFree call and calls no allocating library routine.
 #include <cuda_runtime.h>
