@@ -92,12 +92,6 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
       "r"(c3)
       : "memory");
 }
-__device__ __forceinline__ void tma_prefetch_4d(const CUtensorMap* m, int c0, int c1, int c2, int c3) {
-  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(
-                   reinterpret_cast<uint64_t>(m)),
-               "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-               : "memory");
-}
 __device__ __forceinline__ void tma_store_4d(const CUtensorMap* m, const void* smem_src, int c0, int c1, int c2, int c3) {
   asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
                    reinterpret_cast<uint64_t>(m)),
@@ -109,7 +103,6 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void tma_store_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
-__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 
 // ---- TMEM ----------------------------------------------------------------------------------------
@@ -142,11 +135,6 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N, bool a_mn_m
          | (1u << 10)                    // B format: bf16
          | ((a_mn_major ? 1u : 0u) << 15) | ((b_mn_major ? 1u : 0u) << 16) |
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-// Arrives on the mbarrier once all tcgen05.mma issued so far by this thread have completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
 }
 
 // ---- TMEM loads: 32 lanes x 32-bit, N consecutive columns per thread ------------------------------
@@ -187,12 +175,7 @@ __device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, uint32_t (&r)
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// ---- TMEM stores: 32 lanes x 32-bit, 8 consecutive columns per thread ---------------------------
-__device__ __forceinline__ void tmem_st_x8(uint32_t taddr, const uint32_t (&r)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
+// ---- TMEM stores: 32 lanes x 32-bit, N consecutive columns per thread ---------------------------
 __device__ __forceinline__ void tmem_st_x4(uint32_t taddr, const uint4& r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r.x), "r"(r.y), "r"(r.z),
                "r"(r.w)
@@ -214,12 +197,7 @@ __device__ __forceinline__ void tmem_st_16x128b_x2(uint32_t taddr, const uint32_
                "r"(r[3])
                : "memory");
 }
-// The same with 16 or 32 columns.
-__device__ __forceinline__ void tmem_st_16x128b_x4(uint32_t taddr, const uint32_t (&r)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
-               "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
+// The same with 32 columns.
 __device__ __forceinline__ void tmem_st_16x128b_x8(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], "
@@ -249,20 +227,6 @@ __device__ __forceinline__ uint32_t elect_one() {
   uint32_t el;
   asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(el));
   return el;
-}
-// D[tmem] (+)= A[smem] * B[smem] with descriptors as (low half, common high half); takes effect only
-// in lanes with go != 0.
-__device__ __forceinline__ void umma_bf16_lh(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                             uint32_t idesc, uint32_t accumulate, uint32_t go) {
-  asm volatile(
-      "{\n\t.reg .pred p, g;\n\t.reg .b64 da, db;\n\t"
-      "setp.ne.b32 g, %6, 0;\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
-      "mov.b64 da, {%1, %3};\n\t"
-      "mov.b64 db, {%2, %3};\n\t"
-      "@g tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(go)
-      : "memory");
 }
 // A whole K loop in one instruction sequence: NK tensor-core instructions D[tmem] (+)= A_k * B_k, k = 0..NK-1,
 // all predicated on `go`, the first one accumulating only if `acc0`.  Operand k is operand 0 moved by a
@@ -394,6 +358,7 @@ __device__ __forceinline__ void umma_tri4(uint32_t d_tmem, uint32_t a_lo, uint32
       : "memory");
 }
 #undef LA_UMMA_TRI_STEP
+// Arrives on the mbarrier once all tcgen05.mma issued so far by this thread have completed; takes effect only in lanes with go != 0.
 __device__ __forceinline__ void umma_commit_if(uint64_t* bar, uint32_t go) {
   asm volatile(
       "{\n\t.reg .pred g;\n\tsetp.ne.b32 g, %1, 0;\n\t"
