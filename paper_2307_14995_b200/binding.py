@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 from typing import Optional
 
 import torch
@@ -48,12 +49,17 @@ class LaError(RuntimeError):
 
 _lib = None
 _call, _address = None, {}  # _la_call.call, and where the C functions are
+_loading = threading.Lock()
 
 
 def load():
     """Load the shared library (raises if it has not been built)."""
-    global _lib
-    if _lib is None:
+    global _lib, _call, _address
+    if _lib is not None:
+        return _lib
+    with _loading:
+        if _lib is not None:
+            return _lib
         if not os.path.exists(LIB_PATH):
             raise RuntimeError("CUDA library %s is missing; run `python -m paper_2307_14995_b200.build`"
                                % LIB_PATH)
@@ -124,10 +130,11 @@ def load():
             from . import _la_call
         except ImportError as e:
             raise RuntimeError("extension module _la_call is missing; run `python -m paper_2307_14995_b200.build`") from e
-        global _call
-        _address.update((name, ctypes.cast(getattr(lib, name), ctypes.c_void_p).value) for name in EXPORTS)
+        address = {name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in EXPORTS}
+        address["la_bwd"] = address["la_bwd_reuse"]  # (the same with a NULL fwd_workspace)
         _la_call.bind(LaShape, lambda stream: _stream(stream))
-        _address["la_bwd"] = _address["la_bwd_reuse"]  # (the same with a NULL fwd_workspace)
+        # whoever sees _call finds the whole table behind it
+        _address = address
         _call = _la_call.call
         _lib = lib
     return _lib

@@ -91,3 +91,37 @@ def test_arguments_that_are_refused(args, error):
     first, q = args
     with pytest.raises(error):
         la.la_decode_step(shape if first == "shape" else first, q, None, None, [1.0], None, None)
+
+
+def test_first_use_from_several_threads(monkeypatch):
+    """No thread may find a call that is ready to be made while the table of addresses still changes."""
+    import sys
+    import threading
+    la.load()
+    want = dict(la._address)
+    assert want["la_bwd"] == want["la_bwd_reuse"]  # (la_bwd passes the forward pass's workspace too)
+    wrong = []
+
+    def first_use(start):
+        start.wait()
+        if la._call is None:
+            la.load()
+        for _ in range(50):
+            if dict(la._address) != want:
+                wrong.append(dict(la._address))
+
+    interval = sys.getswitchinterval()
+    sys.setswitchinterval(1e-6)
+    try:
+        for _ in range(100):
+            for name, value in (("_lib", None), ("_call", None), ("_address", {})):
+                monkeypatch.setattr(la, name, value)
+            start = threading.Barrier(4)
+            threads = [threading.Thread(target=first_use, args=(start,)) for _ in range(4)]
+            for t in threads:
+                t.start()
+            for t in threads:
+                t.join()
+    finally:
+        sys.setswitchinterval(interval)
+    assert not wrong
