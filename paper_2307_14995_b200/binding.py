@@ -132,7 +132,7 @@ def load():
             raise RuntimeError("extension module _la_call is missing; run `python -m paper_2307_14995_b200.build`") from e
         address = {name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in EXPORTS}
         address["la_bwd"] = address["la_bwd_reuse"]  # (the same with a NULL fwd_workspace)
-        _la_call.bind(LaShape, lambda stream: _stream(stream))
+        _la_call.bind(LaShape, _handle)
         # whoever sees _call finds the whole table behind it
         _address = address
         _call = _la_call.call
@@ -243,6 +243,12 @@ def _stream(stream):
     if _RAW_STREAM is None or _CURRENT_DEVICE is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
     return _RAW_STREAM(_CURRENT_DEVICE())
+
+
+def _handle(stream) -> int:
+    h = _stream(stream)
+    # (another library's stream object may keep None or a c_void_p)
+    return h if type(h) is int else ctypes.cast(h, ctypes.c_void_p).value or 0
 
 
 def alloc_workspace(op: int, shape: LaShape, device) -> Optional[torch.Tensor]:

@@ -125,3 +125,25 @@ def test_first_use_from_several_threads(monkeypatch):
     finally:
         sys.setswitchinterval(interval)
     assert not wrong
+
+
+@pytest.mark.parametrize("handle,want", [(77, 77), (None, 0), (ctypes.c_void_p(77), 77), (ctypes.c_void_p(None), 0)])
+def test_streams_of_other_libraries(handle, want):
+    """A stream is any object with a handle; what ctypes takes for a pointer is one."""
+    class Stream:
+        cuda_stream = handle
+
+    got = []
+    callback = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p)(lambda p: got.append(p or 0) or 0)
+    la.load()
+    assert la._call(ctypes.cast(callback, ctypes.c_void_p).value, "r", Stream) == 0
+    assert got == [want]
+
+
+def test_a_stream_that_is_no_handle_is_refused():
+    class Stream:
+        cuda_stream = 1.5
+
+    la.load()
+    with pytest.raises((TypeError, ctypes.ArgumentError)):
+        la._call(la._address["la_version"], "r", Stream)
