@@ -3,7 +3,9 @@
     python -m paper_2307_14995_b200.build [--force] [--verbose]
 
 Produces ``paper_2307_14995_b200/libla_b200.so`` (C ABI declared in
-``include/la.h``) and ``paper_2307_14995_b200/_la_call.so``.  nvcc cross-compiles without a GPU.
+``include/la.h``) and the extension module ``_la_call``, whose file name carries the tag of the interpreter that it was
+built for, so that no other one loads it.  Needs nvcc (which cross-compiles without a GPU), a C compiler ($CC, or gcc) and
+Python's headers.
 """
 from __future__ import annotations
 
@@ -15,7 +17,8 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libla_b200.so")
-CALL = os.path.join(HERE, "_la_call.so")
+CALL = os.path.join(HERE, "_la_call" + sysconfig.get_config_var("EXT_SUFFIX"))
+UNTAGGED_CALL = os.path.join(HERE, "_la_call.so")  # as it was once built: any interpreter would load it
 SOURCES = ["la_api.cu", "la_simt.cu", "la_decode.cu", "la_tc.cu", "la_noalloc.cu", "la_gate.cu", "la_lrpe.cu"]
 HEADERS = ["la_common.cuh", os.path.join("..", "..", "include", "la.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -64,6 +67,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
                                src, "-o", tmp])
         os.replace(tmp, CALL)
+    if os.path.exists(UNTAGGED_CALL):
+        os.remove(UNTAGGED_CALL)
     return LIB
 
 

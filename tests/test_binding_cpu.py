@@ -147,3 +147,13 @@ def test_a_stream_that_is_no_handle_is_refused():
     la.load()
     with pytest.raises((TypeError, ctypes.ArgumentError)):
         la._call(la._address["la_version"], "r", Stream)
+
+
+def test_the_extension_module_is_this_interpreters():
+    import importlib.machinery
+    from paper_2307_14995_b200 import build
+    build.build()
+    la.load()
+    from paper_2307_14995_b200 import _la_call
+    suffix = importlib.machinery.EXTENSION_SUFFIXES[0]  # the one with the interpreter's tag
+    assert suffix != ".so" and _la_call.__file__.endswith("_la_call" + suffix)
