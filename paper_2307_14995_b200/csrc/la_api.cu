@@ -50,6 +50,26 @@ struct Packed {
   int total_tokens;
 };
 
+// Part of the table of a packed batch, as a kernel's argument: a launch keeps its own copy, in a stream and in a captured graph alike.  (A copy from
+// host memory that is gone when the call returns would be read again by every replay.)
+template <int N>
+struct TablePart {
+  int v[N];
+};
+template <int N>
+__global__ void __launch_bounds__(256) table_kernel(int* dst, int n, const __grid_constant__ TablePart<N> part) {
+  grid_dep_wait();
+  grid_dep_launch();
+  for (int i = threadIdx.x; i < n; i += 256) dst[i] = part.v[i];
+}
+template <int N>
+cudaError_t put_table(int* dst, const int* src, int n, cudaStream_t cs) {
+  TablePart<N> part;
+  std::copy(src, src + n, part.v);
+  std::fill(part.v + n, part.v + N, 0);
+  return launch_early(table_kernel<N>, dim3(1), dim3(256), 0, cs, 1, dst, n, part);
+}
+
 // A folded batch: entries t and t + batches of the shape's B = 2 * batches read the same entry t of the tensors named here;
 // of the output `out` the second half goes to out2.
 struct Folded {
@@ -966,7 +986,7 @@ bool packed_fits(int op, const la_shape* sp, const void* workspace, size_t works
          workspace_bytes >= packed_table_bytes(sp->B) + w;
 }
 
-// Copies first tokens and lengths to the head of the workspace (stream-ordered) and describes them.
+// Puts first tokens and lengths at the head of the workspace (stream-ordered) and describes them.
 la_status packed_upload(const int* cu, int S, int total, void* workspace, cudaStream_t cs, Packed* pk) {
   std::vector<int> host(3 * (size_t)S);
   for (int i = 0; i < S; ++i) {
@@ -976,9 +996,13 @@ la_status packed_upload(const int* cu, int S, int total, void* workspace, cudaSt
   }
   // longest first (ties in the caller's order): the thread blocks of a launch are handed out in index order
   std::stable_sort(host.begin() + 2 * S, host.end(), [&](int a, int b) { return host[S + a] > host[S + b]; });
-  // pageable source: the runtime has taken its copy of the table by the time the call returns
-  if (cudaMemcpyAsync(workspace, host.data(), host.size() * sizeof(int), cudaMemcpyHostToDevice, cs) != cudaSuccess)
-    return LA_ERR_CUDA;
+  // (arguments of a launch: 4 KB for up to 333 sequences, else 32 KB at a time)
+  constexpr size_t SMALL = 1000, LARGE = 8000;
+  int* const dst = static_cast<int*>(workspace);
+  for (size_t at = 0; at < host.size(); at += LARGE) {
+    const size_t n = std::min(LARGE, host.size() - at);
+    LA_TRY_CUDA(n <= SMALL ? put_table<SMALL>(dst + at, &host[at], (int)n, cs) : put_table<LARGE>(dst + at, &host[at], (int)n, cs));
+  }
   pk->start = static_cast<const int*>(workspace);
   pk->len = pk->start + S;
   pk->order = pk->start + 2 * S;

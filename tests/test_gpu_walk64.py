@@ -94,3 +94,69 @@ def test_state_after_the_last_block(N, precision):
     for g, r in zip((o, kv), ref):
         rms = np.sqrt(np.mean(r * r, axis=(2, 3), keepdims=True))
         assert np.all(np.abs(g.cpu().double().numpy() - r) <= tol * rms + 2 * tol * np.abs(r))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_packed_calls_in_a_graph(d):
+    """A captured call keeps its own copy of the sequences' places."""
+    lens = [300, 1, 127, 128, 700, 5]
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    T = cu[-1]
+    shape = la.make_shape(1, H, T, d, d, torch.bfloat16, torch.float32, 256, layout=la.LA_LAYOUT_BNHD)
+    ws = [torch.empty(la.varlen_workspace_bytes(op, shape, cu), dtype=torch.uint8, device="cuda") for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    gen = torch.Generator().manual_seed(9)
+    inputs = [[torch.randn(1, T, H, d, generator=gen).bfloat16().cuda() for _ in range(4)] for _ in range(2)]
+    x = [torch.empty_like(t) for t in inputs[0]]
+    out = [torch.empty(1, T, H, d, device="cuda") for _ in range(4)]
+
+    def step():
+        la.la_fwd_varlen(shape, *x[:3], LAM, out[0], cu, None, None, ws[0])
+        la.la_bwd_varlen(shape, *x, LAM, *out[1:], cu, workspace=ws[1])
+
+    want = []
+    for given in inputs:
+        for t, s in zip(x, given):
+            t.copy_(s)
+        step()
+        want.append([t.clone() for t in out])
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        step()
+    for w in ws:  # what an earlier call left is not what the replay reads
+        w.zero_()
+    for given, expect in zip(inputs, want):
+        for t, s in zip(x, given):
+            t.copy_(s)
+        for t in out:
+            t.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(out, expect))
+    la.device_status()
+
+
+@pytest.mark.parametrize("S", [333, 334, 2666, 2667, 5334])
+def test_packed_tables_of_many_sequences(S):
+    """The table goes in launches of up to 1000 or 8000 numbers, three for a sequence."""
+    cu = np.concatenate([[0], np.cumsum(1 + np.arange(S) % 3)]).tolist()
+    T = cu[-1]
+    gen = torch.Generator().manual_seed(S)
+    q, k, v = [torch.randn(1, T, 1, D, generator=gen).bfloat16().cuda() for _ in range(3)]
+    shape = la.make_shape(1, 1, T, D, D, torch.bfloat16, torch.float32, layout=la.LA_LAYOUT_BNHD)
+    o = torch.full((1, T, 1, D), float("nan"), device="cuda")
+    ws = torch.empty(la.varlen_workspace_bytes(la.LA_OP_FWD, shape, cu), dtype=torch.uint8, device="cuda")
+    n = la.launch_count()
+    la.la_fwd_varlen(shape, q, k, v, torch.tensor([0.5]), o, cu, None, None, ws)
+    assert la.launch_count() - n == 1
+    torch.cuda.synchronize()
+    la.device_status()
+    # every sequence has up to three tokens: token t sees itself and the one or two before it in its sequence
+    q, k, v = [t[0, :, 0].double().cpu() for t in (q, k, v)]
+    want = torch.zeros(T, D, dtype=torch.float64)
+    place = torch.arange(T) - torch.tensor(cu)[torch.searchsorted(torch.tensor(cu), torch.arange(T), right=True) - 1]
+    for back in range(3):
+        t = torch.nonzero(place >= back)[:, 0]
+        want[t] += 0.5 ** back * (q[t] * k[t - back]).sum(1, keepdim=True) * v[t - back]
+    rms = want.pow(2).mean().sqrt()
+    assert (o[0, :, 0].double().cpu() - want).abs().max() <= 1.7e-4 * rms * 5  # (single rows reach several times the tensor's RMS)
