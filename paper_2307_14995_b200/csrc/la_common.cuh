@@ -170,8 +170,9 @@ unsigned int tc_read_status(bool clear);
 void count_launch(int n = 1);
 
 // Launches that may begin while the launch before them on the stream ends (programmatic dependent launch).  A kernel lets its
-// successor begin (grid_dep_launch) only after its own wait for its predecessor (grid_dep_wait), so whatever came before the predecessor is complete when a kernel begins; what the predecessor itself writes
-// needs the wait.  Kernels that do not say otherwise (Follows) wait before their first access to memory.
+// successor begin (grid_dep_launch) only after its own wait for its predecessor (grid_dep_wait), so whatever came before the
+// predecessor is complete when a kernel begins; what the predecessor itself writes needs the wait.  Kernels that do not say
+// otherwise (Follows) wait before their first access to memory.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_kernel(bool early, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster,
                           Args&&... args) {
@@ -204,6 +205,9 @@ __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.w
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // What a walk needs of the launch before it on the stream.
+// Tensor memory: a kernel takes its columns before it lets its successor begin, so a walk behind a launch of its own call (FOLLOWS_STATES,
+// FOLLOWS_WALK) may take its own at once.  The first launch of a call waits first: what is ahead of it may be another library's kernel
+// that let it begin with columns of its own still to come, which would then wait for a thread block that waits for it.
 enum Follows {
   FOLLOWS_ANY = 0,     // the first launch of a call: everything
   FOLLOWS_STATES = 1,  // the states that it chains; its other inputs were complete before that launch began

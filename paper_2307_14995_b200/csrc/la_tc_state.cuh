@@ -136,6 +136,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap map_b, const __grid_constant
     tma_prefetch_desc(&map_c);
   }
   if (warp == 1) {
+    grid_dep_wait();  // (see Follows)
     tmem_alloc(&sm.tmem_slot, S_TMEM_COLS);
     tmem_relinquish();
   }

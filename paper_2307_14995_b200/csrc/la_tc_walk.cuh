@@ -224,6 +224,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
     fence_mbar_init();
   }
   if (warp == 1) {
+    if (EARLY && args.follows == FOLLOWS_ANY) grid_dep_wait();  // (see Follows)
     tmem_alloc(&sm.tmem_slot, TMEM_COLS);
     tmem_relinquish();
   }

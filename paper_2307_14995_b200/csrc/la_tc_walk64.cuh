@@ -122,6 +122,7 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
     fence_mbar_init();
   }
   if (warp == 1) {
+    if (args.follows == FOLLOWS_ANY) grid_dep_wait();  // (see Follows)
     tmem_alloc(&sm.tmem_slot, TMEM_COLS);
     tmem_relinquish();
   }
