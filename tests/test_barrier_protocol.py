@@ -141,19 +141,23 @@ def test_walk_kernel_with_one_barrier_for_every_block_would_be_overrun():
     assert ("producer", "dz0", 0) in found and ("producer", "o0", 0) in found
 
 
-def walk64_kernel(blocks, last_m3, ahead):
-    """tc_walk64_kernel (one warp of each group).  ahead: the state group fetches its value rows a block ahead."""
+def walk64_kernel(blocks, last_m3, ahead, tail=None, final=False):
+    """tc_walk64_kernel (one warp of each group, of the state group one with the hi and one with the lo terms).  ahead: the state
+    group fetches its value rows a block ahead.  tail: the block, if any, that a packed sequence ends in, whose rows past the end it
+    clears and whose results leave row by row.  final: the state is handed out (last_m3)."""
     two, three = (lambda name, n: name + str(n % 2)), (lambda name, n: name + str(n % 3))
     m3 = lambda n: n + 1 < blocks or last_m3
     producer, p, output = [], [], []
     mma = [("wait", "ab0", 0), ("arrive", "s0")]
     state = []
+    fc = lambda n: [("wait", three("ab", n), n // 3)] * (n == tail) + [("arrive", "fc")]
     if m3(0):
         mma += [("wait", "fc", 0), ("arrive", "dz")]
-        state += [("wait", "c0", 0), ("arrive", "fc")]
+        state += [("wait", "c0", 0)] + fc(0)
     if ahead and m3(1) and blocks > 1:
         state.append(("wait", "c1", 0))
     state.append(("arrive", "z"))
+    staged = 0
     for n in range(blocks):
         if n >= 3:
             producer.append(("wait", three("free", n), n // 3 - 1))
@@ -174,14 +178,21 @@ def walk64_kernel(blocks, last_m3, ahead):
             state.append(("wait", "dz", n))
         if more:
             if m3(n + 1):
-                state.append(("arrive", "fc"))
+                state += fc(n + 1)
             if ahead and n + 2 < blocks and m3(n + 2):
                 state.append(("wait", three("c", n + 2), (n + 2) // 3))
             state += [("wait", "m2", n), ("arrive", "z")]
-        output += [("wait", "o", n), ("arrive", "o_free")] + [("wait", "stored", n - 1)] * (n > 0)
-        output += [("arrive", "staged"), ("wait", "staged", n), ("arrive", "stored")]
-    roles = {"producer": producer, "mma": mma, "p": p, "state": state, "output": output}
-    return roles, {op[1]: 1 for ops in roles.values() for op in ops}
+        output += [("wait", "o", n), ("arrive", "o_free")]
+        if n != tail:
+            output += [("wait", "stored", staged - 1)] * (staged > 0) + [("arrive", "staged"), ("wait", "staged", staged), ("arrive", "stored")]
+            staged += 1
+    # the lo terms' state leaves through the place of the state operand, once the last product has read that
+    lo = [("wait", "m2", blocks - 1), ("arrive", "final")] if final else []
+    hi = [("wait", "final", 0)] if final else []
+    roles = {"producer": producer, "mma": mma, "p": p, "state_hi": state + hi, "state_lo": state + lo, "output": output}
+    counts = {op[1]: 1 for ops in roles.values() for op in ops}
+    counts.update({"fc": 2, "z": 2})
+    return roles, counts
 
 
 @pytest.mark.parametrize("ahead", [False, True])
@@ -189,3 +200,16 @@ def walk64_kernel(blocks, last_m3, ahead):
 @pytest.mark.parametrize("blocks", [1, 2, 3, 4, 5, 11])
 def test_walk64_kernel_phases_are_never_overrun(blocks, last_m3, ahead):
     assert overruns(*walk64_kernel(blocks, last_m3, ahead)) == []
+
+
+@pytest.mark.parametrize("ahead", [False, True])
+@pytest.mark.parametrize("final", [False, True])
+@pytest.mark.parametrize("reverse", [False, True])
+@pytest.mark.parametrize("blocks", [1, 2, 3, 4, 5, 11])
+def test_walk64_kernel_phases_are_never_overrun_at_the_ends_of_sequences(blocks, reverse, final, ahead):
+    """The state that is handed out, and a packed sequence that ends inside a block: the last one of a forward walk, which then has
+    an M3 so that the rows past the end are cleared before M4, or the first one of a reverse walk."""
+    last_m3 = final or not reverse or blocks == 1
+    assert overruns(*walk64_kernel(blocks, last_m3, ahead, tail=0 if reverse else blocks - 1, final=final)) == []
+    if final:
+        assert overruns(*walk64_kernel(blocks, True, ahead, final=True)) == []
