@@ -202,6 +202,14 @@ cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
 // 333 and 320.
 inline bool early_walks(int bh, int nseg, int seg_len) { return (long)bh * nseg <= 148 && seg_len <= 4096; }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... and loads come behind it: never through the read-only path (ld.global.nc: __ldg, or a const __restrict__ parameter of the kernel),
+// which is for memory that nobody writes from a kernel's beginning on, nor by an instruction that the compiler may move ahead of the
+// wait.  Evict-first:
+__device__ __forceinline__ float4 ld_f4_streaming(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // What a walk needs of the launch before it on the stream.

@@ -23,8 +23,7 @@ constexpr int CHUNK = 8;  // tokens whose inputs are on chip at a time
 
 template <typename TIn, typename TOut, int D, int E>
 __global__ void __launch_bounds__(THREADS)
-decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v,
-              float* __restrict__ kv, TOut* __restrict__ o, int H, int T, long long sT, long long sH, long long sB,
+decode_kernel(const TIn* q, const TIn* k, const TIn* v, float* kv, TOut* o, int H, int T, long long sT, long long sH, long long sB,
               const __grid_constant__ RateTable rates) {
   constexpr int LPR = E / 4;              // lanes per state row (float4 each)
   constexpr int RPP = THREADS / LPR;      // rows per pass
@@ -50,7 +49,7 @@ decode_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* _
   // issue every state load first: PASSES independent 16-byte loads per thread
   float4 s[PASSES];
 #pragma unroll
-  for (int p = 0; p < PASSES; ++p) s[p] = __ldcs(&state[(size_t)(row0 + p * RPP) * LPR + col4]);
+  for (int p = 0; p < PASSES; ++p) s[p] = ld_f4_streaming(&state[(size_t)(row0 + p * RPP) * LPR + col4]);
 
   for (int t = 0; t < T; ++t) {
     const int u = t % CHUNK;

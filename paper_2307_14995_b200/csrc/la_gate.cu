@@ -20,8 +20,7 @@ __device__ __forceinline__ float row_sum(float x, int lanes) {
 
 // TO: dtype of o and y (the library's out_dtype), TU: dtype of u (in_dtype).  o and y may be the same buffer.
 template <typename TO, typename TU>
-__global__ void __launch_bounds__(256) norm_gate_fwd_kernel(const TO* o, const TU* __restrict__ u, TO* y,
-                                                            float* __restrict__ rstd, long rows, int e) {
+__global__ void __launch_bounds__(256) norm_gate_fwd_kernel(const TO* o, const TU* u, TO* y, float* rstd, long rows, int e) {
   grid_dep_wait();
   grid_dep_launch();
   const int lanes = e >> 2;  // lanes per row: 16 or 32
@@ -49,9 +48,7 @@ __global__ void __launch_bounds__(256) norm_gate_fwd_kernel(const TO* o, const T
 
 // o in TO (out_dtype); u, dy and d_o in TU (in_dtype: d_o feeds la_bwd); d_u in TO.
 template <typename TO, typename TU>
-__global__ void __launch_bounds__(256) norm_gate_bwd_kernel(const TO* __restrict__ o, const TU* __restrict__ u,
-                                                            const TU* __restrict__ dy, TU* __restrict__ d_o,
-                                                            TO* __restrict__ d_u, long rows, int e) {
+__global__ void __launch_bounds__(256) norm_gate_bwd_kernel(const TO* o, const TU* u, const TU* dy, TU* d_o, TO* d_u, long rows, int e) {
   grid_dep_wait();
   grid_dep_launch();
   const int lanes = e >> 2;

@@ -50,7 +50,7 @@ struct Geometry {   // where token t of (b,h) lives: element offset b*sB + h*sH 
 // step angle, four multiply-adds instead of a sincos per element; over 16 steps the recurrence
 // drifts by a few 1e-7, far below the bf16 features' 2^-9.  With the double products and sincos in the kernels themselves
 // a warp spent most of its 2100 instructions on them with nothing in flight (this kernel: 7 us at 16 heads x 8192 tokens).
-__global__ void __launch_bounds__(256) lrpe_angle_kernel(const float* __restrict__ theta, float2* __restrict__ table, int H, int d,
+__global__ void __launch_bounds__(256) lrpe_angle_kernel(const float* theta, float2* table, int H, int d,
                                                          int runs, long long pos0) {
   grid_dep_wait();
   grid_dep_launch();
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(256) lrpe_angle_kernel(const float* __restrict
 }
 
 // (cos, sin) of four consecutive features.
-__device__ __forceinline__ void load_angles(const float2* __restrict__ at, float (&c)[4], float (&s)[4]) {
+__device__ __forceinline__ void load_angles(const float2* at, float (&c)[4], float (&s)[4]) {
   const float4 x = *reinterpret_cast<const float4*>(at), y = *reinterpret_cast<const float4*>(at + 2);
   c[0] = x.x; s[0] = x.y; c[1] = x.z; s[1] = x.w;
   c[2] = y.x; s[2] = y.y; c[3] = y.z; s[3] = y.w;
@@ -102,7 +102,7 @@ __device__ __forceinline__ void store_features(const FeatureArgs<T>& io, size_t 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256, 4) lrpe_feature_kernel(const FeatureArgs<T> io, const float2* __restrict__ table, Geometry g) {
+__global__ void __launch_bounds__(256, 4) lrpe_feature_kernel(const FeatureArgs<T> io, const float2* table, Geometry g) {
   grid_dep_wait();
   grid_dep_launch();
   const int lanes = g.d >> 2;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256, 4) lrpe_feature_kernel(const FeatureArgs<
 
 // dst = a + b (fp32 operands; dst may be a itself), four elements per thread.
 template <typename TOut>
-__global__ void __launch_bounds__(256) lrpe_sum_kernel(const float* a, const float* __restrict__ b, TOut* dst, long n4) {
+__global__ void __launch_bounds__(256) lrpe_sum_kernel(const float* a, const float* b, TOut* dst, long n4) {
   grid_dep_wait();
   grid_dep_launch();
   const long nthreads = (long)gridDim.x * blockDim.x;
@@ -174,17 +174,17 @@ struct GradArgs {
 };
 
 template <typename TIn, typename TOut>
-__global__ void __launch_bounds__(256) lrpe_grad_kernel(const GradArgs<TIn, TOut> io, const float2* __restrict__ table, Geometry g,
+__global__ void __launch_bounds__(256) lrpe_grad_kernel(const GradArgs<TIn, TOut> io, const float2* table, Geometry g,
                                                            long long pos0, int ntiles) {
   __shared__ float red[2048];  // [tokens per pass][d]: 8 x 128 or 16 x 64
   grid_dep_wait();
   grid_dep_launch();
   const bool second = blockIdx.y != 0;
-  const TIn* __restrict__ const x = second ? io.x[1] : io.x[0];
-  const float* __restrict__ const gc = second ? io.gc[1] : io.gc[0];
-  const float* __restrict__ const gs = second ? io.gs[1] : io.gs[0];
-  TOut* __restrict__ const dx = second ? io.dx[1] : io.dx[0];
-  float* __restrict__ const part = second ? io.part[1] : io.part[0];
+  const TIn* const x = second ? io.x[1] : io.x[0];
+  const float* const gc = second ? io.gc[1] : io.gc[0];
+  const float* const gs = second ? io.gs[1] : io.gs[0];
+  TOut* const dx = second ? io.dx[1] : io.dx[0];
+  float* const part = second ? io.part[1] : io.part[0];
   const int lanes = g.d >> 2;
   const int rows_per_pass = 256 / lanes;  // 8 (d = 128) or 16 (d = 64)
   const int lane = threadIdx.x % lanes, row0 = threadIdx.x / lanes;
@@ -229,9 +229,9 @@ __global__ void __launch_bounds__(256) lrpe_grad_kernel(const GradArgs<TIn, TOut
 // dtheta[h][i] = sum over the batch and the tiles of the two partial arrays, in double, in an order that depends on
 // the shape only (32 slices per feature: slice l adds the partials l, l + 32, ...; the slices are then added in
 // order through shared memory), so the result is reproducible bit for bit.  Eight consecutive features per block.
-__global__ void __launch_bounds__(256) lrpe_theta_reduce_kernel(const float* __restrict__ part_q,
-                                                                const float* __restrict__ part_k,
-                                                                float* __restrict__ dtheta, int B, int H, int ntiles, int d) {
+__global__ void __launch_bounds__(256) lrpe_theta_reduce_kernel(const float* part_q,
+                                                                const float* part_k,
+                                                                float* dtheta, int B, int H, int ntiles, int d) {
   grid_dep_wait();
   grid_dep_launch();
   const int slice = threadIdx.x >> 3, fi = threadIdx.x & 7;

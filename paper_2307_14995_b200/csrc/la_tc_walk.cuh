@@ -149,7 +149,7 @@ __device__ __forceinline__ void store_below(T* p, uint32_t stride_bytes, int x, 
 // The 32 bits at p + x * stride, likewise.
 __device__ __forceinline__ uint32_t load_u32_at(const void* p, uint32_t stride_bytes, int x) {
   uint32_t r;
-  asm volatile("{\n\t.reg .b64 a;\n\tmad.wide.u32 a, %1, %2, %3;\n\tld.global.nc.b32 %0, [a];\n\t}"
+  asm volatile("{\n\t.reg .b64 a;\n\tmad.wide.u32 a, %1, %2, %3;\n\tld.global.b32 %0, [a];\n\t}"
                : "=r"(r)
                : "r"(stride_bytes), "r"((uint32_t)x), "l"(reinterpret_cast<uint64_t>(p)));
   return r;
@@ -451,7 +451,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           const float4* r4 = reinterpret_cast<const float4*>(src + (size_t)(q * 32 + lane) * 128 + w4 * 32);
 #pragma unroll
           for (int x = 0; x < 8; ++x) {
-            const float4 v = __ldg(r4 + x);
+            const float4 v = r4[x];
             zreg[4 * x + 0] = fmaf(g, zreg[4 * x + 0], v.x);
             zreg[4 * x + 1] = fmaf(g, zreg[4 * x + 1], v.y);
             zreg[4 * x + 2] = fmaf(g, zreg[4 * x + 2], v.z);
@@ -460,7 +460,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
         } else {
           const float* r1 = src + (size_t)(w4 * 32) * 128 + q * 32 + lane;
 #pragma unroll
-          for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], __ldg(r1 + x * 128));
+          for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], r1[x * 128]);
         }
       };
       if (EARLY && args.follows == FOLLOWS_STATES) {
@@ -485,9 +485,9 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
             const float* r2 = r1 + (REV ? -1 : 1) * (128 * 128);
             float v[32];
 #pragma unroll
-            for (int x = 0; x < 32; ++x) v[x] = __ldg(r1 + x * 128);
+            for (int x = 0; x < 32; ++x) v[x] = r1[x * 128];
 #pragma unroll
-            for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g2, fmaf(g1, zreg[x], v[x]), __ldg(r2 + x * 128));
+            for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g2, fmaf(g1, zreg[x], v[x]), r2[x * 128]);
             --k;
             continue;
           }

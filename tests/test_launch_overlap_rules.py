@@ -24,3 +24,11 @@ def test_tensor_memory_is_taken_behind_the_wait(name, unless_known):
     assert len(allocs) == 1
     before = " ".join(text[:allocs[0]].split())
     assert before.endswith("if (warp == 1) { " + unless_known + "grid_dep_wait();")
+
+
+@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))))
+def test_loads_take_no_path_for_memory_that_nobody_writes(name):
+    """A kernel that begins early runs while the launch ahead still writes what it will read: ld.global.nc (__ldg, or the compiler's
+    choice for const __restrict__ parameters) is for memory that is read-only from the kernel's beginning on, and the other load
+    intrinsics may be moved ahead of the wait."""
+    assert re.findall(r"__ldg|__ldc[gsav]|__ldlu|ld\.global\.nc|__restrict__", source(name)) == []
