@@ -82,8 +82,7 @@ struct Folded {
 
 struct Plan {
   int BH, seg_len, nseg;
-  bool tensor;      // tensor-core kernels
-  bool chains;      // the walk chains the segments' local states itself (tensor-core kernels): no scan ...
+  bool tensor;      // tensor-core kernels: the walk chains the segments' local states itself, no scan ...
   bool scanned;     // ... but running sums of the slowly decaying heads' states
   bool rows;        // CUDA-core kernels: short segments, every row tile by itself (no chain of blocks)
   int precision;    // LA_SPLIT_* bits (tensor path)
@@ -127,7 +126,6 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
   p->BH = s->B * s->H;
   if (s->path == LA_PATH_TENSOR && !tensor_path_available(s)) return LA_ERR_UNSUPPORTED;
   p->tensor = (s->path == LA_PATH_TENSOR) || (s->path == LA_PATH_AUTO && tensor_path_available(s));
-  p->chains = p->tensor;
   p->scanned = false;
   p->precision = (s->precision == LA_PRECISION_DEFAULT)
                      ? (LA_SPLIT_SCORES | LA_SPLIT_STATE | LA_SPLIT_DECAYED)
@@ -136,11 +134,11 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
   if (seg_len == 0) {
     // One thread block per (batch*head, segment) and one block per SM at a time: pick the segment count with the least
     // cost.  Depends on the shape only.
-    // Where the walk chains the segment states itself, in us: forward walk and dQ walk, the dV and dK walks in one launch (twice
+    // Tensor cores, in us: forward walk and dQ walk, the dV and dK walks in one launch (twice
     // the thread blocks), each in waves over the 148 SMs of (blocks of a segment + start and end), and the launches that make the
     // states, with what each further state costs to write, read and chain, as far as they are not hidden behind the launches
-    // around them.  Segments of one block leave nothing to hide them behind.  Measured, forward and backward: 32 heads x 777 as one
-    // segment 23.8 + 46.1, 256 tokens 20.8 + 48.1, 128 34.1 + 76.7; 8 x 512 14.8 + 27.3, 19.8 + 26.7 and 19.4 + 23.4; 24 x 2048 with
+    // around them.  Segments of one block leave nothing to hide them behind.  Measured at d = 128, forward and backward: 32 heads x 777
+    // as one segment 23.8 + 46.1, 256 tokens 20.8 + 48.1, 128 34.1 + 76.7; 8 x 512 14.8 + 27.3, 19.8 + 26.7 and 19.4 + 23.4; 24 x 2048 with
     // 768 tokens 34.0 + 70.0, 384 26.1 + 66.4, 256 43.3 + 100.9; 8 x 8192 with 1024 43.7 + 84.6, 512 34.6 + 82.2, 256 49.6 + 123.9;
     // 64 x 1500 as one segment 40.9 + 84.3, two 40.0 + 96.9; 2 x 16 x 8192 with 2048 72.5 + 197.9, 1024 96.4 + 256.4.
     // CUDA-core kernels: row tiles up to ROWS_MAX_SEG tokens, whose work grows with the segment's length but which end after
@@ -149,9 +147,12 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
     // and 65; 2 x 2048 205 with 512-token segments, 122 with 256, 81 with 128; 16 x 2048, d = 128, 946, 652 and 488.  Where the heads
     // fill the chip a state costs more than it saves: 256 x 512, d = 64, 747 with 128-token segments and 605 as one; 256 x 4096
     // 7769 with 1024 and 6383 as one; 128 x 2048, d = 128, 6560 with 1024 and 5384 as one.
-    // Tensor cores at d = 64: waves of blocks too, in units of one block (about 2.2 us).  Measured, forward and backward: 8 heads x 777
-    // as one segment 18.4 + 32.3 us, 256 tokens 12.6 + 18.6, 128 13.7 + 20.0; 4 x 16 x 2048 40.9 + 84.6, with 1024 tokens 32.7 + 80.1,
-    // 512 37.5 + 96.6; 16 x 8192 with 2048 48.0 + 93.6, 1024 36.0 + 87.2, 512 44.0 + 104.4.
+    // At d = 64 blocks and states cost less, but in much the same proportion: over 82 sizes of 8 to 128 heads x 300 to 16384 the rule
+    // is within 1 % of the best segment length at 67 and 1.8 % from it on average (costs of its own, 2.2 us a block and 21 + 0.15 a
+    // state, 2.5 %; it took 57 instead of 49 us at 32 x 1024, 86 instead of 73 at 48 x 1536).  Forward plus backward, us: 4 x 16 x 2048
+    // as one segment 122, with 1024 tokens 112, 768 157; 4 x 16 x 1536 93, with 768 96; 32 x 777 50, with 256 tokens 49, 128 87; 16 x
+    // 8192 with 2048 141, 1024 124, 512 166.  Where it loses: 4 x 16 x 1920 116 as one, 110 with 1024; 8 x 2048 with 256 tokens 41.5, 384
+    // 38.4; 8 x 512 as one segment 30, with segments of one block, which it does not consider, 23.
     // Packed batches: waves of (blocks + pipeline fill), segments no shorter than 1024 tokens.  On the tensor cores la_chunk_state
     // takes the same rule: 32 heads x 777 22.5 us with the walk's segments, 16.4 with one; 16 x 2048 20.5 and 16.4; 8 x 8192 20.5
     // and 16.4; d = 64, 4 x 16 x 2048 20.5 and 14.4.
@@ -192,15 +193,10 @@ la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states
       }
     } else if (states_only || packed) {
       // as it stands
-    } else if (p->chains) {
+    } else {
       best_n = choose((s->N + 255) / 256, limit, [&](long nseg, long blocks) {
         return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (3.0 * blocks + 2.0) +
                (nseg > 1 ? 17.0 + 0.75 * nseg + 0.11 * p->BH * nseg + 1e-4 * p->BH * s->N : 0.0);
-      });
-    } else {
-      best_n = choose((s->N + 127) / 128, limit, [&](long nseg, long blocks) {
-        const double units = (double)p->BH * nseg;
-        return (2.0 * waves(p->BH * nseg) + waves(2 * p->BH * nseg)) * (blocks + 0.67) + (nseg > 1 ? 9.6 + 0.068 * units : 0.0);
       });
     }
     seg_len = ((s->N + best_n - 1) / best_n + 127) / 128 * 128;
@@ -219,8 +215,8 @@ size_t state_set_bytes(const la_shape* s, const Plan& p) {
 // State sets that la_workspace_bytes asks for.  Walks that chain the segments' states need one for the forward pass and those of
 // KV^T and of dKV for the backward pass; a scan also writes their transposes.  (At d = 64 the tensor-core walk had a scan before
 // it; what it asks for has stayed.)
-int fwd_sets(const la_shape* s, const Plan& p) { return p.nseg == 1 ? 0 : p.chains && s->d == 128 ? 1 : 2; }
-int bwd_sets(const la_shape* s, const Plan& p) { return p.chains && s->d == 128 ? 2 : 3; }
+int fwd_sets(const la_shape* s, const Plan& p) { return p.nseg == 1 ? 0 : p.tensor && s->d == 128 ? 1 : 2; }
+int bwd_sets(const la_shape* s, const Plan& p) { return p.tensor && s->d == 128 ? 2 : 3; }
 
 // (logarithms and a table twice as large are half a microsecond of a decode step: it takes the rates as they are)
 la_status make_rates(const la_shape* s, const float* lambda_host, RateTable* rates) {
@@ -317,7 +313,7 @@ cudaError_t run_scan(const la_shape* s, const Plan& p, const DecayTable& tab, fl
 // Running sums pay where a slow head would read many states: 7B-like shape, nine segments, 8 us of chain against 5 us of
 // launch; with four segments 3 against 5.  Packed batches: always, their sequences differ in how many segments they have.
 bool wants_running(const la_shape* s, const Plan& p, const DecayTable& tab) {
-  if (!p.chains || p.nseg < 3 || p.BH > 65535 || !(p.pk.start || p.nseg > 6)) return false;
+  if (!p.tensor || p.nseg < 3 || p.BH > 65535 || !(p.pk.start || p.nseg > 6)) return false;
   for (int h = 0; h < s->H; ++h)
     if (slow_head((float)tab.s2[h], p.seg_len)) return true;
   return false;
@@ -338,7 +334,7 @@ cudaError_t run_prefix(const la_shape* s, const Plan& p, const DecayTable& tab, 
 }
 
 // What a walk starts from: the state entering each segment (entry), or, where the walk chains the segments itself
-// (Plan::chains), the state entering the sequence and the segments' local states, each possibly stored transposed.
+// (tensor cores), the state entering the sequence and the segments' local states, each possibly stored transposed.
 struct Carried {
   const float* entry = nullptr;
   const float* z_in = nullptr;
@@ -501,7 +497,7 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   Carried from;
   float* const buf = static_cast<float*>(workspace);
   if (p.nseg > 1) LA_TRY_CUDA(run_prepass(shape, p, tab, k, v, 0, buf, false, cs));
-  if (p.chains) {
+  if (p.tensor) {
     if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf, 0, cs));
     from = chained(kv_in, false, buf, false);
   } else if (p.nseg > 1) {
@@ -511,13 +507,13 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   } else {
     from.entry = kv_in;  // single segment: the caller's state is the entry state
   }
-  from.follows = p.chains && p.nseg > 1 ? FOLLOWS_STATES : FOLLOWS_ANY;
+  from.follows = p.tensor && p.nseg > 1 ? FOLLOWS_STATES : FOLLOWS_ANY;
   if (!u) {
     LA_TRY_CUDA(run_walk(shape, p, tab, q, k, v, o, from, kv_out, 0, cs));
     return LA_OK;
   }
   // the d = 128 walk has the output stage as an epilogue
-  if (p.chains && shape->d == 128) {
+  if (p.tensor && shape->d == 128) {
     OpArgs wa = walk_args(shape, p, q, k, v, o, from, kv_out, 0);
     wa.u = u;
     wa.y = y;
@@ -589,7 +585,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
 
   // dQ = fwd(a = dO, b = V, c = K); its state is KV^T, so the caller's kv_in (and what la_fwd left) enters transposed.
   Carried from_q;
-  if (p.chains) {
+  if (p.tensor) {
     if (multi && !fwd_workspace) {
       LA_TRY_CUDA(run_prepass(shape, p, tab, v, k, 0, buf_kvt, false, cs));
       if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf_kvt, 0, cs));
@@ -606,13 +602,13 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   // Where launches begin early the states of both directions come before all walks: the dQ walk begins while they end and the other
   // two while it ends, so that the thread blocks of a launch fill the multiprocessors that the last ones of the launch before leave
   // idle.
-  const bool together = p.chains && early_walks(p.BH, p.nseg, p.seg_len);
+  const bool together = p.tensor && early_walks(p.BH, p.nseg, p.seg_len);
   if (!p.rows && !together) LA_TRY_CUDA(run_walk(shape, p, tab, d_o, v, k, dq, from_q, nullptr, 0, cs));
 
   // dV = rev(a = K, b = Q, c = dO) carries dKV; dK = rev(a = V, b = dO, c = Q) carries dKV^T.
   Carried from_v, from_k;
   if (multi) LA_TRY_CUDA(run_prepass(shape, p, tab, q, d_o, 1, buf_e, false, cs));
-  if (p.chains) {
+  if (p.tensor) {
     if (p.scanned) LA_TRY_CUDA(run_prefix(shape, p, tab, buf_e, 1, cs));
     from_v = chained(grad_kv_out, false, buf_e, false);
     from_k = chained(grad_kv_out, true, buf_e, true);
@@ -658,7 +654,7 @@ static la_shape doubled(const la_shape* half) {
 size_t halves_workspace(int op, const la_shape* half) {
   const la_shape s = doubled(half);
   Plan p;
-  if (half->B > (1 << 20) || check_shape(&s, true) != LA_OK || make_plan(&s, &p) != LA_OK || !p.chains) return (size_t)-1;
+  if (half->B > (1 << 20) || check_shape(&s, true) != LA_OK || make_plan(&s, &p) != LA_OK || !p.tensor) return (size_t)-1;
   return la_workspace_bytes(op, &s);
 }
 la_status halves_fwd(const la_shape* half, const void* q, const void* k, const void* v, const float* lambda_host, void* o, void* o2,

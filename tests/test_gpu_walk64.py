@@ -160,3 +160,11 @@ def test_packed_tables_of_many_sequences(S):
         want[t] += 0.5 ** back * (q[t] * k[t - back]).sum(1, keepdim=True) * v[t - back]
     rms = want.pow(2).mean().sqrt()
     assert (o[0, :, 0].double().cpu() - want).abs().max() <= 1.7e-4 * rms * 5  # (single rows reach several times the tensor's RMS)
+
+
+@pytest.mark.parametrize("B,heads,N,segment", [
+    (1, 8, 512, 512), (1, 8, 2048, 256), (1, 16, 8192, 1024), (1, 32, 777, 256), (1, 32, 1024, 256), (3, 16, 1536, 512),
+    (4, 16, 1536, 1536), (4, 16, 1920, 1920), (4, 16, 2048, 1024), (4, 16, 16384, 8192)])
+def test_segments_at_64_features(B, heads, N, segment):
+    """The rule that its comment describes is the one that runs (the sizes are among those that were measured)."""
+    assert la.segment_length(la.make_shape(B, heads, N, D, D, torch.bfloat16, torch.float32)) == segment
