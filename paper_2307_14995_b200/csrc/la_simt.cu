@@ -362,12 +362,12 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanArgs args, const De
 // with two thread blocks on the chip.  Here the work grows with the square of the segment, but all tiles run at once, and the
 // walks of a launch do too (B = 1, H = 2, N = 256, d = 64 in fp32, forward plus backward: 240 us before, 38 now; with N = 2048
 // and 128-token segments 1155 and 81).
-// 128 threads; at d = 128 57 KB and 178 registers, which let two thread blocks share an SM; the next tiles are loaded into
+// 128 threads; at d = 128 57 KB and 168 registers, which let three thread blocks share an SM; the next tiles are loaded into
 // registers while the present ones are multiplied.
 //
 // The tiles that a thread block adds up are shared out over G groups of 128 threads, each with its own pair of tiles in shared
 // memory, whose sums meet at the end: with one group a tile costs 4400 clocks, a warp per scheduler waiting for its own loads.
-// Where thread blocks fill the chip several times over, groups only add their meeting (rows_groups).
+// Where thread blocks fill the chip several times over, groups only add their meeting (rows_shared).
 constexpr int ROWS_THREADS = 128;  // of a group
 constexpr int ROWS_MAX_JOBS = 3;
 static_assert(ROWS_MAX_SEG % C == 0, "whole tiles");
@@ -634,17 +634,31 @@ cudaError_t launch_rows_g(const RowsArgs& ra, const DecayTable& tab, cudaStream_
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   KernelTimer timer(ra.units[0] ? K_WALK : K_PREPASS, stream);
-  err = launch_early(kern, dim3((unsigned)ra.first_block[ROWS_MAX_JOBS]), dim3(ROWS_THREADS * G), smem, stream, 1, ra, tab);
+  // One walk of one segment by one group, all thread blocks at once: placed while the launch before still drains, long tiles come to
+  // share multiprocessors (d = 64, 250 heads x 64 tokens 20.3 us, launched after it 14.4; d = 128, 100 x 128 35.8 and 30.9; the three
+  // walks of a backward pass, d = 128, 74 x 64, 20.0 and 21.1).
+  const bool early = G > 1 || !ra.units[0] || ra.units[1] || ra.job[0].nseg > 1 || ra.first_block[ROWS_MAX_JOBS] > 148 * (D == 64 ? 4 : 3);
+  err = launch_kernel(early, kern, dim3((unsigned)ra.first_block[ROWS_MAX_JOBS]), dim3(ROWS_THREADS * G), smem, stream, 1, ra, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }
-// Thread blocks up to which their tiles are shared out over groups: as many as run at once, two or four to a multiprocessor.
-constexpr int rows_groups_limit(int d) { return d == 64 ? 592 : 296; }
+// Whether a launch's tiles are shared out over groups.  With groups fewer thread blocks run at once (two to a multiprocessor at
+// d = 64, where one group lets four run, and one instead of three at d = 128), but each ends sooner: the more tiles its rows add up,
+// the more thread blocks a launch may have.  Measured, us, one group and four at d = 64: 37 heads x 512 (592 thread blocks, 16 tiles)
+// 59 and 36, 64 x 512 (1024) 63 and 58, 75 x 512 (1200) 66 and 69, 90 x 200 (630, 7 tiles) 32.5 and 30.8, 90 x 300 (900, 10 tiles) 43
+// and 47, 140 x 128 (560, 4 tiles) 22.5 and 24.3, 200 x 64 (400, 2 tiles) 12.4 and 15.9; one and two at d = 128: 19 x 500 (304) 92 and
+// 50, 37 x 512 (592) 93 and 56, 64 x 512 (1024) 106 and 95, 75 x 512 (1200) 112 and 112, 64 x 300 (640, 10 tiles) 68 and 54, 100 x 300
+// (1000) 74 and 82, 300 x 64 (600, 2 tiles) 25 and 31.  Short segments of a longer sequence, and states, as before: 592 and 296.
+inline bool rows_shared(int d, const RowsArgs& ra) {
+  const int blocks = ra.first_block[ROWS_MAX_JOBS], tiles = ra.units[0] ? (ra.job[0].seg_len + C - 1) / C : 0;
+  if (tiles >= 5) return blocks <= (d == 64 ? 350 + 50 * tiles : 550 + 40 * tiles);
+  if (d == 64 && tiles > 0 && ra.job[0].nseg == 1) return blocks <= (tiles == 4 ? 444 : 296);
+  return blocks <= (d == 64 ? 592 : 296);
+}
 template <typename TIn, typename TOut, int D>
 cudaError_t launch_rows_t(const RowsArgs& ra, const DecayTable& tab, cudaStream_t stream) {
   constexpr int MANY = D == 64 ? 4 : 2;
-  return ra.first_block[ROWS_MAX_JOBS] <= rows_groups_limit(D) ? launch_rows_g<TIn, TOut, D, MANY>(ra, tab, stream)
-                                                               : launch_rows_g<TIn, TOut, D, 1>(ra, tab, stream);
+  return rows_shared(D, ra) ? launch_rows_g<TIn, TOut, D, MANY>(ra, tab, stream) : launch_rows_g<TIn, TOut, D, 1>(ra, tab, stream);
 }
 template <int D>
 cudaError_t launch_rows_dims(const RowsArgs& ra, const DecayTable& tab, int in_dt, int out_dt, cudaStream_t stream) {

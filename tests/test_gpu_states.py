@@ -209,3 +209,21 @@ def test_full_precision_tiles_shared_by_groups_or_not(B, H, N, d):
     ref = tuple(orc.fwd_rec(q, k, v, lam64, want_state=True)) + tuple(orc.bwd_rec(q, k, v, do, lam64))
     for name, g, r in zip(("o", "kv", "dq", "dk", "dv"), (o, kv) + tuple(grads), ref):
         assert_close(g, r, 3.6e-4, name)
+
+
+@pytest.mark.parametrize("B,H,N,d", [
+    (1, 25, 400, 128), (1, 8, 300, 128), (2, 32, 512, 128), (1, 75, 512, 128), (4, 25, 128, 128), (5, 30, 64, 128),  # one group or two
+    (1, 45, 512, 64), (1, 19, 500, 64), (1, 90, 300, 64), (1, 70, 300, 64), (5, 28, 128, 64), (4, 50, 64, 64)])      # one or four
+def test_full_precision_groups_by_the_tiles_of_a_row(B, H, N, d):
+    """On both sides of where a launch's tiles are shared out, by how many a row adds up.  Tolerance as above: at most 640 products."""
+    gen = torch.Generator().manual_seed(B * H * N)
+    q, k, v, do = [torch.randn(B, H, N, d, generator=gen) * d ** -0.5 for _ in range(4)]
+    lam = torch.linspace(0.5, 1.0, H)
+    dev = [x.cuda() for x in (q, k, v, do)]
+    o = la.fwd(*dev[:3], lam)
+    grads = la.bwd(*dev, lam)
+    torch.cuda.synchronize()
+    lam64 = lam.double().numpy()
+    ref = (orc.fwd_rec(q, k, v, lam64),) + tuple(orc.bwd_rec(q, k, v, do, lam64))
+    for name, g, r in zip(("o", "dq", "dk", "dv"), (o,) + tuple(grads), ref):
+        assert_close(g, r, 3.6e-4, name)
