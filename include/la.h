@@ -266,9 +266,9 @@ la_status la_chain_states(const la_shape* shape, long long total_tokens, long lo
  * bf16 inputs (and more than one sequence) run as ONE set of
  * launches over all sequences: every (sequence, head[, segment]) is a thread block of the tensor-core kernels, which
  * take each sequence's first token and length from a small table that the call writes to the head of the workspace
- * (a kernel with the table as its argument; a captured call keeps its own copy of it).  At d = e = 64 only with a
- * workspace of la_varlen_workspace_bytes, else, and with fp32 inputs, they
- * enqueue one la_fwd / la_bwd per sequence on `stream`.  la_varlen_workspace_bytes covers both.
+ * (a kernel with the table as its argument; a captured call keeps its own copy of it).  With fp32 inputs, and at
+ * d = e = 64 with less workspace than la_varlen_workspace_bytes or where one sequence is much longer than the others
+ * together (and seg_len = 0), they enqueue one la_fwd / la_bwd per sequence on `stream`.  la_varlen_workspace_bytes covers both.
  */
 size_t la_varlen_workspace_bytes(int op, const la_shape* shape, const int* cu_seqlens_host, int num_seqs);
 la_status la_fwd_varlen(const la_shape* shape, const void* q, const void* k, const void* v, const float* lambda_host,

@@ -168,3 +168,35 @@ def test_packed_tables_of_many_sequences(S):
 def test_segments_at_64_features(B, heads, N, segment):
     """The rule that its comment describes is the one that runs (the sizes are among those that were measured)."""
     assert la.segment_length(la.make_shape(B, heads, N, D, D, torch.bfloat16, torch.float32)) == segment
+
+
+@pytest.mark.parametrize("lens,together", [([32768] + [100] * 10, False), ([8192] + [100] * 10, True), ([32768, 64], False)])
+def test_packed_batches_of_uneven_lengths(lens, together):
+    """One long sequence among short ones goes sequence by sequence, like the calls on each alone; others in one set of launches."""
+    heads = 8
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    gen = torch.Generator("cuda")
+    gen.manual_seed(7)
+    q, k, v, do = [torch.randn(1, cu[-1], heads, D, generator=gen, device="cuda").bfloat16() for _ in range(4)]
+    lam = torch.linspace(0.9, 1.0, heads)
+    shape = la.make_shape(1, heads, cu[-1], D, D, torch.bfloat16, torch.float32, layout=la.LA_LAYOUT_BNHD)
+    ws = [torch.empty(la.varlen_workspace_bytes(op, shape, cu), dtype=torch.uint8, device="cuda") for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    out = [torch.full(q.shape, float("nan"), device="cuda") for _ in range(4)]
+    n = la.launch_count()
+    la.la_fwd_varlen(shape, q, k, v, lam, out[0], cu, None, None, ws[0])
+    assert (la.launch_count() - n <= 3) == together
+    la.la_bwd_varlen(shape, q, k, v, do, lam, *out[1:], cu, workspace=ws[1])
+    want = [torch.empty_like(t) for t in out]
+    for a, b in zip(cu, cu[1:]):
+        one = la.make_shape(1, heads, b - a, D, D, torch.bfloat16, torch.float32, layout=la.LA_LAYOUT_BNHD)
+        x, y = [t[:, a:b] for t in (q, k, v, do)], [t[:, a:b] for t in want]
+        w = [torch.empty(max(256, la.workspace_bytes(op, one)), dtype=torch.uint8, device="cuda") for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+        la.la_fwd(one, *x[:3], lam, y[0], workspace=w[0])
+        la.la_bwd(one, *x, lam, *y[1:], workspace=w[1])
+    torch.cuda.synchronize()
+    la.device_status()
+    for a, b in zip(out, want):
+        if together:  # two-term operands, 2^-17 of each product, in other segments: each side as above
+            assert (a - b).abs().max() <= 2 * 1.7e-4 * b.pow(2).mean().sqrt() * 5
+        else:
+            assert torch.equal(a, b)
