@@ -48,6 +48,8 @@ struct Packed {
   const int* len;
   const int* order;  // sequence indices, longest first
   int total_tokens;
+  const int* cu;     // HOST: first token of each sequence, and total_tokens
+  int S;
 };
 
 // Part of the table of a packed batch, as a kernel's argument: a launch keeps its own copy, in a stream and in a captured graph alike.  (A copy from
@@ -121,7 +123,7 @@ bool tensor_path_available(const la_shape* s) {
 // `packed`: the plan of a packed batch, whose sequences of different lengths share one segment length.  `states_only`: of
 // la_chunk_state, which has no walk to shorten; each further segment is a state to write, read and chain.
 la_status make_plan(const la_shape* s, Plan* p, bool packed = false, bool states_only = false) {
-  p->pk = Packed{nullptr, nullptr, nullptr, 0};
+  p->pk = Packed{};
   p->fold = Folded{0, {nullptr, nullptr}, nullptr, nullptr};
   p->BH = s->B * s->H;
   if (s->path == LA_PATH_TENSOR && !tensor_path_available(s)) return LA_ERR_UNSUPPORTED;
@@ -254,6 +256,27 @@ la_status check_device() {
   do {                                          \
     if ((expr) != cudaSuccess) return LA_ERR_CUDA; \
   } while (0)
+
+// Writes first tokens, lengths and order of a packed batch (stream-ordered).
+la_status packed_upload(const Packed& pk, cudaStream_t cs) {
+  const int S = pk.S;
+  std::vector<int> host(3 * (size_t)S);
+  for (int i = 0; i < S; ++i) {
+    host[i] = pk.cu[i];
+    host[S + i] = pk.cu[i + 1] - pk.cu[i];
+    host[2 * S + i] = i;
+  }
+  // longest first (ties in the caller's order): the thread blocks of a launch are handed out in index order
+  std::stable_sort(host.begin() + 2 * S, host.end(), [&](int a, int b) { return host[S + a] > host[S + b]; });
+  // (arguments of a launch: 4 KB for up to 333 sequences, else 32 KB at a time)
+  constexpr size_t SMALL = 1000, LARGE = 8000;
+  int* const dst = const_cast<int*>(pk.start);
+  for (size_t at = 0; at < host.size(); at += LARGE) {
+    const size_t n = std::min(LARGE, host.size() - at);
+    LA_TRY_CUDA(n <= SMALL ? put_table<SMALL>(dst + at, &host[at], (int)n, cs) : put_table<LARGE>(dst + at, &host[at], (int)n, cs));
+  }
+  return LA_OK;
+}
 
 // Element strides of the token tensors for the shape's layout (d == e in every supported shape).
 void set_strides(const la_shape* s, int tokens, OpArgs* a) {
@@ -493,6 +516,7 @@ la_status fwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   if (need > 0 && (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_INVALID_ARG;
   if ((st = check_device()) != LA_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  if (pk && (st = packed_upload(*pk, cs)) != LA_OK) return st;
 
   Carried from;
   float* const buf = static_cast<float*>(workspace);
@@ -577,6 +601,7 @@ la_status bwd_impl(const la_shape* shape, const void* q, const void* k, const vo
   if (reinterpret_cast<uintptr_t>(workspace) & 255u) return LA_ERR_INVALID_ARG;
   if ((st = check_device()) != LA_OK) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  if (pk && (st = packed_upload(*pk, cs)) != LA_OK) return st;
 
   float* buf_kvt = static_cast<float*>(workspace);                 // KV^T entering each segment
   float* buf_e = buf_kvt + one / sizeof(float);                    // dKV entering each segment (from the right)
@@ -1007,28 +1032,10 @@ bool packed_fits(int op, const la_shape* sp, const int* cu, const void* workspac
          workspace_bytes >= packed_table_bytes(sp->B) + w && !better_one_by_one(sp, cu);  // ... or if it ends later for it
 }
 
-// Puts first tokens and lengths at the head of the workspace (stream-ordered) and describes them.
-la_status packed_upload(const int* cu, int S, int total, void* workspace, cudaStream_t cs, Packed* pk) {
-  std::vector<int> host(3 * (size_t)S);
-  for (int i = 0; i < S; ++i) {
-    host[i] = cu[i];
-    host[S + i] = cu[i + 1] - cu[i];
-    host[2 * S + i] = i;
-  }
-  // longest first (ties in the caller's order): the thread blocks of a launch are handed out in index order
-  std::stable_sort(host.begin() + 2 * S, host.end(), [&](int a, int b) { return host[S + a] > host[S + b]; });
-  // (arguments of a launch: 4 KB for up to 333 sequences, else 32 KB at a time)
-  constexpr size_t SMALL = 1000, LARGE = 8000;
-  int* const dst = static_cast<int*>(workspace);
-  for (size_t at = 0; at < host.size(); at += LARGE) {
-    const size_t n = std::min(LARGE, host.size() - at);
-    LA_TRY_CUDA(n <= SMALL ? put_table<SMALL>(dst + at, &host[at], (int)n, cs) : put_table<LARGE>(dst + at, &host[at], (int)n, cs));
-  }
-  pk->start = static_cast<const int*>(workspace);
-  pk->len = pk->start + S;
-  pk->order = pk->start + 2 * S;
-  pk->total_tokens = total;
-  return LA_OK;
+// The table of a packed batch at the head of its workspace (packed_upload fills it).
+Packed packed_at(void* workspace, const int* cu, int S, int total) {
+  const int* const at = static_cast<const int*>(workspace);
+  return Packed{at, at + S, at + 2 * S, total, cu, S};
 }
 }  // namespace
 
@@ -1062,10 +1069,7 @@ la_status la_fwd_varlen(const la_shape* shape, const void* q, const void* k, con
   if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp) && packed_fits(LA_OP_FWD, &sp, cu_seqlens_host, workspace, workspace_bytes)) {
     const size_t tb = packed_table_bytes(num_seqs);
     if (!workspace || workspace_bytes < tb || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_WORKSPACE;
-    if ((st = check_device()) != LA_OK) return st;
-    Packed pk;
-    if ((st = packed_upload(cu_seqlens_host, num_seqs, shape->N, workspace, static_cast<cudaStream_t>(stream), &pk)) != LA_OK)
-      return st;
+    const Packed pk = packed_at(workspace, cu_seqlens_host, num_seqs, shape->N);
     return fwd_impl(&sp, q, k, v, nullptr, lambda_host, nullptr, o, nullptr, kv_in, kv_out,
                     static_cast<char*>(workspace) + tb, workspace_bytes - tb, stream, &pk);
   }
@@ -1096,10 +1100,7 @@ la_status la_bwd_varlen(const la_shape* shape, const void* q, const void* k, con
   if (packed_shape(shape, cu_seqlens_host, num_seqs, &sp) && packed_fits(LA_OP_BWD, &sp, cu_seqlens_host, workspace, workspace_bytes)) {
     const size_t tb = packed_table_bytes(num_seqs);
     if (!workspace || workspace_bytes < tb || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return LA_ERR_WORKSPACE;
-    if ((st = check_device()) != LA_OK) return st;
-    Packed pk;
-    if ((st = packed_upload(cu_seqlens_host, num_seqs, shape->N, workspace, static_cast<cudaStream_t>(stream), &pk)) != LA_OK)
-      return st;
+    const Packed pk = packed_at(workspace, cu_seqlens_host, num_seqs, shape->N);
     return bwd_impl(&sp, q, k, v, d_o, lambda_host, dq, dk, dv, kv_in, grad_kv_out, grad_kv_in, nullptr,
                     static_cast<char*>(workspace) + tb, workspace_bytes - tb, stream, &pk);
   }

@@ -200,3 +200,19 @@ def test_packed_batches_of_uneven_lengths(lens, together):
             assert (a - b).abs().max() <= 2 * 1.7e-4 * b.pow(2).mean().sqrt() * 5
         else:
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_packed_calls_with_wrong_arguments_launch_nothing(d):
+    cu = [0, 100, 300]
+    shape = la.make_shape(1, H, cu[-1], d, d, torch.bfloat16, torch.float32, layout=la.LA_LAYOUT_BNHD)
+    q, o = torch.zeros(1, cu[-1], H, d, device="cuda").bfloat16(), torch.zeros(1, cu[-1], H, d, device="cuda")
+    ws = [torch.full((max(256, la.varlen_workspace_bytes(op, shape, cu)),), 7, dtype=torch.uint8, device="cuda")
+          for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    wrong = torch.tensor([1.0, 2.0, 0.5])  # a rate above 1
+    with pytest.raises(la.LaError):
+        la.la_fwd_varlen(shape, q, q, q, wrong, o, cu, None, None, ws[0])
+    with pytest.raises(la.LaError):
+        la.la_bwd_varlen(shape, q, q, q, q, wrong, o, o.clone(), o.clone(), cu, workspace=ws[1])
+    torch.cuda.synchronize()
+    assert all(bool((w == 7).all()) for w in ws)
