@@ -66,3 +66,76 @@ def test_calls_that_read_one_another(B, H, N, d, dtype):
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(want, x + kv))
     la.device_status()
+
+
+def everything(d, wait):
+    """Every kind of call that launches early, each from what the ones before it wrote, on one workspace per pass; and in between
+    launches that do not begin early (more thread blocks than multiprocessors)."""
+    H, T, dtype = 16, 1300, torch.bfloat16
+    gen = torch.Generator("cuda")
+    gen.manual_seed(d)
+    new = lambda: (torch.randn(1, T, H, d, generator=gen, device="cuda") * d ** -0.5).to(dtype)
+    q, k, v, u, o, o2, y, d_o, du, dq, dk, dv = x = [new() for _ in range(12)]
+    kv = [torch.zeros(1, H, d, d, device="cuda") for _ in range(3)]
+    kvs, part, dtheta = torch.zeros(3, H, d, d, device="cuda"), torch.zeros(1, H, d, d, device="cuda"), torch.zeros(H, d, device="cuda")
+    theta = inputs.make_theta(H, d, seed=1).cuda()
+    lam, cu = inputs.decay_rates(H, 0.5), [0, 500, 501, T]
+    shape = la.make_shape(1, H, T, d, d, dtype, dtype, layout=la.LA_LAYOUT_BNHD)
+    plain = la.make_shape(1, H, T, d, d, dtype, dtype, 128, layout=la.LA_LAYOUT_BNHD)  # 176 thread blocks
+    step = la.make_shape(1, H, 1, d, d, dtype, dtype)
+    need = [max(la.workspace_bytes(op, shape), la.workspace_bytes(op, plain), la.varlen_workspace_bytes(op, shape, cu),
+                la.lrpe_workspace_bytes(op, shape), la.chunk_state_workspace_bytes(shape)) for op in (la.LA_OP_FWD, la.LA_OP_BWD)]
+    wf, wb = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in need]
+    norm = lambda *t: [lambda t=t: la.la_gate_fwd(shape, t, u, t) for t in t]  # in place: the numbers stay in range
+    calls = [
+        lambda: la.la_fwd_varlen(shape, q, k, v, lam, o, cu, None, kvs, wf),
+        lambda: la.la_fwd_gated(shape, o, k, v, u, lam, y, o2, kv_out=kv[0], workspace=wf),
+        lambda: la.la_gate_bwd(shape, o2, u, y, d_o, du), *norm(o2, d_o),
+        lambda: la.la_bwd_varlen(shape, o2, k, v, d_o, lam, dq, dk, dv, cu, workspace=wb), *norm(dq, dk, dv),
+        lambda: la.la_lrpe_fwd(shape, dq, dk, dv, theta, lam, o, workspace=wf), *norm(o),
+        lambda: la.la_fwd(plain, o, dk, dv, lam, y, kv[0], kv[1], wf), *norm(y),
+        lambda: la.la_lrpe_bwd(shape, o, k, y, d_o, theta, lam, dq, dk, dv, dtheta, workspace=wb), *norm(dq, dk),
+        lambda: la.la_bwd(plain, dq, dk, v, o, lam, o2, q, k, workspace=wb), *norm(q, k),
+        lambda: la.la_chunk_state(shape, 0, k, v, lam, part, wf),
+        lambda: la.la_chain_states(shape, 3 * T, T, 0, kvs, 3, 2, part, lam, kv[2]),
+        lambda: la.la_fwd_gated(plain, q, k, v, u, lam, y, kv_in=kv[2], kv_out=kv[0], workspace=wf),
+        lambda: la.la_gate_fwd(shape, o, y, d_o),
+    ] + [lambda t=t: la.la_decode_step(step, y[:, t], d_o[:, t], v[:, t], lam, kv[0], o[:, t]) for t in range(6)] + [
+        lambda: la.la_fwd(shape, o, d_o, v, lam, du, kv[0], kv[1], wf),
+    ]
+    tensors = x + kv + [kvs, part, dtheta]
+
+    def run():
+        for f in calls:
+            f()
+            if wait:
+                torch.cuda.synchronize()
+
+    return run, tensors
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_every_kind_of_call_in_one_stream(d):
+    want = None
+    for wait in (True, False, False, False):
+        run, tensors = everything(d, wait)
+        torch.cuda.synchronize()
+        run()
+        torch.cuda.synchronize()
+        want = want or [t.clone() for t in tensors]
+        assert all(bool(t.float().abs().amax() < 1e20) for t in tensors)  # (no NaN, which equals nothing, either)
+        assert all(torch.equal(a, b) for a, b in zip(want, tensors))
+    la.device_status()
+    run, tensors = everything(d, False)
+    start = [t.clone() for t in tensors]
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        run()
+    for _ in range(2):
+        for t, s in zip(tensors, start):
+            t.copy_(s)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, tensors))
+    la.device_status()
