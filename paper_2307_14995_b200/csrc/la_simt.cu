@@ -642,9 +642,9 @@ cudaError_t launch_rows_g(const RowsArgs& ra, const DecayTable& tab, cudaStream_
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }
-// Whether a launch's tiles are shared out over groups.  With groups fewer thread blocks run at once (two to a multiprocessor at
-// d = 64, where one group lets four run, and one instead of three at d = 128), but each ends sooner: the more tiles its rows add up,
-// the more thread blocks a launch may have.  Measured, us, one group and four at d = 64: 37 heads x 512 (592 thread blocks, 16 tiles)
+// Whether a launch's tiles are shared out over groups.  With groups one thread block has a multiprocessor to itself (its registers),
+// with one group four run at d = 64 and three at d = 128, but each ends sooner: the more tiles its rows add up, the more thread blocks a
+// launch may have.  Measured, us, one group and four at d = 64: 37 heads x 512 (592 thread blocks, 16 tiles)
 // 59 and 36, 64 x 512 (1024) 63 and 58, 75 x 512 (1200) 66 and 69, 90 x 200 (630, 7 tiles) 32.5 and 30.8, 90 x 300 (900, 10 tiles) 43
 // and 47, 140 x 128 (560, 4 tiles) 22.5 and 24.3, 200 x 64 (400, 2 tiles) 12.4 and 15.9; one and two at d = 128: 19 x 500 (304) 92 and
 // 50, 37 x 512 (592) 93 and 56, 64 x 512 (1024) 106 and 95, 75 x 512 (1200) 112 and 112, 64 x 300 (640, 10 tiles) 68 and 54, 100 x 300
