@@ -204,8 +204,19 @@ inline bool early_walks(int bh, int nseg, int seg_len) { return (long)bh * nseg 
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // ... and loads come behind it: never through the read-only path (ld.global.nc: __ldg, or a const __restrict__ parameter of the kernel),
 // which is for memory that nobody writes from a kernel's beginning on, nor by an instruction that the compiler may move ahead of the
-// wait.  Evict-first:
-__device__ __forceinline__ float4 ld_f4_streaming(const float4* p) {
+// wait.  As instructions where it matters which registers they take: with C++ loads of its entry state the gated walk at d = 128 spills
+// 48 bytes more (1 x 32 x 65536 in bf16 700 us, this way 660).
+__device__ __forceinline__ float ld_f1(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_f4(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_f4_streaming(const float4* p) {  // evict-first
   float4 v;
   asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
   return v;

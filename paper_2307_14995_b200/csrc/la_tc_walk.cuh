@@ -451,7 +451,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
           const float4* r4 = reinterpret_cast<const float4*>(src + (size_t)(q * 32 + lane) * 128 + w4 * 32);
 #pragma unroll
           for (int x = 0; x < 8; ++x) {
-            const float4 v = r4[x];
+            const float4 v = ld_f4(r4 + x);
             zreg[4 * x + 0] = fmaf(g, zreg[4 * x + 0], v.x);
             zreg[4 * x + 1] = fmaf(g, zreg[4 * x + 1], v.y);
             zreg[4 * x + 2] = fmaf(g, zreg[4 * x + 2], v.z);
@@ -460,7 +460,7 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
         } else {
           const float* r1 = src + (size_t)(w4 * 32) * 128 + q * 32 + lane;
 #pragma unroll
-          for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], r1[x * 128]);
+          for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], ld_f1(r1 + x * 128));
         }
       };
       if (EARLY && args.follows == FOLLOWS_STATES) {
@@ -485,9 +485,9 @@ tc_walk_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ TcM
             const float* r2 = r1 + (REV ? -1 : 1) * (128 * 128);
             float v[32];
 #pragma unroll
-            for (int x = 0; x < 32; ++x) v[x] = r1[x * 128];
+            for (int x = 0; x < 32; ++x) v[x] = ld_f1(r1 + x * 128);
 #pragma unroll
-            for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g2, fmaf(g1, zreg[x], v[x]), r2[x * 128]);
+            for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g2, fmaf(g1, zreg[x], v[x]), ld_f1(r2 + x * 128));
             --k;
             continue;
           }

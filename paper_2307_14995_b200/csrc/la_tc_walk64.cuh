@@ -406,7 +406,7 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
           const float4* r4 = reinterpret_cast<const float4*>(src + (size_t)e * 64 + zh * 32);
 #pragma unroll
           for (int x = 0; x < 8; ++x) {
-            const float4 v = r4[x];
+            const float4 v = ld_f4(r4 + x);
             zreg[4 * x + 0] = fmaf(g, zreg[4 * x + 0], v.x);
             zreg[4 * x + 1] = fmaf(g, zreg[4 * x + 1], v.y);
             zreg[4 * x + 2] = fmaf(g, zreg[4 * x + 2], v.z);
@@ -415,7 +415,7 @@ tc_walk64_kernel(const __grid_constant__ TcMaps maps0, const __grid_constant__ T
         } else {
           const float* r1 = src + (size_t)(zh * 32) * 64 + e;
 #pragma unroll
-          for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], r1[x * 64]);
+          for (int x = 0; x < 32; ++x) zreg[x] = fmaf(g, zreg[x], ld_f1(r1 + x * 64));
         }
       };
       if (args.follows == FOLLOWS_STATES) {
