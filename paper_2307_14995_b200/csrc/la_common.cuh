@@ -199,7 +199,7 @@ cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
 // come in several waves or run for long a launch's end matters less, and held at the power limit the step is slower for it: 1 x 32
 // heads x 65536, 288 thread blocks a walk, 2333 us with launches one after the other and 2368 with early ones; 1 x 16 x 51521, 144
 // thread blocks of 45 blocks, 920 and 932; 128 thread blocks: 1 x 32 x 16384, 32 blocks each, 639 and 634; 2 x 16 x 8192, 16 blocks,
-// 333 and 320.
+// 333 and 320 (all on one box, in turn; runs of one side differ by half a percent).
 inline bool early_walks(int bh, int nseg, int seg_len) { return (long)bh * nseg <= 148 && seg_len <= 4096; }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // ... and loads come behind it: never through the read-only path (ld.global.nc: __ldg, or a const __restrict__ parameter of the kernel),
