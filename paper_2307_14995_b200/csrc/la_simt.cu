@@ -482,16 +482,19 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
   for (int n = threadIdx.x; n <= L; n += ROWS_THREADS * G) sm.dtab[n] = decay_pow_d(s2, (double)n);
   __syncthreads();
 
+  // The tiles of the entry state, after the others: one group at d = 128 takes them in a loop of their own (16 heads x 2048 tokens
+  // forward 260 us in one loop, 253 this way; one group at d = 64 103.6 and 106.2).
+  constexpr bool APART = D == 128 && G == 1;
   int items = count;
   if (!state) {
     // leave out the tiles whose every weight is zero in fp32, and add those of the entry state
     items = 1;
     while (items < count && sm.dtab[(items - 1) * C + 1] != 0.f) ++items;
     count = items;
-    if (Z && sm.dtab[rev ? max(L - tile * C - C, 0) : tile * C + 1] != 0.f) items += D / C;
+    if (!APART && Z && sm.dtab[rev ? max(L - tile * C - C, 0) : tile * C + 1] != 0.f) items += D / C;
   }
   const auto fetch = [&](int n) {
-    if (n < count) fetch_pair(n);
+    if (APART || n < count) fetch_pair(n);
     else fetch_tile<float, D>(nc, Z + (size_t)(n - count) * C * D, D, C, tid);
   };
   if (grp >= count && grp < items) fetch(grp);
@@ -504,8 +507,28 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
 #pragma unroll
     for (int m = 0; m < EM; ++m) acc[r][m] = 0.f;
 
+  const auto accumulate = [&]() {
+    // acc += w^T t over 32 rows; a thread has rows i4 .. i4 + 3 and columns e0 .. e0 + 3 (d = 128: and 64 + those)
+#pragma unroll 4
+    for (int j = 0; j < C; ++j) {
+      const float4 w = *reinterpret_cast<const float4*>(&gm.w[j][i4]);
+      const float wr[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int g = 0; g < EM / 4; ++g) {
+        const float4 t = *reinterpret_cast<const float4*>(&gm.t[j][e0 + 64 * g]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          acc[r][4 * g + 0] = fmaf(wr[r], t.x, acc[r][4 * g + 0]);
+          acc[r][4 * g + 1] = fmaf(wr[r], t.y, acc[r][4 * g + 1]);
+          acc[r][4 * g + 2] = fmaf(wr[r], t.z, acc[r][4 * g + 2]);
+          acc[r][4 * g + 3] = fmaf(wr[r], t.w, acc[r][4 * g + 3]);
+        }
+      }
+    }
+  };
+
   for (int n = grp; n < items; n += G) {
-    const bool pair = n < count;  // else 32 rows of the entry state
+    const bool pair = APART || n < count;  // else 32 rows of the entry state
     const int jt = first + n * dir;
     if (pair) put_tile<D, D + 4>(gm.b, nb, tid);
     put_tile<D, D>(gm.t, nc, tid);
@@ -559,24 +582,22 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
         }
     }
     group_sync<G>(grp);
-    // acc += w^T t over 32 rows; a thread has rows i4 .. i4 + 3 and columns e0 .. e0 + 3 (d = 128: and 64 + those)
-#pragma unroll 4
-    for (int j = 0; j < C; ++j) {
-      const float4 w = *reinterpret_cast<const float4*>(&gm.w[j][i4]);
-      const float wr[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int g = 0; g < EM / 4; ++g) {
-        const float4 t = *reinterpret_cast<const float4*>(&gm.t[j][e0 + 64 * g]);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          acc[r][4 * g + 0] = fmaf(wr[r], t.x, acc[r][4 * g + 0]);
-          acc[r][4 * g + 1] = fmaf(wr[r], t.y, acc[r][4 * g + 1]);
-          acc[r][4 * g + 2] = fmaf(wr[r], t.z, acc[r][4 * g + 2]);
-          acc[r][4 * g + 3] = fmaf(wr[r], t.w, acc[r][4 * g + 3]);
-        }
-      }
-    }
+    accumulate();
     group_sync<G>(grp);
+  }
+  if (APART && !state && Z && sm.dtab[rev ? max(L - tile * C - C, 0) : tile * C + 1] != 0.f) {
+    for (int k0 = 0; k0 < D; k0 += C) {
+      fetch_tile<float, D>(nc, Z + (size_t)k0 * D, D, C, tid);
+      put_tile<D, D>(gm.t, nc, tid);
+      for (int x = tid; x < C * C; x += ROWS_THREADS) {
+        const int k = x / C, i = x % C;
+        const int dist = rev ? L - 1 - (tile * C + i) : tile * C + i + 1;
+        gm.w[k][i] = dist >= 0 && dist <= L ? sm.a[i][k0 + k] * sm.dtab[dist] : 0.f;
+      }
+      __syncthreads();
+      accumulate();
+      __syncthreads();
+    }
   }
   if (G > 1) {
     // the groups' sums, in order, through their own tiles
@@ -627,11 +648,39 @@ simt_rows_kernel(const __grid_constant__ RowsArgs all, const __grid_constant__ D
   }
 }
 
+// Whether a launch's tiles are shared out over groups.  With groups one thread block has a multiprocessor to itself (its registers),
+// with one group four run at d = 64 and three at d = 128, but each ends sooner: the more tiles its rows add up, the more thread blocks a
+// launch may have.  Measured, us, one group and four at d = 64: 37 heads x 512 (592 thread blocks, 16 tiles) 59 and 36, 64 x 512 (1024)
+// 63 and 58, 75 x 512 (1200) 66 and 69, 90 x 200 (630, 7 tiles) 32.5 and 30.8, 90 x 300 (900, 10 tiles) 43 and 47, 140 x 128 (560, 4
+// tiles) 22.5 and 24.3, 200 x 64 (400, 2 tiles) 12.4 and 15.9; one (two thread blocks to a multiprocessor, see rows_two_at_a_time) and
+// two at d = 128: 19 x 500 (304) 70 and 50, 55 x 512 (880) 90 and 81, 64 x 512 (1024) 88 and 95, 50 x 300 (500, 10 tiles) 54 and 42, 70 x
+// 300 (700) 56 and 58, 90 x 300 (900) 65 and 72, 60 x 200 (420, 7 tiles) 37 and 33, 90 x 200 (630) 43 and 47, 70 x 160 (350, 5 tiles) 29 and
+// 26, 100 x 150 (500) 33 and 36; a backward pass's three walks at d = 128: 19 x 500 (912) 111 and 100, 30 x 300 (900) 84 and 76, 70 x 160
+// (1050, 5 tiles) 64 and 70.  Short segments of a longer sequence, and states: 592 and 296.
+inline bool rows_shared(int d, const RowsArgs& ra) {
+  const int blocks = ra.first_block[ROWS_MAX_JOBS], tiles = ra.units[0] ? (ra.job[0].seg_len + C - 1) / C : 0;
+  if (tiles >= 5 && d == 64) return blocks <= 300 + 55 * tiles;
+  if (tiles >= 5) return blocks <= (ra.units[1] ? 550 + 40 * tiles : 200 + 44 * tiles);
+  if (d == 64 && tiles > 0 && ra.job[0].nseg == 1) return blocks <= (tiles == 4 ? 444 : 296);
+  return blocks <= (d == 64 ? 592 : 296);
+}
+// d = 128, one group, one walk of one segment: where a multiprocessor has two or three thread blocks' worth of rows, two at a time end
+// before three do, whose longest rows wait for one another.  us, three and two: 100 heads x 128 (400 thread blocks, 4 tiles) 31 and 27, 125 x
+// 128 (500) 33 and 28, 140 x 128 (560) 31 and 33, 75 x 512 (1200, 16 tiles) 108 and 99, 100 x 300 (1000, 10 tiles) 72 and 72, 100 x 400
+// (1300, 13 tiles) 94 and 101, 200 x 160 (1000, 5 tiles) 53 and 59.
+inline bool rows_two_at_a_time(const RowsArgs& ra) {
+  if (!ra.units[0] || ra.units[1] || ra.job[0].nseg > 1) return false;
+  const int blocks = ra.first_block[ROWS_MAX_JOBS], tiles = (ra.job[0].seg_len + C - 1) / C;
+  return tiles >= 5 ? blocks <= 400 + 55 * tiles : blocks < 140 * tiles;
+}
 template <typename TIn, typename TOut, int D, int G>
 cudaError_t launch_rows_g(const RowsArgs& ra, const DecayTable& tab, cudaStream_t stream) {
-  const size_t smem = sizeof(RowsSmem<D, G>);
+  constexpr size_t OWN = sizeof(RowsSmem<D, G>), TWO = 80 * 1024;  // (of TWO a multiprocessor has no room for three)
+  constexpr bool CHOICE = D == 128 && G == 1;
+  const size_t smem = CHOICE && rows_two_at_a_time(ra) ? TWO : OWN;
   auto kern = simt_rows_kernel<TIn, TOut, D, G>;
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (the same limit from every thread that launches)
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(CHOICE ? TWO : OWN));
   if (err != cudaSuccess) return err;
   KernelTimer timer(ra.units[0] ? K_WALK : K_PREPASS, stream);
   // One walk of one segment by one group, all thread blocks at once: placed while the launch before still drains, long tiles come to
@@ -641,19 +690,6 @@ cudaError_t launch_rows_g(const RowsArgs& ra, const DecayTable& tab, cudaStream_
   err = launch_kernel(early, kern, dim3((unsigned)ra.first_block[ROWS_MAX_JOBS]), dim3(ROWS_THREADS * G), smem, stream, 1, ra, tab);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
-}
-// Whether a launch's tiles are shared out over groups.  With groups one thread block has a multiprocessor to itself (its registers),
-// with one group four run at d = 64 and three at d = 128, but each ends sooner: the more tiles its rows add up, the more thread blocks a
-// launch may have.  Measured, us, one group and four at d = 64: 37 heads x 512 (592 thread blocks, 16 tiles)
-// 59 and 36, 64 x 512 (1024) 63 and 58, 75 x 512 (1200) 66 and 69, 90 x 200 (630, 7 tiles) 32.5 and 30.8, 90 x 300 (900, 10 tiles) 43
-// and 47, 140 x 128 (560, 4 tiles) 22.5 and 24.3, 200 x 64 (400, 2 tiles) 12.4 and 15.9; one and two at d = 128: 19 x 500 (304) 92 and
-// 50, 37 x 512 (592) 93 and 56, 64 x 512 (1024) 106 and 95, 75 x 512 (1200) 112 and 112, 64 x 300 (640, 10 tiles) 68 and 54, 100 x 300
-// (1000) 74 and 82, 300 x 64 (600, 2 tiles) 25 and 31.  Short segments of a longer sequence, and states, as before: 592 and 296.
-inline bool rows_shared(int d, const RowsArgs& ra) {
-  const int blocks = ra.first_block[ROWS_MAX_JOBS], tiles = ra.units[0] ? (ra.job[0].seg_len + C - 1) / C : 0;
-  if (tiles >= 5) return blocks <= (d == 64 ? 350 + 50 * tiles : 550 + 40 * tiles);
-  if (d == 64 && tiles > 0 && ra.job[0].nseg == 1) return blocks <= (tiles == 4 ? 444 : 296);
-  return blocks <= (d == 64 ? 592 : 296);
 }
 template <typename TIn, typename TOut, int D>
 cudaError_t launch_rows_t(const RowsArgs& ra, const DecayTable& tab, cudaStream_t stream) {

@@ -212,7 +212,8 @@ def test_full_precision_tiles_shared_by_groups_or_not(B, H, N, d):
 
 
 @pytest.mark.parametrize("B,H,N,d", [
-    (1, 25, 400, 128), (1, 8, 300, 128), (2, 32, 512, 128), (1, 75, 512, 128), (4, 25, 128, 128), (5, 30, 64, 128),  # one group or two
+    (1, 25, 400, 128), (1, 8, 300, 128), (2, 32, 512, 128), (1, 75, 512, 128), (4, 25, 128, 128), (5, 30, 64, 128),  # one group or two,
+    (5, 28, 128, 128), (1, 90, 300, 128), (1, 55, 512, 128), (2, 50, 160, 128),                                      # two at a time
     (1, 45, 512, 64), (1, 19, 500, 64), (1, 90, 300, 64), (1, 70, 300, 64), (5, 28, 128, 64), (4, 50, 64, 64)])      # one or four
 def test_full_precision_groups_by_the_tiles_of_a_row(B, H, N, d):
     """On both sides of where a launch's tiles are shared out, by how many a row adds up.  Tolerance as above: at most 640 products."""
